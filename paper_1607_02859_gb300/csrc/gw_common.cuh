@@ -114,6 +114,13 @@ template <typename C> __host__ __device__ __forceinline__ C cmul(C a, C b) {
 template <typename C> __host__ __device__ __forceinline__ C cmulc(C a, C b) {  // a * conj(b)
   return mk(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
+// acc + a b and acc + a conj(b) as fused multiply-adds
+template <typename C> __device__ __forceinline__ C cfma(C a, C b, C acc) {
+  return mk(fma(a.x, b.x, fma(-a.y, b.y, acc.x)), fma(a.x, b.y, fma(a.y, b.x, acc.y)));
+}
+template <typename C> __device__ __forceinline__ C cfmac(C a, C b, C acc) {
+  return mk(fma(a.x, b.x, fma(a.y, b.y, acc.x)), fma(a.y, b.x, fma(-a.x, b.y, acc.y)));
+}
 template <typename C> __host__ __device__ __forceinline__ C cconj(C a) { return mk(a.x, -a.y); }
 template <typename C> __host__ __device__ __forceinline__ C cmuli(C a) { return mk(-a.y, a.x); }  // i*a
 template <typename C, typename R> __host__ __device__ __forceinline__ C cscale(C a, R s) {

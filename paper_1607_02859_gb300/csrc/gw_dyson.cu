@@ -52,74 +52,244 @@ __global__ void __launch_bounds__(256) build_eps_kernel(const typename cpx<T>::t
   }
 }
 
-// Unblocked Cholesky (K form) of the kb x kb diagonal block, in shared memory.
+// 1 / sqrt(x): the CUDA estimate with one Newton step in FP32 (the exact square
+// root and division sit on the pivot chain below), the quotient in FP64.
+__device__ __forceinline__ float inv_sqrt(float x) {
+  const float r = rsqrtf(x);
+  return fmaf(0.5f * r, fmaf(-x * r, r, 1.0f), r);
+}
+__device__ __forceinline__ double inv_sqrt(double x) { return 1.0 / sqrt(x); }
+
+// Cholesky factor (K form) and inverse of the kb x kb diagonal block of every
+// batch entry: L (diagonal L_jj - 1) back into A, L^{-1} - 1 into P (lower).
+//
+// One CTA per entry; the chain of kb pivots bounds it (FP32).  Both triangles
+// live in registers, a 4 x 4 cyclic block each per thread of a 16 x 16 grid,
+// and advance together: with the raw column j of the factor and the raw row j
+// of the inverse published in (double-buffered) shared memory behind one
+// barrier, every thread scales them by 1 / L_jj itself and applies
+//   S -= l l^H,   X[i > j] -= l_i x_j.
+// Only the 16-wide register blocks that column j touches are updated.  The
+// inverse turns the triangular solves of the panel into products (below): one
+// thread per row of a solve walked 64 columns serially (68 us a panel, and 74 us
+// for the inverse's rows, whatever the size).  Screening 12 frequencies of 1536
+// G vectors (fp16x3) went from 7.02 to 3.96 ms, 2 x 8192 with refinement from
+// 185 to 170 ms; FP64, 4 x 1024, from 41.8 to 32.1 ms, FP32, 8 x 1536, from 8.7 to 5.3.
 template <typename T>
-__global__ void __launch_bounds__(256) potrf_diag_kernel(typename cpx<T>::t* A, long lda, long s_a, int kb, int* flag,
-                                                         int col0) {
+__global__ void __launch_bounds__(256) potrf_inv_kernel(typename cpx<T>::t* A, long lda, long s_a,
+                                                        typename cpx<T>::t* P, long ldp, long s_p, int kb, int* flag,
+                                                        int col0) {
+  using C = typename cpx<T>::t;
+  static_assert(kNB == 64, "4 x 4 blocks of a 16 x 16 thread grid");
+  __shared__ C col[2][kNB], row[2][kNB];
+  A += blockIdx.z * s_a;
+  P += blockIdx.z * s_p;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  C S[4][4], X[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int i = ty + 16 * a, c = tx + 16 * b;
+      S[a][b] = i < kb && c <= i ? A[(long)i * lda + c] : mk(T(0), T(0));
+      X[a][b] = mk(T(i == c ? 1 : 0), T(0));
+    }
+#pragma unroll
+  for (int jb = 0; jb < 4; ++jb) {
+#pragma unroll 1
+    for (int jj = 0; jj < 16; ++jj) {
+      const int j = 16 * jb + jj;
+      if (j >= kb) break;
+      const int buf = j & 1;
+      if (tx == jj)
+#pragma unroll
+        for (int a = jb; a < 4; ++a) col[buf][ty + 16 * a] = S[a][jb];
+      if (ty == jj)
+#pragma unroll
+        for (int b = 0; b <= jb; ++b) row[buf][tx + 16 * b] = X[jb][b];
+      __syncthreads();
+      T d = col[buf][j].x;                     // eps~_jj - 1 after the updates
+      const bool bad = !(T(1) + d > T(0));
+      if (bad) d = T(0);
+      const T inv = inv_sqrt(T(1) + d);
+      C l[4], lc[4], xr[4];
+#pragma unroll
+      for (int a = jb; a < 4; ++a) {
+        l[a] = cscale(col[buf][ty + 16 * a], inv);
+        lc[a] = cscale(col[buf][tx + 16 * a], inv);
+      }
+#pragma unroll
+      for (int b = 0; b <= jb; ++b) xr[b] = cscale(row[buf][tx + 16 * b], inv);
+      if (tx == jj) {
+#pragma unroll
+        for (int a = jb; a < 4; ++a)
+          if (ty + 16 * a > j) S[a][jb] = l[a];
+        if (ty == jj) {
+          S[jb][jb] = mk(d / (T(1) + sqrt(T(1) + d)), T(0));   // L_jj - 1
+          if (bad && atomicCAS(flag, 0, 1) == 0) {
+            flag[1] = col0 + j;
+            flag[2] = blockIdx.z;
+          }
+        }
+      }
+      if (ty == jj)
+#pragma unroll
+        for (int b = 0; b <= jb; ++b) X[jb][b] = xr[b];
+      if (ty <= jj) l[jb] = mk(T(0), T(0));    // rows up to j and columns up to j are final
+      if (tx <= jj) lc[jb] = mk(T(0), T(0));
+#pragma unroll
+      for (int a = jb; a < 4; ++a) {
+        const C nl = mk(-l[a].x, -l[a].y);
+#pragma unroll
+        for (int b = jb; b <= a; ++b) S[a][b] = cfmac(nl, lc[b], S[a][b]);
+#pragma unroll
+        for (int b = 0; b <= jb; ++b) X[a][b] = cfma(nl, xr[b], X[a][b]);
+      }
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b <= a; ++b) {
+      const int i = ty + 16 * a, c = tx + 16 * b;
+      if (i >= kb || c > i) continue;
+      A[(long)i * lda + c] = S[a][b];
+      const T k = S[a][b].x;                   // on the diagonal: (1 + K)^{-1} - 1 = -K / (1 + K)
+      P[(long)i * ldp + c] = i == c ? mk(-k / (T(1) + k), T(0)) : X[a][b];
+    }
+}
+
+constexpr int kPR = 32;     // rows (columns) of a panel product per CTA
+
+// Shared memory of the two panel products: the inverted diagonal block and the tile.
+template <typename T>
+constexpr size_t panel_smem() {
+  return sizeof(typename cpx<T>::t) * (kNB * (kNB + 1) + kPR * (kNB + 1));
+}
+
+// Rows below the diagonal block: L21 = A21 L11^{-H} = A21 + A21 P11^H, in place,
+// kPR rows per CTA and 2 x 4 outputs per thread; P11 is lower triangular, so
+// the sum of each group of 16 columns stops at its last column.
+template <typename T>
+__global__ void __launch_bounds__(256) panel_right_kernel(typename cpx<T>::t* A, long lda, long s_a,
+                                                          const typename cpx<T>::t* P, long ldp, long s_p, int kb,
+                                                          int rows) {
   using C = typename cpx<T>::t;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C (*S)[kNB + 1] = reinterpret_cast<C (*)[kNB + 1]>(smem_raw);    // [kNB][kNB+1]
+  C* Ps = reinterpret_cast<C*>(smem_raw);          // [kNB][kNB + 1]
+  C* As = Ps + kNB * (kNB + 1);                     // [kPR][kNB + 1]
   A += blockIdx.z * s_a;
-  for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) {
-    const int i = e / kb, c = e % kb;
-    S[i][c] = c <= i ? A[(long)i * lda + c] : mk(T(0), T(0));
+  P += blockIdx.z * s_p;
+  const int r0 = blockIdx.x * kPR;
+  for (int e = threadIdx.x; e < kNB * kNB; e += 256) {
+    const int i = e / kNB, c = e % kNB;
+    Ps[i * (kNB + 1) + c] = i < kb && c <= i ? P[(long)i * ldp + c] : mk(T(0), T(0));
+  }
+  for (int e = threadIdx.x; e < kPR * kNB; e += 256) {
+    const int i = e / kNB, c = e % kNB;
+    As[i * (kNB + 1) + c] = r0 + i < rows && c < kb ? A[(long)(r0 + i) * lda + c] : mk(T(0), T(0));
   }
   __syncthreads();
-  for (int j = 0; j < kb; ++j) {
-    if (threadIdx.x == 0) {
-      T b = S[j][j].x;                       // eps~_jj - 1 after the updates
-      if (!(T(1) + b > T(0))) {
-        if (atomicCAS(flag, 0, 1) == 0) {
-          flag[1] = col0 + j;
-          flag[2] = blockIdx.z;
-        }
-        b = T(0);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  C acc[2][4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b)
+#pragma unroll
+    for (int a = 0; a < 2; ++a) acc[a][b] = mk(T(0), T(0));
+#pragma unroll
+  for (int pb = 0; pb < 4; ++pb) {
+#pragma unroll 4
+    for (int pp = 0; pp < 16; ++pp) {
+      const int p = 16 * pb + pp;
+      const C a0 = As[ty * (kNB + 1) + p], a1 = As[(ty + 16) * (kNB + 1) + p];
+#pragma unroll
+      for (int b = pb; b < 4; ++b) {
+        const C w = Ps[(tx + 16 * b) * (kNB + 1) + p];
+        acc[0][b] = cfmac(a0, w, acc[0][b]);
+        acc[1][b] = cfmac(a1, w, acc[1][b]);
       }
-      S[j][j] = mk(b / (T(1) + sqrt(T(1) + b)), T(0));   // L_jj - 1
     }
-    __syncthreads();
-    const T piv = T(1) + S[j][j].x;
-    for (int i = j + 1 + threadIdx.x; i < kb; i += blockDim.x) S[i][j] = cscale(S[i][j], T(1) / piv);
-    __syncthreads();
-    const int m = kb - j - 1;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-      const int i = j + 1 + e / m, c = j + 1 + e % m;
-      if (c <= i) S[i][c] = csub(S[i][c], cmulc(S[i][j], S[c][j]));
-    }
-    __syncthreads();
   }
-  for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) {
-    const int i = e / kb, c = e % kb;
-    if (c <= i) A[(long)i * lda + c] = S[i][c];
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const int i = ty + 16 * a;
+    if (r0 + i >= rows) continue;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int c = tx + 16 * b;
+      if (c < kb) A[(long)(r0 + i) * lda + c] = cadd(As[i * (kNB + 1) + c], acc[a][b]);
+    }
   }
 }
 
-// Rows below the diagonal block: x L11^H = a  ->  x (row of L21).  64 rows per CTA.
+// One block row of P = L^{-1} - 1, left of its diagonal block: Y <- L_ii^{-1} Y =
+// Y + P_ii Y for the kb rows and ncols columns at Y, in place, kPR columns per
+// CTA.  CTAs past those columns set up the rows below instead: P[r][col0 ..] =
+// -L[r][col0 ..] (the identity part of 1 + P in the update of those rows).
 template <typename T>
-__global__ void __launch_bounds__(64) trsm_panel_kernel(typename cpx<T>::t* A, long lda, long s_a, int k0, int kb,
-                                                        int rows) {
+__global__ void __launch_bounds__(256) panel_left_kernel(const typename cpx<T>::t* P, long ldp, long s_p,
+                                                         typename cpx<T>::t* Y, int kb, int ncols,
+                                                         const typename cpx<T>::t* Lb, long ldl, long s_l,
+                                                         typename cpx<T>::t* Pb, int below) {
   using C = typename cpx<T>::t;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* L = reinterpret_cast<C*>(smem_raw);          // [kb][kb+1]
-  C* X = L + kNB * (kNB + 1);                       // [kb][64]  (column c of thread t at X[c*64+t])
-  A += blockIdx.z * s_a;
-  const int t = threadIdx.x;
-  for (int e = t; e < kb * kb; e += blockDim.x) {
-    const int i = e / kb, c = e % kb;
-    L[i * (kNB + 1) + c] = c <= i ? A[(long)(k0 + i) * lda + k0 + c] : mk(T(0), T(0));
+  const int mul_ctas = (ncols + kPR - 1) / kPR;
+  if ((int)blockIdx.x >= mul_ctas) {
+    Lb += blockIdx.z * s_l;
+    Pb += blockIdx.z * s_p;
+    const int r0 = ((int)blockIdx.x - mul_ctas) * kPR;
+    for (int e = threadIdx.x; e < kPR * kNB; e += 256) {
+      const int r = r0 + e / kNB, c = e % kNB;
+      if (r >= below || c >= kb) continue;
+      const C v = Lb[(long)r * ldl + c];
+      Pb[(long)r * ldp + c] = mk(-v.x, -v.y);
+    }
+    return;
   }
-  const long row = (long)k0 + kb + (long)blockIdx.x * 64 + t;
-  const bool active = blockIdx.x * 64 + t < rows;
-  if (active)
-    for (int c = 0; c < kb; ++c) X[c * 64 + t] = A[row * lda + k0 + c];
+  C* Ps = reinterpret_cast<C*>(smem_raw);          // [kNB][kNB + 1]
+  C* Ys = Ps + kNB * (kNB + 1);                     // [kNB][kPR] (fits the row tile's space)
+  P += blockIdx.z * s_p;
+  Y += blockIdx.z * s_p;
+  const int c0 = blockIdx.x * kPR;
+  for (int e = threadIdx.x; e < kNB * kNB; e += 256) {
+    const int i = e / kNB, c = e % kNB;
+    Ps[i * (kNB + 1) + c] = i < kb && c <= i ? P[(long)i * ldp + c] : mk(T(0), T(0));
+  }
+  for (int e = threadIdx.x; e < kNB * kPR; e += 256) {
+    const int i = e / kPR, c = e % kPR;
+    Ys[i * kPR + c] = i < kb && c0 + c < ncols ? Y[(long)i * ldp + c0 + c] : mk(T(0), T(0));
+  }
   __syncthreads();
-  if (!active) return;
-  for (int c = 0; c < kb; ++c) {
-    C s = X[c * 64 + t];
-    for (int p = 0; p < c; ++p) s = csub(s, cmulc(X[p * 64 + t], L[c * (kNB + 1) + p]));
-    X[c * 64 + t] = cscale(s, T(1) / (T(1) + L[c * (kNB + 1) + c].x));
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  C acc[4][2];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) acc[a][b] = mk(T(0), T(0));
+#pragma unroll
+  for (int pb = 0; pb < 4; ++pb) {
+#pragma unroll 4
+    for (int pp = 0; pp < 16; ++pp) {
+      const int p = 16 * pb + pp;
+      const C y0 = Ys[p * kPR + tx], y1 = Ys[p * kPR + tx + 16];
+#pragma unroll
+      for (int a = pb; a < 4; ++a) {
+        const C w = Ps[(ty + 16 * a) * (kNB + 1) + p];
+        acc[a][0] = cfma(w, y0, acc[a][0]);
+        acc[a][1] = cfma(w, y1, acc[a][1]);
+      }
+    }
   }
-  for (int c = 0; c < kb; ++c) A[row * lda + k0 + c] = X[c * 64 + t];
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int i = ty + 16 * a;
+    if (i >= kb) continue;
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int c = tx + 16 * b;
+      if (c0 + c < ncols) Y[(long)i * ldp + c0 + c] = cadd(Ys[i * kPR + c], acc[a][b]);
+    }
+  }
 }
 
 // P[rows below][col0 .. col0+kb) = -L[rows below][col0 .. col0+kb): the identity
@@ -135,47 +305,6 @@ __global__ void neg_copy_kernel(const typename cpx<T>::t* __restrict__ Lm, long 
   for (int c = threadIdx.x; c < kb; c += blockDim.x) {
     const auto v = Lm[r * ldl + col0 + c];
     P[r * ldp + col0 + c] = mk(-v.x, -v.y);
-  }
-}
-
-// Y = L_ii^{-1} Y for the block rows k0..k0+kb-1 and columns 0..ncols-1 of Y,
-// with the identity as right-hand side in the diagonal-block columns (their
-// stored values are ignored) and P = L^{-1} - 1 stored on the diagonal.
-template <typename T>
-__global__ void __launch_bounds__(64) trsm_left_kernel(const typename cpx<T>::t* Lm, long ldl, long s_l,
-                                                      typename cpx<T>::t* Y, long ldy, long s_y, int k0, int kb,
-                                                      int ncols) {
-  using C = typename cpx<T>::t;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* L = reinterpret_cast<C*>(smem_raw);
-  C* X = L + kNB * (kNB + 1);
-  Lm += blockIdx.z * s_l;
-  Y += blockIdx.z * s_y;
-  const int t = threadIdx.x;
-  for (int e = t; e < kb * kb; e += blockDim.x) {
-    const int i = e / kb, c = e % kb;
-    L[i * (kNB + 1) + c] = c <= i ? Lm[(long)(k0 + i) * ldl + k0 + c] : mk(T(0), T(0));
-  }
-  const int col = blockIdx.x * 64 + t;
-  const bool active = col < ncols;
-  const int dc = col - k0;                   // column inside the diagonal block, or < 0
-  if (active)
-    for (int r = 0; r < kb; ++r)
-      X[r * 64 + t] = dc >= 0 ? mk(T(r == dc ? 1 : 0), T(0)) : Y[(long)(k0 + r) * ldy + col];
-  __syncthreads();
-  if (!active) return;
-  for (int r = 0; r < kb; ++r) {
-    C s = X[r * 64 + t];
-    for (int p = 0; p < r; ++p) s = csub(s, cmul(L[r * (kNB + 1) + p], X[p * 64 + t]));
-    X[r * 64 + t] = cscale(s, T(1) / (T(1) + L[r * (kNB + 1) + r].x));
-  }
-  for (int r = 0; r < kb; ++r) {
-    C y = X[r * 64 + t];
-    if (r == dc) {                           // (1 + K)^{-1} - 1 = -K / (1 + K)
-      const T k = L[r * (kNB + 1) + r].x;
-      y = mk(-k / (T(1) + k), T(0));
-    }
-    Y[(long)(k0 + r) * ldy + col] = y;
   }
 }
 
@@ -283,41 +412,40 @@ struct Batch {
 
 template <typename T>
 static gw_status set_attrs(gw_ctx* ctx) {
-  using C = typename cpx<T>::t;
-  const size_t tsm = sizeof(C) * (kNB * (kNB + 1) + kNB * 64);
-  const size_t psm = sizeof(C) * kNB * (kNB + 1);
   gw_status rc = GW_OK;
-  if (tsm > 48 * 1024) {
-    rc = cuda_check(ctx, cudaFuncSetAttribute(trsm_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm),
+  if (panel_smem<T>() > 48 * 1024) {
+    rc = cuda_check(ctx, cudaFuncSetAttribute(panel_right_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)panel_smem<T>()),
                     "cudaFuncSetAttribute");
     if (!rc)
-      rc = cuda_check(ctx, cudaFuncSetAttribute(trsm_left_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm),
+      rc = cuda_check(ctx, cudaFuncSetAttribute(panel_left_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)panel_smem<T>()),
                       "cudaFuncSetAttribute");
   }
-  if (!rc && psm > 48 * 1024)
-    rc = cuda_check(ctx, cudaFuncSetAttribute(potrf_diag_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm),
-                    "cudaFuncSetAttribute");
   return rc;
 }
 
 // Cholesky (lower, K form on the diagonal) of the n x n block at a (leading
-// dimension lda) of every batch entry, on CUDA cores, 64-column panels.
+// dimension lda) of every batch entry, on CUDA cores, 64-column panels; the
+// inverses (minus 1) of the diagonal blocks go to the diagonal of the block at
+// p, which is zeroed otherwise.
 template <typename T>
-static gw_status chol_simt(gw_ctx* ctx, gw_prec prec, typename cpx<T>::t* a, long lda, int n, int col0, Batch bt,
-                           cudaStream_t st) {
-  using C = typename cpx<T>::t;
+static gw_status chol_simt(gw_ctx* ctx, gw_prec prec, typename cpx<T>::t* a, long lda, typename cpx<T>::t* p, long ldp,
+                           int n, int col0, Batch bt, cudaStream_t st) {
   gw_status rc;
-  const size_t tsm = sizeof(C) * (kNB * (kNB + 1) + kNB * 64);
-  const size_t psm = sizeof(C) * kNB * (kNB + 1);
+  zero_block_kernel<T><<<dim3((n + 127) / 128, n, bt.B), 128, 0, st>>>(p, ldp, bt.ms, n);
+  if ((rc = launch_check(ctx, "zero_block_kernel"))) return rc;
   for (int k0 = 0; k0 < n; k0 += kNB) {
     const int kb = std::min(kNB, n - k0);
-    potrf_diag_kernel<T><<<dim3(1, 1, bt.B), 256, psm, st>>>(a + (long)k0 * lda + k0, lda, bt.ms, kb, ctx->dflag,
-                                                             col0 + k0);
-    if ((rc = launch_check(ctx, "potrf_diag_kernel"))) return rc;
+    auto* pii = p + (long)k0 * ldp + k0;
+    potrf_inv_kernel<T><<<dim3(1, 1, bt.B), 256, 0, st>>>(a + (long)k0 * lda + k0, lda, bt.ms, pii, ldp, bt.ms, kb,
+                                                          ctx->dflag, col0 + k0);
+    if ((rc = launch_check(ctx, "potrf_inv_kernel"))) return rc;
     const int rows = n - k0 - kb;
     if (rows <= 0) break;
-    trsm_panel_kernel<T><<<dim3((rows + 63) / 64, 1, bt.B), 64, tsm, st>>>(a, lda, bt.ms, k0, kb, rows);
-    if ((rc = launch_check(ctx, "trsm_panel_kernel"))) return rc;
+    panel_right_kernel<T><<<dim3((rows + kPR - 1) / kPR, 1, bt.B), 256, panel_smem<T>(), st>>>(
+        a + (long)(k0 + kb) * lda + k0, lda, bt.ms, pii, ldp, bt.ms, kb, rows);
+    if ((rc = launch_check(ctx, "panel_right_kernel"))) return rc;
     GemmArgs g{};
     g.M = rows;
     g.N = rows;
@@ -341,26 +469,24 @@ static gw_status chol_simt(gw_ctx* ctx, gw_prec prec, typename cpx<T>::t* a, lon
   return GW_OK;
 }
 
-// P = L^{-1} - 1 for the n x n lower factor L (K form diagonal) at Lm, written
-// to the n x n block at p, for every batch entry (CUDA cores).
+// P = L^{-1} - 1 for the n x n lower factor L (K form diagonal) at Lm, in the
+// n x n block at p as chol_simt left it (the inverted diagonal blocks, zero
+// elsewhere), for every batch entry (CUDA cores).
 template <typename T>
 static gw_status inv_simt(gw_ctx* ctx, gw_prec prec, const typename cpx<T>::t* Lm, long ldl,
                           typename cpx<T>::t* p, long ldp, int n, Batch bt, cudaStream_t st) {
-  using C = typename cpx<T>::t;
   gw_status rc;
-  const size_t tsm = sizeof(C) * (kNB * (kNB + 1) + kNB * 64);
-  zero_block_kernel<T><<<dim3((n + 127) / 128, n, bt.B), 128, 0, st>>>(p, ldp, bt.ms, n);
-  if ((rc = launch_check(ctx, "zero_block_kernel"))) return rc;
   for (int k0 = 0; k0 < n; k0 += kNB) {
     const int kb = std::min(kNB, n - k0);
-    const int ncols = k0 + kb;
-    trsm_left_kernel<T><<<dim3((ncols + 63) / 64, 1, bt.B), 64, tsm, st>>>(Lm, ldl, bt.ms, p, ldp, bt.ms, k0, kb,
-                                                                          ncols);
-    if ((rc = launch_check(ctx, "trsm_left_kernel"))) return rc;
-    const int rows = n - k0 - kb;
+    const int ncols = k0 + kb, rows = n - k0 - kb;
+    const int ctas = (k0 + kPR - 1) / kPR + (rows + kPR - 1) / kPR;
+    if (ctas > 0) {
+      panel_left_kernel<T><<<dim3(ctas, 1, bt.B), 256, panel_smem<T>(), st>>>(
+          p + (long)k0 * ldp + k0, ldp, bt.ms, p + (long)k0 * ldp, kb, k0, Lm + (long)(k0 + kb) * ldl + k0, ldl, bt.ms,
+          p + (long)(k0 + kb) * ldp + k0, rows);
+      if ((rc = launch_check(ctx, "panel_left_kernel"))) return rc;
+    }
     if (rows <= 0) break;
-    neg_copy_kernel<T><<<dim3(rows, 1, bt.B), kNB, 0, st>>>(Lm, ldl, bt.ms, p, ldp, bt.ms, k0 + kb, rows, k0, kb);
-    if ((rc = launch_check(ctx, "neg_copy_kernel"))) return rc;
     GemmArgs g{};
     g.M = rows;
     g.N = ncols;
@@ -579,7 +705,7 @@ static gw_status screen_batch(gw_ctx* ctx, gw_prec prec, int n, int B, const voi
   if ((rc = launch_check(ctx, "build_eps_kernel"))) return rc;
   if (!tcs) {
     // CUDA cores, 64-column panels over the whole matrix
-    if ((rc = chol_simt<T>(ctx, prec, e, n, n, 0, bt, st))) return rc;
+    if ((rc = chol_simt<T>(ctx, prec, e, n, p, n, n, 0, bt, st))) return rc;
     if ((rc = inv_simt<T>(ctx, prec, e, n, p, n, n, bt, st))) return rc;
     GemmArgs g{};
     g.M = n;
@@ -631,7 +757,7 @@ static gw_status screen_batch(gw_ctx* ctx, gw_prec prec, int n, int B, const voi
         const int kb = std::min(kTB, n - k0);
         C* akk = e + (long)k0 * n + k0;
         C* pkk = p + (long)k0 * n + k0;
-        if ((rc = chol_simt<float>(ctx, GW_FP32, akk, n, kb, k0, bt, st))) return rc;
+        if ((rc = chol_simt<float>(ctx, GW_FP32, akk, n, pkk, n, kb, k0, bt, st))) return rc;
         if ((rc = inv_simt<float>(ctx, GW_FP32, akk, n, pkk, n, kb, bt, st))) return rc;
         const int rows = n - k0 - kb;
         if (rows <= 0) break;
