@@ -83,21 +83,35 @@ __global__ void __launch_bounds__(256) stripe_chi_kernel(const typename cpx<T>::
   }
 }
 
-// slab[r][q*n_chi + j] *= exp(sgn i q.r)
+// exp(i q.r) for every cell point r and every q: tab[r][q].  One table per call
+// instead of the FP64 trigonometry in every thread of q_phase_kernel: at a 12^3
+// cell on 2x2x2 with 509 G vectors the phase pass of one tau was bound by the
+// FP64 pipe (580 us); reading the table it moves its 2 x 56 MB.
 template <typename T>
-__global__ void __launch_bounds__(256) q_phase_kernel(typename cpx<T>::t* slab, long ld, int n_chi, int n1, int n2,
-                                                      int n3, int nk1, int nk2, int nk3, double sgn) {
-  const long r = blockIdx.x;
-  const int i1 = (int)(r / (n2 * n3)), rem = (int)(r - (long)i1 * n2 * n3), i2 = rem / n3, i3 = rem - i2 * n3;
+__global__ void __launch_bounds__(128) q_phase_table_kernel(typename cpx<T>::t* __restrict__ tab, int nr, int n1,
+                                                            int n2, int n3, int nk1, int nk2, int nk3) {
   const int n_k = nk1 * nk2 * nk3;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= nr * n_k) return;
+  const int r = e / n_k, q = e - r * n_k;
+  const int i1 = r / (n2 * n3), rem = r - i1 * n2 * n3, i2 = rem / n3, i3 = rem - i2 * n3;
+  const int q1 = q / (nk2 * nk3), qr = q - q1 * nk2 * nk3, q2 = qr / nk3, q3 = qr - q2 * nk3;
+  // q.r / 2 pi = sum_d q_d i_d / (nk_d n_d), reduced mod 1 before the trigonometry
+  double f = (double)q1 * i1 / (nk1 * n1) + (double)q2 * i2 / (nk2 * n2) + (double)q3 * i3 / (nk3 * n3);
+  f -= floor(f);
+  double s, c;
+  sincospi(2.0 * f, &s, &c);
+  tab[e] = mk(T(c), T(s));
+}
+
+// slab[r][q*n_chi + j] *= exp(sgn i q.r), the phases from q_phase_table_kernel
+template <typename T>
+__global__ void __launch_bounds__(256) q_phase_kernel(typename cpx<T>::t* slab, long ld, int n_chi, int n_k,
+                                                      const typename cpx<T>::t* __restrict__ tab, T sgn) {
+  const long r = blockIdx.x;
   for (int q = blockIdx.y; q < n_k; q += gridDim.y) {
-    const int q1 = q / (nk2 * nk3), qr = q - q1 * nk2 * nk3, q2 = qr / nk3, q3 = qr - q2 * nk3;
-    // q.r / 2 pi = sum_d q_d i_d / (nk_d n_d), reduced mod 1 before the trigonometry
-    double f = (double)q1 * i1 / (nk1 * n1) + (double)q2 * i2 / (nk2 * n2) + (double)q3 * i3 / (nk3 * n3);
-    f -= floor(f);
-    double s, c;
-    sincospi(2.0 * sgn * f, &s, &c);
-    const T cr = T(c), ci = T(s);
+    const auto ph = tab[r * n_k + q];
+    const T cr = ph.x, ci = sgn * ph.y;
     auto* p = slab + r * ld + (long)q * n_chi;
     for (int j = threadIdx.x; j < n_chi; j += blockDim.x) {
       const auto v = p[j];
@@ -245,14 +259,24 @@ static gw_status launch_stripe(gw_ctx* ctx, gw_prec prec, const GridInfo& g, con
   return go(stripe_chi_kernel<float, PRODUCT>, (float2*)nullptr);
 }
 
-static gw_status launch_q_phase(gw_ctx* ctx, gw_prec prec, const GridInfo& g, const int* nk, void* slab, long ld,
-                                int n_chi, double sgn, cudaStream_t s) {
+// The phase table of a call: N_r N_k complex numbers at tab.
+static gw_status fill_q_phases(gw_ctx* ctx, gw_prec prec, const GridInfo& g, const int* nk, void* tab, cudaStream_t s) {
+  const int blocks = (g.nr * nk[0] * nk[1] * nk[2] + 127) / 128;
+  if (is_fp64(prec))
+    q_phase_table_kernel<double><<<blocks, 128, 0, s>>>((double2*)tab, g.nr, g.n1, g.n2, g.n3, nk[0], nk[1], nk[2]);
+  else
+    q_phase_table_kernel<float><<<blocks, 128, 0, s>>>((float2*)tab, g.nr, g.n1, g.n2, g.n3, nk[0], nk[1], nk[2]);
+  return launch_check(ctx, "q_phase_table_kernel");
+}
+
+static gw_status launch_q_phase(gw_ctx* ctx, gw_prec prec, const GridInfo& g, const int* nk, const void* tab,
+                                void* slab, long ld, int n_chi, double sgn, cudaStream_t s) {
   const int n_k = nk[0] * nk[1] * nk[2];
   const dim3 gq(g.nr, std::min(n_k, 8));
   if (is_fp64(prec))
-    q_phase_kernel<double><<<gq, 256, 0, s>>>((double2*)slab, ld, n_chi, g.n1, g.n2, g.n3, nk[0], nk[1], nk[2], sgn);
+    q_phase_kernel<double><<<gq, 256, 0, s>>>((double2*)slab, ld, n_chi, n_k, (const double2*)tab, sgn);
   else
-    q_phase_kernel<float><<<gq, 256, 0, s>>>((float2*)slab, ld, n_chi, g.n1, g.n2, g.n3, nk[0], nk[1], nk[2], sgn);
+    q_phase_kernel<float><<<gq, 256, 0, s>>>((float2*)slab, ld, n_chi, n_k, (const float2*)tab, (float)sgn);
   return launch_check(ctx, "q_phase_kernel");
 }
 
@@ -293,6 +317,7 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   probe.take<double>((size_t)n_k * n_b);
   probe.take<double>((size_t)n * n);
   probe.take<double2>((size_t)n_k * n_k);
+  probe.take<char>((size_t)g.nr * n_k * es);
   probe.take<char>(slab * n * es);
   probe.take<char>((size_t)n_k * rb * g.nr * es);
   probe.take<char>((size_t)n_k * rb * g.nr * es);
@@ -308,6 +333,7 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   char* dscale = cv.take<char>((size_t)n_k * n_b * 8);
   char* dcw = cv.take<char>((size_t)n * n * 8);
   char* dph = cv.take<char>((size_t)n_k * n_k * 16);
+  char* dqph = cv.take<char>((size_t)g.nr * n_k * es);
   char* slabs = cv.take<char>(slab * n * es);
   char* gok = cv.take<char>((size_t)n_k * rb * g.nr * es);
   char* guk = cv.take<char>((size_t)n_k * rb * g.nr * es);
@@ -319,6 +345,7 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   if ((st = upload(ctx, dsmap, smap.data(), sizeof(int) * n_k * n_chi, s))) return st;
   if ((st = upload(ctx, dsinv, sinv.data(), sizeof(int) * gs.nr, s))) return st;
   if ((st = upload_phases(ctx, dph, kl_phases(nk), prec, s))) return st;
+  if ((st = fill_q_phases(ctx, prec, g, nk, dqph, s))) return st;
   const double fac = g.dv * g.dv / g.volume;   // Eq. FFTX2 normalisation
   std::vector<float> cw32;
   if (is_fp64(prec)) {
@@ -354,7 +381,7 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
                                n_k * n_chi, rows, 1.0, s, dsinv, tmp_s)))
         return st;
     }
-    if ((st = launch_q_phase(ctx, prec, g, nk, slab_j, ld, n_chi, -1.0, s))) return st;
+    if ((st = launch_q_phase(ctx, prec, g, nk, dqph, slab_j, ld, n_chi, -1.0, s))) return st;
     if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, ld, (int)ld, 1.0, s))) return st;
   }
   for (int q = 0; q < n_k; ++q) {
@@ -437,6 +464,7 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
   probe.take<char>((size_t)n_k * n_b * 8);
   probe.take<char>((size_t)n * n * 8);
   probe.take<double>(2 * (size_t)n_b);
+  probe.take<char>((size_t)g.nr * n_k * es);
   probe.take<char>(slab * n * es);
   probe.take<char>((size_t)n_b * g.nr * es);
   probe.take<char>((size_t)n_k * n_b * n_pw * es);
@@ -456,6 +484,7 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
   char* dscale = cv.take<char>((size_t)n_k * n_b * 8);
   char* dcw = cv.take<char>((size_t)n * n * 8);
   double* dnorm = cv.take<double>(2 * (size_t)n_b);
+  char* dqph = cv.take<char>((size_t)g.nr * n_k * es);
   char* slabs = cv.take<char>(slab * n * es);
   char* u = cv.take<char>((size_t)n_b * g.nr * es);
   char* dc = cv.take<char>((size_t)n_k * n_b * n_pw * es);
@@ -480,6 +509,7 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
     cw32 = split_weights(C_h, n * n, fac);
     if ((st = upload(ctx, dcw, cw32.data(), sizeof(float) * 2 * n * n, s))) return st;
   }
+  if ((st = fill_q_phases(ctx, prec, g, nk, dqph, s))) return st;
   // the coefficients of u_ak over the set for every k (checked to span every band)
   for (int k = 0; k < n_k; ++k) {
     const int kv[3] = {k / (nk[1] * nk[2]), (k / nk[2]) % nk[1], k % nk[2]};
@@ -516,13 +546,13 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
       }
     }
     // exp(-i k.r) on the block of each k, then per row: expand, multiply, transform onto {q + g}
-    if ((st = launch_q_phase(ctx, prec, g, nk, to, ldt, n_pw, -1.0, s))) return st;
-    if ((st = launch_q_phase(ctx, prec, g, nk, tu, ldt, n_pw, -1.0, s))) return st;
+    if ((st = launch_q_phase(ctx, prec, g, nk, dqph, to, ldt, n_pw, -1.0, s))) return st;
+    if ((st = launch_q_phase(ctx, prec, g, nk, dqph, tu, ldt, n_pw, -1.0, s))) return st;
     char* slab_j = slabs + (size_t)j * slab * es;
     if ((st = launch_row_pw_chi(ctx, gs, prec, tu, to, ldt, slab_j, ld, dinv_pws, n_pws, dsinv, n_chis, g.nr,
                                 row_scale, s)))
       return st;
-    if ((st = launch_q_phase(ctx, prec, g, nk, slab_j, ld, n_chi, -1.0, s))) return st;
+    if ((st = launch_q_phase(ctx, prec, g, nk, dqph, slab_j, ld, n_chi, -1.0, s))) return st;
     if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, ld, (int)ld, 1.0, s))) return st;
   }
   for (int q = 0; q < n_k; ++q) {
@@ -586,6 +616,7 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   probe.take<int>(3 * (size_t)n_n);
   probe.take<double>((size_t)n_k * n_b);
   probe.take<double2>((size_t)n_k * n_k);
+  probe.take<char>((size_t)g.nr * n_k * es);
   probe.take<double>(2 * (size_t)n * n + n + nreal1);
   probe.take<double>(2 * (size_t)n_n * n);
   probe.take<double2>((size_t)n_n * (n + nreal1));
@@ -606,6 +637,7 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   int* dbid = dbk + 2 * n_n;
   char* dscale = cv.take<char>((size_t)n_k * n_b * 8);
   char* dph = cv.take<char>((size_t)n_k * n_k * 16);
+  char* dqph = cv.take<char>((size_t)g.nr * n_k * es);
   double* tab = cv.take<double>(2 * (size_t)n * n + n + nreal1);
   double* acc = cv.take<double>(2 * (size_t)n_n * n);
   double2* out = cv.take<double2>((size_t)n_n * (n + nreal1));
@@ -628,6 +660,7 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   for (int i = 0; i < n_n; ++i) bk[2 * n_n + i] = i;
   if ((st = upload(ctx, dbk, bk.data(), sizeof(int) * 3 * n_n, s))) return st;
   if ((st = upload_phases(ctx, dph, kl_phases(nk), prec, s))) return st;
+  if ((st = fill_q_phases(ctx, prec, g, nk, dqph, s))) return st;
   if ((st = upload(ctx, tab, C_h, sizeof(double) * n * n, s))) return st;
   if ((st = upload(ctx, tab + (size_t)n * n, S_h, sizeof(double) * n * n, s))) return st;
   if ((st = upload(ctx, tab + 2 * (size_t)n * n, omega_h, sizeof(double) * n, s))) return st;
@@ -660,7 +693,7 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
       if ((st = launch_col_line(ctx, g, prec, +1, 1, wq, n_chi, blk, ld, n_chi, dinv, 1.0, s))) return st;
       if ((st = launch_col_plane(ctx, g, prec, +1, blk, ld, n_chi, 1.0, s))) return st;
     }
-    if ((st = launch_q_phase(ctx, prec, g, nk, wrg, ld, n_chi, +1.0, s))) return st;
+    if ((st = launch_q_phase(ctx, prec, g, nk, dqph, wrg, ld, n_chi, +1.0, s))) return st;
     for (int r0 = 0; r0 < g.nr; r0 += rb) {
       const int rows = std::min(rb, g.nr - r0);
       for (int k = 0; k < n_k; ++k) {
