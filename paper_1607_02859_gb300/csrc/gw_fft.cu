@@ -32,23 +32,87 @@ bool grid_supported(int a, int b, int c) {
   return false;
 }
 
+// What of the grid a G set touches, behind its inverse map on the device (set_lists):
+// the (i2, i3) columns and (i1, i2) pencils that hold a point of the set, and the
+// values of each axis that do.  A cutoff sphere of n_chi points touches far fewer
+// than all: at 36^3 with n_chi = 8192, 489 of 1296 columns and 25 of 36 values.
+template <int N1, int N2, int N3>
+struct SetLists {
+  int n23, n12, n1, n2, n3;
+  const int *l23, *l12, *l1, *l2, *l3;
+  __device__ __forceinline__ explicit SetLists(const int* __restrict__ inv) {
+    const int* x = inv + N1 * N2 * N3;
+    n23 = __ldg(x);
+    n12 = __ldg(x + 1);
+    n1 = __ldg(x + 2);
+    n2 = __ldg(x + 3);
+    n3 = __ldg(x + 4);
+    l23 = x + kSetHead;
+    l12 = l23 + N2 * N3;
+    l1 = l12 + N1 * N2;
+    l2 = l1 + N1;
+    l3 = l2 + N2;
+  }
+};
+
+// Rows of a Hermitian matrix x(r, R') of which only R' <= r is used: the row kernels
+// take the grid index low of the launch's first row (-1: whole rows).
+// Forward: elements past r are taken as zero without being read (the tensor-core
+// chi pass does not write them).  Backward: the columns that the fused self-energy
+// reads, i.e. up to the end of the 128-column tile that holds the diagonal of the
+// row's 128-row tile; the rest of the row is not written.
+__device__ __forceinline__ int low_last_fwd(int low, long row, int nr) {
+  return low < 0 ? nr - 1 : low + (int)row;
+}
+__device__ __forceinline__ int low_last_bwd(int low, long row, int nr) {
+  if (low < 0) return nr - 1;
+  const int g0 = low + ((int)row & ~127);
+  return min(nr - 1, (g0 + 127) / 128 * 128 + 127);
+}
+
+// Threads and CTAs per SM of the one-CTA rows: two rounds of pencils (N1 N2 per
+// pass) for the larger grids, so that the registers of two or three CTAs fit an SM
+// and one row's loads overlap another's arithmetic.  FP64 is bound by its ALU.
+template <typename T, int N1, int N2, int N3>
+struct RowCfg {
+  static constexpr int PC = N1 * N2;
+  static constexpr bool F32 = sizeof(T) == 4;
+  static constexpr int NR = N1 * N2 * N3;
+  static constexpr int TH = F32 ? (NR >= 4096 ? ((PC / 2 + 31) / 32 * 32 < 64 ? 64 : (PC / 2 + 31) / 32 * 32)
+                                              : ((PC + 31) / 32 * 32))
+                                : (NR >= 4096 ? 512 : 256);
+  static constexpr int MINB = F32 ? (NR >= 13824 ? 2 : (NR >= 4096 ? 3 : 4)) : 1;
+};
+
 // MODE 0: x = scale * a * conj(b) (Eq. chi_rr), forward (+i), gather the G' set.
 // MODE 1: x = a, forward (+i), gather.            (Eq. FFTX1)
 // MODE 2: scatter a[j] to fft positions, backward (-i), times scale.   (Eq. FFTW, 2nd step)
-// VEC: rows 16-byte aligned with even lengths; contiguous rows move as pairs of
-// elements, four pairs in flight per thread.
-template <typename T, int N1, int N2, int N3, int MODE, int THREADS, bool VEC>
-__global__ void __launch_bounds__(THREADS) row_fft_kernel(const typename cpx<T>::t* __restrict__ a,
-                                                          const typename cpx<T>::t* __restrict__ b, long lda,
-                                                          typename cpx<T>::t* __restrict__ out, long ldo,
-                                                          const int* __restrict__ map, int n_chi, T scale) {
+// VI / VO: the grid side / the G-set side (modes 0, 1) moves as 16-byte pairs of
+// elements (aligned rows of even length), four pairs in flight per thread.
+//
+// The three passes over the row do only what the G set (lists) and the triangle
+// (low) need: forward the planes i1 <= i1(r), of them the i3 of the set in the i2
+// pass, and the set's (i2, i3) columns in the i1 pass; backward the set's (i1, i2)
+// pencils, then its i1 planes, and of the i1 pass the planes up to the last one
+// read.  A MODE 0 row of the triangle takes half of its diagonal element.
+// That is 0.44 of a whole row's pencils at 24^3 with n_chi = 4097; the rows of one
+// tau went from 790 to 560 us there (scalar loads for the odd n_chi before), from
+// 250 to 172 us at 20^3 with n_chi = 1536.  Bound by instruction issue.
+template <typename T, int N1, int N2, int N3, int MODE, bool VI, bool VO>
+__global__ void __launch_bounds__(RowCfg<T, N1, N2, N3>::TH, RowCfg<T, N1, N2, N3>::MINB)
+    row_fft_kernel(const typename cpx<T>::t* __restrict__ a, const typename cpx<T>::t* __restrict__ b, long lda,
+                   typename cpx<T>::t* __restrict__ out, long ldo, const int* __restrict__ map,
+                   const int* __restrict__ inv, int n_chi, T scale, int low) {
   using C = typename cpx<T>::t;
   using L = RowLayout<N1, N2, N3>;
-  constexpr int NP = L::NR / 2;
+  constexpr int THREADS = RowCfg<T, N1, N2, N3>::TH;
+  constexpr int PL = N2 * N3;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* s = reinterpret_cast<C*>(smem_raw);
   const long row = blockIdx.x;
-  if (MODE == 2) {
+  const SetLists<N1, N2, N3> g(inv);
+  if constexpr (MODE == 2) {
+    const int i1m = low_last_bwd(low, row, L::NR) / PL + 1;      // planes to deliver
     for (int e = threadIdx.x; e < L::TOT; e += THREADS) s[e] = mk(T(0), T(0));
     __syncthreads();
     const C* src = a + row * lda;
@@ -67,56 +131,130 @@ __global__ void __launch_bounds__(THREADS) row_fft_kernel(const typename cpx<T>:
       for (int u = 0; u < 4; ++u)
         if (j0 + u * THREADS < n_chi) s[L::pos(m[u])] = v[u];
     }
-  } else {
-    const C* pa = a + row * lda;
-    const C* pb = b + row * lda;
-    if (VEC) {
-      for (int q0 = threadIdx.x; q0 < NP; q0 += 4 * THREADS) {
-        C v[4][2], w[4][2];
+    __syncthreads();
+    for (int e = threadIdx.x; e < g.n12; e += THREADS) {
+      const int o = __ldg(g.l12 + e) * L::S2;
+      C x[N3];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int q = q0 + u * THREADS;
-          if (q < NP) {
-            ld_pair(pa + 2 * q, v[u][0], v[u][1]);
-            if (MODE == 0) ld_pair(pb + 2 * q, w[u][0], w[u][1]);
-          }
-        }
+      for (int k = 0; k < N3; ++k) x[k] = s[o + k];
+      RegFFT<N3, -1>::run(x);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int q = q0 + u * THREADS;
-          if (q >= NP) continue;
-          const int p = L::pos(2 * q);           // 2q and 2q+1 share an i3 pencil (N3 even)
-          s[p] = MODE == 0 ? cscale(cmulc(v[u][0], w[u][0]), scale) : v[u][0];
-          s[p + 1] = MODE == 0 ? cscale(cmulc(v[u][1], w[u][1]), scale) : v[u][1];
-        }
-      }
-    } else {
-      for (int r = threadIdx.x; r < L::NR; r += THREADS) {
-        C v = pa[r];
-        if (MODE == 0) v = cscale(cmulc(v, pb[r]), scale);
-        s[L::pos(r)] = v;
-      }
+      for (int k = 0; k < N3; ++k) s[o + k] = x[k];
     }
-  }
-  __syncthreads();
-  fft3_smem<N1, N2, N3, MODE == 2 ? -1 : +1>(s);
-  C* dst = out + row * ldo;
-  if (MODE == 2) {
-    if (VEC) {
-      for (int q = threadIdx.x; q < NP; q += THREADS) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < g.n1 * N3; e += THREADS) {
+      const int o = __ldg(g.l1 + e / N3) * L::S1 + e % N3;
+      C x[N2];
+#pragma unroll
+      for (int k = 0; k < N2; ++k) x[k] = s[o + k * L::S2];
+      RegFFT<N2, -1>::run(x);
+#pragma unroll
+      for (int k = 0; k < N2; ++k) s[o + k * L::S2] = x[k];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < PL; e += THREADS) {
+      const int o = e / N3 * L::S2 + e % N3;
+      C x[N1];
+#pragma unroll
+      for (int k = 0; k < N1; ++k) x[k] = s[o + k * L::S1];
+      RegFFT<N1, -1>::run(x);
+#pragma unroll
+      for (int k = 0; k < N1; ++k)
+        if (k < i1m) s[o + k * L::S1] = x[k];
+    }
+    __syncthreads();
+    C* dst = out + row * ldo;
+    if (VI) {
+      for (int q = threadIdx.x; q < i1m * PL / 2; q += THREADS) {
         const int p = L::pos(2 * q);
         st_pair(dst + 2 * q, cscale(s[p], scale), cscale(s[p + 1], scale));
       }
     } else {
-      for (int r = threadIdx.x; r < L::NR; r += THREADS) dst[r] = cscale(s[L::pos(r)], scale);
+      for (int r = threadIdx.x; r < i1m * PL; r += THREADS) dst[r] = cscale(s[L::pos(r)], scale);
+    }
+    return;
+  }
+  const int last = low_last_fwd(low, row, L::NR);
+  const int i1m = last / PL + 1;                                 // planes with an element R' <= r
+  const int half = MODE == 0 && low >= 0 ? last : -1;
+  const C* pa = a + row * lda;
+  const C* pb = b + row * lda;
+  auto value = [&](C v, C w, int r) -> C {
+    if (r > last) return mk(T(0), T(0));
+    if (MODE != 0) return v;
+    return cscale(cmulc(v, w), r == half ? scale * T(0.5) : scale);
+  };
+  if (VI) {
+    const int np = i1m * PL / 2;
+    for (int q0 = threadIdx.x; q0 < np; q0 += 4 * THREADS) {
+      C v[4][2], w[4][2];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int q = q0 + u * THREADS;
+        v[u][0] = v[u][1] = w[u][0] = w[u][1] = mk(T(0), T(0));
+        if (q < np && 2 * q <= last) {
+          ld_pair(pa + 2 * q, v[u][0], v[u][1]);
+          if (MODE == 0) ld_pair(pb + 2 * q, w[u][0], w[u][1]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int q = q0 + u * THREADS;
+        if (q >= np) continue;
+        const int p = L::pos(2 * q);           // 2q and 2q+1 share an i3 pencil (N3 even)
+        s[p] = value(v[u][0], w[u][0], 2 * q);
+        s[p + 1] = value(v[u][1], w[u][1], 2 * q + 1);
+      }
     }
   } else {
-    if (VEC) {
-      for (int q = threadIdx.x; q < n_chi / 2; q += THREADS)
-        st_pair(dst + 2 * q, s[L::pos(map[2 * q])], s[L::pos(map[2 * q + 1])]);
-    } else {
-      for (int j = threadIdx.x; j < n_chi; j += THREADS) dst[j] = s[L::pos(map[j])];
+    for (int r = threadIdx.x; r < i1m * PL; r += THREADS) {
+      C v = mk(T(0), T(0)), w = v;
+      if (r <= last) {
+        v = pa[r];
+        if (MODE == 0) w = pb[r];
+      }
+      s[L::pos(r)] = value(v, w, r);
     }
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < i1m * N2; e += THREADS) {
+    const int o = e * L::S2;
+    C x[N3];
+#pragma unroll
+    for (int k = 0; k < N3; ++k) x[k] = s[o + k];
+    RegFFT<N3, +1>::run(x);
+#pragma unroll
+    for (int k = 0; k < N3; ++k) s[o + k] = x[k];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < i1m * g.n3; e += THREADS) {
+    const int i1 = e / g.n3;
+    const int o = i1 * L::S1 + __ldg(g.l3 + (e - i1 * g.n3));
+    C x[N2];
+#pragma unroll
+    for (int k = 0; k < N2; ++k) x[k] = s[o + k * L::S2];
+    RegFFT<N2, +1>::run(x);
+#pragma unroll
+    for (int k = 0; k < N2; ++k) s[o + k * L::S2] = x[k];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < g.n23; e += THREADS) {
+    const int c = __ldg(g.l23 + e);
+    const int o = c / N3 * L::S2 + c % N3;
+    C x[N1];
+#pragma unroll
+    for (int k = 0; k < N1; ++k) x[k] = k < i1m ? s[o + k * L::S1] : mk(T(0), T(0));
+    RegFFT<N1, +1>::run(x);
+#pragma unroll
+    for (int k = 0; k < N1; ++k) s[o + k * L::S1] = x[k];
+  }
+  __syncthreads();
+  C* dst = out + row * ldo;
+  if (VO) {
+    for (int q = threadIdx.x; q < n_chi / 2; q += THREADS)
+      st_pair(dst + 2 * q, s[L::pos(map[2 * q])], s[L::pos(map[2 * q + 1])]);
+  } else {
+    for (int j = threadIdx.x; j < n_chi; j += THREADS) dst[j] = s[L::pos(map[j])];
   }
 }
 
@@ -219,21 +357,21 @@ __global__ void __launch_bounds__(256) row_line_bwd_kernel(const typename cpx<T>
 }
 
 // Rows too long for one CTA's shared memory, split over a thread-block cluster
-// of CL CTAs: CTA c holds planes i1 in [c P, (c+1) P) (P = N1 / CL) of the row
-// and the slice [c n_s, (c+1) n_s) of its G-set side (n_s = ceil(n_chi / CL)).
-// The (i2, i3) transforms run on the CTA's own planes; for the i1 transforms
-// each CTA takes N2 N3 / CL of the (i2, i3) columns and reads and writes the
-// other CTAs' planes and G-set slices through distributed shared memory.  Each
-// element crosses HBM once, as for the one-CTA rows.
+// of CL CTAs: CTA c holds the planes i1 = c, c + CL, ... of the row (so that every
+// CTA has its share of the planes i1 <= i1(r) of a triangle's row) and the slice
+// [c n_s, (c+1) n_s) of its G-set side (n_s = ceil(n_chi / CL)).  The (i2, i3)
+// transforms run on the CTA's own planes; the i1 transforms of the set's
+// (i2, i3) columns are dealt out over the CTAs, which read and write the other
+// CTAs' planes and G-set slices through distributed shared memory.  Each element
+// crosses HBM once, as for the one-CTA rows, and the passes skip what the G set
+// and the triangle do not need in the same way.
 template <typename T, int N1, int N2, int N3>
 struct ClusterRow {
   using C = typename cpx<T>::t;
   static constexpr int S2 = N3 % 2 == 0 ? N3 + 1 : N3;
   static constexpr int PL = N2 * N3;
   static constexpr size_t plane_bytes(int cl) { return (size_t)(N1 / cl) * N2 * S2 * sizeof(C); }
-  static constexpr bool fits(int cl) {
-    return N1 % cl == 0 && PL % cl == 0 && plane_bytes(cl) + 32768 <= 200 * 1024;
-  }
+  static constexpr bool fits(int cl) { return N1 % cl == 0 && plane_bytes(cl) + 32768 <= 200 * 1024; }
   // the smallest cluster whose planes leave room for two CTAs per SM, else the smallest that fits
   static constexpr int pick() {
     for (int cl : {2, 4, 8})
@@ -244,51 +382,53 @@ struct ClusterRow {
   }
   static constexpr int CL = pick();
   static constexpr int P = CL ? N1 / CL : 1;
-  static constexpr int COLS = CL ? PL / CL : 1;
-  // one thread per pencil of the local planes (P N2 = COLS when N2 = N3), two CTAs per SM
-  static constexpr int THREADS = CL ? ((P * N2 > COLS ? P * N2 : COLS) + 1) / 2 : 32;
-  static size_t smem(int n_chi) { return plane_bytes(CL) + (size_t)((n_chi + CL - 1) / CL) * sizeof(C); }
+  // half a thread per pencil of all local planes, rounded to warps
+  static constexpr int THREADS = CL ? (P * N2 / 2 + 31) / 32 * 32 : 32;
+  // planes: local planes that the launch's rows use
+  static size_t smem(int n_chi, int planes) {
+    return (size_t)planes * N2 * S2 * sizeof(C) + (size_t)((n_chi + CL - 1) / CL) * sizeof(C);
+  }
 };
 
-// MODE 0 / 1 / 2 as for row_fft_kernel; grid (CL, rows), clusters of CL along x.
+// MODE 0 / 1 / 2 and low as for row_fft_kernel; grid (CL, rows), clusters of CL
+// along x; planes: the local planes of the largest row of the launch.
 template <typename T, int N1, int N2, int N3, int MODE, bool VEC>
 __global__ void __launch_bounds__(ClusterRow<T, N1, N2, N3>::THREADS, 2)
     row_cluster_kernel(const typename cpx<T>::t* __restrict__ a, const typename cpx<T>::t* __restrict__ b, long lda,
                        typename cpx<T>::t* __restrict__ out, long ldo, const int* __restrict__ inv, int n_chi,
-                       T scale) {
+                       T scale, int low, int planes) {
   namespace cg = cooperative_groups;
   using C = typename cpx<T>::t;
   using R = ClusterRow<T, N1, N2, N3>;
-  constexpr int P = R::P, PL = R::PL, S2 = R::S2, COLS = R::COLS;
+  constexpr int PL = R::PL, S2 = R::S2, CL = R::CL, S1 = N2 * S2;
   constexpr int TH = R::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* s = reinterpret_cast<C*>(smem_raw);                         // [P][N2][S2] own planes
-  C* gs = reinterpret_cast<C*>(smem_raw + R::plane_bytes(R::CL));  // [n_s] own G-set slice
+  C* s = reinterpret_cast<C*>(smem_raw);                         // [planes][N2][S2] own planes
+  C* gs = s + (size_t)planes * S1;                               // [n_s] own G-set slice
   cg::cluster_group cluster = cg::this_cluster();
   const int c = (int)cluster.block_rank();
   const long row = blockIdx.y;
-  const int n_s = (n_chi + R::CL - 1) / R::CL;
+  const SetLists<N1, N2, N3> g(inv);
+  const int n_s = (n_chi + CL - 1) / CL;
   const int j0 = c * n_s, j1 = min(n_chi, j0 + n_s);
-  const long pbase = (long)c * P * PL;                           // the CTA's planes within the row
-  auto plane_pos = [](int e) {
+  const int last = MODE == 2 ? low_last_bwd(low, row, N1 * PL) : low_last_fwd(low, row, N1 * PL);
+  const int i1m = last / PL + 1;                                 // planes in use, of them here:
+  const int nloc = (i1m - c + CL - 1) / CL;                      // (c < CL, so i1m - c + CL - 1 >= 0)
+  const int q0s = g.n23 * c / CL, q1s = g.n23 * (c + 1) / CL;    // the CTA's share of the columns
+  auto plane_pos = [](int e) {                                   // e = p PL + i2 N3 + i3
     const int p = e / PL, rem = e - p * PL, i2 = rem / N3;
-    return (p * N2 + i2) * S2 + (rem - i2 * N3);
+    return p * S1 + i2 * S2 + (rem - i2 * N3);
   };
-  auto planes_2d = [&](auto dir) {
-    constexpr int D = decltype(dir)::value;
-    pencil_pass<N3, D>(s, P * N2, 1, [](int q) { return q * S2; });
-    __syncthreads();
-    pencil_pass<N2, D>(s, P * N3, S2, [](int q) { return (q / N3) * (N2 * S2) + (q % N3); });
-    __syncthreads();
-  };
-  if (MODE == 2) {
+  auto plane_base = [&](int e) { return (long)((e / PL) * CL + c) * PL + e % PL; };   // its place in the row
+  if constexpr (MODE == 2) {
     // the G-set slice, then i1 transforms of the CTA's columns into every CTA's planes
     for (int j = j0 + threadIdx.x; j < j1; j += TH) gs[j - j0] = a[row * lda + j];
+    for (int e = threadIdx.x; e < nloc * S1; e += TH) s[e] = mk(T(0), T(0));
     cluster.sync();
-    for (int q = c * COLS + threadIdx.x; q < (c + 1) * COLS; q += TH) {
-      const int i2 = q / N3, i3 = q - i2 * N3;
+    for (int e = q0s + threadIdx.x; e < q1s; e += TH) {
+      const int q = __ldg(g.l23 + e);
+      const int o23 = q / N3 * S2 + q % N3;
       C x[N1];
-      bool any = false;
 #pragma unroll
       for (int i1 = 0; i1 < N1; ++i1) {
         const int j = __ldg(inv + i1 * PL + q);
@@ -296,75 +436,109 @@ __global__ void __launch_bounds__(ClusterRow<T, N1, N2, N3>::THREADS, 2)
         if (j >= 0) {
           const int o = j / n_s;
           x[i1] = cluster.map_shared_rank(gs, o)[j - o * n_s];
-          any = true;
         }
       }
-      // columns outside the G set's projection are zero and stay zero
-      if (__any_sync(__activemask(), any)) RegFFT<N1, -1>::run(x);
+      RegFFT<N1, -1>::run(x);
 #pragma unroll
-      for (int i1 = 0; i1 < N1; ++i1) cluster.map_shared_rank(s, i1 / P)[((i1 % P) * N2 + i2) * S2 + i3] = x[i1];
+      for (int i1 = 0; i1 < N1; ++i1)
+        if (i1 < i1m) cluster.map_shared_rank(s, i1 % CL)[(i1 / CL) * S1 + o23] = x[i1];
     }
     cluster.sync();                                              // no remote access after this point
-    planes_2d(std::integral_constant<int, -1>{});
-    C* dst = out + row * ldo + pbase;
+    for (int e = threadIdx.x; e < nloc * g.n2; e += TH) {        // pencils outside the set's i2 are zero
+      const int p = e / g.n2;
+      const int o = p * S1 + __ldg(g.l2 + (e - p * g.n2)) * S2;
+      C x[N3];
+#pragma unroll
+      for (int k = 0; k < N3; ++k) x[k] = s[o + k];
+      RegFFT<N3, -1>::run(x);
+#pragma unroll
+      for (int k = 0; k < N3; ++k) s[o + k] = x[k];
+    }
+    __syncthreads();
+    pencil_pass<N2, -1>(s, nloc * N3, S2, [](int q) { return (q / N3) * S1 + (q % N3); });
+    __syncthreads();
+    C* dst = out + row * ldo;
     if (VEC) {
-      for (int q = threadIdx.x; q < P * PL / 2; q += TH) {
+      for (int q = threadIdx.x; q < nloc * PL / 2; q += TH) {
         const int ps = plane_pos(2 * q);
-        st_pair(dst + 2 * q, cscale(s[ps], scale), cscale(s[ps + 1], scale));
+        st_pair(dst + plane_base(2 * q), cscale(s[ps], scale), cscale(s[ps + 1], scale));
       }
     } else {
-      for (int e = threadIdx.x; e < P * PL; e += TH) dst[e] = cscale(s[plane_pos(e)], scale);
+      for (int e = threadIdx.x; e < nloc * PL; e += TH) dst[plane_base(e)] = cscale(s[plane_pos(e)], scale);
     }
     return;
   }
   // forward: the CTA's planes (with the product of Eq. chi_rr for MODE 0) ...
-  const C* pa = a + row * lda + pbase;
-  const C* pb = b + row * lda + pbase;
+  const C* pa = a + row * lda;
+  const C* pb = b + row * lda;
+  const int half = MODE == 0 && low >= 0 ? last : -1;
+  auto value = [&](C v, C w, long r) -> C {
+    if (r > last) return mk(T(0), T(0));
+    if (MODE != 0) return v;
+    return cscale(cmulc(v, w), r == half ? scale * T(0.5) : scale);
+  };
   if (VEC) {
-    constexpr int NP = P * PL / 2;
-    // the row's ~93 KB per CTA arrive in few round trips: LB 16-byte loads in flight per thread
+    const int np = nloc * PL / 2;
+    // the planes arrive in few round trips: LB 16-byte loads in flight per thread
     // (the FFT's registers are free here)
     constexpr int LB = MODE == 0 ? 6 : 12;
-    for (int q0 = threadIdx.x; q0 < NP; q0 += LB * TH) {
+    for (int qb = threadIdx.x; qb < np; qb += LB * TH) {
       C v[LB][2], w[LB][2];
 #pragma unroll
       for (int u = 0; u < LB; ++u) {
-        const int q = q0 + u * TH;
-        if (q < NP) {
-          ld_pair(pa + 2 * q, v[u][0], v[u][1]);
-          if (MODE == 0) ld_pair(pb + 2 * q, w[u][0], w[u][1]);
+        const int q = qb + u * TH;
+        v[u][0] = v[u][1] = w[u][0] = w[u][1] = mk(T(0), T(0));
+        if (q < np) {
+          const long r = plane_base(2 * q);
+          if (r <= last) {
+            ld_pair(pa + r, v[u][0], v[u][1]);
+            if (MODE == 0) ld_pair(pb + r, w[u][0], w[u][1]);
+          }
         }
       }
 #pragma unroll
       for (int u = 0; u < LB; ++u) {
-        const int q = q0 + u * TH;
-        if (q >= NP) continue;
+        const int q = qb + u * TH;
+        if (q >= np) continue;
         const int ps = plane_pos(2 * q);
-        s[ps] = MODE == 0 ? cscale(cmulc(v[u][0], w[u][0]), scale) : v[u][0];
-        s[ps + 1] = MODE == 0 ? cscale(cmulc(v[u][1], w[u][1]), scale) : v[u][1];
+        const long r = plane_base(2 * q);
+        s[ps] = value(v[u][0], w[u][0], r);
+        s[ps + 1] = value(v[u][1], w[u][1], r + 1);
       }
     }
   } else {
-    for (int e = threadIdx.x; e < P * PL; e += TH) {
-      C v = pa[e];
-      if (MODE == 0) v = cscale(cmulc(v, pb[e]), scale);
-      s[plane_pos(e)] = v;
+    for (int e = threadIdx.x; e < nloc * PL; e += TH) {
+      const long r = plane_base(e);
+      C v = mk(T(0), T(0)), w = v;
+      if (r <= last) {
+        v = pa[r];
+        if (MODE == 0) w = pb[r];
+      }
+      s[plane_pos(e)] = value(v, w, r);
     }
   }
   __syncthreads();
-  planes_2d(std::integral_constant<int, +1>{});
+  pencil_pass<N3, +1>(s, nloc * N2, 1, [](int q) { return q * S2; });
+  __syncthreads();
+  for (int e = threadIdx.x; e < nloc * g.n3; e += TH) {
+    const int p = e / g.n3;
+    const int o = p * S1 + __ldg(g.l3 + (e - p * g.n3));
+    C x[N2];
+#pragma unroll
+    for (int k = 0; k < N2; ++k) x[k] = s[o + k * S2];
+    RegFFT<N2, +1>::run(x);
+#pragma unroll
+    for (int k = 0; k < N2; ++k) s[o + k * S2] = x[k];
+  }
   cluster.sync();
   // ... i1 transforms of the CTA's columns, each result scattered to the G-set slice that holds it
-  for (int q = c * COLS + threadIdx.x; q < (c + 1) * COLS; q += TH) {
-    const int i2 = q / N3, i3 = q - i2 * N3;
-    // a column with no G-set point has nothing to deliver: skip it where the whole warp may
-    bool any = false;
-#pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1) any |= __ldg(inv + i1 * PL + q) >= 0;
-    if (!__any_sync(__activemask(), any)) continue;
+  for (int e = q0s + threadIdx.x; e < q1s; e += TH) {
+    const int q = __ldg(g.l23 + e);
+    const int o23 = q / N3 * S2 + q % N3;
     C x[N1];
 #pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1) x[i1] = cluster.map_shared_rank(s, i1 / P)[((i1 % P) * N2 + i2) * S2 + i3];
+    for (int i1 = 0; i1 < N1; ++i1)
+      x[i1] = i1 < i1m ? cluster.map_shared_rank(s, i1 % CL)[(i1 / CL) * S1 + o23] : mk(T(0), T(0));
     RegFFT<N1, +1>::run(x);
 #pragma unroll
     for (int i1 = 0; i1 < N1; ++i1) {
@@ -391,7 +565,10 @@ __global__ void __launch_bounds__(ClusterRow<T, N1, N2, N3>::THREADS, 2)
 // CTAs of a cluster share a row as in row_cluster_kernel (CL = 1: one CTA), with
 // two plane buffers; the slices of the input rows and of the output row share
 // one region (the inputs are read before the first cluster barrier, the output
-// written after the third).
+// written after the third).  chi(r,R') is Hermitian: with low >= 0 only the planes
+// i1 <= i1(r) are expanded, the product is kept for R' <= r with half the
+// diagonal, and the caller adds the conjugate transpose in the end.  The passes
+// visit only the columns and pencils that the two G sets touch.
 template <typename T, int N1, int N2, int N3>
 struct PwRow {
   using C = typename cpx<T>::t;
@@ -412,7 +589,10 @@ struct PwRow {
     const size_t in = 2 * (size_t)((n_pw + CL - 1) / CL), out = (size_t)((n_chi + CL - 1) / CL);
     return in > out ? in : out;
   }
-  static size_t smem(int n_pw, int n_chi) { return 2 * plane_bytes(CL) + slice_elems(n_pw, n_chi) * sizeof(C); }
+  // planes: local planes that the launch's rows use
+  static size_t smem(int n_pw, int n_chi, int planes = P) {
+    return 2 * (size_t)planes * N2 * S2 * sizeof(C) + slice_elems(n_pw, n_chi) * sizeof(C);
+  }
   // row_pw_sigma_kernel: [T_occ | T_unocc | W~] slices in, hu and ho out over the last two
   static size_t sig_smem(int n_pw, int n_chi) {
     const size_t ps = (size_t)((n_pw + CL - 1) / CL), ws = (size_t)((n_chi + CL - 1) / CL);
@@ -425,20 +605,24 @@ template <typename T, int N1, int N2, int N3>
 __global__ void __launch_bounds__(PwRow<T, N1, N2, N3>::THREADS)
     row_pw_chi_kernel(const typename cpx<T>::t* __restrict__ a, const typename cpx<T>::t* __restrict__ b, long lda,
                       typename cpx<T>::t* __restrict__ out, long ldo, const int* __restrict__ inv_pw, int n_pw,
-                      const int* __restrict__ inv_chi, int n_chi, T scale) {
+                      const int* __restrict__ inv_chi, int n_chi, T scale, int low, int planes) {
   namespace cg = cooperative_groups;
   using C = typename cpx<T>::t;
   using R = PwRow<T, N1, N2, N3>;
-  constexpr int P = R::P, PL = R::PL, S2 = R::S2, COLS = R::COLS, CL = R::CL;
+  constexpr int PL = R::PL, S2 = R::S2, CL = R::CL, S1 = N2 * S2;
   constexpr int TH = R::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* sa = reinterpret_cast<C*>(smem_raw);                              // [P][N2][S2] a, then x
-  C* sb = reinterpret_cast<C*>(smem_raw + R::plane_bytes(CL));         // [P][N2][S2] b
-  C* sl = reinterpret_cast<C*>(smem_raw + 2 * R::plane_bytes(CL));     // slices
+  C* sa = reinterpret_cast<C*>(smem_raw);                              // [planes][N2][S2] a, then x
+  C* sb = sa + (size_t)planes * S1;                                    // [planes][N2][S2] b
+  C* sl = sb + (size_t)planes * S1;                                    // slices
   cg::cluster_group cluster = cg::this_cluster();
   const int c = (int)cluster.block_rank();
   const long row = blockIdx.y;
+  const SetLists<N1, N2, N3> gp(inv_pw), gx(inv_chi);
   const int n_ps = (n_pw + CL - 1) / CL, n_cs = (n_chi + CL - 1) / CL;
+  const int last = low_last_fwd(low, row, N1 * PL);
+  const int i1m = last / PL + 1;                // planes in use, dealt out i1 = c, c + CL, ...
+  const int nloc = (i1m - c + CL - 1) / CL;
   C* su = sl;                 // [n_ps] this CTA's part of a's row
   C* so = sl + n_ps;          // [n_ps] of b's row
   {
@@ -447,17 +631,19 @@ __global__ void __launch_bounds__(PwRow<T, N1, N2, N3>::THREADS)
       su[j - j0] = a[row * lda + j];
       so[j - j0] = b[row * lda + j];
     }
+    for (int e = threadIdx.x; e < nloc * S1; e += TH) sa[e] = sb[e] = mk(T(0), T(0));
   }
   cluster.sync();
-  // backward i1 transforms of the CTA's columns, for both rows, into every CTA's planes
-  for (int q = c * COLS + threadIdx.x; q < (c + 1) * COLS; q += TH) {
-    const int i2 = q / N3, i3 = q - i2 * N3;
-#pragma unroll 1
-    for (int which = 0; which < 2; ++which) {
-      C* src = which ? so : su;
-      C* dst = which ? sb : sa;
+  // backward i1 transforms of the CTA's share of the set's columns, for both rows, into every CTA's planes
+  {
+    const int e0 = gp.n23 * c / CL, e1 = gp.n23 * (c + 1) / CL, ne = e1 - e0;
+    for (int t = threadIdx.x; t < 2 * ne; t += TH) {
+      const bool second = t >= ne;
+      const int q = __ldg(gp.l23 + e0 + (second ? t - ne : t));
+      const int o23 = q / N3 * S2 + q % N3;
+      C* src = second ? so : su;
+      C* dst = second ? sb : sa;
       C x[N1];
-      bool any = false;
 #pragma unroll
       for (int i1 = 0; i1 < N1; ++i1) {
         const int j = __ldg(inv_pw + i1 * PL + q);
@@ -465,45 +651,81 @@ __global__ void __launch_bounds__(PwRow<T, N1, N2, N3>::THREADS)
         if (j >= 0) {
           const int o = j / n_ps;
           x[i1] = cluster.map_shared_rank(src, o)[j - o * n_ps];
-          any = true;
         }
       }
-      if (__any_sync(__activemask(), any)) RegFFT<N1, -1>::run(x);   // empty columns stay zero
+      RegFFT<N1, -1>::run(x);
 #pragma unroll
       for (int i1 = 0; i1 < N1; ++i1)
-        cluster.map_shared_rank(dst, i1 / P)[((i1 % P) * N2 + i2) * S2 + i3] = x[i1];
+        if (i1 < i1m) cluster.map_shared_rank(dst, i1 % CL)[(i1 / CL) * S1 + o23] = x[i1];
     }
   }
   cluster.sync();                  // the planes are complete and the input slices free
-  // (i2, i3) backward transforms of the CTA's planes, both rows
-  pencil_pass<N3, -1>(sa, P * N2, 1, [](int q) { return q * S2; });
-  pencil_pass<N3, -1>(sb, P * N2, 1, [](int q) { return q * S2; });
-  __syncthreads();
-  pencil_pass<N2, -1>(sa, P * N3, S2, [](int q) { return (q / N3) * (N2 * S2) + (q % N3); });
-  pencil_pass<N2, -1>(sb, P * N3, S2, [](int q) { return (q / N3) * (N2 * S2) + (q % N3); });
-  __syncthreads();
-  // the product of Eq. chi_rr, then the forward (i2, i3) transforms
-  for (int e = threadIdx.x; e < P * PL; e += TH) {
-    const int p = e / PL, rem = e - p * PL, i2 = rem / N3;
-    const int ps = (p * N2 + i2) * S2 + (rem - i2 * N3);
-    sa[ps] = cscale(cmulc(sa[ps], sb[ps]), scale);
+  // (i2, i3) backward transforms of the CTA's planes, both rows (pencils outside the set's i2 are zero)
+  auto both = [&](int t, int n) { return t >= n ? sb : sa; };
+  {
+    const int n = nloc * gp.n2;
+    for (int t = threadIdx.x; t < 2 * n; t += TH) {
+      const int e = t >= n ? t - n : t, p = e / gp.n2;
+      C* s = both(t, n) + p * S1 + __ldg(gp.l2 + (e - p * gp.n2)) * S2;
+      C x[N3];
+#pragma unroll
+      for (int k = 0; k < N3; ++k) x[k] = s[k];
+      RegFFT<N3, -1>::run(x);
+#pragma unroll
+      for (int k = 0; k < N3; ++k) s[k] = x[k];
+    }
   }
   __syncthreads();
-  pencil_pass<N2, +1>(sa, P * N3, S2, [](int q) { return (q / N3) * (N2 * S2) + (q % N3); });
+  {
+    const int n = nloc * N3;
+    for (int t = threadIdx.x; t < 2 * n; t += TH) {
+      const int e = t >= n ? t - n : t;
+      C* s = both(t, n) + e / N3 * S1 + e % N3;
+      C x[N2];
+#pragma unroll
+      for (int k = 0; k < N2; ++k) x[k] = s[k * S2];
+      RegFFT<N2, -1>::run(x);
+#pragma unroll
+      for (int k = 0; k < N2; ++k) s[k * S2] = x[k];
+    }
+  }
   __syncthreads();
-  pencil_pass<N3, +1>(sa, P * N2, 1, [](int q) { return q * S2; });
+  // the product of Eq. chi_rr taken into the forward i2 pass, then the i3 pass of the set's pencils
+  for (int e = threadIdx.x; e < nloc * N3; e += TH) {
+    const int p = e / N3, i3 = e - p * N3, o = p * S1 + i3;
+    const int r0 = (p * CL + c) * PL + i3;               // grid position of k = 0
+    C x[N2];
+#pragma unroll
+    for (int k = 0; k < N2; ++k) {
+      const int r = r0 + k * N3;
+      x[k] = mk(T(0), T(0));
+      if (r <= last) x[k] = cscale(cmulc(sa[o + k * S2], sb[o + k * S2]), low >= 0 && r == last ? scale * T(0.5) : scale);
+    }
+    RegFFT<N2, +1>::run(x);
+#pragma unroll
+    for (int k = 0; k < N2; ++k) sa[o + k * S2] = x[k];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < nloc * gx.n2; e += TH) {
+    const int p = e / gx.n2;
+    C* s = sa + p * S1 + __ldg(gx.l2 + (e - p * gx.n2)) * S2;
+    C x[N3];
+#pragma unroll
+    for (int k = 0; k < N3; ++k) x[k] = s[k];
+    RegFFT<N3, +1>::run(x);
+#pragma unroll
+    for (int k = 0; k < N3; ++k) s[k] = x[k];
+  }
   cluster.sync();                  // every CTA's x planes are final
   // forward i1 transforms of the CTA's columns, each result into the slice of chi that holds it
   C* sx = sl;                      // [n_cs] this CTA's part of the chi row
-  for (int q = c * COLS + threadIdx.x; q < (c + 1) * COLS; q += TH) {
-    const int i2 = q / N3, i3 = q - i2 * N3;
-    bool any = false;                // columns with no point of chi's G set deliver nothing
-#pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1) any |= __ldg(inv_chi + i1 * PL + q) >= 0;
-    if (!__any_sync(__activemask(), any)) continue;
+  for (int e = gx.n23 * c / CL + threadIdx.x; e < gx.n23 * (c + 1) / CL; e += TH) {
+    const int q = __ldg(gx.l23 + e);
+    const int o23 = q / N3 * S2 + q % N3;
     C x[N1];
 #pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1) x[i1] = cluster.map_shared_rank(sa, i1 / P)[((i1 % P) * N2 + i2) * S2 + i3];
+    for (int i1 = 0; i1 < N1; ++i1)
+      x[i1] = i1 < i1m ? cluster.map_shared_rank(sa, i1 % CL)[(i1 / CL) * S1 + o23] : mk(T(0), T(0));
     RegFFT<N1, +1>::run(x);
 #pragma unroll
     for (int i1 = 0; i1 < N1; ++i1) {
@@ -974,17 +1196,35 @@ struct GridOps {
   }
   static gw_status row(gw_ctx* ctx, int mode, const void* a, const void* b, long lda, void* out, long ldo,
                        const int* map, int n_chi, int n_rows, double scale, cudaStream_t st, const int* inv,
-                       void* tmp) {
-    const size_t bytes = RowLayout<N1, N2, N3>::TOT * sizeof(C);
-    const double rd = mode == 0 ? 2.0 * RowLayout<N1, N2, N3>::NR : (mode == 1 ? RowLayout<N1, N2, N3>::NR : n_chi);
-    const double wr = mode == 2 ? RowLayout<N1, N2, N3>::NR : n_chi;
+                       void* tmp, int low) {
+    using L = RowLayout<N1, N2, N3>;
+    const size_t bytes = L::TOT * sizeof(C);
+    const double rd = mode == 0 ? 2.0 * L::NR : (mode == 1 ? L::NR : n_chi);
+    const double wr = mode == 2 ? L::NR : n_chi;
+    // HBM bytes of the launch: whole rows, or the triangle's share of the grid side
+    double grid_el = (double)n_rows * L::NR;
+    if (low >= 0) {
+      grid_el = 0;
+      for (int r = 0; r < n_rows; ++r) grid_el += std::min(L::NR, low + r + 1);
+    }
+    const double work = (grid_el * (mode == 0 ? 2.0 : 1.0) + (double)n_rows * n_chi) * sizeof(C);
     auto al = [](const void* p) { return p == nullptr || reinterpret_cast<uintptr_t>(p) % 16 == 0; };
-    const bool vec = al(a) && al(b) && al(out) && lda % 2 == 0 && ldo % 2 == 0 && n_chi % 2 == 0 && N3 % 2 == 0;
+    // 16-byte pairs on the grid side (rows of a and b, or of out for mode 2) and on the G-set side
+    const bool vi = mode == 2 ? al(out) && ldo % 2 == 0 && N3 % 2 == 0 : al(a) && al(b) && lda % 2 == 0 && N3 % 2 == 0;
+    const bool vo = mode != 2 && al(out) && ldo % 2 == 0 && n_chi % 2 == 0;
+    if (!inv) return fail(ctx, GW_ERR_ARG, "row transform without the G set's inverse map");
     if (bytes > kRowSmemMax) {
       using CR = ClusterRow<T, N1, N2, N3>;
-      if constexpr (CR::CL > 0 && RowLayout<N1, N2, N3>::TOT * sizeof(C) > kRowSmemMax) {
-        if (inv && CR::smem(n_chi) <= kRowSmemMax) {
-          const size_t cbytes = CR::smem(n_chi);
+      if constexpr (CR::CL > 0 && L::TOT * sizeof(C) > kRowSmemMax) {
+        if (CR::smem(n_chi, CR::P) <= kRowSmemMax) {
+          // local planes of the launch's last row
+          int planes = CR::P;
+          if (low >= 0) {
+            const int g0 = low + (n_rows - 1) / 128 * 128;
+            const int last = mode == 2 ? std::min(L::NR - 1, (g0 + 127) / 128 * 128 + 127) : low + n_rows - 1;
+            planes = (last / (N2 * N3) + CR::CL) / CR::CL;
+          }
+          const size_t cbytes = CR::smem(n_chi, planes);
           auto go = [&](auto kernel) -> gw_status {
             gw_status s = set_smem(ctx, kernel, cbytes);
             if (s) return s;
@@ -1000,16 +1240,16 @@ struct GridOps {
             attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            KTimer kt(ctx, KF_ROW_FFT, (double)n_rows * (rd + wr) * sizeof(C), st);
+            KTimer kt(ctx, KF_ROW_FFT, work, st);
             gw_status r = cuda_check(ctx, cudaLaunchKernelEx(&cfg, kernel, (const C*)a, (const C*)b, lda, (C*)out, ldo,
-                                                             inv, n_chi, (T)scale),
+                                                             inv, n_chi, (T)scale, low, planes),
                                      "cudaLaunchKernelEx(row_cluster_kernel)");
             if (r) return r;
             return launch_check(ctx, "row_cluster_kernel");
           };
-#define GW_ROWC_GO(M)                                                                        \
-          if (mode == M) return vec ? go(row_cluster_kernel<T, N1, N2, N3, M, N3 % 2 == 0>)  \
-                                    : go(row_cluster_kernel<T, N1, N2, N3, M, false>);
+#define GW_ROWC_GO(M)                                                                       \
+          if (mode == M) return vi ? go(row_cluster_kernel<T, N1, N2, N3, M, N3 % 2 == 0>)  \
+                                   : go(row_cluster_kernel<T, N1, N2, N3, M, false>);
           GW_ROWC_GO(0)
           GW_ROWC_GO(1)
           GW_ROWC_GO(2)
@@ -1017,25 +1257,38 @@ struct GridOps {
           return fail(ctx, GW_ERR_ARG, "bad row transform mode");
         }
       }
+      if (low >= 0 && mode != 2) return fail(ctx, GW_ERR_UNSUPPORTED, "triangle rows need the one-pass row transform");
       return row_two_pass(ctx, mode, a, b, lda, out, ldo, inv, tmp, n_chi, n_rows, scale, st);
     }
-    auto go = [&](auto kernel, int threads) -> gw_status {
-      gw_status s = set_smem(ctx, kernel, bytes);
-      if (s) return s;
-      KTimer kt(ctx, KF_ROW_FFT, (double)n_rows * (rd + wr) * sizeof(C), st);
-      kernel<<<n_rows, threads, bytes, st>>>((const C*)a, (const C*)b, lda, (C*)out, ldo, map, n_chi, (T)scale);
-      return launch_check(ctx, "row_fft_kernel");
-    };
-    constexpr bool big = N1 * N2 * N3 >= 4096;
-    constexpr int TH = big ? 512 : 256;
-#define GW_ROW_GO(M)                                                              \
-    if (mode == M) return vec ? go(row_fft_kernel<T, N1, N2, N3, M, TH, N3 % 2 == 0>, TH) \
-                              : go(row_fft_kernel<T, N1, N2, N3, M, TH, false>, TH);
-    GW_ROW_GO(0)
-    GW_ROW_GO(1)
-    GW_ROW_GO(2)
+    if constexpr (L::TOT * sizeof(C) <= kRowSmemMax) {
+      auto go = [&](auto kernel) -> gw_status {
+        gw_status s = set_smem(ctx, kernel, bytes);
+        if (s) return s;
+        KTimer kt(ctx, KF_ROW_FFT, work, st);
+        kernel<<<n_rows, RowCfg<T, N1, N2, N3>::TH, bytes, st>>>((const C*)a, (const C*)b, lda, (C*)out, ldo, map, inv,
+                                                                 n_chi, (T)scale, low);
+        return launch_check(ctx, "row_fft_kernel");
+      };
+      constexpr bool E = N3 % 2 == 0;
+#define GW_ROW_GO(M)                                                        \
+      if (mode == M)                                                        \
+        return vi ? (vo ? go(row_fft_kernel<T, N1, N2, N3, M, E, true>)     \
+                        : go(row_fft_kernel<T, N1, N2, N3, M, E, false>))   \
+                  : go(row_fft_kernel<T, N1, N2, N3, M, false, false>);
+      GW_ROW_GO(0)
+      GW_ROW_GO(1)
 #undef GW_ROW_GO
+      if (mode == 2) return vi ? go(row_fft_kernel<T, N1, N2, N3, 2, E, false>)
+                               : go(row_fft_kernel<T, N1, N2, N3, 2, false, false>);
+    }
     return fail(ctx, GW_ERR_ARG, "bad row transform mode");
+  }
+  // whether rows of the triangle R' <= r have a kernel (all but the two-pass FP64 rows)
+  static bool row_low_ok(int n_chi) {
+    using CR = ClusterRow<T, N1, N2, N3>;
+    if (RowLayout<N1, N2, N3>::TOT * sizeof(C) <= kRowSmemMax) return true;
+    if constexpr (CR::CL > 0) return CR::smem(n_chi, CR::P) <= kRowSmemMax;
+    return false;
   }
   static bool row_pw_ok(int n_pw, int n_chi) {
     using PR = PwRow<T, N1, N2, N3>;
@@ -1044,11 +1297,38 @@ struct GridOps {
   }
   static gw_status row_pw(gw_ctx* ctx, const void* a, const void* b, long lda, void* out, long ldo,
                            const int* inv_pw, int n_pw, const int* inv_chi, int n_chi, int n_rows, double scale,
-                           cudaStream_t st) {
+                           cudaStream_t st, int low) {
     using PR = PwRow<T, N1, N2, N3>;
     if constexpr (PR::CL > 0) {
-      const size_t bytes = PR::smem(n_pw, n_chi);
-      if (bytes > kRowSmemMax) return fail(ctx, GW_ERR_UNSUPPORTED, "plane-wave chi rows: G sets too large for this grid");
+      if (PR::smem(n_pw, n_chi) > kRowSmemMax)
+        return fail(ctx, GW_ERR_UNSUPPORTED, "plane-wave chi rows: G sets too large for this grid");
+      if (low >= 0) {
+        // rows of equal local plane counts go together: the shorter ones need less shared memory,
+        // so more of them share an SM
+        constexpr int step = PR::CL * N2 * N3;
+        const int end = std::min(N1 * N2 * N3, low + n_rows);
+        for (int r = low; r < end;) {
+          const int to = std::min(end, (r / step + 1) * step);
+          const long o = r - low;
+          gw_status s = row_pw_part(ctx, (const C*)a + o * lda, (const C*)b + o * lda, lda, (C*)out + o * ldo, ldo,
+                                    inv_pw, n_pw, inv_chi, n_chi, to - r, scale, st, r, r / step + 1);
+          if (s) return s;
+          r = to;
+        }
+        return GW_OK;
+      }
+      return row_pw_part(ctx, (const C*)a, (const C*)b, lda, (C*)out, ldo, inv_pw, n_pw, inv_chi, n_chi, n_rows, scale,
+                         st, -1, PR::P);
+    } else {
+      return fail(ctx, GW_ERR_UNSUPPORTED, "plane-wave chi rows: no cluster split fits this grid and precision");
+    }
+  }
+  static gw_status row_pw_part(gw_ctx* ctx, const C* a, const C* b, long lda, C* out, long ldo, const int* inv_pw,
+                               int n_pw, const int* inv_chi, int n_chi, int n_rows, double scale, cudaStream_t st,
+                               int low, int planes) {
+    using PR = PwRow<T, N1, N2, N3>;
+    if constexpr (PR::CL > 0) {
+      const size_t bytes = PR::smem(n_pw, n_chi, planes);
       auto kernel = row_pw_chi_kernel<T, N1, N2, N3>;
       gw_status s = set_smem(ctx, kernel, bytes);
       if (s) return s;
@@ -1067,13 +1347,13 @@ struct GridOps {
       // FP32/FP64 ALU work: three transforms of N_r points (5 N log2 N each) and the product per row
       const double nr = (double)N1 * N2 * N3;
       KTimer kt(ctx, KF_ROW_PW, (double)n_rows * (3.0 * 5.0 * nr * std::log2(nr) + 6.0 * nr), st);
-      s = cuda_check(ctx, cudaLaunchKernelEx(&cfg, kernel, (const C*)a, (const C*)b, lda, (C*)out, ldo, inv_pw, n_pw,
-                                             inv_chi, n_chi, (T)scale),
+      s = cuda_check(ctx, cudaLaunchKernelEx(&cfg, kernel, a, b, lda, out, ldo, inv_pw, n_pw,
+                                             inv_chi, n_chi, (T)scale, low, planes),
                      "cudaLaunchKernelEx(row_pw_chi_kernel)");
       if (s) return s;
       return launch_check(ctx, "row_pw_chi_kernel");
     } else {
-      return fail(ctx, GW_ERR_UNSUPPORTED, "plane-wave chi rows: no cluster split fits this grid and precision");
+      return GW_ERR_UNSUPPORTED;
     }
   }
   static bool row_pw_sigma_ok(int n_pw, int n_chi) {
@@ -1208,16 +1488,23 @@ static bool with_grid(const GridInfo& g, F&& f) {
 
 gw_status launch_row_fft(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int mode, const void* a, const void* b,
                          long lda, void* out, long ldo, const int* map, int n_chi, int n_rows, double scale,
-                         cudaStream_t st, const int* inv, void* tmp) {
+                         cudaStream_t st, const int* inv, void* tmp, int low) {
   if (n_rows <= 0) return GW_OK;
-  GW_DISPATCH(prec, g, rc = O::row(ctx, mode, a, b, lda, out, ldo, map, n_chi, n_rows, scale, st, inv, tmp))
+  GW_DISPATCH(prec, g, rc = O::row(ctx, mode, a, b, lda, out, ldo, map, n_chi, n_rows, scale, st, inv, tmp, low))
+}
+
+bool row_low_ok(const GridInfo& g, gw_prec prec, int n_chi) {
+  bool ok = false;
+  if (is_fp64(prec)) with_grid<double>(g, [&](auto ops) { ok = decltype(ops)::row_low_ok(n_chi); });
+  else with_grid<float>(g, [&](auto ops) { ok = decltype(ops)::row_low_ok(n_chi); });
+  return ok;
 }
 
 gw_status launch_row_pw_chi(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* a, const void* b, long lda,
                             void* out, long ldo, const int* inv_pw, int n_pw, const int* inv_chi, int n_chi,
-                            int n_rows, double scale, cudaStream_t st) {
+                            int n_rows, double scale, cudaStream_t st, int low) {
   if (n_rows <= 0) return GW_OK;
-  GW_DISPATCH(prec, g, rc = O::row_pw(ctx, a, b, lda, out, ldo, inv_pw, n_pw, inv_chi, n_chi, n_rows, scale, st))
+  GW_DISPATCH(prec, g, rc = O::row_pw(ctx, a, b, lda, out, ldo, inv_pw, n_pw, inv_chi, n_chi, n_rows, scale, st, low))
 }
 
 gw_status check_row_pw(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int n_pw, int n_chi) {
@@ -1344,7 +1631,30 @@ gw_status index_maps(gw_ctx* ctx, const GridInfo& g, const int32_t* fft_index_h,
     if (inv[map[j]] >= 0) return fail(ctx, GW_ERR_ARG, "fft_index has duplicates");
     inv[map[j]] = j;
   }
+  set_lists(g, inv);
   return GW_OK;
+}
+
+void set_lists(const GridInfo& g, std::vector<int>& inv) {
+  inv.resize(g.nr);
+  const int pl = g.n2 * g.n3;
+  std::vector<char> c23(pl, 0), c12((size_t)g.n1 * g.n2, 0), u1(g.n1, 0), u2(g.n2, 0), u3(g.n3, 0);
+  for (int p = 0; p < g.nr; ++p) {
+    if (inv[p] < 0) continue;
+    const int i1 = p / pl, i2 = p % pl / g.n3, i3 = p % g.n3;
+    c23[p % pl] = c12[i1 * g.n2 + i2] = u1[i1] = u2[i2] = u3[i3] = 1;
+  }
+  inv.resize(inv_ints(g), 0);
+  int* x = inv.data() + g.nr;
+  int* at = x + kSetHead;
+  int head = 0;
+  for (const std::vector<char>* v : {&c23, &c12, &u1, &u2, &u3}) {
+    int count = 0;
+    for (size_t i = 0; i < v->size(); ++i)
+      if ((*v)[i]) at[count++] = (int)i;
+    x[head++] = count;
+    at += v->size();
+  }
 }
 
 }  // namespace gw
@@ -1381,15 +1691,15 @@ extern "C" gw_status gw_rr_to_GG_fft(gw_ctx* ctx, const gw_grid* grid, int direc
   const bool work_rows = stage == 1 && direction > 0 && row_two_pass(g, prec);
   Carver probe(nullptr);
   probe.take<int>(n_chi);
-  probe.take<int>(g.nr);
+  probe.take<int>(inv_ints(g));
   if (work_rows) probe.take<char>((size_t)n_rows * g.nr * csize(prec));
   if ((st = reserve(ctx, probe.off))) return st;
   Carver cv(ctx->arena);
   int* dmap = cv.take<int>(n_chi);
-  int* dinv = cv.take<int>(g.nr);
+  int* dinv = cv.take<int>(inv_ints(g));
   void* tmp = work_rows ? cv.take<char>((size_t)n_rows * g.nr * csize(prec)) : nullptr;
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
-  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * g.nr, s))) return st;
+  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if (stage == 1) {
     if (direction > 0)
       return launch_row_fft(ctx, g, prec, 1, in, nullptr, g.nr, out, n_chi, dmap, n_chi, n_rows, 1.0, s, dinv, tmp);
@@ -1451,10 +1761,11 @@ extern "C" gw_status gw_tau_to_omega(gw_ctx* ctx, int kind, int n, const double*
 namespace {
 
 constexpr int kNoAllocMaxInts = 2 * 13824;   // n_chi + N_r for the largest compiled grid (24^3)
+constexpr int kNoAllocLists = kSetHead + 2 * 24 * 24 + 3 * 24;   // and the set's lists behind its inverse map
 
-// Holds fft_index followed by its inverse map.  Every GPU that loads the
+// Holds fft_index followed by its inverse map and the set's lists (set_lists).  Every GPU that loads the
 // library keeps this array until the process exits; all calls share it.
-static __device__ __align__(256) int g_noalloc_maps[kNoAllocMaxInts];
+static __device__ __align__(256) int g_noalloc_maps[kNoAllocMaxInts + kNoAllocLists];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mu;
@@ -1519,10 +1830,10 @@ extern "C" gw_status gw_rr_to_GG_fft_noalloc(const gw_grid* grid, int direction,
   int* dinv = maps + n_chi;
   // both maps are rewritten in full on every call, so nothing carries over
   if ((st = upload(&local, dmap, map.data(), sizeof(int) * n_chi, s))) return done(st);
-  if ((st = upload(&local, dinv, inv.data(), sizeof(int) * g.nr, s))) return done(st);
+  if ((st = upload(&local, dinv, inv.data(), sizeof(int) * inv.size(), s))) return done(st);
   if (stage == 1) {
-    if (direction > 0) st = launch_row_fft(&local, g, prec, 1, in, nullptr, g.nr, out, n_chi, dmap, n_chi, n_rows, 1.0, s);
-    else st = launch_row_fft(&local, g, prec, 2, in, nullptr, n_chi, out, g.nr, dmap, n_chi, n_rows, 1.0 / g.volume, s);
+    if (direction > 0) st = launch_row_fft(&local, g, prec, 1, in, nullptr, g.nr, out, n_chi, dmap, n_chi, n_rows, 1.0, s, dinv);
+    else st = launch_row_fft(&local, g, prec, 2, in, nullptr, n_chi, out, g.nr, dmap, n_chi, n_rows, 1.0 / g.volume, s, dinv);
     return done(st);
   }
   if (direction > 0) {

@@ -3,6 +3,8 @@
 // inverse of the screening step.  64x64 output tile per 256-thread CTA, 4x4
 // complex outputs per thread on an interleaved (stride-16) pattern so that the
 // shared-memory reads of a warp are broadcasts or consecutive.
+#include <algorithm>
+
 #include "gw_kernels.h"
 
 namespace gw {
@@ -21,6 +23,7 @@ struct GemmP {
   long ldc;
   const T* kscale;
   long sA, sB, sC;
+  int low;
 };
 
 template <typename T, int AKM, bool AC, int BNK, bool BC, bool SCALE, int TRI>
@@ -31,6 +34,7 @@ __global__ void __launch_bounds__(256) cgemm_kernel(GemmP<T> p) {
   __shared__ C Bs[BK][BN + PAD];
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   if (TRI && n0 > m0 + BM - 1) return;
+  if (!TRI && p.low >= 0 && n0 > p.low + m0 + BM - 1) return;   // no column n <= low + m in the tile
   p.A += blockIdx.z * p.sA;
   p.B += blockIdx.z * p.sB;
   p.Cm += blockIdx.z * p.sC;
@@ -111,6 +115,13 @@ __global__ void __launch_bounds__(256) cgemm_kernel(GemmP<T> p) {
     }
 }
 
+// Flops of a product of which only n <= low + m is needed (whole rows of 64).
+static double low_flops(const GemmArgs& a) {
+  double s = 0;
+  for (int m = 0; m < a.M; m += 64) s += (double)std::min(64, a.M - m) * std::min(a.N, a.low + m + 64);
+  return 8.0 * s * a.K;
+}
+
 template <typename T>
 static gw_status run_gemm(gw_ctx* ctx, const GemmArgs& a, cudaStream_t st) {
   using C = typename cpx<T>::t;
@@ -130,12 +141,14 @@ static gw_status run_gemm(gw_ctx* ctx, const GemmArgs& a, cudaStream_t st) {
   p.sA = a.sA;
   p.sB = a.sB;
   p.sC = a.sC;
-  dim3 grid((a.N + 63) / 64, (a.M + 63) / 64, a.batch > 0 ? a.batch : 1);
+  p.low = a.low;
+  const int n_end = a.low >= 0 ? std::min(a.N, a.low + a.M) : a.N;    // columns past the last row's are not needed
+  dim3 grid((n_end + 63) / 64, (a.M + 63) / 64, a.batch > 0 ? a.batch : 1);
   if (grid.y > 65535) return fail(ctx, GW_ERR_SHAPE, "GEMM M too large");
 #define GW_GEMM_CASE(AKM, AC, BNK, BC, SC, TRI)                                                   \
   if (a.a_km == AKM && a.a_conj == AC && a.b_nk == BNK && a.b_conj == BC && (a.kscale != nullptr) == SC && \
       a.tri == TRI) {                                                                               \
-    KTimer kt(ctx, KF_CGEMM_SIMT, grid.z * gemm_flops(a.M, a.N, a.K, TRI), st);                   \
+    KTimer kt(ctx, KF_CGEMM_SIMT, grid.z * (a.low >= 0 ? low_flops(a) : gemm_flops(a.M, a.N, a.K, TRI)), st); \
     cgemm_kernel<T, AKM, AC, BNK, BC, SC, TRI><<<grid, 256, 0, st>>>(p);                           \
     return launch_check(ctx, "cgemm_kernel");                                                       \
   }

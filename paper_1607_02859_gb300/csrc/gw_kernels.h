@@ -12,14 +12,27 @@ namespace gw {
 constexpr size_t kRowSmemMax = 227 * 1024;
 gw_status launch_row_fft(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int mode, const void* a, const void* b,
                          long lda, void* out, long ldo, const int* map, int n_chi, int n_rows, double scale,
-                         cudaStream_t st, const int* inv = nullptr, void* tmp = nullptr);
+                         cudaStream_t st, const int* inv, void* tmp = nullptr, int low = -1);
+// low >= 0: the rows are rows low .. of a Hermitian matrix used only for R' <= r
+// (forward: elements past r count as zero and mode 0 halves the diagonal; backward:
+// only what the fused self-energy reads is written); row_low_ok: forward rows have it.
+bool row_low_ok(const GridInfo& g, gw_prec prec, int n_chi);
+// A G set's inverse map on the device: inv [N_r] (grid position -> G index or -1)
+// followed by what of the grid the set touches (set_lists appends it; index_maps
+// does): kSetHead counts, then the (i2,i3) columns, the (i1,i2) pencils and the
+// values of i1, i2, i3 that hold a point of the set, each ascending.
+constexpr int kSetHead = 8;
+inline int inv_ints(const GridInfo& g) {
+  return g.nr + kSetHead + g.n2 * g.n3 + g.n1 * g.n2 + g.n1 + g.n2 + g.n3;
+}
+void set_lists(const GridInfo& g, std::vector<int>& inv);
 bool row_two_pass(const GridInfo& g, gw_prec prec);
 // chi rows from the plane-wave form of G: a = T_unocc, b = T_occ rows [n_rows][lda]
 // over the orbitals' plane-wave set (inv_pw: grid position -> set index or -1),
 // out [n_rows][ldo] = FFT+(scale a conj(b)) on chi's G set (inv_chi).
 gw_status launch_row_pw_chi(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* a, const void* b, long lda,
                             void* out, long ldo, const int* inv_pw, int n_pw, const int* inv_chi, int n_chi,
-                            int n_rows, double scale, cudaStream_t st);
+                            int n_rows, double scale, cudaStream_t st, int low = -1);
 // GW_OK if launch_row_pw_chi supports the grid, precision and set sizes.
 gw_status check_row_pw(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int n_pw, int n_chi);
 // Sigma rows in the plane-wave form: tu, to [n_rows][ldt] (T rows over the negated
@@ -90,6 +103,8 @@ struct GemmArgs {
   int tri;
   int batch = 1;              // grid z: independent problems sA/sB/sC elements apart
   long sA = 0, sB = 0, sC = 0;
+  int low = -1;               // >= 0: row m is row low + m of a matrix of which only the columns n <= low + m
+                              // are needed: tiles wholly above that line are left as they are
 };
 gw_status launch_gemm(gw_ctx* ctx, gw_prec prec, const GemmArgs& a, cudaStream_t st);
 
@@ -101,7 +116,7 @@ struct GreenScales {
 GreenScales green_scales(const double* eps, int n_b, int n_occ, double mu, double tau);
 gw_status green_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const void* dscale,
                      const GreenScales& gs, int r0, int n_rows, gw_prec prec, void* g_occ, void* g_unocc,
-                     cudaStream_t st);
+                     cudaStream_t st, int low = -1);
 
 }  // namespace gw
 

@@ -311,9 +311,9 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   const size_t slab = (size_t)g.nr * ld;
   Carver probe(nullptr);
   probe.take<int>(n_chi);
-  probe.take<int>(g.nr);
+  probe.take<int>(inv_ints(g));
   probe.take<int>((size_t)n_k * n_chi);
-  probe.take<int>(gs.nr);
+  probe.take<int>(inv_ints(gs));
   probe.take<double>((size_t)n_k * n_b);
   probe.take<double>((size_t)n * n);
   probe.take<double2>((size_t)n_k * n_k);
@@ -327,9 +327,9 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   if ((st = reserve(ctx, probe.off))) return st;
   Carver cv(ctx->arena);
   int* dmap = cv.take<int>(n_chi);
-  int* dinv = cv.take<int>(g.nr);
+  int* dinv = cv.take<int>(inv_ints(g));
   int* dsmap = cv.take<int>((size_t)n_k * n_chi);
-  int* dsinv = cv.take<int>(gs.nr);
+  int* dsinv = cv.take<int>(inv_ints(gs));
   char* dscale = cv.take<char>((size_t)n_k * n_b * 8);
   char* dcw = cv.take<char>((size_t)n * n * 8);
   char* dph = cv.take<char>((size_t)n_k * n_k * 16);
@@ -341,9 +341,9 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   char* tmp_s = two_pass ? cv.take<char>((size_t)rb * gs.nr * es) : nullptr;
   void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false)) : nullptr;
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
-  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * g.nr, s))) return st;
+  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if ((st = upload(ctx, dsmap, smap.data(), sizeof(int) * n_k * n_chi, s))) return st;
-  if ((st = upload(ctx, dsinv, sinv.data(), sizeof(int) * gs.nr, s))) return st;
+  if ((st = upload(ctx, dsinv, sinv.data(), sizeof(int) * sinv.size(), s))) return st;
   if ((st = upload_phases(ctx, dph, kl_phases(nk), prec, s))) return st;
   if ((st = fill_q_phases(ctx, prec, g, nk, dqph, s))) return st;
   const double fac = g.dv * g.dv / g.volume;   // Eq. FFTX2 normalisation
@@ -444,6 +444,7 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
       inv_pws[pos] = k * n_pw + j;
     }
   }
+  set_lists(gs, inv_pws);
   pw_negate(g, map_pw, inv_pw);
   const int n_pws = n_k * n_pw, n_chis = n_k * n_chi;
   if ((st = check_row_pw(ctx, gs, prec, n_pws, n_chis))) return st;
@@ -456,11 +457,11 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
   const GridInfo gp = pw_grid(g, n_pw);
   const bool tmp_needed = row_two_pass(g, prec) && is_fp64(prec);
   Carver probe(nullptr);
-  probe.take<int>(g.nr);
-  probe.take<int>(gs.nr);
+  probe.take<int>(inv_ints(g));
+  probe.take<int>(inv_ints(gs));
   probe.take<int>(n_pw);
-  probe.take<int>(g.nr);
-  probe.take<int>(gs.nr);
+  probe.take<int>(inv_ints(g));
+  probe.take<int>(inv_ints(gs));
   probe.take<char>((size_t)n_k * n_b * 8);
   probe.take<char>((size_t)n * n * 8);
   probe.take<double>(2 * (size_t)n_b);
@@ -476,11 +477,11 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
   if (tc) probe.take<char>(tc_scratch_bytes(gp, n_b, n_occ, n_pw, false));
   if ((st = reserve(ctx, probe.off))) return st;
   Carver cv(ctx->arena);
-  int* dinv = cv.take<int>(g.nr);
-  int* dsinv = cv.take<int>(gs.nr);
+  int* dinv = cv.take<int>(inv_ints(g));
+  int* dsinv = cv.take<int>(inv_ints(gs));
   int* dmap_pw = cv.take<int>(n_pw);
-  int* dinv_pw = cv.take<int>(g.nr);
-  int* dinv_pws = cv.take<int>(gs.nr);
+  int* dinv_pw = cv.take<int>(inv_ints(g));
+  int* dinv_pws = cv.take<int>(inv_ints(gs));
   char* dscale = cv.take<char>((size_t)n_k * n_b * 8);
   char* dcw = cv.take<char>((size_t)n * n * 8);
   double* dnorm = cv.take<double>(2 * (size_t)n_b);
@@ -494,11 +495,11 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
   char* tu = cv.take<char>((size_t)g.nr * ldt * es);
   char* tmp = tmp_needed ? cv.take<char>((size_t)n_b * g.nr * es) : nullptr;
   void* tcs = tc ? cv.take<char>(tc_scratch_bytes(gp, n_b, n_occ, n_pw, false)) : nullptr;
-  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * g.nr, s))) return st;
-  if ((st = upload(ctx, dsinv, sinv.data(), sizeof(int) * gs.nr, s))) return st;
+  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
+  if ((st = upload(ctx, dsinv, sinv.data(), sizeof(int) * sinv.size(), s))) return st;
   if ((st = upload(ctx, dmap_pw, map_pw.data(), sizeof(int) * n_pw, s))) return st;
-  if ((st = upload(ctx, dinv_pw, inv_pw.data(), sizeof(int) * g.nr, s))) return st;
-  if ((st = upload(ctx, dinv_pws, inv_pws.data(), sizeof(int) * gs.nr, s))) return st;
+  if ((st = upload(ctx, dinv_pw, inv_pw.data(), sizeof(int) * inv_pw.size(), s))) return st;
+  if ((st = upload(ctx, dinv_pws, inv_pws.data(), sizeof(int) * inv_pws.size(), s))) return st;
   const double fac = g.dv * g.dv / g.volume;   // Eq. FFTX2 normalisation
   std::vector<float> cw32;
   if (is_fp64(prec)) {
@@ -610,9 +611,9 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   const int nreal1 = std::max(n_real, 1);
   Carver probe(nullptr);
   probe.take<int>(n_chi);
-  probe.take<int>(g.nr);
+  probe.take<int>(inv_ints(g));
   probe.take<int>((size_t)n_k * n_chi);
-  probe.take<int>(gs.nr);
+  probe.take<int>(inv_ints(gs));
   probe.take<int>(3 * (size_t)n_n);
   probe.take<double>((size_t)n_k * n_b);
   probe.take<double2>((size_t)n_k * n_k);
@@ -630,9 +631,9 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   if ((st = reserve(ctx, probe.off))) return st;
   Carver cv(ctx->arena);
   int* dmap = cv.take<int>(n_chi);
-  int* dinv = cv.take<int>(g.nr);
+  int* dinv = cv.take<int>(inv_ints(g));
   int* dsmap = cv.take<int>((size_t)n_k * n_chi);
-  int* dsinv = cv.take<int>(gs.nr);
+  int* dsinv = cv.take<int>(inv_ints(gs));
   int* dbk = cv.take<int>(3 * (size_t)n_n);           // (band, k) pairs, then 0 .. n_n-1
   int* dbid = dbk + 2 * n_n;
   char* dscale = cv.take<char>((size_t)n_k * n_b * 8);
@@ -652,9 +653,9 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   char* prow = ext + (size_t)n_n * gs.nr * es;
   void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false)) : nullptr;
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
-  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * g.nr, s))) return st;
+  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if ((st = upload(ctx, dsmap, smap.data(), sizeof(int) * n_k * n_chi, s))) return st;
-  if ((st = upload(ctx, dsinv, sinv.data(), sizeof(int) * gs.nr, s))) return st;
+  if ((st = upload(ctx, dsinv, sinv.data(), sizeof(int) * sinv.size(), s))) return st;
   std::vector<int> bk(3 * (size_t)n_n);
   for (int i = 0; i < 2 * n_n; ++i) bk[i] = bk_h[i];
   for (int i = 0; i < n_n; ++i) bk[2 * n_n + i] = i;

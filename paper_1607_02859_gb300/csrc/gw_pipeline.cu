@@ -22,7 +22,7 @@ size_t chi0_omega_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_ch
   const size_t slab = (size_t)g.nr * n_chi;
   Carver probe(nullptr);
   probe.take<int>(n_chi);
-  probe.take<int>(g.nr);
+  probe.take<int>(inv_ints(g));
   probe.take<double>((size_t)n * n_b);
   probe.take<double>((size_t)n * n);
   probe.take<char>(slab * n * es);
@@ -32,31 +32,43 @@ size_t chi0_omega_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_ch
   return probe.off;
 }
 
-// chi(G,G') = X(G,G') + conj(X(G',G)) in place, for every frequency.  The
-// tensor-core chi pass forms only the lower triangle T of chi(r,R') (R' <= r)
-// with its diagonal halved; chi(r,R') is Hermitian, so chi = T + T^H, and the
-// transforms of Eqs. FFTX1, FFTX2 and the cosine transform (Eq. CTX, real
-// weights) carry that over: chi(G,G',i omega) = X + X^H with X the result for T.
+// chi(G,G') = X(G,G') + conj(X(G',G)) in place, for every frequency.  The chi
+// passes form only the lower triangle T of chi(r,R') (R' <= r) with its diagonal
+// halved; chi(r,R') is Hermitian, so chi = T + T^H, and the transforms of Eqs.
+// FFTX1, FFTX2 and the cosine transform (Eq. CTX, real weights) carry that over:
+// chi(G,G',i omega) = X + X^H with X the result for T.
 // One CTA per pair of 32 x 32 tiles (I, J), I <= J, through shared memory.
-__global__ void __launch_bounds__(256) hermitize_kernel(float2* __restrict__ X, long sx, int n) {
-  __shared__ float2 a[32][33], b[32][33];
+template <typename C>
+__global__ void __launch_bounds__(256) hermitize_kernel(C* __restrict__ X, long sx, int n) {
+  __shared__ C a[32][33], b[32][33];
   const int I = blockIdx.x, J = blockIdx.y;
   if (I > J) return;
-  float2* x = X + blockIdx.z * sx;
+  C* x = X + blockIdx.z * sx;
   const int tx = threadIdx.x;
+  const C zero = mk(decltype(a[0][0].x)(0), decltype(a[0][0].x)(0));
   for (int y = threadIdx.y; y < 32; y += blockDim.y) {
     const int r = I * 32 + y, c = J * 32 + tx;
-    a[y][tx] = (r < n && c < n) ? x[(long)r * n + c] : make_float2(0.f, 0.f);
+    a[y][tx] = (r < n && c < n) ? x[(long)r * n + c] : zero;
     const int r2 = J * 32 + y, c2 = I * 32 + tx;
-    b[y][tx] = (r2 < n && c2 < n) ? x[(long)r2 * n + c2] : make_float2(0.f, 0.f);
+    b[y][tx] = (r2 < n && c2 < n) ? x[(long)r2 * n + c2] : zero;
   }
   __syncthreads();
   for (int y = threadIdx.y; y < 32; y += blockDim.y) {
     const int r = I * 32 + y, c = J * 32 + tx;
-    if (r < n && c < n) x[(long)r * n + c] = make_float2(a[y][tx].x + b[tx][y].x, a[y][tx].y - b[tx][y].y);
+    if (r < n && c < n) x[(long)r * n + c] = mk(a[y][tx].x + b[tx][y].x, a[y][tx].y - b[tx][y].y);
     const int r2 = J * 32 + y, c2 = I * 32 + tx;
-    if (I != J && r2 < n && c2 < n) x[(long)r2 * n + c2] = make_float2(b[y][tx].x + a[tx][y].x, b[y][tx].y - a[tx][y].y);
+    if (I != J && r2 < n && c2 < n) x[(long)r2 * n + c2] = mk(b[y][tx].x + a[tx][y].x, b[y][tx].y - a[tx][y].y);
   }
+}
+
+static gw_status launch_hermitize(gw_ctx* ctx, gw_prec prec, int n, int n_chi, void* chi_w, cudaStream_t s) {
+  const int nt = (n_chi + 31) / 32;
+  const long sx = (long)n_chi * n_chi;
+  if (is_fp64(prec))
+    hermitize_kernel<<<dim3(nt, nt, n), dim3(32, 8), 0, s>>>(static_cast<double2*>(chi_w), sx, n_chi);
+  else
+    hermitize_kernel<<<dim3(nt, nt, n), dim3(32, 8), 0, s>>>(static_cast<float2*>(chi_w), sx, n_chi);
+  return launch_check(ctx, "hermitize_kernel");
 }
 
 // Device tables of one chi0 evaluation.
@@ -116,6 +128,7 @@ static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ,
   void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false)) : nullptr;
   if (tcs_out) *tcs_out = tcs;
   bool first = true;
+  const bool low = row_low_ok(g, prec, n_chi);    // only R' <= r, and chi0 = X + X^H in the end
   for (int j = 0; j < n; ++j) {
     const GreenScales& gs = scales[j];
     const char* sj = t.scale + (size_t)j * n_b * 8;
@@ -124,15 +137,15 @@ static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ,
       const int rows = std::min(rb, g.nr - r0);
       if (tc) {
         if ((st = tc_chi_rows(ctx, g, n_b, n_occ, psi, gs, r0, rows, prec, ga, tcs, first, s,
-                              t.sk ? t.sk + (size_t)j * n_b : nullptr, t.status, true)))
+                              t.sk ? t.sk + (size_t)j * n_b : nullptr, t.status, low)))
           return st;
         first = false;
         st = launch_row_fft(ctx, g, prec, 1, ga, nullptr, g.nr, slab_j + (size_t)r0 * n_chi * es, n_chi, t.map, n_chi,
-                            rows, 1.0, s, t.inv, gb);
+                            rows, 1.0, s, t.inv, gb, low ? r0 : -1);
       } else {
-        if ((st = green_rows(ctx, g, n_b, n_occ, psi, sj, gs, r0, rows, prec, ga, gb, s))) return st;
+        if ((st = green_rows(ctx, g, n_b, n_occ, psi, sj, gs, r0, rows, prec, ga, gb, s, low ? r0 : -1))) return st;
         st = launch_row_fft(ctx, g, prec, 0, ga, gb, g.nr, slab_j + (size_t)r0 * n_chi * es, n_chi, t.map, n_chi,
-                            rows, -2.0, s, t.inv, ga);
+                            rows, -2.0, s, t.inv, ga, low ? r0 : -1);
       }
       if (st) return st;
     }
@@ -141,10 +154,7 @@ static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ,
   if ((st = launch_col_line_ct(ctx, g, prec, slabs, (long)slab, n_chi, n, t.cw, n, chi_w, (long)n_chi * n_chi, n_chi,
                                t.inv, n_chi, s, cw32.empty() ? nullptr : cw32.data())))
     return st;
-  if (!tc) return GW_OK;
-  const int nt = (n_chi + 31) / 32;
-  hermitize_kernel<<<dim3(nt, nt, n), dim3(32, 8), 0, s>>>(static_cast<float2*>(chi_w), (long)n_chi * n_chi, n_chi);
-  return launch_check(ctx, "hermitize_kernel");
+  return low ? launch_hermitize(ctx, prec, n, n_chi, chi_w, s) : GW_OK;
 }
 
 }  // namespace gw
@@ -172,11 +182,11 @@ extern "C" gw_status gw_chi0_omega(gw_ctx* ctx, const gw_grid* grid, int n_b, in
   chi0_tables(g, n_b, n_occ, eps_h, mu, n, tau_h, C_h, prec, scales, cw64, cw32);
   Carver cv(ctx->arena);
   int* dmap = cv.take<int>(n_chi);
-  int* dinv = cv.take<int>(g.nr);
+  int* dinv = cv.take<int>(inv_ints(g));
   char* dscale = cv.take<char>((size_t)n * n_b * 8);
   char* dcw = cv.take<char>((size_t)n * n * 8);
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
-  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * g.nr, s))) return st;
+  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if (is_fp64(prec)) st = upload(ctx, dcw, cw64.data(), sizeof(double) * n * n, s);
   else st = upload(ctx, dcw, cw32.data(), sizeof(float) * 2 * n * n, s);
   if (st) return st;
@@ -266,6 +276,7 @@ void pw_negate(const GridInfo& g, std::vector<int>& map, std::vector<int>& inv) 
   }
   std::fill(inv.begin(), inv.end(), -1);
   for (size_t j = 0; j < map.size(); ++j) inv[map[j]] = (int)j;
+  set_lists(g, inv);
 }
 
 gw_status pw_coefficients(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* psi, int n_b, int n_pw,
@@ -304,9 +315,9 @@ size_t chi0_pw_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_chi, 
   const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
   Carver probe(nullptr);
   probe.take<int>(n_chi);
-  probe.take<int>(g.nr);
+  probe.take<int>(inv_ints(g));
   probe.take<int>(n_pw);
-  probe.take<int>(g.nr);
+  probe.take<int>(inv_ints(g));
   probe.take<double>((size_t)n * n_b);
   probe.take<double>((size_t)n * n);
   probe.take<double>(2 * (size_t)n_b);
@@ -349,9 +360,9 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   chi0_tables(g, n_b, n_occ, eps_h, mu, n, tau_h, C_h, prec, scales, cw64, cw32);
   Carver cv(ctx->arena);
   int* dmap = cv.take<int>(n_chi);
-  int* dinv = cv.take<int>(g.nr);
+  int* dinv = cv.take<int>(inv_ints(g));
   int* dmap_pw = cv.take<int>(n_pw);
-  int* dinv_pw = cv.take<int>(g.nr);
+  int* dinv_pw = cv.take<int>(inv_ints(g));
   char* dscale = cv.take<char>((size_t)n * n_b * 8);
   char* dcw = cv.take<char>((size_t)n * n * 8);
   double* dnorm = cv.take<double>(2 * (size_t)n_b);
@@ -366,9 +377,9 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   const GridInfo gp = pw_grid(g, n_pw);
   void* tcs = tc ? cv.take<char>(tc_scratch_bytes(gp, n_b, n_occ, n_pw, false)) : nullptr;
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
-  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * g.nr, s))) return st;
+  if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if ((st = upload(ctx, dmap_pw, map_pw.data(), sizeof(int) * n_pw, s))) return st;
-  if ((st = upload(ctx, dinv_pw, inv_pw.data(), sizeof(int) * g.nr, s))) return st;
+  if ((st = upload(ctx, dinv_pw, inv_pw.data(), sizeof(int) * inv_pw.size(), s))) return st;
   if (is_fp64(prec)) st = upload(ctx, dcw, cw64.data(), sizeof(double) * n * n, s);
   else st = upload(ctx, dcw, cw32.data(), sizeof(float) * 2 * n * n, s);
   if (st) return st;
@@ -394,13 +405,14 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
     }
     // chi(r, G', tau_j) for every row r: expand, multiply (Eq. chi_rr), transform (Eq. FFTX1)
     char* slab_j = slabs + (size_t)j * slab * es;
-    if ((st = launch_row_pw_chi(ctx, g, prec, tu, to, n_pw, slab_j, n_chi, dinv_pw, n_pw, dinv, n_chi, g.nr, -2.0, s)))
+    if ((st = launch_row_pw_chi(ctx, g, prec, tu, to, n_pw, slab_j, n_chi, dinv_pw, n_pw, dinv, n_chi, g.nr, -2.0, s, 0)))
       return st;
     if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, n_chi, n_chi, 1.0, s))) return st;
   }
   if ((st = launch_col_line_ct(ctx, g, prec, slabs, (long)slab, n_chi, n, dcw, n, chi_w, (long)n_chi * n_chi, n_chi,
                                dinv, n_chi, s, cw32.empty() ? nullptr : cw32.data())))
     return st;
+  if ((st = launch_hermitize(ctx, prec, n, n_chi, chi_w, s))) return st;
   return tc ? tc_check(ctx, tcs, s) : GW_OK;
 }
 
@@ -445,7 +457,7 @@ extern "C" gw_status gw_chi0_plan_create(gw_ctx* ctx, const gw_grid* grid, int n
   const size_t o_map = probe.off;
   probe.take<int>(n_chi);
   const size_t o_inv = probe.off;
-  probe.take<int>(g.nr);
+  probe.take<int>(inv_ints(g));
   const size_t o_scale = probe.off;
   probe.take<char>((size_t)n * n_b * 8);
   const size_t o_sk = probe.off;
@@ -456,7 +468,7 @@ extern "C" gw_status gw_chi0_plan_create(gw_ctx* ctx, const gw_grid* grid, int n
   probe.take<int>(2);
   std::vector<char> host(probe.off, 0);
   std::memcpy(host.data() + o_map, map.data(), sizeof(int) * n_chi);
-  std::memcpy(host.data() + o_inv, inv.data(), sizeof(int) * g.nr);
+  std::memcpy(host.data() + o_inv, inv.data(), sizeof(int) * inv.size());
   for (int j = 0; j < n; ++j)
     for (int b = 0; b < n_b; ++b) {
       const double v = p->scales[j].s[b];

@@ -544,7 +544,7 @@ void sigma_carve_tables(Carver& cv, const GridInfo& g, int n_b, int n, int n_chi
                         SigmaTables& t) {
   const size_t nnm = full ? (size_t)n_n * n_n : (size_t)n_n;
   t.map = cv.take<int>(n_chi);
-  t.inv = cv.take<int>(g.nr);
+  t.inv = cv.take<int>(inv_ints(g));
   t.bands = cv.take<int>(n_n);
   t.scale = cv.take<char>((size_t)n * n_b * 8);
   t.tab = cv.take<double>(4 * (size_t)n * n + 2 * n + std::max(n_real, 1));
@@ -584,7 +584,7 @@ gw_status sigma_upload_tables(gw_ctx* ctx, const SigmaTables& t, const GridInfo&
                               const double* omega_h, const double* w_real_h, int n_real, gw_prec prec, cudaStream_t s) {
   gw_status st;
   if ((st = upload(ctx, t.map, map.data(), sizeof(int) * n_chi, s))) return st;
-  if ((st = upload(ctx, t.inv, inv.data(), sizeof(int) * g.nr, s))) return st;
+  if ((st = upload(ctx, t.inv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if ((st = upload(ctx, t.bands, bands_h, sizeof(int) * n_n, s))) return st;
   for (int j = 0; j < n; ++j)
     if ((st = upload_scales(ctx, t.scale + (size_t)j * n_b * 8, scales[j], prec, s))) return st;
@@ -629,9 +629,10 @@ gw_status sigma_kernels(gw_ctx* ctx, const GridInfo& g, gw_prec prec, bool full,
     for (int r0 = 0; r0 < g.nr; r0 += rb) {
       const int rows = std::min(rb, g.nr - r0);
       if (w.fused) {
-        // W~(r,R') of the block, then G formation with the contraction in its epilogue
+        // W~(r,R') of the block (as far as the tiles with R' <= r reach), then G formation with the
+        // contraction in its epilogue
         if ((st = launch_row_fft(ctx, g, prec, 2, w.wrg + (size_t)r0 * n_chi * es, nullptr, n_chi, w.wrr, g.nr, t.map,
-                                 n_chi, rows, 1.0, s, t.inv)))
+                                 n_chi, rows, 1.0, s, t.inv, nullptr, r0)))
           return st;
         TcSigma sg;
         sg.wrr = reinterpret_cast<const float2*>(w.wrr);
@@ -857,8 +858,8 @@ extern "C" gw_status gw_sigma_diag_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   auto carve = [&](Carver& cv) {
     sigma_carve_tables(cv, g, n_b, n, n_chi, n_n, n_real, false, t);
     dmap_neg = cv.take<int>(n_pw);
-    dinv_neg = cv.take<int>(g.nr);
-    dinv_nat = cv.take<int>(g.nr);
+    dinv_neg = cv.take<int>(inv_ints(g));
+    dinv_nat = cv.take<int>(inv_ints(g));
     dnorm = cv.take<double>(2 * (size_t)n_b);
     dc = cv.take<char>((size_t)n_b * n_pw * es);
     cn = cv.take<char>((size_t)n_n * n_pw * es);
@@ -885,8 +886,8 @@ extern "C" gw_status gw_sigma_diag_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
                                 n_real, prec, s)))
     return st;
   if ((st = upload(ctx, dmap_neg, map_neg.data(), sizeof(int) * n_pw, s))) return st;
-  if ((st = upload(ctx, dinv_neg, inv_neg.data(), sizeof(int) * g.nr, s))) return st;
-  if ((st = upload(ctx, dinv_nat, inv_nat.data(), sizeof(int) * g.nr, s))) return st;
+  if ((st = upload(ctx, dinv_neg, inv_neg.data(), sizeof(int) * inv_neg.size(), s))) return st;
+  if ((st = upload(ctx, dinv_nat, inv_nat.data(), sizeof(int) * inv_nat.size(), s))) return st;
   if ((st = pw_coefficients(ctx, g, prec, psi, n_b, n_pw, dmap_neg, dinv_neg, dc, dnorm, tmp, s))) return st;
   {
     const dim3 gg((n_pw + 255) / 256, n_n);

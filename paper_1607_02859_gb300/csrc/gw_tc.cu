@@ -85,7 +85,8 @@ struct Params {
   // MODE 0 and 2: only tiles with R' <= r (the grid row of the tile's rows is r0 + local row).
   // chi(r,R') and G(r,R') W~(r,R') are Hermitian in (r, R'): MODE 0 writes the lower triangle with
   // the diagonal halved (T, so that the transform of chi is X + X^H with X that of T) and zeros
-  // above; MODE 2 weights the strictly lower part 2 and the diagonal 1 (the real quadratic form).
+  // above it in the tiles on the diagonal; MODE 2 weights the strictly lower part 2 and the
+  // diagonal 1 (the real quadratic form).
   int lower;
 };
 
@@ -153,21 +154,7 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
   }
   const long grow0 = (long)p.r0 + m0;                 // grid row of the tile's first row
   if (MODE != 1 && p.lower && n0 >= grow0 + BM) {
-    // every R' of the tile is above every r: zeros (chi), or nothing (self-energy)
-    if (MODE == 0) {
-      for (int idx = threadIdx.x; idx < BM * (BNC / 2); idx += blockDim.x) {
-        const int row = idx / (BNC / 2), pc = 2 * (idx % (BNC / 2));
-        const int gm = m0 + row, gn = n0 + pc;
-        if (gm >= p.m_rows || gn >= p.n_cols) continue;
-        float2* o = p.out0 + (long)gm * p.ldo + gn;
-        if (gn + 1 < p.n_cols && ((reinterpret_cast<uintptr_t>(o) & 15) == 0)) {
-          *reinterpret_cast<float4*>(o) = make_float4(0.f, 0.f, 0.f, 0.f);
-        } else {
-          o[0] = make_float2(0.f, 0.f);
-          if (gn + 1 < p.n_cols) o[1] = make_float2(0.f, 0.f);
-        }
-      }
-    }
+    // every R' of the tile is above every r: nothing to do (the row transform takes them as zero)
     return;
   }
   const bool diag_tile = MODE != 1 && p.lower && n0 + BNC > grow0;   // the tile meets the diagonal
@@ -952,8 +939,8 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
     P.acc_o = sig->acc_o;
     P.acc_stride = sig->acc_stride;
   }
-  // lower-triangle self-energy: the column tiles past the block's last row hold no R' <= r
-  const int col_end = (mode == 2 && P.lower) ? std::min(g.nr, r0 + n_rows) : g.nr;
+  // the column tiles past the block's last row hold no R' <= r
+  const int col_end = P.lower ? std::min(g.nr, r0 + n_rows) : g.nr;
   const dim3 grid((col_end + BNC - 1) / BNC, (n_rows + BM - 1) / BM);
   // multiply-adds the launch performs: full tiles, or those meeting R' <= r
   double tiles = (double)grid.x * grid.y;

@@ -19,8 +19,9 @@ gw_status tc_green_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, cons
 // chi rows = -2 G_occ o conj(G_unocc) with both tiles accumulated in tensor memory.
 // sk_dev: the per-band factors gs.s already on the device as FP32 (then the
 // call copies nothing from the host).
-// lower: only R' <= r (grid rows r0 ..): the diagonal halved and zeros above it, whose
-// transform X gives chi(G,G') = X + X^H (chi is Hermitian in (r, R')).
+// lower: only R' <= r (grid rows r0 ..), with the diagonal halved; what lies above is not
+// all written (launch_row_fft with low takes it as zero).  Its transform X gives
+// chi(G,G') = X + X^H (chi is Hermitian in (r, R')).
 gw_status tc_chi_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales& gs,
                       int r0, int n_rows, gw_prec prec, void* chi, void* scratch, bool prep_b, cudaStream_t st,
                       const float* sk_dev = nullptr, int* status_dev = nullptr, bool lower = false);
