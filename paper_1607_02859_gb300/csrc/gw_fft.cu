@@ -258,193 +258,72 @@ __global__ void __launch_bounds__(RowCfg<T, N1, N2, N3>::TH, RowCfg<T, N1, N2, N
   }
 }
 
-// Rows too long for shared memory (36^3 = 46656 points, 373 KB) take two
-// passes through HBM.  The plane pass does the (i2, i3) 2-D transform of
-// kRowPlanes consecutive planes of one row per CTA; the line pass does the i1
-// transforms of one row per CTA in registers, with the G-set side of the row
-// (n_chi values) held in shared memory: forward, the results are scattered
-// there through inv and the row is written out in order; backward, the input
-// row is staged there and gathered through inv.
-constexpr int kRowPlanes = 4;
-
-// MODE 0: x = scale a conj(b) -> out;  MODE 1: x = a -> out;  MODE 2: out in place, times scale.
-template <typename T, int N1, int N2, int N3, int MODE, int DIR>
-__global__ void __launch_bounds__(256) row_plane_kernel(const typename cpx<T>::t* a,
-                                                        const typename cpx<T>::t* b, long lda,
-                                                        typename cpx<T>::t* out, long ldo, T scale) {
-  using C = typename cpx<T>::t;
-  constexpr int S2 = N3 % 2 == 0 ? N3 + 1 : N3;      // odd pencil stride
-  constexpr int PL = N2 * N3;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* s = reinterpret_cast<C*>(smem_raw);               // [kRowPlanes][N2][S2]
-  const long row = blockIdx.y;
-  const int i10 = blockIdx.x * kRowPlanes;
-  const int np = min(kRowPlanes, N1 - i10);
-  const long base = (long)i10 * PL;
-  for (int e = threadIdx.x; e < np * PL; e += blockDim.x) {
-    const int p = e / PL, rem = e - p * PL, i2 = rem / N3, i3 = rem - i2 * N3;
-    C v;
-    if (MODE == 2) {
-      v = out[row * ldo + base + e];
-    } else {
-      v = a[row * lda + base + e];
-      if (MODE == 0) v = cscale(cmulc(v, b[row * lda + base + e]), scale);
-    }
-    s[(p * N2 + i2) * S2 + i3] = v;
-  }
-  __syncthreads();
-  pencil_pass<N3, DIR>(s, np * N2, 1, [](int q) { return q * S2; });
-  __syncthreads();
-  pencil_pass<N2, DIR>(s, np * N3, S2, [](int q) { return (q / N3) * (N2 * S2) + (q % N3); });
-  __syncthreads();
-  for (int e = threadIdx.x; e < np * PL; e += blockDim.x) {
-    const int p = e / PL, rem = e - p * PL, i2 = rem / N3, i3 = rem - i2 * N3;
-    const C v = s[(p * N2 + i2) * S2 + i3];
-    out[row * ldo + base + e] = MODE == 2 ? cscale(v, scale) : v;
-  }
-}
-
-// Forward line pass: i1 transforms (+i) of tmp's row, the G set scattered into
-// shared memory through inv, then out[row][j], j < n_chi, in order.
+// Rows too long for one CTA's shared memory (36^3 = 46656 points, 373 KB) take two
+// kernels, and what passes between them is only the (i2, i3) columns that the G
+// set touches (n23 of N2 N3: 489 of 1296 for 8192 G vectors at 36^3):
+//   plane kernel: the (i2, i3) transforms of a few planes of one row per CTA;
+//   line kernel: the i1 transforms of the set's columns of one row per CTA, with
+//   the G-set side of the row in shared memory where it fits.
+// Column e of the set's list of plane i1 of a row lies at
+// row * t_row + i1 * t_plane + e of the workspace, which may be the grid-side
+// rows themselves (t_plane = N2 N3: a plane's columns lie at the start of the
+// plane).  Both kernels keep many small CTAs on an SM.  A thread-block cluster
+// holding the whole row in distributed shared memory (one pass over HBM, but 76
+// rows in flight, three cluster barriers and scattered remote accesses) took
+// 204 ns a row of the triangle at 36^3 with n_chi = 8192, these take 152 ns
+// forward and 128 ns backward; with all pencils of whole rows it was 340 ns.
 template <typename T, int N1, int N2, int N3>
-__global__ void __launch_bounds__(256) row_line_fwd_kernel(const typename cpx<T>::t* __restrict__ tmp, long ldt,
-                                                           typename cpx<T>::t* __restrict__ out, long ldo,
-                                                           const int* __restrict__ inv, int n_chi) {
-  using C = typename cpx<T>::t;
-  constexpr int PL = N2 * N3;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* so = reinterpret_cast<C*>(smem_raw);              // [n_chi]
-  const long row = blockIdx.x;
-  for (int i23 = threadIdx.x; i23 < PL; i23 += blockDim.x) {
-    C x[N1];
-#pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1) x[i1] = tmp[row * ldt + (long)i1 * PL + i23];
-    RegFFT<N1, +1>::run(x);
-#pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1) {
-      const int j = inv[i1 * PL + i23];
-      if (j >= 0) so[j] = x[i1];
-    }
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < n_chi; j += blockDim.x) out[row * ldo + j] = so[j];
-}
-
-// Backward line pass: a's row (n_chi values of the G set) staged in shared
-// memory, gathered through inv into the grid, i1 transforms (-i) into out.
-template <typename T, int N1, int N2, int N3>
-__global__ void __launch_bounds__(256) row_line_bwd_kernel(const typename cpx<T>::t* __restrict__ a, long lda,
-                                                           typename cpx<T>::t* __restrict__ out, long ldo,
-                                                           const int* __restrict__ inv, int n_chi) {
-  using C = typename cpx<T>::t;
-  constexpr int PL = N2 * N3;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* si = reinterpret_cast<C*>(smem_raw);              // [n_chi]
-  const long row = blockIdx.x;
-  for (int j = threadIdx.x; j < n_chi; j += blockDim.x) si[j] = a[row * lda + j];
-  __syncthreads();
-  for (int i23 = threadIdx.x; i23 < PL; i23 += blockDim.x) {
-    C x[N1];
-#pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1) {
-      const int j = inv[i1 * PL + i23];
-      x[i1] = j >= 0 ? si[j] : mk(T(0), T(0));
-    }
-    RegFFT<N1, -1>::run(x);
-#pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1) out[row * ldo + (long)i1 * PL + i23] = x[i1];
-  }
-}
-
-// Rows too long for one CTA's shared memory, split over a thread-block cluster
-// of CL CTAs: CTA c holds the planes i1 = c, c + CL, ... of the row (so that every
-// CTA has its share of the planes i1 <= i1(r) of a triangle's row) and the slice
-// [c n_s, (c+1) n_s) of its G-set side (n_s = ceil(n_chi / CL)).  The (i2, i3)
-// transforms run on the CTA's own planes; the i1 transforms of the set's
-// (i2, i3) columns are dealt out over the CTAs, which read and write the other
-// CTAs' planes and G-set slices through distributed shared memory.  Each element
-// crosses HBM once, as for the one-CTA rows, and the passes skip what the G set
-// and the triangle do not need in the same way.
-template <typename T, int N1, int N2, int N3>
-struct ClusterRow {
+struct PlaneCfg {
   using C = typename cpx<T>::t;
   static constexpr int S2 = N3 % 2 == 0 ? N3 + 1 : N3;
+  static constexpr int S1 = N2 * S2;
   static constexpr int PL = N2 * N3;
-  static constexpr size_t plane_bytes(int cl) { return (size_t)(N1 / cl) * N2 * S2 * sizeof(C); }
-  static constexpr bool fits(int cl) { return N1 % cl == 0 && plane_bytes(cl) + 32768 <= 200 * 1024; }
-  // the smallest cluster whose planes leave room for two CTAs per SM, else the smallest that fits
-  static constexpr int pick() {
-    for (int cl : {2, 4, 8})
-      if (fits(cl) && plane_bytes(cl) <= 96 * 1024) return cl;
-    for (int cl : {2, 4, 8})
-      if (fits(cl)) return cl;
-    return 0;
-  }
-  static constexpr int CL = pick();
-  static constexpr int P = CL ? N1 / CL : 1;
-  // half a thread per pencil of all local planes, rounded to warps
-  static constexpr int THREADS = CL ? (P * N2 / 2 + 31) / 32 * 32 : 32;
-  // planes: local planes that the launch's rows use
-  static size_t smem(int n_chi, int planes) {
-    return (size_t)planes * N2 * S2 * sizeof(C) + (size_t)((n_chi + CL - 1) / CL) * sizeof(C);
-  }
+  static constexpr int PP = N2 >= 40 ? 2 : 4;                      // planes per CTA
+  static constexpr int TH = (PP * N2 + 31) / 32 * 32;              // one pencil per thread and pass
+  static constexpr int MINB = sizeof(T) == 4 ? (N2 >= 30 ? 4 : 6) : 2;
+  static constexpr size_t bytes = (size_t)PP * S1 * sizeof(C);
+  static constexpr int LT = 128;                                    // threads of the line kernels
+  static constexpr int LMINB = sizeof(T) == 4 ? 4 : 2;
+  // the longest G-set row that the line kernels stage in shared memory (two CTAs per SM)
+  static constexpr size_t kStage = 110 * 1024;
 };
 
-// MODE 0 / 1 / 2 and low as for row_fft_kernel; grid (CL, rows), clusters of CL
-// along x; planes: the local planes of the largest row of the launch.
+// MODE 0 / 1 as for row_fft_kernel: planes of x = scale a conj(b) or a, (+i) over
+// i3 and the set's i3 of i2, the set's columns to t.  MODE 2: the columns from t,
+// (-i) over the set's i2 of i3 and i2, times scale, to the planes of out.
 template <typename T, int N1, int N2, int N3, int MODE, bool VEC>
-__global__ void __launch_bounds__(ClusterRow<T, N1, N2, N3>::THREADS, 2)
-    row_cluster_kernel(const typename cpx<T>::t* __restrict__ a, const typename cpx<T>::t* __restrict__ b, long lda,
-                       typename cpx<T>::t* __restrict__ out, long ldo, const int* __restrict__ inv, int n_chi,
-                       T scale, int low, int planes) {
-  namespace cg = cooperative_groups;
+__global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::TH, PlaneCfg<T, N1, N2, N3>::MINB)
+    row_plane_kernel(const typename cpx<T>::t* a, const typename cpx<T>::t* b, long lda, typename cpx<T>::t* t,
+                     long t_row, long t_plane, typename cpx<T>::t* out, long ldo, const int* __restrict__ inv, T scale,
+                     int low) {
   using C = typename cpx<T>::t;
-  using R = ClusterRow<T, N1, N2, N3>;
-  constexpr int PL = R::PL, S2 = R::S2, CL = R::CL, S1 = N2 * S2;
-  constexpr int TH = R::THREADS;
+  using R = PlaneCfg<T, N1, N2, N3>;
+  constexpr int PL = R::PL, S1 = R::S1, S2 = R::S2, TH = R::TH;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* s = reinterpret_cast<C*>(smem_raw);                         // [planes][N2][S2] own planes
-  C* gs = s + (size_t)planes * S1;                               // [n_s] own G-set slice
-  cg::cluster_group cluster = cg::this_cluster();
-  const int c = (int)cluster.block_rank();
+  C* s = reinterpret_cast<C*>(smem_raw);                           // [PP][N2][S2]
   const long row = blockIdx.y;
-  const SetLists<N1, N2, N3> g(inv);
-  const int n_s = (n_chi + CL - 1) / CL;
-  const int j0 = c * n_s, j1 = min(n_chi, j0 + n_s);
+  const int p0 = blockIdx.x * R::PP;
   const int last = MODE == 2 ? low_last_bwd(low, row, N1 * PL) : low_last_fwd(low, row, N1 * PL);
-  const int i1m = last / PL + 1;                                 // planes in use, of them here:
-  const int nloc = (i1m - c + CL - 1) / CL;                      // (c < CL, so i1m - c + CL - 1 >= 0)
-  const int q0s = g.n23 * c / CL, q1s = g.n23 * (c + 1) / CL;    // the CTA's share of the columns
-  auto plane_pos = [](int e) {                                   // e = p PL + i2 N3 + i3
+  const int np = min(R::PP, last / PL + 1 - p0);                   // planes of this CTA in use
+  if (np <= 0) return;
+  const SetLists<N1, N2, N3> g(inv);
+  auto pos = [](int e) {                                           // e = p PL + i2 N3 + i3
     const int p = e / PL, rem = e - p * PL, i2 = rem / N3;
     return p * S1 + i2 * S2 + (rem - i2 * N3);
   };
-  auto plane_base = [&](int e) { return (long)((e / PL) * CL + c) * PL + e % PL; };   // its place in the row
+  C* tp = t + row * t_row + (long)p0 * t_plane;
   if constexpr (MODE == 2) {
-    // the G-set slice, then i1 transforms of the CTA's columns into every CTA's planes
-    for (int j = j0 + threadIdx.x; j < j1; j += TH) gs[j - j0] = a[row * lda + j];
-    for (int e = threadIdx.x; e < nloc * S1; e += TH) s[e] = mk(T(0), T(0));
-    cluster.sync();
-    for (int e = q0s + threadIdx.x; e < q1s; e += TH) {
+    for (int e = threadIdx.x; e < np * S1; e += TH) s[e] = mk(T(0), T(0));
+    __syncthreads();
+    for (int e = threadIdx.x; e < g.n23; e += TH) {
       const int q = __ldg(g.l23 + e);
-      const int o23 = q / N3 * S2 + q % N3;
-      C x[N1];
+      const int o = q / N3 * S2 + q % N3;
 #pragma unroll
-      for (int i1 = 0; i1 < N1; ++i1) {
-        const int j = __ldg(inv + i1 * PL + q);
-        x[i1] = mk(T(0), T(0));
-        if (j >= 0) {
-          const int o = j / n_s;
-          x[i1] = cluster.map_shared_rank(gs, o)[j - o * n_s];
-        }
-      }
-      RegFFT<N1, -1>::run(x);
-#pragma unroll
-      for (int i1 = 0; i1 < N1; ++i1)
-        if (i1 < i1m) cluster.map_shared_rank(s, i1 % CL)[(i1 / CL) * S1 + o23] = x[i1];
+      for (int p = 0; p < R::PP; ++p)
+        if (p < np) s[p * S1 + o] = tp[p * t_plane + e];
     }
-    cluster.sync();                                              // no remote access after this point
-    for (int e = threadIdx.x; e < nloc * g.n2; e += TH) {        // pencils outside the set's i2 are zero
+    __syncthreads();
+    for (int e = threadIdx.x; e < np * g.n2; e += TH) {            // pencils outside the set's i2 are zero
       const int p = e / g.n2;
       const int o = p * S1 + __ldg(g.l2 + (e - p * g.n2)) * S2;
       C x[N3];
@@ -455,72 +334,64 @@ __global__ void __launch_bounds__(ClusterRow<T, N1, N2, N3>::THREADS, 2)
       for (int k = 0; k < N3; ++k) s[o + k] = x[k];
     }
     __syncthreads();
-    pencil_pass<N2, -1>(s, nloc * N3, S2, [](int q) { return (q / N3) * S1 + (q % N3); });
+    pencil_pass<N2, -1>(s, np * N3, S2, [](int q) { return (q / N3) * S1 + (q % N3); });
     __syncthreads();
-    C* dst = out + row * ldo;
+    C* dst = out + row * ldo + (long)p0 * PL;
     if (VEC) {
-      for (int q = threadIdx.x; q < nloc * PL / 2; q += TH) {
-        const int ps = plane_pos(2 * q);
-        st_pair(dst + plane_base(2 * q), cscale(s[ps], scale), cscale(s[ps + 1], scale));
+      for (int q = threadIdx.x; q < np * PL / 2; q += TH) {
+        const int o = pos(2 * q);
+        st_pair(dst + 2 * q, cscale(s[o], scale), cscale(s[o + 1], scale));
       }
     } else {
-      for (int e = threadIdx.x; e < nloc * PL; e += TH) dst[plane_base(e)] = cscale(s[plane_pos(e)], scale);
+      for (int e = threadIdx.x; e < np * PL; e += TH) dst[e] = cscale(s[pos(e)], scale);
     }
     return;
   }
-  // forward: the CTA's planes (with the product of Eq. chi_rr for MODE 0) ...
-  const C* pa = a + row * lda;
-  const C* pb = b + row * lda;
-  const int half = MODE == 0 && low >= 0 ? last : -1;
-  auto value = [&](C v, C w, long r) -> C {
-    if (r > last) return mk(T(0), T(0));
+  const int last0 = last - p0 * PL;                                // the last element in use, from the CTA's first
+  const int half = MODE == 0 && low >= 0 ? last0 : -1;
+  const C* pa = a + row * lda + (long)p0 * PL;
+  const C* pb = b + row * lda + (long)p0 * PL;
+  auto value = [&](C v, C w, int e) -> C {
+    if (e > last0) return mk(T(0), T(0));
     if (MODE != 0) return v;
-    return cscale(cmulc(v, w), r == half ? scale * T(0.5) : scale);
+    return cscale(cmulc(v, w), e == half ? scale * T(0.5) : scale);
   };
   if (VEC) {
-    const int np = nloc * PL / 2;
-    // the planes arrive in few round trips: LB 16-byte loads in flight per thread
-    // (the FFT's registers are free here)
-    constexpr int LB = MODE == 0 ? 6 : 12;
-    for (int qb = threadIdx.x; qb < np; qb += LB * TH) {
+    constexpr int LB = MODE == 0 ? 4 : 8;                          // 16-byte loads in flight per thread
+    for (int q0 = threadIdx.x; q0 < np * PL / 2; q0 += LB * TH) {
       C v[LB][2], w[LB][2];
 #pragma unroll
       for (int u = 0; u < LB; ++u) {
-        const int q = qb + u * TH;
+        const int q = q0 + u * TH;
         v[u][0] = v[u][1] = w[u][0] = w[u][1] = mk(T(0), T(0));
-        if (q < np) {
-          const long r = plane_base(2 * q);
-          if (r <= last) {
-            ld_pair(pa + r, v[u][0], v[u][1]);
-            if (MODE == 0) ld_pair(pb + r, w[u][0], w[u][1]);
-          }
+        if (q < np * PL / 2 && 2 * q <= last0) {
+          ld_pair_rw(pa + 2 * q, v[u][0], v[u][1]);
+          if (MODE == 0) ld_pair_rw(pb + 2 * q, w[u][0], w[u][1]);
         }
       }
 #pragma unroll
       for (int u = 0; u < LB; ++u) {
-        const int q = qb + u * TH;
-        if (q >= np) continue;
-        const int ps = plane_pos(2 * q);
-        const long r = plane_base(2 * q);
-        s[ps] = value(v[u][0], w[u][0], r);
-        s[ps + 1] = value(v[u][1], w[u][1], r + 1);
+        const int q = q0 + u * TH;
+        if (q >= np * PL / 2) continue;
+        const int o = pos(2 * q);
+        s[o] = value(v[u][0], w[u][0], 2 * q);
+        s[o + 1] = value(v[u][1], w[u][1], 2 * q + 1);
       }
     }
   } else {
-    for (int e = threadIdx.x; e < nloc * PL; e += TH) {
-      const long r = plane_base(e);
+    for (int e = threadIdx.x; e < np * PL; e += TH) {
       C v = mk(T(0), T(0)), w = v;
-      if (r <= last) {
-        v = pa[r];
-        if (MODE == 0) w = pb[r];
+      if (e <= last0) {
+        v = pa[e];
+        if (MODE == 0) w = pb[e];
       }
-      s[plane_pos(e)] = value(v, w, r);
+      s[pos(e)] = value(v, w, e);
     }
   }
   __syncthreads();
-  pencil_pass<N3, +1>(s, nloc * N2, 1, [](int q) { return q * S2; });
+  pencil_pass<N3, +1>(s, np * N2, 1, [](int q) { return q * S2; });
   __syncthreads();
-  for (int e = threadIdx.x; e < nloc * g.n3; e += TH) {
+  for (int e = threadIdx.x; e < np * g.n3; e += TH) {
     const int p = e / g.n3;
     const int o = p * S1 + __ldg(g.l3 + (e - p * g.n3));
     C x[N2];
@@ -530,27 +401,80 @@ __global__ void __launch_bounds__(ClusterRow<T, N1, N2, N3>::THREADS, 2)
 #pragma unroll
     for (int k = 0; k < N2; ++k) s[o + k * S2] = x[k];
   }
-  cluster.sync();
-  // ... i1 transforms of the CTA's columns, each result scattered to the G-set slice that holds it
-  for (int e = q0s + threadIdx.x; e < q1s; e += TH) {
+  __syncthreads();
+  for (int e = threadIdx.x; e < g.n23; e += TH) {
     const int q = __ldg(g.l23 + e);
-    const int o23 = q / N3 * S2 + q % N3;
+    const int o = q / N3 * S2 + q % N3;
+#pragma unroll
+    for (int p = 0; p < R::PP; ++p)
+      if (p < np) tp[p * t_plane + e] = s[p * S1 + o];
+  }
+}
+
+// Forward line pass of one row per CTA: i1 transforms (+i) of the set's columns,
+// the results to out[row][inv], in order through shared memory where STAGE.
+template <typename T, int N1, int N2, int N3, bool STAGE>
+__global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::LT, PlaneCfg<T, N1, N2, N3>::LMINB)
+    row_line_fwd_kernel(const typename cpx<T>::t* t, long t_row, long t_plane, typename cpx<T>::t* __restrict__ out,
+                        long ldo, const int* __restrict__ inv, int n_chi, int low) {
+  using C = typename cpx<T>::t;
+  constexpr int PL = N2 * N3, LT = PlaneCfg<T, N1, N2, N3>::LT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* so = reinterpret_cast<C*>(smem_raw);                          // [n_chi]
+  const long row = blockIdx.x;
+  const int i1m = low_last_fwd(low, row, N1 * PL) / PL + 1;
+  const SetLists<N1, N2, N3> g(inv);
+  C* o = STAGE ? so : out + row * ldo;
+  for (int e = threadIdx.x; e < g.n23; e += LT) {
+    const int q = __ldg(g.l23 + e);
     C x[N1];
 #pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1)
-      x[i1] = i1 < i1m ? cluster.map_shared_rank(s, i1 % CL)[(i1 / CL) * S1 + o23] : mk(T(0), T(0));
+    for (int i1 = 0; i1 < N1; ++i1) x[i1] = i1 < i1m ? t[row * t_row + i1 * t_plane + e] : mk(T(0), T(0));
     RegFFT<N1, +1>::run(x);
 #pragma unroll
     for (int i1 = 0; i1 < N1; ++i1) {
       const int j = __ldg(inv + i1 * PL + q);
-      if (j >= 0) {
-        const int o = j / n_s;
-        cluster.map_shared_rank(gs, o)[j - o * n_s] = x[i1];
-      }
+      if (j >= 0) o[j] = x[i1];
     }
   }
-  cluster.sync();                                                // no remote access after this point
-  for (int j = j0 + threadIdx.x; j < j1; j += TH) out[row * ldo + j] = gs[j - j0];
+  if (!STAGE) return;
+  __syncthreads();
+  for (int j = threadIdx.x; j < n_chi; j += LT) out[row * ldo + j] = so[j];
+}
+
+// Backward line pass: the row's n_chi values (through shared memory where STAGE)
+// gathered through inv, i1 transforms (-i) of the set's columns, the planes in use to t.
+template <typename T, int N1, int N2, int N3, bool STAGE>
+__global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::LT, PlaneCfg<T, N1, N2, N3>::LMINB)
+    row_line_bwd_kernel(const typename cpx<T>::t* __restrict__ a, long lda, typename cpx<T>::t* __restrict__ t,
+                        long t_row, long t_plane, const int* __restrict__ inv, int n_chi, int low, int fwd_rows) {
+  using C = typename cpx<T>::t;
+  constexpr int PL = N2 * N3, LT = PlaneCfg<T, N1, N2, N3>::LT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* si = reinterpret_cast<C*>(smem_raw);                          // [n_chi]
+  const long row = blockIdx.x;
+  const int last = fwd_rows ? low_last_fwd(low, row, N1 * PL) : low_last_bwd(low, row, N1 * PL);
+  const int i1m = last / PL + 1;
+  const SetLists<N1, N2, N3> g(inv);
+  const C* src = a + row * lda;
+  if (STAGE) {
+    for (int j = threadIdx.x; j < n_chi; j += LT) si[j] = src[j];
+    __syncthreads();
+    src = si;
+  }
+  for (int e = threadIdx.x; e < g.n23; e += LT) {
+    const int q = __ldg(g.l23 + e);
+    C x[N1];
+#pragma unroll
+    for (int i1 = 0; i1 < N1; ++i1) {
+      const int j = __ldg(inv + i1 * PL + q);
+      x[i1] = j >= 0 ? src[j] : mk(T(0), T(0));
+    }
+    RegFFT<N1, -1>::run(x);
+#pragma unroll
+    for (int i1 = 0; i1 < N1; ++i1)
+      if (i1 < i1m) t[row * t_row + i1 * t_plane + e] = x[i1];
+  }
 }
 
 // chi rows from the plane-wave form of G (the paper evaluates G in a plane-wave
@@ -560,15 +484,128 @@ __global__ void __launch_bounds__(ClusterRow<T, N1, N2, N3>::THREADS, 2)
 // (the column-transformed plane-wave G, length n_pw) are expanded over the grid
 // R' (backward transform), multiplied as
 //   x(R') = scale a(R') conj(b(R'))            (Eq. chi_rr)
-// and transformed forward onto the n_chi-long G set of chi (Eq. FFTX1).  Each
-// element of a row crosses HBM once: n_pw + n_pw values in, n_chi out.  The CL
-// CTAs of a cluster share a row as in row_cluster_kernel (CL = 1: one CTA), with
-// two plane buffers; the slices of the input rows and of the output row share
-// one region (the inputs are read before the first cluster barrier, the output
-// written after the third).  chi(r,R') is Hermitian: with low >= 0 only the planes
-// i1 <= i1(r) are expanded, the product is kept for R' <= r with half the
-// diagonal, and the caller adds the conjugate transpose in the end.  The passes
-// visit only the columns and pencils that the two G sets touch.
+// and transformed forward onto the n_chi-long G set of chi (Eq. FFTX1): the
+// backward line kernel for a and b, this kernel per plane (a few planes of both
+// rows in shared memory: (i2, i3) backward, product, forward), and the forward
+// line kernel.  Between them go only the columns that the sets touch, for a
+// chunk of rows that stays in L2.  chi(r,R') is Hermitian: with low >= 0 only the
+// planes i1 <= i1(r) are visited and the product is kept for R' <= r with half the
+// diagonal; the caller adds the conjugate transpose in the end.  One tau at 36^3
+// with 4224 plane waves and n_chi = 8192: 51.5 ms with a cluster of four CTAs per
+// whole row, 34.7 ms with that cluster on the triangle, 15.2 ms as here (FFT
+// instruction issue bounds it).
+template <typename T, int N1, int N2, int N3>
+struct PwPlane {
+  using C = typename cpx<T>::t;
+  using R = PlaneCfg<T, N1, N2, N3>;
+  static constexpr int PP = N2 >= 30 ? 2 : 4;
+  static constexpr int TH = (2 * PP * N2 + 31) / 32 * 32;          // one pencil of the two rows per thread
+  static constexpr int MINB = sizeof(T) == 4 ? (N2 >= 30 ? 4 : 3) : 1;
+  static constexpr size_t bytes = 2 * (size_t)PP * R::S1 * sizeof(C);
+};
+
+template <typename T, int N1, int N2, int N3>
+__global__ void __launch_bounds__(PwPlane<T, N1, N2, N3>::TH, PwPlane<T, N1, N2, N3>::MINB)
+    row_pw_plane_kernel(const typename cpx<T>::t* __restrict__ ta, const typename cpx<T>::t* __restrict__ tb,
+                        long ta_row, long ta_plane, typename cpx<T>::t* __restrict__ tx, long tx_row, long tx_plane,
+                        const int* __restrict__ inv_pw, const int* __restrict__ inv_chi, T scale, int low) {
+  using C = typename cpx<T>::t;
+  using R = PlaneCfg<T, N1, N2, N3>;
+  constexpr int PL = R::PL, S1 = R::S1, S2 = R::S2, PP = PwPlane<T, N1, N2, N3>::PP, TH = PwPlane<T, N1, N2, N3>::TH;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* sa = reinterpret_cast<C*>(smem_raw);                          // [PP][N2][S2] a, then x
+  C* sb = sa + PP * S1;                                            // [PP][N2][S2] b
+  const long row = blockIdx.y;
+  const int p0 = blockIdx.x * PP;
+  const int last = low_last_fwd(low, row, N1 * PL);
+  const int np = min(PP, last / PL + 1 - p0);
+  if (np <= 0) return;
+  const int last0 = last - p0 * PL;
+  const SetLists<N1, N2, N3> gp(inv_pw), gx(inv_chi);
+  for (int e = threadIdx.x; e < 2 * PP * S1; e += TH) sa[e] = mk(T(0), T(0));
+  __syncthreads();
+  {
+    const C* pa = ta + row * ta_row + (long)p0 * ta_plane;
+    const C* pb = tb + row * ta_row + (long)p0 * ta_plane;
+    for (int e = threadIdx.x; e < gp.n23; e += TH) {
+      const int q = __ldg(gp.l23 + e);
+      const int o = q / N3 * S2 + q % N3;
+#pragma unroll
+      for (int p = 0; p < PP; ++p)
+        if (p < np) {
+          sa[p * S1 + o] = pa[p * ta_plane + e];
+          sb[p * S1 + o] = pb[p * ta_plane + e];
+        }
+    }
+  }
+  __syncthreads();
+  {                                                                // pencils outside the set's i2 are zero
+    const int n = np * gp.n2;
+    for (int t = threadIdx.x; t < 2 * n; t += TH) {
+      const int e = t >= n ? t - n : t, p = e / gp.n2;
+      C* s = (t >= n ? sb : sa) + p * S1 + __ldg(gp.l2 + (e - p * gp.n2)) * S2;
+      C x[N3];
+#pragma unroll
+      for (int k = 0; k < N3; ++k) x[k] = s[k];
+      RegFFT<N3, -1>::run(x);
+#pragma unroll
+      for (int k = 0; k < N3; ++k) s[k] = x[k];
+    }
+  }
+  __syncthreads();
+  {
+    const int n = np * N3;
+    for (int t = threadIdx.x; t < 2 * n; t += TH) {
+      const int e = t >= n ? t - n : t;
+      C* s = (t >= n ? sb : sa) + e / N3 * S1 + e % N3;
+      C x[N2];
+#pragma unroll
+      for (int k = 0; k < N2; ++k) x[k] = s[k * S2];
+      RegFFT<N2, -1>::run(x);
+#pragma unroll
+      for (int k = 0; k < N2; ++k) s[k * S2] = x[k];
+    }
+  }
+  __syncthreads();
+  // the product of Eq. chi_rr as the input of the forward i2 pass, then the i3 pass of the set's pencils
+  for (int e = threadIdx.x; e < np * N3; e += TH) {
+    const int p = e / N3, i3 = e - p * N3, o = p * S1 + i3, r0 = p * PL + i3;
+    C x[N2];
+#pragma unroll
+    for (int k = 0; k < N2; ++k) {
+      const int r = r0 + k * N3;
+      x[k] = mk(T(0), T(0));
+      if (r <= last0)
+        x[k] = cscale(cmulc(sa[o + k * S2], sb[o + k * S2]), low >= 0 && r == last0 ? scale * T(0.5) : scale);
+    }
+    RegFFT<N2, +1>::run(x);
+#pragma unroll
+    for (int k = 0; k < N2; ++k) sa[o + k * S2] = x[k];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < np * gx.n2; e += TH) {
+    const int p = e / gx.n2;
+    C* s = sa + p * S1 + __ldg(gx.l2 + (e - p * gx.n2)) * S2;
+    C x[N3];
+#pragma unroll
+    for (int k = 0; k < N3; ++k) x[k] = s[k];
+    RegFFT<N3, +1>::run(x);
+#pragma unroll
+    for (int k = 0; k < N3; ++k) s[k] = x[k];
+  }
+  __syncthreads();
+  C* px = tx + row * tx_row + (long)p0 * tx_plane;
+  for (int e = threadIdx.x; e < gx.n23; e += TH) {
+    const int q = __ldg(gx.l23 + e);
+    const int o = q / N3 * S2 + q % N3;
+#pragma unroll
+    for (int p = 0; p < PP; ++p)
+      if (p < np) px[p * tx_plane + e] = sa[p * S1 + o];
+  }
+}
+
+// Rows too long for one CTA in the plane-wave self-energy: the CL CTAs of a
+// cluster share a row's planes and columns through distributed shared memory.
 template <typename T, int N1, int N2, int N3>
 struct PwRow {
   using C = typename cpx<T>::t;
@@ -589,10 +626,8 @@ struct PwRow {
     const size_t in = 2 * (size_t)((n_pw + CL - 1) / CL), out = (size_t)((n_chi + CL - 1) / CL);
     return in > out ? in : out;
   }
-  // planes: local planes that the launch's rows use
-  static size_t smem(int n_pw, int n_chi, int planes = P) {
-    return 2 * (size_t)planes * N2 * S2 * sizeof(C) + slice_elems(n_pw, n_chi) * sizeof(C);
-  }
+  // the sizes the plane-wave rows take: two expanded rows and their slices in a cluster's shared memory
+  static size_t smem(int n_pw, int n_chi) { return 2 * plane_bytes(CL) + slice_elems(n_pw, n_chi) * sizeof(C); }
   // row_pw_sigma_kernel: [T_occ | T_unocc | W~] slices in, hu and ho out over the last two
   static size_t sig_smem(int n_pw, int n_chi) {
     const size_t ps = (size_t)((n_pw + CL - 1) / CL), ws = (size_t)((n_chi + CL - 1) / CL);
@@ -600,148 +635,6 @@ struct PwRow {
     return 2 * plane_bytes(CL) + e * sizeof(C);
   }
 };
-
-template <typename T, int N1, int N2, int N3>
-__global__ void __launch_bounds__(PwRow<T, N1, N2, N3>::THREADS)
-    row_pw_chi_kernel(const typename cpx<T>::t* __restrict__ a, const typename cpx<T>::t* __restrict__ b, long lda,
-                      typename cpx<T>::t* __restrict__ out, long ldo, const int* __restrict__ inv_pw, int n_pw,
-                      const int* __restrict__ inv_chi, int n_chi, T scale, int low, int planes) {
-  namespace cg = cooperative_groups;
-  using C = typename cpx<T>::t;
-  using R = PwRow<T, N1, N2, N3>;
-  constexpr int PL = R::PL, S2 = R::S2, CL = R::CL, S1 = N2 * S2;
-  constexpr int TH = R::THREADS;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* sa = reinterpret_cast<C*>(smem_raw);                              // [planes][N2][S2] a, then x
-  C* sb = sa + (size_t)planes * S1;                                    // [planes][N2][S2] b
-  C* sl = sb + (size_t)planes * S1;                                    // slices
-  cg::cluster_group cluster = cg::this_cluster();
-  const int c = (int)cluster.block_rank();
-  const long row = blockIdx.y;
-  const SetLists<N1, N2, N3> gp(inv_pw), gx(inv_chi);
-  const int n_ps = (n_pw + CL - 1) / CL, n_cs = (n_chi + CL - 1) / CL;
-  const int last = low_last_fwd(low, row, N1 * PL);
-  const int i1m = last / PL + 1;                // planes in use, dealt out i1 = c, c + CL, ...
-  const int nloc = (i1m - c + CL - 1) / CL;
-  C* su = sl;                 // [n_ps] this CTA's part of a's row
-  C* so = sl + n_ps;          // [n_ps] of b's row
-  {
-    const int j0 = c * n_ps, j1 = min(n_pw, j0 + n_ps);
-    for (int j = j0 + threadIdx.x; j < j1; j += TH) {
-      su[j - j0] = a[row * lda + j];
-      so[j - j0] = b[row * lda + j];
-    }
-    for (int e = threadIdx.x; e < nloc * S1; e += TH) sa[e] = sb[e] = mk(T(0), T(0));
-  }
-  cluster.sync();
-  // backward i1 transforms of the CTA's share of the set's columns, for both rows, into every CTA's planes
-  {
-    const int e0 = gp.n23 * c / CL, e1 = gp.n23 * (c + 1) / CL, ne = e1 - e0;
-    for (int t = threadIdx.x; t < 2 * ne; t += TH) {
-      const bool second = t >= ne;
-      const int q = __ldg(gp.l23 + e0 + (second ? t - ne : t));
-      const int o23 = q / N3 * S2 + q % N3;
-      C* src = second ? so : su;
-      C* dst = second ? sb : sa;
-      C x[N1];
-#pragma unroll
-      for (int i1 = 0; i1 < N1; ++i1) {
-        const int j = __ldg(inv_pw + i1 * PL + q);
-        x[i1] = mk(T(0), T(0));
-        if (j >= 0) {
-          const int o = j / n_ps;
-          x[i1] = cluster.map_shared_rank(src, o)[j - o * n_ps];
-        }
-      }
-      RegFFT<N1, -1>::run(x);
-#pragma unroll
-      for (int i1 = 0; i1 < N1; ++i1)
-        if (i1 < i1m) cluster.map_shared_rank(dst, i1 % CL)[(i1 / CL) * S1 + o23] = x[i1];
-    }
-  }
-  cluster.sync();                  // the planes are complete and the input slices free
-  // (i2, i3) backward transforms of the CTA's planes, both rows (pencils outside the set's i2 are zero)
-  auto both = [&](int t, int n) { return t >= n ? sb : sa; };
-  {
-    const int n = nloc * gp.n2;
-    for (int t = threadIdx.x; t < 2 * n; t += TH) {
-      const int e = t >= n ? t - n : t, p = e / gp.n2;
-      C* s = both(t, n) + p * S1 + __ldg(gp.l2 + (e - p * gp.n2)) * S2;
-      C x[N3];
-#pragma unroll
-      for (int k = 0; k < N3; ++k) x[k] = s[k];
-      RegFFT<N3, -1>::run(x);
-#pragma unroll
-      for (int k = 0; k < N3; ++k) s[k] = x[k];
-    }
-  }
-  __syncthreads();
-  {
-    const int n = nloc * N3;
-    for (int t = threadIdx.x; t < 2 * n; t += TH) {
-      const int e = t >= n ? t - n : t;
-      C* s = both(t, n) + e / N3 * S1 + e % N3;
-      C x[N2];
-#pragma unroll
-      for (int k = 0; k < N2; ++k) x[k] = s[k * S2];
-      RegFFT<N2, -1>::run(x);
-#pragma unroll
-      for (int k = 0; k < N2; ++k) s[k * S2] = x[k];
-    }
-  }
-  __syncthreads();
-  // the product of Eq. chi_rr taken into the forward i2 pass, then the i3 pass of the set's pencils
-  for (int e = threadIdx.x; e < nloc * N3; e += TH) {
-    const int p = e / N3, i3 = e - p * N3, o = p * S1 + i3;
-    const int r0 = (p * CL + c) * PL + i3;               // grid position of k = 0
-    C x[N2];
-#pragma unroll
-    for (int k = 0; k < N2; ++k) {
-      const int r = r0 + k * N3;
-      x[k] = mk(T(0), T(0));
-      if (r <= last) x[k] = cscale(cmulc(sa[o + k * S2], sb[o + k * S2]), low >= 0 && r == last ? scale * T(0.5) : scale);
-    }
-    RegFFT<N2, +1>::run(x);
-#pragma unroll
-    for (int k = 0; k < N2; ++k) sa[o + k * S2] = x[k];
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < nloc * gx.n2; e += TH) {
-    const int p = e / gx.n2;
-    C* s = sa + p * S1 + __ldg(gx.l2 + (e - p * gx.n2)) * S2;
-    C x[N3];
-#pragma unroll
-    for (int k = 0; k < N3; ++k) x[k] = s[k];
-    RegFFT<N3, +1>::run(x);
-#pragma unroll
-    for (int k = 0; k < N3; ++k) s[k] = x[k];
-  }
-  cluster.sync();                  // every CTA's x planes are final
-  // forward i1 transforms of the CTA's columns, each result into the slice of chi that holds it
-  C* sx = sl;                      // [n_cs] this CTA's part of the chi row
-  for (int e = gx.n23 * c / CL + threadIdx.x; e < gx.n23 * (c + 1) / CL; e += TH) {
-    const int q = __ldg(gx.l23 + e);
-    const int o23 = q / N3 * S2 + q % N3;
-    C x[N1];
-#pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1)
-      x[i1] = i1 < i1m ? cluster.map_shared_rank(sa, i1 % CL)[(i1 / CL) * S1 + o23] : mk(T(0), T(0));
-    RegFFT<N1, +1>::run(x);
-#pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1) {
-      const int j = __ldg(inv_chi + i1 * PL + q);
-      if (j >= 0) {
-        const int o = j / n_cs;
-        cluster.map_shared_rank(sx, o)[j - o * n_cs] = x[i1];
-      }
-    }
-  }
-  cluster.sync();                  // no remote access after this point
-  {
-    const int j0 = c * n_cs, j1 = min(n_chi, j0 + n_cs);
-    for (int j = j0 + threadIdx.x; j < j1; j += TH) out[row * ldo + j] = sx[j - j0];
-  }
-}
 
 // The self-energy's rows in the same plane-wave form (first term of Eq.
 // Sigma_occ_reduce with Eq. Sigma_rr): for each row r, the W~ row over chi's G
@@ -1155,44 +1048,73 @@ static gw_status set_smem(gw_ctx* ctx, K kernel, size_t bytes) {
 template <typename T, int N1, int N2, int N3>
 struct GridOps {
   using C = typename cpx<T>::t;
-  static gw_status row_two_pass(gw_ctx* ctx, int mode, const void* a, const void* b, long lda, void* out, long ldo,
-                                const int* inv, void* tmp, int n_chi, int n_rows, double scale, cudaStream_t st) {
-    constexpr int NR = N1 * N2 * N3;
-    constexpr int S2 = N3 % 2 == 0 ? N3 + 1 : N3;
-    const size_t pbytes = (size_t)kRowPlanes * N2 * S2 * sizeof(C);
-    const size_t lbytes = (size_t)n_chi * sizeof(C);
-    if (!inv || (mode != 2 && !tmp))
-      return fail(ctx, GW_ERR_UNSUPPORTED, "this grid's rows need the two-pass transform (index map and workspace)");
-    if (lbytes > 200 * 1024) return fail(ctx, GW_ERR_UNSUPPORTED, "G set too large for the two-pass row transform");
-    const dim3 pgrid((N1 + kRowPlanes - 1) / kRowPlanes, n_rows);
-    const double rd = mode == 0 ? 2.0 * NR : (mode == 1 ? NR : n_chi);
-    const double wr = mode == 2 ? NR : n_chi;
-    gw_status rc;
-    auto plane = [&](auto kernel, const void* pa, const void* pb, long pld, void* po, long pldo) -> gw_status {
-      gw_status r = set_smem(ctx, kernel, pbytes);
+  using PC = PlaneCfg<T, N1, N2, N3>;
+  static gw_status line_fwd(gw_ctx* ctx, const void* t, long t_row, long t_plane, void* out, long ldo, const int* inv,
+                            int n_chi, int n_rows, int low, double work, int fam, cudaStream_t st) {
+    const size_t bytes = (size_t)n_chi * sizeof(C);
+    auto go = [&](auto kernel, size_t sm) -> gw_status {
+      gw_status r = set_smem(ctx, kernel, sm);
       if (r) return r;
-      KTimer kt(ctx, KF_ROW_FFT, 0.0, st);
-      kernel<<<pgrid, 256, pbytes, st>>>((const C*)pa, (const C*)pb, pld, (C*)po, pldo, (T)scale);
+      KTimer kt(ctx, fam, work, st);
+      kernel<<<n_rows, PC::LT, sm, st>>>((const C*)t, t_row, t_plane, (C*)out, ldo, inv, n_chi, low);
+      return launch_check(ctx, "row_line_fwd_kernel");
+    };
+    return bytes <= PC::kStage ? go(row_line_fwd_kernel<T, N1, N2, N3, true>, bytes)
+                               : go(row_line_fwd_kernel<T, N1, N2, N3, false>, 0);
+  }
+  static gw_status line_bwd(gw_ctx* ctx, const void* a, long lda, void* t, long t_row, long t_plane, const int* inv,
+                            int n_chi, int n_rows, int low, bool fwd_rows, double work, int fam, cudaStream_t st) {
+    const size_t bytes = (size_t)n_chi * sizeof(C);
+    auto go = [&](auto kernel, size_t sm) -> gw_status {
+      gw_status r = set_smem(ctx, kernel, sm);
+      if (r) return r;
+      KTimer kt(ctx, fam, work, st);
+      kernel<<<n_rows, PC::LT, sm, st>>>((const C*)a, lda, (C*)t, t_row, t_plane, inv, n_chi, low, fwd_rows ? 1 : 0);
+      return launch_check(ctx, "row_line_bwd_kernel");
+    };
+    return bytes <= PC::kStage ? go(row_line_bwd_kernel<T, N1, N2, N3, true>, bytes)
+                               : go(row_line_bwd_kernel<T, N1, N2, N3, false>, 0);
+  }
+  // planes of the launch's longest row
+  static int row_planes(int low, int n_rows, bool bwd) {
+    if (low < 0) return N1;
+    const int g0 = low + (n_rows - 1) / 128 * 128;
+    const int last = bwd ? (g0 + 127) / 128 * 128 + 127 : low + n_rows - 1;
+    return std::min(N1, last / PC::PL + 1);
+  }
+  static gw_status row_two_pass(gw_ctx* ctx, int mode, const void* a, const void* b, long lda, void* out, long ldo,
+                                const int* inv, void* tmp, int n_chi, int n_rows, double scale, cudaStream_t st,
+                                bool vec, int low, double work) {
+    constexpr int NR = N1 * N2 * N3;
+    if (mode != 2 && !tmp)
+      return fail(ctx, GW_ERR_UNSUPPORTED, "this grid's rows need the two-pass transform (index map and workspace)");
+    if (sizeof(T) == 8 && (size_t)n_chi * sizeof(C) > 200 * 1024)
+      return fail(ctx, GW_ERR_UNSUPPORTED, "G set too large for the two-pass row transform");
+    const dim3 pgrid((row_planes(low, n_rows, mode == 2) + PC::PP - 1) / PC::PP, n_rows);
+    auto plane = [&](auto kernel, void* t, long t_row) -> gw_status {
+      gw_status r = set_smem(ctx, kernel, PC::bytes);
+      if (r) return r;
+      KTimer kt(ctx, KF_ROW_FFT, work, st);
+      kernel<<<pgrid, PC::TH, PC::bytes, st>>>((const C*)a, (const C*)b, lda, (C*)t, t_row, (long)PC::PL, (C*)out, ldo,
+                                               inv, (T)scale, low);
       return launch_check(ctx, "row_plane_kernel");
     };
+    constexpr bool E = N3 % 2 == 0;
+    gw_status rc;
     if (mode == 2) {
-      auto kl = row_line_bwd_kernel<T, N1, N2, N3>;
-      if ((rc = set_smem(ctx, kl, lbytes))) return rc;
-      {
-        KTimer kt(ctx, KF_ROW_FFT, (double)n_rows * (rd + wr) * sizeof(C), st);
-        kl<<<n_rows, 256, lbytes, st>>>((const C*)a, lda, (C*)out, ldo, inv, n_chi);
-        if ((rc = launch_check(ctx, "row_line_bwd_kernel"))) return rc;
-      }
-      return plane(row_plane_kernel<T, N1, N2, N3, 2, -1>, nullptr, nullptr, 0, out, ldo);
+      // the columns lie in out itself, at the start of each plane
+      if ((rc = line_bwd(ctx, a, lda, out, ldo, PC::PL, inv, n_chi, n_rows, low, false, 0.0, KF_ROW_FFT, st))) return rc;
+      return vec ? plane(row_plane_kernel<T, N1, N2, N3, 2, E>, out, ldo)
+                 : plane(row_plane_kernel<T, N1, N2, N3, 2, false>, out, ldo);
     }
-    if (mode == 0) rc = plane(row_plane_kernel<T, N1, N2, N3, 0, +1>, a, b, lda, tmp, NR);
-    else rc = plane(row_plane_kernel<T, N1, N2, N3, 1, +1>, a, nullptr, lda, tmp, NR);
+    if (mode == 0)
+      rc = vec ? plane(row_plane_kernel<T, N1, N2, N3, 0, E>, tmp, NR)
+               : plane(row_plane_kernel<T, N1, N2, N3, 0, false>, tmp, NR);
+    else
+      rc = vec ? plane(row_plane_kernel<T, N1, N2, N3, 1, E>, tmp, NR)
+               : plane(row_plane_kernel<T, N1, N2, N3, 1, false>, tmp, NR);
     if (rc) return rc;
-    auto kl = row_line_fwd_kernel<T, N1, N2, N3>;
-    if ((rc = set_smem(ctx, kl, lbytes))) return rc;
-    KTimer kt(ctx, KF_ROW_FFT, (double)n_rows * (rd + wr) * sizeof(C), st);
-    kl<<<n_rows, 256, lbytes, st>>>((const C*)tmp, NR, (C*)out, ldo, inv, n_chi);
-    return launch_check(ctx, "row_line_fwd_kernel");
+    return line_fwd(ctx, tmp, NR, PC::PL, out, ldo, inv, n_chi, n_rows, low, 0.0, KF_ROW_FFT, st);
   }
   static gw_status row(gw_ctx* ctx, int mode, const void* a, const void* b, long lda, void* out, long ldo,
                        const int* map, int n_chi, int n_rows, double scale, cudaStream_t st, const int* inv,
@@ -1213,53 +1135,8 @@ struct GridOps {
     const bool vi = mode == 2 ? al(out) && ldo % 2 == 0 && N3 % 2 == 0 : al(a) && al(b) && lda % 2 == 0 && N3 % 2 == 0;
     const bool vo = mode != 2 && al(out) && ldo % 2 == 0 && n_chi % 2 == 0;
     if (!inv) return fail(ctx, GW_ERR_ARG, "row transform without the G set's inverse map");
-    if (bytes > kRowSmemMax) {
-      using CR = ClusterRow<T, N1, N2, N3>;
-      if constexpr (CR::CL > 0 && L::TOT * sizeof(C) > kRowSmemMax) {
-        if (CR::smem(n_chi, CR::P) <= kRowSmemMax) {
-          // local planes of the launch's last row
-          int planes = CR::P;
-          if (low >= 0) {
-            const int g0 = low + (n_rows - 1) / 128 * 128;
-            const int last = mode == 2 ? std::min(L::NR - 1, (g0 + 127) / 128 * 128 + 127) : low + n_rows - 1;
-            planes = (last / (N2 * N3) + CR::CL) / CR::CL;
-          }
-          const size_t cbytes = CR::smem(n_chi, planes);
-          auto go = [&](auto kernel) -> gw_status {
-            gw_status s = set_smem(ctx, kernel, cbytes);
-            if (s) return s;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(CR::CL, (unsigned)n_rows);
-            cfg.blockDim = dim3(CR::THREADS);
-            cfg.dynamicSmemBytes = cbytes;
-            cfg.stream = st;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = CR::CL;
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            KTimer kt(ctx, KF_ROW_FFT, work, st);
-            gw_status r = cuda_check(ctx, cudaLaunchKernelEx(&cfg, kernel, (const C*)a, (const C*)b, lda, (C*)out, ldo,
-                                                             inv, n_chi, (T)scale, low, planes),
-                                     "cudaLaunchKernelEx(row_cluster_kernel)");
-            if (r) return r;
-            return launch_check(ctx, "row_cluster_kernel");
-          };
-#define GW_ROWC_GO(M)                                                                       \
-          if (mode == M) return vi ? go(row_cluster_kernel<T, N1, N2, N3, M, N3 % 2 == 0>)  \
-                                   : go(row_cluster_kernel<T, N1, N2, N3, M, false>);
-          GW_ROWC_GO(0)
-          GW_ROWC_GO(1)
-          GW_ROWC_GO(2)
-#undef GW_ROWC_GO
-          return fail(ctx, GW_ERR_ARG, "bad row transform mode");
-        }
-      }
-      if (low >= 0 && mode != 2) return fail(ctx, GW_ERR_UNSUPPORTED, "triangle rows need the one-pass row transform");
-      return row_two_pass(ctx, mode, a, b, lda, out, ldo, inv, tmp, n_chi, n_rows, scale, st);
-    }
+    if constexpr (L::TOT * sizeof(C) > kRowSmemMax)
+      return row_two_pass(ctx, mode, a, b, lda, out, ldo, inv, tmp, n_chi, n_rows, scale, st, vi, low, work);
     if constexpr (L::TOT * sizeof(C) <= kRowSmemMax) {
       auto go = [&](auto kernel) -> gw_status {
         gw_status s = set_smem(ctx, kernel, bytes);
@@ -1283,78 +1160,44 @@ struct GridOps {
     }
     return fail(ctx, GW_ERR_ARG, "bad row transform mode");
   }
-  // whether rows of the triangle R' <= r have a kernel (all but the two-pass FP64 rows)
-  static bool row_low_ok(int n_chi) {
-    using CR = ClusterRow<T, N1, N2, N3>;
-    if (RowLayout<N1, N2, N3>::TOT * sizeof(C) <= kRowSmemMax) return true;
-    if constexpr (CR::CL > 0) return CR::smem(n_chi, CR::P) <= kRowSmemMax;
-    return false;
-  }
   static bool row_pw_ok(int n_pw, int n_chi) {
     using PR = PwRow<T, N1, N2, N3>;
     if constexpr (PR::CL > 0) return PR::smem(n_pw, n_chi) <= kRowSmemMax;
     return false;
   }
   static gw_status row_pw(gw_ctx* ctx, const void* a, const void* b, long lda, void* out, long ldo,
-                           const int* inv_pw, int n_pw, const int* inv_chi, int n_chi, int n_rows, double scale,
-                           cudaStream_t st, int low) {
-    using PR = PwRow<T, N1, N2, N3>;
-    if constexpr (PR::CL > 0) {
-      if (PR::smem(n_pw, n_chi) > kRowSmemMax)
-        return fail(ctx, GW_ERR_UNSUPPORTED, "plane-wave chi rows: G sets too large for this grid");
-      if (low >= 0) {
-        // rows of equal local plane counts go together: the shorter ones need less shared memory,
-        // so more of them share an SM
-        constexpr int step = PR::CL * N2 * N3;
-        const int end = std::min(N1 * N2 * N3, low + n_rows);
-        for (int r = low; r < end;) {
-          const int to = std::min(end, (r / step + 1) * step);
-          const long o = r - low;
-          gw_status s = row_pw_part(ctx, (const C*)a + o * lda, (const C*)b + o * lda, lda, (C*)out + o * ldo, ldo,
-                                    inv_pw, n_pw, inv_chi, n_chi, to - r, scale, st, r, r / step + 1);
-          if (s) return s;
-          r = to;
-        }
-        return GW_OK;
-      }
-      return row_pw_part(ctx, (const C*)a, (const C*)b, lda, (C*)out, ldo, inv_pw, n_pw, inv_chi, n_chi, n_rows, scale,
-                         st, -1, PR::P);
-    } else {
+                          const int* inv_pw, int n_pw, int pw_cols, const int* inv_chi, int n_chi, int chi_cols,
+                          int n_rows, double scale, cudaStream_t st, int low, void* work) {
+    if (!row_pw_ok(n_pw, n_chi))
       return fail(ctx, GW_ERR_UNSUPPORTED, "plane-wave chi rows: no cluster split fits this grid and precision");
+    using PP = PwPlane<T, N1, N2, N3>;
+    auto kernel = row_pw_plane_kernel<T, N1, N2, N3>;
+    gw_status s = set_smem(ctx, kernel, PP::bytes);
+    if (s) return s;
+    const int ch = std::min(n_rows, kPwChunk);
+    const long tp = pw_cols, tr = (long)N1 * tp, xp = chi_cols, xr = (long)N1 * xp;
+    C* ta = static_cast<C*>(work);
+    C* tb = ta + ch * tr;
+    C* tx = tb + ch * tr;
+    const double nr = (double)N1 * N2 * N3;
+    for (int r = 0; r < n_rows; r += ch) {
+      const int rows = std::min(ch, n_rows - r), lo = low >= 0 ? low + r : -1;
+      // ALU work: three transforms of N_r points (5 N log2 N each) and the product per row, booked on the planes
+      const C* pa = static_cast<const C*>(a) + (long)r * lda;
+      const C* pb = static_cast<const C*>(b) + (long)r * lda;
+      if ((s = line_bwd(ctx, pa, lda, ta, tr, tp, inv_pw, n_pw, rows, lo, true, 0.0, KF_ROW_PW, st))) return s;
+      if ((s = line_bwd(ctx, pb, lda, tb, tr, tp, inv_pw, n_pw, rows, lo, true, 0.0, KF_ROW_PW, st))) return s;
+      {
+        const dim3 grid((row_planes(lo, rows, false) + PP::PP - 1) / PP::PP, rows);
+        KTimer kt(ctx, KF_ROW_PW, (double)rows * (3.0 * 5.0 * nr * std::log2(nr) + 6.0 * nr), st);
+        kernel<<<grid, PP::TH, PP::bytes, st>>>(ta, tb, tr, tp, tx, xr, xp, inv_pw, inv_chi, (T)scale, lo);
+        if ((s = launch_check(ctx, "row_pw_plane_kernel"))) return s;
+      }
+      if ((s = line_fwd(ctx, tx, xr, xp, static_cast<C*>(out) + (long)r * ldo, ldo, inv_chi, n_chi, rows, lo, 0.0,
+                        KF_ROW_PW, st)))
+        return s;
     }
-  }
-  static gw_status row_pw_part(gw_ctx* ctx, const C* a, const C* b, long lda, C* out, long ldo, const int* inv_pw,
-                               int n_pw, const int* inv_chi, int n_chi, int n_rows, double scale, cudaStream_t st,
-                               int low, int planes) {
-    using PR = PwRow<T, N1, N2, N3>;
-    if constexpr (PR::CL > 0) {
-      const size_t bytes = PR::smem(n_pw, n_chi, planes);
-      auto kernel = row_pw_chi_kernel<T, N1, N2, N3>;
-      gw_status s = set_smem(ctx, kernel, bytes);
-      if (s) return s;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(PR::CL, (unsigned)n_rows);
-      cfg.blockDim = dim3(PR::THREADS);
-      cfg.dynamicSmemBytes = bytes;
-      cfg.stream = st;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = PR::CL;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      // FP32/FP64 ALU work: three transforms of N_r points (5 N log2 N each) and the product per row
-      const double nr = (double)N1 * N2 * N3;
-      KTimer kt(ctx, KF_ROW_PW, (double)n_rows * (3.0 * 5.0 * nr * std::log2(nr) + 6.0 * nr), st);
-      s = cuda_check(ctx, cudaLaunchKernelEx(&cfg, kernel, a, b, lda, out, ldo, inv_pw, n_pw,
-                                             inv_chi, n_chi, (T)scale, low, planes),
-                     "cudaLaunchKernelEx(row_pw_chi_kernel)");
-      if (s) return s;
-      return launch_check(ctx, "row_pw_chi_kernel");
-    } else {
-      return GW_ERR_UNSUPPORTED;
-    }
+    return GW_OK;
   }
   static bool row_pw_sigma_ok(int n_pw, int n_chi) {
     using PR = PwRow<T, N1, N2, N3>;
@@ -1493,18 +1336,16 @@ gw_status launch_row_fft(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int mode,
   GW_DISPATCH(prec, g, rc = O::row(ctx, mode, a, b, lda, out, ldo, map, n_chi, n_rows, scale, st, inv, tmp, low))
 }
 
-bool row_low_ok(const GridInfo& g, gw_prec prec, int n_chi) {
-  bool ok = false;
-  if (is_fp64(prec)) with_grid<double>(g, [&](auto ops) { ok = decltype(ops)::row_low_ok(n_chi); });
-  else with_grid<float>(g, [&](auto ops) { ok = decltype(ops)::row_low_ok(n_chi); });
-  return ok;
+gw_status launch_row_pw_chi(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* a, const void* b, long lda,
+                            void* out, long ldo, const int* inv_pw, int n_pw, int pw_cols, const int* inv_chi,
+                            int n_chi, int chi_cols, int n_rows, double scale, void* work, cudaStream_t st, int low) {
+  if (n_rows <= 0) return GW_OK;
+  GW_DISPATCH(prec, g, rc = O::row_pw(ctx, a, b, lda, out, ldo, inv_pw, n_pw, pw_cols, inv_chi, n_chi, chi_cols, n_rows,
+                                      scale, st, low, work))
 }
 
-gw_status launch_row_pw_chi(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* a, const void* b, long lda,
-                            void* out, long ldo, const int* inv_pw, int n_pw, const int* inv_chi, int n_chi,
-                            int n_rows, double scale, cudaStream_t st, int low) {
-  if (n_rows <= 0) return GW_OK;
-  GW_DISPATCH(prec, g, rc = O::row_pw(ctx, a, b, lda, out, ldo, inv_pw, n_pw, inv_chi, n_chi, n_rows, scale, st, low))
+size_t row_pw_work(const GridInfo& g, gw_prec prec, int pw_cols, int chi_cols) {
+  return (size_t)std::min(g.nr, kPwChunk) * g.n1 * (2 * (size_t)pw_cols + chi_cols) * csize(prec);
 }
 
 gw_status check_row_pw(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int n_pw, int n_chi) {

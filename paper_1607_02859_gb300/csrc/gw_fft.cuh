@@ -30,6 +30,16 @@ __device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b
   a = __ldg(p);
   b = __ldg(p + 1);
 }
+// the same from memory that the kernel also writes
+__device__ __forceinline__ void ld_pair_rw(const float2* p, float2& a, float2& b) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  a = make_float2(v.x, v.y);
+  b = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void ld_pair_rw(const double2* p, double2& a, double2& b) {
+  a = p[0];
+  b = p[1];
+}
 __device__ __forceinline__ void st_pair(float2* p, float2 a, float2 b) {
   *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
 }

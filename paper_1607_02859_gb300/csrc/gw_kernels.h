@@ -6,17 +6,17 @@
 namespace gw {
 
 // gw_fft.cu
-// Rows whose shared-memory copy exceeds kRowSmemMax go through two passes
-// (row_two_pass(g, prec)); those need inv (grid position -> G index or -1) and,
-// forward, a [n_rows][N_r] workspace tmp (which may be a itself for mode 0).
+// inv: the G set's inverse map with its lists (below).  Rows whose shared-memory
+// copy exceeds kRowSmemMax take two kernels (row_two_pass(g, prec)); forward,
+// those need a [n_rows][N_r] workspace tmp (which may be a itself).
 constexpr size_t kRowSmemMax = 227 * 1024;
 gw_status launch_row_fft(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int mode, const void* a, const void* b,
                          long lda, void* out, long ldo, const int* map, int n_chi, int n_rows, double scale,
-                         cudaStream_t st, const int* inv, void* tmp = nullptr, int low = -1);
+                         cudaStream_t st, const int* inv, void* tmp = nullptr,
+                         int low = -1);
 // low >= 0: the rows are rows low .. of a Hermitian matrix used only for R' <= r
 // (forward: elements past r count as zero and mode 0 halves the diagonal; backward:
-// only what the fused self-energy reads is written); row_low_ok: forward rows have it.
-bool row_low_ok(const GridInfo& g, gw_prec prec, int n_chi);
+// only what the fused self-energy reads is written).
 // A G set's inverse map on the device: inv [N_r] (grid position -> G index or -1)
 // followed by what of the grid the set touches (set_lists appends it; index_maps
 // does): kSetHead counts, then the (i2,i3) columns, the (i1,i2) pencils and the
@@ -26,13 +26,20 @@ inline int inv_ints(const GridInfo& g) {
   return g.nr + kSetHead + g.n2 * g.n3 + g.n1 * g.n2 + g.n1 + g.n2 + g.n3;
 }
 void set_lists(const GridInfo& g, std::vector<int>& inv);
+inline int set_columns(const GridInfo& g, const std::vector<int>& inv) { return inv[g.nr]; }   // (i2,i3) columns touched
 bool row_two_pass(const GridInfo& g, gw_prec prec);
 // chi rows from the plane-wave form of G: a = T_unocc, b = T_occ rows [n_rows][lda]
 // over the orbitals' plane-wave set (inv_pw: grid position -> set index or -1),
 // out [n_rows][ldo] = FFT+(scale a conj(b)) on chi's G set (inv_chi).
+// pw_cols, chi_cols: the columns that the two sets touch (set_columns); work: row_pw_work
+// bytes, the columns of a chunk of kPwChunk rows (95 MB for the triangle at 36^3 with
+// 4224 plane waves: it stays in L2).
+constexpr int kPwChunk = 1024;
+size_t row_pw_work(const GridInfo& g, gw_prec prec, int pw_cols, int chi_cols);
 gw_status launch_row_pw_chi(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* a, const void* b, long lda,
-                            void* out, long ldo, const int* inv_pw, int n_pw, const int* inv_chi, int n_chi,
-                            int n_rows, double scale, cudaStream_t st, int low = -1);
+                            void* out, long ldo, const int* inv_pw, int n_pw, int pw_cols, const int* inv_chi,
+                            int n_chi, int chi_cols, int n_rows, double scale, void* work, cudaStream_t st,
+                            int low = -1);
 // GW_OK if launch_row_pw_chi supports the grid, precision and set sizes.
 gw_status check_row_pw(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int n_pw, int n_chi);
 // Sigma rows in the plane-wave form: tu, to [n_rows][ldt] (T rows over the negated
@@ -51,8 +58,9 @@ gw_status check_row_pw_sigma(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int n
 // after checking (one synchronisation) that every band lies in the set's span;
 // pw_grid is the GridInfo of the G formation over the set.
 void pw_negate(const GridInfo& g, std::vector<int>& map, std::vector<int>& inv);
+// tmp: a workspace of tmp_rows >= 1 rows of N_r elements (used where row_two_pass).
 gw_status pw_coefficients(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* psi, int n_b, int n_pw,
-                          const int* dmap_neg, const int* dinv_neg, void* dc, double* dnorm, void* tmp,
+                          const int* dmap_neg, const int* dinv_neg, void* dc, double* dnorm, void* tmp, int tmp_rows,
                           cudaStream_t s);
 GridInfo pw_grid(const GridInfo& g, int n_pw);
 

@@ -455,7 +455,7 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
   const long ldt = (long)n_pws;                        // T row: all k blocks
   const size_t slab = (size_t)g.nr * ld;
   const GridInfo gp = pw_grid(g, n_pw);
-  const bool tmp_needed = row_two_pass(g, prec) && is_fp64(prec);
+  const int pw_cols = set_columns(gs, inv_pws), chi_cols = set_columns(gs, sinv);
   Carver probe(nullptr);
   probe.take<int>(inv_ints(g));
   probe.take<int>(inv_ints(gs));
@@ -473,7 +473,7 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
   probe.take<char>((size_t)n_pw * n_pw * es);
   probe.take<char>((size_t)g.nr * ldt * es);
   probe.take<char>((size_t)g.nr * ldt * es);
-  if (tmp_needed) probe.take<char>((size_t)n_b * g.nr * es);
+  probe.take<char>(row_pw_work(gs, prec, pw_cols, chi_cols));
   if (tc) probe.take<char>(tc_scratch_bytes(gp, n_b, n_occ, n_pw, false));
   if ((st = reserve(ctx, probe.off))) return st;
   Carver cv(ctx->arena);
@@ -493,7 +493,7 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
   char* mu_ = cv.take<char>((size_t)n_pw * n_pw * es);
   char* to = cv.take<char>((size_t)g.nr * ldt * es);
   char* tu = cv.take<char>((size_t)g.nr * ldt * es);
-  char* tmp = tmp_needed ? cv.take<char>((size_t)n_b * g.nr * es) : nullptr;
+  void* rwork = cv.take<char>(row_pw_work(gs, prec, pw_cols, chi_cols));
   void* tcs = tc ? cv.take<char>(tc_scratch_bytes(gp, n_b, n_occ, n_pw, false)) : nullptr;
   if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if ((st = upload(ctx, dsinv, sinv.data(), sizeof(int) * sinv.size(), s))) return st;
@@ -524,7 +524,7 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
                                                       nk[0], nk[1], nk[2], (float2*)u);
     if ((st = launch_check(ctx, "bloch_unphase_kernel"))) return st;
     if ((st = pw_coefficients(ctx, g, prec, u, n_b, n_pw, dmap_pw, dinv_pw, dc + (size_t)k * n_b * n_pw * es, dnorm,
-                              tmp, s)))
+                              to, n_pw, s)))
       return st;
   }
   const double row_scale = -2.0 / ((double)n_k * n_k);
@@ -550,8 +550,8 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
     if ((st = launch_q_phase(ctx, prec, g, nk, dqph, to, ldt, n_pw, -1.0, s))) return st;
     if ((st = launch_q_phase(ctx, prec, g, nk, dqph, tu, ldt, n_pw, -1.0, s))) return st;
     char* slab_j = slabs + (size_t)j * slab * es;
-    if ((st = launch_row_pw_chi(ctx, gs, prec, tu, to, ldt, slab_j, ld, dinv_pws, n_pws, dsinv, n_chis, g.nr,
-                                row_scale, s)))
+    if ((st = launch_row_pw_chi(ctx, gs, prec, tu, to, ldt, slab_j, ld, dinv_pws, n_pws, pw_cols, dsinv, n_chis,
+                                chi_cols, g.nr, row_scale, rwork, s)))
       return st;
     if ((st = launch_q_phase(ctx, prec, g, nk, dqph, slab_j, ld, n_chi, -1.0, s))) return st;
     if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, ld, (int)ld, 1.0, s))) return st;

@@ -128,7 +128,6 @@ static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ,
   void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false)) : nullptr;
   if (tcs_out) *tcs_out = tcs;
   bool first = true;
-  const bool low = row_low_ok(g, prec, n_chi);    // only R' <= r, and chi0 = X + X^H in the end
   for (int j = 0; j < n; ++j) {
     const GreenScales& gs = scales[j];
     const char* sj = t.scale + (size_t)j * n_b * 8;
@@ -137,15 +136,15 @@ static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ,
       const int rows = std::min(rb, g.nr - r0);
       if (tc) {
         if ((st = tc_chi_rows(ctx, g, n_b, n_occ, psi, gs, r0, rows, prec, ga, tcs, first, s,
-                              t.sk ? t.sk + (size_t)j * n_b : nullptr, t.status, low)))
+                              t.sk ? t.sk + (size_t)j * n_b : nullptr, t.status, true)))
           return st;
         first = false;
         st = launch_row_fft(ctx, g, prec, 1, ga, nullptr, g.nr, slab_j + (size_t)r0 * n_chi * es, n_chi, t.map, n_chi,
-                            rows, 1.0, s, t.inv, gb, low ? r0 : -1);
+                            rows, 1.0, s, t.inv, gb, r0);
       } else {
-        if ((st = green_rows(ctx, g, n_b, n_occ, psi, sj, gs, r0, rows, prec, ga, gb, s, low ? r0 : -1))) return st;
+        if ((st = green_rows(ctx, g, n_b, n_occ, psi, sj, gs, r0, rows, prec, ga, gb, s, r0))) return st;
         st = launch_row_fft(ctx, g, prec, 0, ga, gb, g.nr, slab_j + (size_t)r0 * n_chi * es, n_chi, t.map, n_chi,
-                            rows, -2.0, s, t.inv, ga, low ? r0 : -1);
+                            rows, -2.0, s, t.inv, ga, r0);
       }
       if (st) return st;
     }
@@ -154,7 +153,7 @@ static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ,
   if ((st = launch_col_line_ct(ctx, g, prec, slabs, (long)slab, n_chi, n, t.cw, n, chi_w, (long)n_chi * n_chi, n_chi,
                                t.inv, n_chi, s, cw32.empty() ? nullptr : cw32.data())))
     return st;
-  return low ? launch_hermitize(ctx, prec, n, n_chi, chi_w, s) : GW_OK;
+  return launch_hermitize(ctx, prec, n, n_chi, chi_w, s);    // the rows hold R' <= r only
 }
 
 }  // namespace gw
@@ -280,11 +279,16 @@ void pw_negate(const GridInfo& g, std::vector<int>& map, std::vector<int>& inv) 
 }
 
 gw_status pw_coefficients(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* psi, int n_b, int n_pw,
-                          const int* dmap_neg, const int* dinv_neg, void* dc, double* dnorm, void* tmp,
+                          const int* dmap_neg, const int* dinv_neg, void* dc, double* dnorm, void* tmp, int tmp_rows,
                           cudaStream_t s) {
   gw_status st;
-  if ((st = launch_row_fft(ctx, g, prec, 1, psi, nullptr, g.nr, dc, n_pw, dmap_neg, n_pw, n_b, 1.0, s, dinv_neg, tmp)))
-    return st;
+  const size_t es = csize(prec);
+  const int step = row_two_pass(g, prec) ? tmp_rows : n_b;
+  for (int b = 0; b < n_b; b += step)
+    if ((st = launch_row_fft(ctx, g, prec, 1, static_cast<const char*>(psi) + (size_t)b * g.nr * es, nullptr, g.nr,
+                             static_cast<char*>(dc) + (size_t)b * n_pw * es, n_pw, dmap_neg, n_pw,
+                             std::min(step, n_b - b), 1.0, s, dinv_neg, tmp)))
+      return st;
   if (is_fp64(prec))
     band_norms_kernel<double2><<<n_b, 256, 0, s>>>((const double2*)psi, g.nr, (const double2*)dc, n_pw, dnorm);
   else
@@ -310,7 +314,8 @@ gw_status pw_coefficients(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const vo
   return launch_check(ctx, "conj_scale_kernel");
 }
 
-size_t chi0_pw_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_chi, int n_pw, gw_prec prec) {
+size_t chi0_pw_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_chi, int n_pw, int pw_cols, int chi_cols,
+                       gw_prec prec) {
   const size_t es = csize(prec);
   const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
   Carver probe(nullptr);
@@ -327,7 +332,7 @@ size_t chi0_pw_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_chi, 
   probe.take<char>((size_t)n_pw * n_pw * es);            // Mc unocc
   probe.take<char>((size_t)g.nr * n_pw * es);            // T occ
   probe.take<char>((size_t)g.nr * n_pw * es);            // T unocc
-  if (row_two_pass(g, prec) && is_fp64(prec)) probe.take<char>((size_t)n_b * g.nr * es);
+  probe.take<char>(row_pw_work(g, prec, pw_cols, chi_cols));
   if (tc) probe.take<char>(tc_scratch_bytes(pw_grid(g, n_pw), n_b, n_occ, n_pw, false));
   return probe.off;
 }
@@ -350,10 +355,11 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   if ((st = index_maps(ctx, g, pw_index_h, n_pw, map_pw, inv_pw))) return st;
   pw_negate(g, map_pw, inv_pw);
   if ((st = check_row_pw(ctx, g, prec, n_pw, n_chi))) return st;
+  const int pw_cols = set_columns(g, inv_pw), chi_cols = set_columns(g, inv);
   cudaStream_t s = as_stream(stream);
   const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
   const size_t es = csize(prec);
-  if ((st = reserve(ctx, chi0_pw_scratch(g, n_b, n_occ, n, n_chi, n_pw, prec)))) return st;
+  if ((st = reserve(ctx, chi0_pw_scratch(g, n_b, n_occ, n, n_chi, n_pw, pw_cols, chi_cols, prec)))) return st;
   std::vector<GreenScales> scales;
   std::vector<double> cw64;
   std::vector<float> cw32;
@@ -373,7 +379,7 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   char* mu_ = cv.take<char>((size_t)n_pw * n_pw * es);
   char* to = cv.take<char>((size_t)g.nr * n_pw * es);
   char* tu = cv.take<char>((size_t)g.nr * n_pw * es);
-  char* tmp = row_two_pass(g, prec) && is_fp64(prec) ? cv.take<char>((size_t)n_b * g.nr * es) : nullptr;
+  void* rwork = cv.take<char>(row_pw_work(g, prec, pw_cols, chi_cols));
   const GridInfo gp = pw_grid(g, n_pw);
   void* tcs = tc ? cv.take<char>(tc_scratch_bytes(gp, n_b, n_occ, n_pw, false)) : nullptr;
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
@@ -386,7 +392,7 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   if (!tc)
     for (int j = 0; j < n; ++j)
       if ((st = upload_scales(ctx, dscale + (size_t)j * n_b * 8, scales[j], prec, s))) return st;
-  if ((st = pw_coefficients(ctx, g, prec, psi, n_b, n_pw, dmap_pw, dinv_pw, dc, dnorm, tmp, s))) return st;
+  if ((st = pw_coefficients(ctx, g, prec, psi, n_b, n_pw, dmap_pw, dinv_pw, dc, dnorm, to, n_pw, s))) return st;
   bool first = true;
   for (int j = 0; j < n; ++j) {
     // Mc_occ, Mc_unocc over the plane-wave set, then their column transforms T(r, g')
@@ -405,7 +411,8 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
     }
     // chi(r, G', tau_j) for every row r: expand, multiply (Eq. chi_rr), transform (Eq. FFTX1)
     char* slab_j = slabs + (size_t)j * slab * es;
-    if ((st = launch_row_pw_chi(ctx, g, prec, tu, to, n_pw, slab_j, n_chi, dinv_pw, n_pw, dinv, n_chi, g.nr, -2.0, s, 0)))
+    if ((st = launch_row_pw_chi(ctx, g, prec, tu, to, n_pw, slab_j, n_chi, dinv_pw, n_pw, pw_cols, dinv, n_chi,
+                                chi_cols, g.nr, -2.0, rwork, s, 0)))
       return st;
     if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, n_chi, n_chi, 1.0, s))) return st;
   }

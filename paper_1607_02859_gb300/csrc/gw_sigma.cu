@@ -853,7 +853,7 @@ extern "C" gw_status gw_sigma_diag_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   int *dmap_neg = nullptr, *dinv_neg = nullptr, *dinv_nat = nullptr;
   double* dnorm = nullptr;
   char *dc = nullptr, *cn = nullptr, *mo = nullptr, *mu_ = nullptr, *to = nullptr, *tu = nullptr, *wg = nullptr;
-  char *hu = nullptr, *ho = nullptr, *vu = nullptr, *vo = nullptr, *tmp = nullptr;
+  char *hu = nullptr, *ho = nullptr, *vu = nullptr, *vo = nullptr;
   void* tcs = nullptr;
   auto carve = [&](Carver& cv) {
     sigma_carve_tables(cv, g, n_b, n, n_chi, n_n, n_real, false, t);
@@ -872,7 +872,6 @@ extern "C" gw_status gw_sigma_diag_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
     ho = cv.take<char>((size_t)g.nr * n_pw * es);
     vu = cv.take<char>((size_t)g.nr * n_n * es);
     vo = cv.take<char>((size_t)g.nr * n_n * es);
-    tmp = row_two_pass(g, prec) && is_fp64(prec) ? cv.take<char>((size_t)n_b * g.nr * es) : nullptr;
     tcs = tc ? cv.take<char>(tc_scratch_bytes(gp, n_b, n_occ, n_pw, false)) : nullptr;
   };
   {
@@ -888,7 +887,7 @@ extern "C" gw_status gw_sigma_diag_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   if ((st = upload(ctx, dmap_neg, map_neg.data(), sizeof(int) * n_pw, s))) return st;
   if ((st = upload(ctx, dinv_neg, inv_neg.data(), sizeof(int) * inv_neg.size(), s))) return st;
   if ((st = upload(ctx, dinv_nat, inv_nat.data(), sizeof(int) * inv_nat.size(), s))) return st;
-  if ((st = pw_coefficients(ctx, g, prec, psi, n_b, n_pw, dmap_neg, dinv_neg, dc, dnorm, tmp, s))) return st;
+  if ((st = pw_coefficients(ctx, g, prec, psi, n_b, n_pw, dmap_neg, dinv_neg, dc, dnorm, to, n_pw, s))) return st;
   {
     const dim3 gg((n_pw + 255) / 256, n_n);
     if (is_fp64(prec)) gather_rows_kernel<<<gg, 256, 0, s>>>((const double2*)dc, n_pw, t.bands, n_pw, (double2*)cn);
