@@ -31,9 +31,8 @@ struct BatchSys {
   GridInfo g{};
   gw_chi0_plan* chi0 = nullptr;
   std::vector<GreenScales> scales;
-  std::vector<float> ict32;      // inverse CT weights as FP32 hi/lo (kernel parameters)
   double* dvh = nullptr;         // v^1/2 on the device
-  double* dict = nullptr;        // inverse CT weights on the device (general path)
+  double* dict = nullptr;        // inverse CT weights on the device (FP64, or FP32 hi then lo)
   SigmaTables st{};
   int* status = nullptr;         // [kStatusInts]
 };
@@ -90,8 +89,7 @@ static gw_status record_system(gw_batch* b, BatchSys& y, cudaStream_t s) {
                             nullptr, s)))
       return st;
   }
-  if ((st = launch_ct(ctx, prec, false, in.n, y.dict, slice, in.chi_w, in.w_tau, s,
-                      y.ict32.empty() ? nullptr : y.ict32.data())))
+  if ((st = launch_ct(ctx, prec, false, in.n, y.dict, slice, in.chi_w, in.w_tau, s)))
     return st;
   {
     Carver cv(ctx->arena);
@@ -189,8 +187,8 @@ extern "C" gw_status gw_batch_plan(gw_ctx* ctx, int n_sys, const gw_batch_system
     if (is_fp64(prec)) {
       if ((st = upload(ctx, y.dict, in.Cinv_h, sizeof(double) * in.n * in.n, b->cs))) return bail(st);
     } else {
-      y.ict32 = split_weights(in.Cinv_h, in.n * in.n, 1.0);
-      if ((st = upload(ctx, y.dict, y.ict32.data(), sizeof(float) * 2 * in.n * in.n, b->cs))) return bail(st);
+      const std::vector<float> w32 = split_weights(in.Cinv_h, in.n * in.n, 1.0);
+      if ((st = upload(ctx, y.dict, w32.data(), sizeof(float) * 2 * in.n * in.n, b->cs))) return bail(st);
     }
     if ((st = sigma_upload_tables(ctx, y.st, y.g, in.n_b, in.n, in.n_chi, maps[i], invs[i], in.bands_h, in.n_n,
                                   y.scales, in.C_h, in.S_h, in.omega_h, nullptr, 0, prec, b->cs)))

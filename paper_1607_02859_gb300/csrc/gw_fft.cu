@@ -771,64 +771,126 @@ __global__ void __launch_bounds__(PwRow<T, N1, N2, N3>::THREADS)
   }
 }
 
-constexpr int kPlaneW = 16;
+// Columns per CTA of the plane pass: as many as leave two CTAs (FP32) in an SM's
+// shared memory, at least 64 bytes of a row.
+template <typename T, int N2, int N3>
+constexpr int kPlaneW = N2 * N3 * 16 * sizeof(typename cpx<T>::t) <= 96 * 1024 ? 16 : 8;
+template <typename T, int N2, int N3>
+struct ColPlane {
+  static constexpr int W = kPlaneW<T, N2, N3>;
+  static constexpr size_t bytes = (size_t)N2 * N3 * W * sizeof(typename cpx<T>::t);
+  static constexpr int PEN = (N2 > N3 ? N2 : N3) * W;              // pencils of a pass: one or two rounds
+  static constexpr int TH = ((PEN > 288 ? PEN / 2 : PEN) + 31) / 32 * 32;
+  static constexpr int MINB = sizeof(T) == 8 ? 1 : (bytes > 76 * 1024 ? 2 : 3);
+};
 
-// In-place 2-D FFT over (i2, i3) of the rows of plane i1 = blockIdx.y, for 16
+// In-place 2-D FFT over (i2, i3) of the rows of plane i1 = blockIdx.y, for W
 // contiguous columns per CTA.  PAIRS (FP32 only): rows move as 16-byte pairs
 // of columns; the host takes it when ld and ncols are even (every pair then
 // starts on a 16-byte boundary and lies wholly inside or outside the matrix).
-template <typename T, int N2, int N3, int DIR, bool PAIRS>
-__global__ void __launch_bounds__(256) col_plane_kernel(typename cpx<T>::t* __restrict__ buf, long ld, int ncols,
-                                                        T scale) {
+// Towards the G set (DIR -1) only the (i2, i3) rows that the set touches are
+// written (the i1 pass reads no others) and the i2 pass visits the set's i3;
+// from it (DIR +1) only those rows are read (the others are zero) and the i3
+// pass visits the set's i2.  HBM bounds it: one pass at 36^3, 8192 columns, takes
+// 1.29 ms (3.3 TB/s); with all rows and one 16-column CTA per SM it took 2.28 ms.
+template <typename T, int N1, int N2, int N3, int DIR, bool PAIRS>
+__global__ void __launch_bounds__(ColPlane<T, N2, N3>::TH, ColPlane<T, N2, N3>::MINB)
+    col_plane_kernel(typename cpx<T>::t* __restrict__ buf, long ld, int ncols, T scale, const int* __restrict__ inv) {
   using C = typename cpx<T>::t;
-  constexpr int W = kPlaneW;
+  constexpr int W = ColPlane<T, N2, N3>::W, TH = ColPlane<T, N2, N3>::TH;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* s = reinterpret_cast<C*>(smem_raw);
   const long i1 = blockIdx.y;
   const int c0 = blockIdx.x * W;
   C* base = buf + i1 * (N2 * N3) * ld + c0;
+  const SetLists<N1, N2, N3> g(inv);
+  if constexpr (DIR > 0) {
+    for (int e = threadIdx.x; e < N2 * N3 * W; e += TH) s[e] = mk(T(0), T(0));
+    __syncthreads();
+  }
+  const int n_in = DIR > 0 ? g.n23 : N2 * N3;
+  auto row_in = [&](int e) { return DIR > 0 ? __ldg(g.l23 + e) : e; };
   if constexpr (PAIRS) {
-    for (int e = threadIdx.x; e < N2 * N3 * W / 2; e += blockDim.x) {
-      const int rr = e / (W / 2), w = 2 * (e - rr * (W / 2));
-      C a = mk(T(0), T(0)), b = a;
-      if (c0 + w < ncols) ld_pair(base + rr * ld + w, a, b);
-      s[rr * W + w] = a;
-      s[rr * W + w + 1] = b;
+    constexpr int LB = 6;                                          // loads in flight per thread
+    for (int e0 = threadIdx.x; e0 < n_in * (W / 2); e0 += LB * TH) {
+      C a[LB], b[LB];
+      int at[LB];
+#pragma unroll
+      for (int u = 0; u < LB; ++u) {
+        const int e = e0 + u * TH;
+        a[u] = b[u] = mk(T(0), T(0));
+        at[u] = -1;
+        if (e < n_in * (W / 2)) {
+          const int rr = row_in(e / (W / 2)), w = 2 * (e % (W / 2));
+          at[u] = rr * W + w;
+          if (c0 + w < ncols) ld_pair_rw(base + rr * ld + w, a[u], b[u]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < LB; ++u)
+        if (at[u] >= 0) {
+          s[at[u]] = a[u];
+          s[at[u] + 1] = b[u];
+        }
     }
   } else {
-    for (int e = threadIdx.x; e < N2 * N3 * W; e += blockDim.x) {
-      const int rr = e / W, w = e - rr * W;
-      s[e] = (c0 + w < ncols) ? base[rr * ld + w] : mk(T(0), T(0));
+    for (int e = threadIdx.x; e < n_in * W; e += TH) {
+      const int rr = row_in(e / W), w = e % W;
+      s[rr * W + w] = (c0 + w < ncols) ? base[rr * ld + w] : mk(T(0), T(0));
     }
   }
   __syncthreads();
-  pencil_pass<N3, DIR>(s, N2 * W, W, [](int p) { return (p / W) * (N3 * W) + (p % W); });
+  const int n2 = DIR > 0 ? g.n2 : N2;
+  for (int e = threadIdx.x; e < n2 * W; e += TH) {
+    const int i2 = DIR > 0 ? __ldg(g.l2 + e / W) : e / W;
+    const int o = i2 * (N3 * W) + e % W;
+    C x[N3];
+#pragma unroll
+    for (int k = 0; k < N3; ++k) x[k] = s[o + k * W];
+    RegFFT<N3, DIR>::run(x);
+#pragma unroll
+    for (int k = 0; k < N3; ++k) s[o + k * W] = x[k];
+  }
   __syncthreads();
-  pencil_pass<N2, DIR>(s, N3 * W, N3 * W, [](int p) { return (p / W) * W + (p % W); });
+  const int n3 = DIR > 0 ? N3 : g.n3;
+  for (int e = threadIdx.x; e < n3 * W; e += TH) {
+    const int i3 = DIR > 0 ? e / W : __ldg(g.l3 + e / W);
+    const int o = i3 * W + e % W;
+    C x[N2];
+#pragma unroll
+    for (int k = 0; k < N2; ++k) x[k] = s[o + k * (N3 * W)];
+    RegFFT<N2, DIR>::run(x);
+#pragma unroll
+    for (int k = 0; k < N2; ++k) s[o + k * (N3 * W)] = x[k];
+  }
   __syncthreads();
+  const int n_out = DIR > 0 ? N2 * N3 : g.n23;
+  auto row_out = [&](int e) { return DIR > 0 ? e : __ldg(g.l23 + e); };
   if constexpr (PAIRS) {
-    for (int e = threadIdx.x; e < N2 * N3 * W / 2; e += blockDim.x) {
-      const int rr = e / (W / 2), w = 2 * (e - rr * (W / 2));
+    for (int e = threadIdx.x; e < n_out * (W / 2); e += TH) {
+      const int rr = row_out(e / (W / 2)), w = 2 * (e % (W / 2));
       if (c0 + w < ncols) st_pair(base + rr * ld + w, cscale(s[rr * W + w], scale), cscale(s[rr * W + w + 1], scale));
     }
   } else {
-    for (int e = threadIdx.x; e < N2 * N3 * W; e += blockDim.x) {
-      const int rr = e / W, w = e - rr * W;
-      if (c0 + w < ncols) base[rr * ld + w] = cscale(s[e], scale);
+    for (int e = threadIdx.x; e < n_out * W; e += TH) {
+      const int rr = row_out(e / W), w = e % W;
+      if (c0 + w < ncols) base[rr * ld + w] = cscale(s[rr * W + w], scale);
     }
   }
 }
 
-// In-place 1-D FFT over i1 for the column c and the (i2,i3) pair blockIdx.y.
-// GATHER_IN: read row inv[pos] of `in` (zero if -1) instead of buf[pos].
-// SCATTER_OUT: write row inv[pos] of `out` (skip if -1) instead of buf[pos].
+// 1-D FFT over i1 for the column c and the blockIdx.y-th (i2,i3) that the G set
+// touches (l23, behind the inverse map).
+// GATHER_IN: read row inv[pos] of `in` (zero if -1) instead of row pos.
+// SCATTER_OUT: write row inv[pos] of `out` (skip if -1) instead of row pos.
 template <typename T, int N1, int DIR, bool GATHER_IN, bool SCATTER_OUT>
-__global__ void __launch_bounds__(256) col_line_kernel(const typename cpx<T>::t* __restrict__ in, long ldi,
+__global__ void __launch_bounds__(128) col_line_kernel(const typename cpx<T>::t* __restrict__ in, long ldi,
                                                        typename cpx<T>::t* __restrict__ out, long ldo, int ncols,
-                                                       int plane, const int* __restrict__ inv, T scale) {
+                                                       int plane, const int* __restrict__ inv,
+                                                       const int* __restrict__ l23, T scale) {
   using C = typename cpx<T>::t;
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i23 = blockIdx.y;
+  const int i23 = __ldg(l23 + blockIdx.y);
   if (c >= ncols) return;
   C x[N1];
 #pragma unroll
@@ -861,42 +923,63 @@ __global__ void __launch_bounds__(256) col_line_kernel(const typename cpx<T>::t*
 // accumulates c x as fma(hi, x, fma(lo, x, s)), which removes the weight
 // rounding for one extra FMA per term; the remaining FP32 accumulation error
 // is below the rounding already present in the x_j themselves.  FP64 keeps the
-// plain sum.
-template <typename T>
-struct WSum {
-  T s = 0;
-  __device__ void add(T wh, T, T x) { s += wh * x; }
-  __device__ T value() const { return s; }
-};
-template <>
-struct WSum<float> {
-  float s = 0.f;
-  __device__ void add(float wh, float wl, float x) { s = __fmaf_rn(wh, x, __fmaf_rn(wl, x, s)); }
-  __device__ float value() const { return s; }
-};
-// The weight arrays hold hi[n_k][n_j] and, for FP32, lo[n_k][n_j] right after.
-template <typename T>
-constexpr int kWParts = sizeof(T) == 4 ? 2 : 1;
+// plain sum.  The weight arrays hold hi[n_k][n_j] and, for FP32, lo[n_k][n_j]
+// right after.
+//
+// Two FP32 values (re, im) per 64-bit register pair: one packed multiply-add
+// does both (half the issue slots of scalar FMAs at the same lane rate).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+// Weights in shared memory as (hi, hi, lo, lo), rows padded with zeros to NTB: one
+// 16-byte broadcast read per term feeds the multiply-adds of several elements.
+template <int NTB>
+__device__ __forceinline__ void load_weights(const float* __restrict__ M, int nk, int nj, float4* w) {
+  for (int e = threadIdx.x; e < nk * NTB; e += blockDim.x) {
+    const int k = e / NTB, j = e - k * NTB;
+    const float hi = j < nj ? M[k * nj + j] : 0.f, lo = j < nj ? M[nk * nj + k * nj + j] : 0.f;
+    w[e] = make_float4(hi, hi, lo, lo);
+  }
+}
+// s += sum_j c_kj x_j for E elements, terms in ascending j
+template <int NTB, int E>
+__device__ __forceinline__ void weighted(const float4* w, const f32x2 (&x)[NTB][E], f32x2 (&acc)[E]) {
+#pragma unroll
+  for (int u = 0; u < E; ++u) acc[u] = 0ull;
+#pragma unroll
+  for (int j = 0; j < NTB; ++j) {
+    const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(w + j);
+#pragma unroll
+    for (int u = 0; u < E; ++u) acc[u] = fma2(c.x, x[j][u], fma2(c.y, x[j][u], acc[u]));
+  }
+}
 
 // Last column pass of the chi chain: i1 FFT (-i) of every tau slab, then
 // out[k][inv[pos]][c] = sum_j cw[k][j] * slab_j(pos, c)  (Eq. CTX with the
-// dV^2/Omega of Eq. FFTX2 folded into cw).  32 columns x 8 warps per CTA.
+// dV^2/Omega of Eq. FFTX2 folded into cw).  FP64: 32 columns x 8 warps per CTA.
 template <typename T, int N1>
 __global__ void __launch_bounds__(256) col_line_ct_kernel(const typename cpx<T>::t* __restrict__ slabs,
                                                           long slab_stride, long ld, int ntau,
                                                           const T* __restrict__ cw, int nw,
                                                           typename cpx<T>::t* __restrict__ out, long out_slice,
-                                                          long ldo, const int* __restrict__ inv, int plane,
-                                                          int ncols) {
+                                                          long ldo, const int* __restrict__ inv,
+                                                          const int* __restrict__ l23, int plane, int ncols) {
   using C = typename cpx<T>::t;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* s = reinterpret_cast<C*>(smem_raw);                       // [ntau][N1][32]
-  T* w = reinterpret_cast<T*>(s + (size_t)ntau * N1 * 32);      // [parts][nw][ntau]
-  const T* wl = w + (kWParts<T> - 1) * nw * ntau;
+  T* w = reinterpret_cast<T*>(s + (size_t)ntau * N1 * 32);      // [nw][ntau]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane;
-  const int i23 = blockIdx.y;
-  for (int e = threadIdx.x; e < kWParts<T> * nw * ntau; e += blockDim.x) w[e] = cw[e];
+  const int i23 = __ldg(l23 + blockIdx.y);
+  for (int e = threadIdx.x; e < nw * ntau; e += blockDim.x) w[e] = cw[e];
   for (int j = warp; j < ntau; j += 8) {
     C x[N1];
     const C* src = slabs + (long)j * slab_stride;
@@ -913,38 +996,49 @@ __global__ void __launch_bounds__(256) col_line_ct_kernel(const typename cpx<T>:
     const int k = q / N1, i1 = q - k * N1;
     const int row = inv[(long)i1 * plane + i23];
     if (row < 0) continue;
-    WSum<T> re, im;
+    C acc = mk(T(0), T(0));
     for (int j = 0; j < ntau; ++j) {
       const C v = s[(j * N1 + i1) * 32 + lane];
-      const T wh = w[k * ntau + j], wlo = wl[k * ntau + j];
-      re.add(wh, wlo, v.x);
-      im.add(wh, wlo, v.y);
+      acc.x += w[k * ntau + j] * v.x;
+      acc.y += w[k * ntau + j] * v.y;
     }
-    out[(long)k * out_slice + (long)row * ldo + c] = mk(re.value(), im.value());
+    out[(long)k * out_slice + (long)row * ldo + c] = acc;
   }
 }
 
-// Same pass with a compile-time count of tau points (FP32): each lane keeps the
-// NT values of its column and one i1 in registers and the weights come from a
-// kernel-parameter block (constant bank), so the transform costs one
-// shared-memory read per input instead of three per multiply-add.
-template <int NT>
-struct CtWeights {
-  float hi[NT * NT];
-  float lo[NT * NT];
-};
-
-template <int N1, int NT>
-__global__ void __launch_bounds__(256, (NT * N1 * 32 * 8 <= 110 * 1024) ? 2 : 1) col_line_ct_reg_kernel(const float2* __restrict__ slabs, long slab_stride,
-                                                              long ld, const __grid_constant__ CtWeights<NT> cw,
+// The same pass in FP32 for any count of tau points up to NTB: 32 M columns per
+// CTA, M so that the (tau, 32 columns) pencils fill the eight warps.  Each lane
+// then keeps the values of its column at two i1 that hold a G vector in registers
+// and runs over the frequencies.  At 36^3 with n_chi = 8192 and 2 tau the form
+// with one warp per tau of every (i2, i3) took 7.3 to 8 ms, this one 1.0 ms.
+template <int N1, int NTB>
+__global__ void __launch_bounds__(256, N1 <= 24 || NTB <= 16 ? 2 : 1) col_line_ct_reg_kernel(const float2* __restrict__ slabs, long slab_stride,
+                                                              long ld, int ntau, int m, const float* __restrict__ cw,
                                                               float2* __restrict__ out, long out_slice, long ldo,
-                                                              const int* __restrict__ inv, int plane, int ncols) {
+                                                              const int* __restrict__ inv,
+                                                              const int* __restrict__ l23, int plane, int ncols) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* s = reinterpret_cast<float2*>(smem_raw);             // [NT][N1][32]
+  __shared__ int act[N1], act_row[N1], n_act;
+  float4* w = reinterpret_cast<float4*>(smem_raw);             // [ntau][NTB]
+  float2* s = reinterpret_cast<float2*>(w + ntau * NTB);       // [ntau][N1][32 m]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c = blockIdx.x * 32 + lane;
-  const int i23 = blockIdx.y;
-  for (int j = warp; j < NT; j += 8) {
+  const int cw_cols = 32 * m;
+  const int c0 = blockIdx.x * cw_cols;
+  const int i23 = __ldg(l23 + blockIdx.y);
+  load_weights<NTB>(cw, ntau, ntau, w);
+  if (threadIdx.x == 0) {
+    int n = 0;
+    for (int i1 = 0; i1 < N1; ++i1) {
+      const int row = __ldg(inv + (long)i1 * plane + i23);
+      if (row >= 0) {
+        act[n] = i1;
+        act_row[n++] = row;
+      }
+    }
+    n_act = n;
+  }
+  for (int t = warp; t < ntau * m; t += 8) {
+    const int j = t / m, cl = (t - j * m) * 32 + lane, c = c0 + cl;
     float2 x[N1];
     const float2* src = slabs + (long)j * slab_stride;
 #pragma unroll
@@ -952,77 +1046,96 @@ __global__ void __launch_bounds__(256, (NT * N1 * 32 * 8 <= 110 * 1024) ? 2 : 1)
       x[i1] = c < ncols ? src[((long)i1 * plane + i23) * ld + c] : make_float2(0.f, 0.f);
     RegFFT<N1, -1>::run(x);
 #pragma unroll
-    for (int i1 = 0; i1 < N1; ++i1) s[(j * N1 + i1) * 32 + lane] = x[i1];
+    for (int i1 = 0; i1 < N1; ++i1) s[(j * N1 + i1) * cw_cols + cl] = x[i1];
   }
   __syncthreads();
-  if (c >= ncols) return;
-  for (int i1 = warp; i1 < N1; i1 += 8) {
-    const int row = inv[(long)i1 * plane + i23];
-    if (row < 0) continue;
-    float2 x[NT];
+  const int pairs = (n_act + 1) / 2;
+  for (int t = warp; t < pairs * m; t += 8) {
+    const int a = t / m, cl = (t - a * m) * 32 + lane, c = c0 + cl;
+    if (c >= ncols) continue;
+    const bool two = 2 * a + 1 < n_act;
+    const int ia = act[2 * a], ib = two ? act[2 * a + 1] : ia;
+    const long oa = (long)act_row[2 * a] * ldo + c, ob = two ? (long)act_row[2 * a + 1] * ldo + c : 0;
+    f32x2 x[NTB][2];
 #pragma unroll
-    for (int j = 0; j < NT; ++j) x[j] = s[(j * N1 + i1) * 32 + lane];
-#pragma unroll
-    for (int k = 0; k < NT; ++k) {
-      WSum<float> re, im;
-#pragma unroll
-      for (int j = 0; j < NT; ++j) {
-        re.add(cw.hi[k * NT + j], cw.lo[k * NT + j], x[j].x);
-        im.add(cw.hi[k * NT + j], cw.lo[k * NT + j], x[j].y);
-      }
-      out[(long)k * out_slice + (long)row * ldo + c] = make_float2(re.value(), im.value());
+    for (int j = 0; j < NTB; ++j) {
+      x[j][0] = j < ntau ? *reinterpret_cast<const f32x2*>(s + (j * N1 + ia) * cw_cols + cl) : 0ull;
+      x[j][1] = j < ntau ? *reinterpret_cast<const f32x2*>(s + (j * N1 + ib) * cw_cols + cl) : 0ull;
+    }
+#pragma unroll 1
+    for (int k = 0; k < ntau; ++k) {
+      f32x2 acc[2];
+      weighted<NTB, 2>(w + k * NTB, x, acc);
+      out[(long)k * out_slice + oa] = unpack2(acc[0]);
+      if (two) out[(long)k * out_slice + ob] = unpack2(acc[1]);
     }
   }
 }
 
-// Same map with a compile-time size (FP32, weights in a kernel-parameter
-// block, constant bank): each thread keeps one element of all n slices in
-// registers.  Capped at 80 registers for three CTAs (24 warps) per SM, which
-// keeps enough loads in flight to approach the HBM rate.
-template <int NT, bool ST>
-__global__ void __launch_bounds__(256, 3) ct_reg1_kernel(const float2* __restrict__ in, float2* __restrict__ out,
-                                                      size_t elems, const __grid_constant__ CtWeights<NT> w) {
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < elems; e += (size_t)gridDim.x * blockDim.x) {
-    float2 x[NT];
+// out[k][e] = (i if ST) sum_j M[k][j] in[j][e] in FP32: each thread keeps E
+// elements of all n <= NTB slices in registers and runs over the outputs.  E = 2
+// (16-byte accesses) where the slices allow it.  HBM and the multiply-add pipe
+// bound it about equally at 20 points (four packed FMAs per weight and pair): 20
+// slices of 2048^2 in 287 us (4.7 TB/s), 762 us with the weights in constant
+// memory, whose cache the 800 of them did not fit.
+template <int NTB, bool ST, int E>
+__global__ void __launch_bounds__(128) ct_reg_kernel(const float2* __restrict__ in, float2* __restrict__ out,
+                                                     size_t elems, int n, const float* __restrict__ M) {
+  __shared__ float4 w[32 * NTB];
+  load_weights<NTB>(M, n, n, w);
+  __syncthreads();
+  const size_t count = elems / E;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) {
+    f32x2 x[NTB][E];
 #pragma unroll
-    for (int j = 0; j < NT; ++j) x[j] = __ldg(in + (size_t)j * elems + e);
-#pragma unroll
-    for (int k = 0; k < NT; ++k) {
-      WSum<float> re, im;
-#pragma unroll
-      for (int j = 0; j < NT; ++j) {
-        re.add(w.hi[k * NT + j], w.lo[k * NT + j], x[j].x);
-        im.add(w.hi[k * NT + j], w.lo[k * NT + j], x[j].y);
+    for (int j = 0; j < NTB; ++j) {
+      if constexpr (E == 2) {
+        ulonglong2 v = make_ulonglong2(0ull, 0ull);
+        if (j < n) v = __ldg(reinterpret_cast<const ulonglong2*>(in + (size_t)j * elems) + e);
+        x[j][0] = v.x;
+        x[j][1] = v.y;
+      } else {
+        x[j][0] = j < n ? __ldg(reinterpret_cast<const f32x2*>(in + (size_t)j * elems) + e) : 0ull;
       }
-      out[(size_t)k * elems + e] = ST ? make_float2(-im.value(), re.value()) : make_float2(re.value(), im.value());
+    }
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+      f32x2 acc[E];
+      weighted<NTB, E>(w + k * NTB, x, acc);
+      float2 v[E];
+#pragma unroll
+      for (int u = 0; u < E; ++u) {
+        v[u] = unpack2(acc[u]);
+        if (ST) v[u] = make_float2(-v[u].y, v[u].x);
+      }
+      float2* o = out + (size_t)k * elems + E * e;
+      if constexpr (E == 2) st_pair(o, v[0], v[1]);
+      else o[0] = v[0];
     }
   }
 }
 
-// out[k][e] = (i if ST) sum_j M[k][j] in[j][e]
-template <typename T, bool ST>
-__global__ void __launch_bounds__(256) ct_kernel(const typename cpx<T>::t* __restrict__ in,
-                                                 typename cpx<T>::t* __restrict__ out, size_t elems, int n,
-                                                 const T* __restrict__ M) {
-  using C = typename cpx<T>::t;
-  __shared__ T w[kWParts<T> * 32 * 32];
-  const T* wl = w + (kWParts<T> - 1) * n * n;
-  for (int e = threadIdx.x; e < kWParts<T> * n * n; e += blockDim.x) w[e] = M[e];
+// FP64: out[k][e] = (i if ST) sum_j M[k][j] in[j][e]
+template <bool ST>
+__global__ void __launch_bounds__(256) ct_kernel(const double2* __restrict__ in, double2* __restrict__ out,
+                                                 size_t elems, int n, const double* __restrict__ M) {
+  __shared__ double w[32 * 32];
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) w[e] = M[e];
   __syncthreads();
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < elems; e += (size_t)gridDim.x * blockDim.x) {
-    C x[32];
+    double2 x[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j)
       if (j < n) x[j] = in[(size_t)j * elems + e];
     for (int k = 0; k < n; ++k) {
-      WSum<T> re, im;
+      double re = 0, im = 0;
 #pragma unroll
       for (int j = 0; j < 32; ++j)
         if (j < n) {
-          re.add(w[k * n + j], wl[k * n + j], x[j].x);
-          im.add(w[k * n + j], wl[k * n + j], x[j].y);
+          re += w[k * n + j] * x[j].x;
+          im += w[k * n + j] * x[j].y;
         }
-      out[(size_t)k * elems + e] = ST ? mk(-im.value(), re.value()) : mk(re.value(), im.value());
+      out[(size_t)k * elems + e] = ST ? make_double2(-im, re) : make_double2(re, im);
     }
   }
 }
@@ -1238,75 +1351,77 @@ struct GridOps {
       return fail(ctx, GW_ERR_UNSUPPORTED, "plane-wave Sigma rows: no cluster split fits this grid and precision");
     }
   }
-  static gw_status plane(gw_ctx* ctx, int dir, void* buf, long ld, int ncols, double scale, cudaStream_t st) {
-    const size_t bytes = (size_t)N2 * N3 * kPlaneW * sizeof(C);
-    dim3 grid((ncols + kPlaneW - 1) / kPlaneW, N1);
+  static gw_status plane(gw_ctx* ctx, int dir, void* buf, long ld, int ncols, double scale, const int* inv, int cols,
+                         cudaStream_t st) {
+    using CP = ColPlane<T, N2, N3>;
+    dim3 grid((ncols + CP::W - 1) / CP::W, N1);
     auto go = [&](auto kernel) -> gw_status {
-      gw_status s = set_smem(ctx, kernel, bytes);
+      gw_status s = set_smem(ctx, kernel, CP::bytes);
       if (s) return s;
-      KTimer kt(ctx, KF_COL_FFT, 2.0 * N1 * N2 * N3 * (double)ncols * sizeof(C), st);
-      kernel<<<grid, 256, bytes, st>>>((C*)buf, ld, ncols, (T)scale);
+      KTimer kt(ctx, KF_COL_FFT, ((double)N2 * N3 + cols) * N1 * (double)ncols * sizeof(C), st);
+      kernel<<<grid, CP::TH, CP::bytes, st>>>((C*)buf, ld, ncols, (T)scale, inv);
       return launch_check(ctx, "col_plane_kernel");
     };
     const bool pairs = sizeof(T) == 4 && ld % 2 == 0 && ncols % 2 == 0 && reinterpret_cast<uintptr_t>(buf) % 16 == 0;
-    if (pairs) return dir > 0 ? go(col_plane_kernel<T, N2, N3, +1, true>) : go(col_plane_kernel<T, N2, N3, -1, true>);
-    return dir > 0 ? go(col_plane_kernel<T, N2, N3, +1, false>) : go(col_plane_kernel<T, N2, N3, -1, false>);
+    if (pairs)
+      return dir > 0 ? go(col_plane_kernel<T, N1, N2, N3, +1, sizeof(T) == 4>)
+                     : go(col_plane_kernel<T, N1, N2, N3, -1, sizeof(T) == 4>);
+    return dir > 0 ? go(col_plane_kernel<T, N1, N2, N3, +1, false>) : go(col_plane_kernel<T, N1, N2, N3, -1, false>);
   }
   static gw_status line(gw_ctx* ctx, int dir, int variant, const void* in, long ldi, void* out, long ldo, int ncols,
-                        const int* inv, double scale, cudaStream_t st) {
-    dim3 grid((ncols + 127) / 128, N2 * N3);
+                        const int* inv, int cols, double scale, cudaStream_t st) {
+    dim3 grid((ncols + 127) / 128, cols);
     auto go = [&](auto kernel) -> gw_status {
-      KTimer kt(ctx, KF_COL_FFT, 2.0 * N1 * N2 * N3 * (double)ncols * sizeof(C), st);
-      kernel<<<grid, 128, 0, st>>>((const C*)in, ldi, (C*)out, ldo, ncols, N2 * N3, inv, (T)scale);
+      KTimer kt(ctx, KF_COL_FFT, 2.0 * N1 * cols * (double)ncols * sizeof(C), st);
+      kernel<<<grid, 128, 0, st>>>((const C*)in, ldi, (C*)out, ldo, ncols, N2 * N3, inv, inv + N1 * N2 * N3 + kSetHead,
+                                   (T)scale);
       return launch_check(ctx, "col_line_kernel");
     };
-    // variant 0: in place / plain; 1: gather rows of `in` through inv; 2: scatter rows of `out` through inv
-    if (variant == 0) return dir > 0 ? go(col_line_kernel<T, N1, +1, false, false>)
-                                     : go(col_line_kernel<T, N1, -1, false, false>);
+    // variant 1: gather rows of `in` through inv; 2: scatter rows of `out` through inv
     if (variant == 1) return dir > 0 ? go(col_line_kernel<T, N1, +1, true, false>)
                                      : go(col_line_kernel<T, N1, -1, true, false>);
     return dir > 0 ? go(col_line_kernel<T, N1, +1, false, true>) : go(col_line_kernel<T, N1, -1, false, true>);
   }
-  template <int NT>
-  static gw_status line_ct_reg(gw_ctx* ctx, const void* slabs, long slab_stride, long ld, const float* cw_h, void* out,
-                               long out_slice, long ldo, const int* inv, int ncols, cudaStream_t st) {
-    CtWeights<NT> w;
-    for (int e = 0; e < NT * NT; ++e) {
-      w.hi[e] = cw_h[e];
-      w.lo[e] = cw_h[NT * NT + e];
-    }
-    const size_t bytes = (size_t)NT * N1 * 32 * sizeof(float2);
-    auto kernel = col_line_ct_reg_kernel<N1, NT>;
+  template <int NTB>
+  static gw_status line_ct_reg(gw_ctx* ctx, const void* slabs, long slab_stride, long ld, int ntau, const void* cw,
+                               void* out, long out_slice, long ldo, const int* inv, int cols, int ncols,
+                               cudaStream_t st) {
+    // columns per CTA: enough (tau, 32 columns) pencils for the eight warps
+    const int m = std::max(1, std::min(8 / ntau, (ncols + 31) / 32));
+    const size_t bytes = (size_t)ntau * N1 * 32 * m * sizeof(float2) + (size_t)ntau * NTB * sizeof(float4);
+    auto kernel = col_line_ct_reg_kernel<N1, NTB>;
     gw_status s = set_smem(ctx, kernel, bytes);
     if (s) return s;
-    dim3 grid((ncols + 31) / 32, N2 * N3);
-    KTimer kt(ctx, KF_COL_LINE_CT, ((double)NT * N1 * N2 * N3 + (double)NT * ncols) * ncols * sizeof(float2), st);
-    kernel<<<grid, 256, bytes, st>>>((const float2*)slabs, slab_stride, ld, w, (float2*)out, out_slice, ldo, inv,
-                                     N2 * N3, ncols);
+    dim3 grid((ncols + 32 * m - 1) / (32 * m), cols);
+    KTimer kt(ctx, KF_COL_LINE_CT, ((double)ntau * N1 * cols + (double)ntau * ncols) * ncols * sizeof(float2), st);
+    kernel<<<grid, 256, bytes, st>>>((const float2*)slabs, slab_stride, ld, ntau, m, (const float*)cw, (float2*)out,
+                                     out_slice, ldo, inv, inv + N1 * N2 * N3 + kSetHead, N2 * N3, ncols);
     return launch_check(ctx, "col_line_ct_reg_kernel");
   }
-  static gw_status line_ct(gw_ctx* ctx, const void* slabs, long slab_stride, long ld, int ntau, const void* cw, int nw,
-                           void* out, long out_slice, long ldo, const int* inv, int ncols, cudaStream_t st,
-                           const float* cw_h = nullptr) {
-    if (std::is_same<T, float>::value && cw_h && nw == ntau) {
-      switch (ntau) {
-        case 6: return line_ct_reg<6>(ctx, slabs, slab_stride, ld, cw_h, out, out_slice, ldo, inv, ncols, st);
-        case 8: return line_ct_reg<8>(ctx, slabs, slab_stride, ld, cw_h, out, out_slice, ldo, inv, ncols, st);
-        case 12: return line_ct_reg<12>(ctx, slabs, slab_stride, ld, cw_h, out, out_slice, ldo, inv, ncols, st);
-        case 16: return line_ct_reg<16>(ctx, slabs, slab_stride, ld, cw_h, out, out_slice, ldo, inv, ncols, st);
-        case 20: return line_ct_reg<20>(ctx, slabs, slab_stride, ld, cw_h, out, out_slice, ldo, inv, ncols, st);
-        default: break;
-      }
+  static gw_status line_ct(gw_ctx* ctx, const void* slabs, long slab_stride, long ld, int ntau, const void* cw,
+                           void* out, long out_slice, long ldo, const int* inv, int cols, int ncols, cudaStream_t st) {
+    if constexpr (std::is_same<T, float>::value) {
+      auto reg = [&](auto nt) {
+        return line_ct_reg<decltype(nt)::value>(ctx, slabs, slab_stride, ld, ntau, cw, out, out_slice, ldo, inv, cols,
+                                                ncols, st);
+      };
+      if (ntau <= 8) return reg(std::integral_constant<int, 8>{});
+      if (ntau <= 12) return reg(std::integral_constant<int, 12>{});
+      if (ntau <= 16) return reg(std::integral_constant<int, 16>{});
+      if (ntau <= 20) return reg(std::integral_constant<int, 20>{});
+      if (ntau <= 24) return reg(std::integral_constant<int, 24>{});
+      return reg(std::integral_constant<int, 32>{});
+    } else {
+      const size_t bytes = (size_t)ntau * N1 * 32 * sizeof(C) + (size_t)ntau * ntau * sizeof(T);
+      auto kernel = col_line_ct_kernel<T, N1>;
+      gw_status s = set_smem(ctx, kernel, bytes);
+      if (s) return s;
+      dim3 grid((ncols + 31) / 32, cols);
+      KTimer kt(ctx, KF_COL_LINE_CT, ((double)ntau * N1 * cols + (double)ntau * ncols) * ncols * sizeof(C), st);
+      kernel<<<grid, 256, bytes, st>>>((const C*)slabs, slab_stride, ld, ntau, (const T*)cw, ntau, (C*)out, out_slice,
+                                       ldo, inv, inv + N1 * N2 * N3 + kSetHead, N2 * N3, ncols);
+      return launch_check(ctx, "col_line_ct_kernel");
     }
-    const size_t bytes = (size_t)ntau * N1 * 32 * sizeof(C) + (size_t)kWParts<T> * nw * ntau * sizeof(T);
-    auto kernel = col_line_ct_kernel<T, N1>;
-    gw_status s = set_smem(ctx, kernel, bytes);
-    if (s) return s;
-    dim3 grid((ncols + 31) / 32, N2 * N3);
-    KTimer kt(ctx, KF_COL_LINE_CT, ((double)ntau * N1 * N2 * N3 + (double)nw * ncols) * ncols * sizeof(C), st);
-    kernel<<<grid, 256, bytes, st>>>((const C*)slabs, slab_stride, ld, ntau, (const T*)cw, nw, (C*)out, out_slice,
-                                     ldo, inv, N2 * N3, ncols);
-    return launch_check(ctx, "col_line_ct_kernel");
   }
 };
 
@@ -1376,58 +1491,54 @@ bool row_two_pass(const GridInfo& g, gw_prec prec) {
 }
 
 gw_status launch_col_plane(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int dir, void* buf, long ld, int ncols,
-                           double scale, cudaStream_t st) {
-  GW_DISPATCH(prec, g, rc = O::plane(ctx, dir, buf, ld, ncols, scale, st))
+                           double scale, const int* inv, int cols, cudaStream_t st) {
+  GW_DISPATCH(prec, g, rc = O::plane(ctx, dir, buf, ld, ncols, scale, inv, cols, st))
 }
 
 gw_status launch_col_line(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int dir, int variant, const void* in,
-                          long ldi, void* out, long ldo, int ncols, const int* inv, double scale, cudaStream_t st) {
-  GW_DISPATCH(prec, g, rc = O::line(ctx, dir, variant, in, ldi, out, ldo, ncols, inv, scale, st))
+                          long ldi, void* out, long ldo, int ncols, const int* inv, int cols, double scale,
+                          cudaStream_t st) {
+  GW_DISPATCH(prec, g, rc = O::line(ctx, dir, variant, in, ldi, out, ldo, ncols, inv, cols, scale, st))
 }
 
 gw_status launch_col_line_ct(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* slabs, long slab_stride,
-                             long ld, int ntau, const void* cw, int nw, void* out, long out_slice, long ldo,
-                             const int* inv, int ncols, cudaStream_t st, const float* cw_h) {
+                             long ld, int ntau, const void* cw, void* out, long out_slice, long ldo, const int* inv,
+                             int cols, int ncols, cudaStream_t st) {
   GW_DISPATCH(prec, g,
-              rc = O::line_ct(ctx, slabs, slab_stride, ld, ntau, cw, nw, out, out_slice, ldo, inv, ncols, st, cw_h))
+              rc = O::line_ct(ctx, slabs, slab_stride, ld, ntau, cw, out, out_slice, ldo, inv, cols, ncols, st))
 }
 
-template <int NT>
-static gw_status launch_ct_reg(gw_ctx* ctx, bool st_kind, const float* w_h, size_t elems, const void* in, void* out,
-                               cudaStream_t st) {
-  CtWeights<NT> w;
-  for (int e = 0; e < NT * NT; ++e) {
-    w.hi[e] = w_h[e];
-    w.lo[e] = w_h[NT * NT + e];
-  }
-  KTimer kt(ctx, KF_CT, 2.0 * NT * (double)elems * sizeof(float2), st);
-  const int blocks = (int)std::min<size_t>((elems + 255) / 256, (size_t)ctx->num_sms * 12);
-  if (st_kind) ct_reg1_kernel<NT, true><<<blocks, 256, 0, st>>>((const float2*)in, (float2*)out, elems, w);
-  else ct_reg1_kernel<NT, false><<<blocks, 256, 0, st>>>((const float2*)in, (float2*)out, elems, w);
-  return launch_check(ctx, "ct_reg_kernel");
+template <int NTB>
+static gw_status launch_ct_reg(gw_ctx* ctx, bool st_kind, int n, const void* dM, size_t elems, const void* in,
+                               void* out, cudaStream_t st) {
+  KTimer kt(ctx, KF_CT, 2.0 * n * (double)elems * sizeof(float2), st);
+  const bool two = elems % 2 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0;
+  const size_t items = two ? elems / 2 : elems;
+  const int blocks = (int)std::min<size_t>((items + 127) / 128, (size_t)ctx->num_sms * 24);
+  auto go = [&](auto kernel) -> gw_status {
+    kernel<<<blocks, 128, 0, st>>>((const float2*)in, (float2*)out, elems, n, (const float*)dM);
+    return launch_check(ctx, "ct_reg_kernel");
+  };
+  if (two) return st_kind ? go(ct_reg_kernel<NTB, true, 2>) : go(ct_reg_kernel<NTB, false, 2>);
+  return st_kind ? go(ct_reg_kernel<NTB, true, 1>) : go(ct_reg_kernel<NTB, false, 1>);
 }
 
 gw_status launch_ct(gw_ctx* ctx, gw_prec prec, bool st_kind, int n, const void* dM, size_t elems, const void* in,
-                    void* out, cudaStream_t st, const float* w_h) {
+                    void* out, cudaStream_t st) {
   if (elems == 0) return GW_OK;
-  if (!is_fp64(prec) && w_h) {
-    switch (n) {
-      case 6: return launch_ct_reg<6>(ctx, st_kind, w_h, elems, in, out, st);
-      case 8: return launch_ct_reg<8>(ctx, st_kind, w_h, elems, in, out, st);
-      case 12: return launch_ct_reg<12>(ctx, st_kind, w_h, elems, in, out, st);
-      case 16: return launch_ct_reg<16>(ctx, st_kind, w_h, elems, in, out, st);
-      case 20: return launch_ct_reg<20>(ctx, st_kind, w_h, elems, in, out, st);
-      default: break;
-    }
+  if (!is_fp64(prec)) {
+    if (n <= 4) return launch_ct_reg<4>(ctx, st_kind, n, dM, elems, in, out, st);
+    if (n <= 8) return launch_ct_reg<8>(ctx, st_kind, n, dM, elems, in, out, st);
+    if (n <= 12) return launch_ct_reg<12>(ctx, st_kind, n, dM, elems, in, out, st);
+    if (n <= 16) return launch_ct_reg<16>(ctx, st_kind, n, dM, elems, in, out, st);
+    if (n <= 20) return launch_ct_reg<20>(ctx, st_kind, n, dM, elems, in, out, st);
+    if (n <= 24) return launch_ct_reg<24>(ctx, st_kind, n, dM, elems, in, out, st);
+    return launch_ct_reg<32>(ctx, st_kind, n, dM, elems, in, out, st);
   }
   int blocks = (int)std::min<size_t>((elems + 255) / 256, (size_t)ctx->num_sms * 8);
-  if (is_fp64(prec)) {
-    if (st_kind) ct_kernel<double, true><<<blocks, 256, 0, st>>>((const double2*)in, (double2*)out, elems, n, (const double*)dM);
-    else ct_kernel<double, false><<<blocks, 256, 0, st>>>((const double2*)in, (double2*)out, elems, n, (const double*)dM);
-  } else {
-    if (st_kind) ct_kernel<float, true><<<blocks, 256, 0, st>>>((const float2*)in, (float2*)out, elems, n, (const float*)dM);
-    else ct_kernel<float, false><<<blocks, 256, 0, st>>>((const float2*)in, (float2*)out, elems, n, (const float*)dM);
-  }
+  KTimer kt(ctx, KF_CT, 2.0 * n * (double)elems * sizeof(double2), st);
+  if (st_kind) ct_kernel<true><<<blocks, 256, 0, st>>>((const double2*)in, (double2*)out, elems, n, (const double*)dM);
+  else ct_kernel<false><<<blocks, 256, 0, st>>>((const double2*)in, (double2*)out, elems, n, (const double*)dM);
   return launch_check(ctx, "ct_kernel");
 }
 
@@ -1528,6 +1639,7 @@ extern "C" gw_status gw_rr_to_GG_fft(gw_ctx* ctx, const gw_grid* grid, int direc
   if ((st = index_maps(ctx, g, fft_index_h, n_chi, map, inv))) return st;
   if (stage == 1 && (n_rows < 0 || r0 < 0 || r0 + n_rows > g.nr)) return fail(ctx, GW_ERR_SHAPE, "rows out of range");
   cudaStream_t s = as_stream(stream);
+  const int cols = set_columns(g, inv);
   // rows too long for shared memory need a [n_rows][N_r] workspace forward
   const bool work_rows = stage == 1 && direction > 0 && row_two_pass(g, prec);
   Carver probe(nullptr);
@@ -1550,12 +1662,12 @@ extern "C" gw_status gw_rr_to_GG_fft(gw_ctx* ctx, const gw_grid* grid, int direc
   if (direction > 0) {
     // in [N_r][n_chi] is the work buffer: (i2,i3) planes in place, then the i1 pass writes the G rows of out.
     void* work = const_cast<void*>(in);
-    if ((st = launch_col_plane(ctx, g, prec, -1, work, n_chi, n_chi, 1.0, s))) return st;
-    return launch_col_line(ctx, g, prec, -1, 2, work, n_chi, out, n_chi, n_chi, dinv, g.dv * g.dv / g.volume, s);
+    if ((st = launch_col_plane(ctx, g, prec, -1, work, n_chi, n_chi, 1.0, dinv, cols, s))) return st;
+    return launch_col_line(ctx, g, prec, -1, 2, work, n_chi, out, n_chi, n_chi, dinv, cols, g.dv * g.dv / g.volume, s);
   }
   // W(G,G') -> W(r,G'): i1 pass gathering the G rows, then the (i2,i3) planes in place in out.
-  if ((st = launch_col_line(ctx, g, prec, +1, 1, in, n_chi, out, n_chi, n_chi, dinv, 1.0, s))) return st;
-  return launch_col_plane(ctx, g, prec, +1, out, n_chi, n_chi, 1.0, s);
+  if ((st = launch_col_line(ctx, g, prec, +1, 1, in, n_chi, out, n_chi, n_chi, dinv, cols, 1.0, s))) return st;
+  return launch_col_plane(ctx, g, prec, +1, out, n_chi, n_chi, 1.0, dinv, cols, s);
 }
 
 extern "C" gw_status gw_tau_to_omega(gw_ctx* ctx, int kind, int n, const double* M_h, size_t elems, gw_prec prec,
@@ -1582,7 +1694,7 @@ extern "C" gw_status gw_tau_to_omega(gw_ctx* ctx, int kind, int n, const double*
     m32 = split_weights(M_h, n * n, 1.0);
     if ((st = upload(ctx, ctx->arena, m32.data(), sizeof(float) * 2 * n * n, s))) return st;
   }
-  return launch_ct(ctx, prec, kind != GW_CT, n, ctx->arena, elems, in, out, s, m32.empty() ? nullptr : m32.data());
+  return launch_ct(ctx, prec, kind != GW_CT, n, ctx->arena, elems, in, out, s);
 }
 
 // ---------------------------------------------------------------------- no-allocation variant
@@ -1665,6 +1777,7 @@ extern "C" gw_status gw_rr_to_GG_fft_noalloc(const gw_grid* grid, int direction,
                                                std::to_string(kNoAllocMaxInts) + " entries"));
   if (stage == 1 && (n_rows < 0 || r0 < 0 || r0 + n_rows > g.nr))
     return done(fail(&local, GW_ERR_SHAPE, "rows out of range"));
+  const int cols = set_columns(g, inv);
   int* maps = nullptr;
   if ((st = noalloc_maps_ptr(&local, &maps))) return done(st);
   int* dmap = maps;
@@ -1679,9 +1792,9 @@ extern "C" gw_status gw_rr_to_GG_fft_noalloc(const gw_grid* grid, int direction,
   }
   if (direction > 0) {
     void* work = const_cast<void*>(in);
-    if ((st = launch_col_plane(&local, g, prec, -1, work, n_chi, n_chi, 1.0, s))) return done(st);
-    return done(launch_col_line(&local, g, prec, -1, 2, work, n_chi, out, n_chi, n_chi, dinv, g.dv * g.dv / g.volume, s));
+    if ((st = launch_col_plane(&local, g, prec, -1, work, n_chi, n_chi, 1.0, dinv, cols, s))) return done(st);
+    return done(launch_col_line(&local, g, prec, -1, 2, work, n_chi, out, n_chi, n_chi, dinv, cols, g.dv * g.dv / g.volume, s));
   }
-  if ((st = launch_col_line(&local, g, prec, +1, 1, in, n_chi, out, n_chi, n_chi, dinv, 1.0, s))) return done(st);
-  return done(launch_col_plane(&local, g, prec, +1, out, n_chi, n_chi, 1.0, s));
+  if ((st = launch_col_line(&local, g, prec, +1, 1, in, n_chi, out, n_chi, n_chi, dinv, cols, 1.0, s))) return done(st);
+  return done(launch_col_plane(&local, g, prec, +1, out, n_chi, n_chi, 1.0, dinv, cols, s));
 }

@@ -78,15 +78,21 @@ gw_status launch_sigma_contract(gw_ctx* ctx, gw_prec prec, const void* wrr, cons
 gw_status sigma_finish(gw_ctx* ctx, double* acc, int n_n, int n, const double* tab, int n_real, double2* out,
                        int* stat, const int32_t* labels, double* sigma_tau_h, double* sigma_iw_h,
                        double* sigma_real_h, cudaStream_t s);
+// Column transforms of a matrix with N_r rows (grid points) over its G set (inv on
+// the device, cols = set_columns): only the (i2,i3) rows that the set touches pass
+// between the plane and the line kernels (dir -1: planes, then lines to the G rows;
+// dir +1: lines from the G rows, then planes).
 gw_status launch_col_plane(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int dir, void* buf, long ld, int ncols,
-                           double scale, cudaStream_t st);
+                           double scale, const int* inv, int cols, cudaStream_t st);
 gw_status launch_col_line(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int dir, int variant, const void* in,
-                          long ldi, void* out, long ldo, int ncols, const int* inv, double scale, cudaStream_t st);
+                          long ldi, void* out, long ldo, int ncols, const int* inv, int cols, double scale,
+                          cudaStream_t st);
+// cw: [ntau][ntau] weights on the device (FP64, or FP32 hi then lo).
 gw_status launch_col_line_ct(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* slabs, long slab_stride,
-                             long ld, int ntau, const void* cw, int nw, void* out, long out_slice, long ldo,
-                             const int* inv, int ncols, cudaStream_t st, const float* cw_h = nullptr);
+                             long ld, int ntau, const void* cw, void* out, long out_slice, long ldo, const int* inv,
+                             int cols, int ncols, cudaStream_t st);
 gw_status launch_ct(gw_ctx* ctx, gw_prec prec, bool st_kind, int n, const void* dM, size_t elems, const void* in,
-                    void* out, cudaStream_t st, const float* w_h = nullptr);
+                    void* out, cudaStream_t st);
 gw_status launch_hadamard(gw_ctx* ctx, gw_prec prec, size_t count, const void* a, const void* b, double scale,
                           void* out, cudaStream_t st);
 gw_status upload(gw_ctx* ctx, void* dst, const void* src, size_t bytes, cudaStream_t st);
@@ -151,6 +157,7 @@ gw_status screen_launch(gw_ctx* ctx, int n_chi, int n_omega, gw_prec prec, int r
 struct SigmaTables {
   int* map;
   int* inv;
+  int cols = 0;       // (i2,i3) columns that the G set touches
   int* bands;
   char* scale;
   double* tab;
@@ -178,7 +185,7 @@ gw_status sigma_check(gw_ctx* ctx, const gw_grid* grid, GridInfo* g, int n_b, in
                       const double* omega_h, const double* C_h, const double* S_h, const void* w_tau, int n_chi,
                       const int32_t* fft_index_h, gw_prec prec, bool full, const double* w_real_h, int n_real,
                       std::vector<int>& map, std::vector<int>& inv, std::vector<GreenScales>& scales);
-gw_status sigma_upload_tables(gw_ctx* ctx, const SigmaTables& t, const GridInfo& g, int n_b, int n, int n_chi,
+gw_status sigma_upload_tables(gw_ctx* ctx, SigmaTables& t, const GridInfo& g, int n_b, int n, int n_chi,
                               const std::vector<int>& map, const std::vector<int>& inv, const int32_t* bands_h, int n_n,
                               const std::vector<GreenScales>& scales, const double* C_h, const double* S_h,
                               const double* omega_h, const double* w_real_h, int n_real, gw_prec prec, cudaStream_t s);

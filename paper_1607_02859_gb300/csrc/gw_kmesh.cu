@@ -382,12 +382,12 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
         return st;
     }
     if ((st = launch_q_phase(ctx, prec, g, nk, dqph, slab_j, ld, n_chi, -1.0, s))) return st;
-    if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, ld, (int)ld, 1.0, s))) return st;
+    if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, ld, (int)ld, 1.0, dinv, set_columns(g, inv), s))) return st;
   }
   for (int q = 0; q < n_k; ++q) {
     char* out_q = static_cast<char*>(chi_w) + (size_t)q * n * n_chi * n_chi * es;
-    if ((st = launch_col_line_ct(ctx, g, prec, slabs + (size_t)q * n_chi * es, (long)slab, ld, n, dcw, n, out_q,
-                                 (long)n_chi * n_chi, n_chi, dinv, n_chi, s, cw32.empty() ? nullptr : cw32.data())))
+    if ((st = launch_col_line_ct(ctx, g, prec, slabs + (size_t)q * n_chi * es, (long)slab, ld, n, dcw, out_q,
+                                 (long)n_chi * n_chi, n_chi, dinv, set_columns(g, inv), n_chi, s)))
       return st;
   }
   return tc ? tc_check(ctx, tcs, s) : GW_OK;
@@ -542,8 +542,8 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
       for (int part = 0; part < 2; ++part) {
         const char* m = part ? mu_ : mo;
         char* t = (part ? tu : to) + (size_t)k * n_pw * es;
-        if ((st = launch_col_line(ctx, g, prec, +1, 1, m, n_pw, t, ldt, n_pw, dinv_pw, 1.0, s))) return st;
-        if ((st = launch_col_plane(ctx, g, prec, +1, t, ldt, n_pw, 1.0, s))) return st;
+        if ((st = launch_col_line(ctx, g, prec, +1, 1, m, n_pw, t, ldt, n_pw, dinv_pw, set_columns(g, inv_pw), 1.0, s))) return st;
+        if ((st = launch_col_plane(ctx, g, prec, +1, t, ldt, n_pw, 1.0, dinv_pw, set_columns(g, inv_pw), s))) return st;
       }
     }
     // exp(-i k.r) on the block of each k, then per row: expand, multiply, transform onto {q + g}
@@ -554,12 +554,12 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
                                 chi_cols, g.nr, row_scale, rwork, s)))
       return st;
     if ((st = launch_q_phase(ctx, prec, g, nk, dqph, slab_j, ld, n_chi, -1.0, s))) return st;
-    if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, ld, (int)ld, 1.0, s))) return st;
+    if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, ld, (int)ld, 1.0, dinv, set_columns(g, inv), s))) return st;
   }
   for (int q = 0; q < n_k; ++q) {
     char* out_q = static_cast<char*>(chi_w) + (size_t)q * n * n_chi * n_chi * es;
-    if ((st = launch_col_line_ct(ctx, g, prec, slabs + (size_t)q * n_chi * es, (long)slab, ld, n, dcw, n, out_q,
-                                 (long)n_chi * n_chi, n_chi, dinv, n_chi, s, cw32.empty() ? nullptr : cw32.data())))
+    if ((st = launch_col_line_ct(ctx, g, prec, slabs + (size_t)q * n_chi * es, (long)slab, ld, n, dcw, out_q,
+                                 (long)n_chi * n_chi, n_chi, dinv, set_columns(g, inv), n_chi, s)))
       return st;
   }
   return tc ? tc_check(ctx, tcs, s) : GW_OK;
@@ -691,8 +691,8 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
     for (int q = 0; q < n_k; ++q) {
       const char* wq = static_cast<const char*>(w_tau) + ((size_t)q * n + j) * n_chi * n_chi * es;
       char* blk = wrg + (size_t)q * n_chi * es;
-      if ((st = launch_col_line(ctx, g, prec, +1, 1, wq, n_chi, blk, ld, n_chi, dinv, 1.0, s))) return st;
-      if ((st = launch_col_plane(ctx, g, prec, +1, blk, ld, n_chi, 1.0, s))) return st;
+      if ((st = launch_col_line(ctx, g, prec, +1, 1, wq, n_chi, blk, ld, n_chi, dinv, set_columns(g, inv), 1.0, s))) return st;
+      if ((st = launch_col_plane(ctx, g, prec, +1, blk, ld, n_chi, 1.0, dinv, set_columns(g, inv), s))) return st;
     }
     if ((st = launch_q_phase(ctx, prec, g, nk, dqph, wrg, ld, n_chi, +1.0, s))) return st;
     for (int r0 = 0; r0 < g.nr; r0 += rb) {

@@ -74,7 +74,8 @@ static gw_status launch_hermitize(gw_ctx* ctx, gw_prec prec, int n, int n_chi, v
 // Device tables of one chi0 evaluation.
 struct Chi0Dev {
   const int* map = nullptr;      // [n_chi] FFT positions of the G set
-  const int* inv = nullptr;      // [N_r] position -> G index or -1
+  const int* inv = nullptr;      // [N_r] position -> G index or -1, and the set's lists
+  int cols = 0;                  // (i2,i3) columns that the set touches
   const char* scale = nullptr;   // CUDA-core path: [n][n_b] per-band factors in 8-byte slots
   const float* sk = nullptr;     // tensor path: [n][n_b] FP32 factors, or NULL to copy them per call
   const void* cw = nullptr;      // transform weights, dV^2/Omega folded in (FP32 hi/lo or FP64)
@@ -116,7 +117,7 @@ static void chi0_tables(const GridInfo& g, int n_b, int n_occ, const double* eps
 // status region for tc_check.
 static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, int n,
                              const std::vector<GreenScales>& scales, int n_chi, gw_prec prec, int rb,
-                             const Chi0Dev& t, const std::vector<float>& cw32, Carver& cv, void* chi_w,
+                             const Chi0Dev& t, Carver& cv, void* chi_w,
                              cudaStream_t s, void** tcs_out) {
   gw_status st;
   const size_t es = csize(prec);
@@ -148,10 +149,10 @@ static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ,
       }
       if (st) return st;
     }
-    if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, n_chi, n_chi, 1.0, s))) return st;
+    if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, n_chi, n_chi, 1.0, t.inv, t.cols, s))) return st;
   }
-  if ((st = launch_col_line_ct(ctx, g, prec, slabs, (long)slab, n_chi, n, t.cw, n, chi_w, (long)n_chi * n_chi, n_chi,
-                               t.inv, n_chi, s, cw32.empty() ? nullptr : cw32.data())))
+  if ((st = launch_col_line_ct(ctx, g, prec, slabs, (long)slab, n_chi, n, t.cw, chi_w, (long)n_chi * n_chi, n_chi,
+                               t.inv, t.cols, n_chi, s)))
     return st;
   return launch_hermitize(ctx, prec, n, n_chi, chi_w, s);    // the rows hold R' <= r only
 }
@@ -195,10 +196,11 @@ extern "C" gw_status gw_chi0_omega(gw_ctx* ctx, const gw_grid* grid, int n_b, in
   Chi0Dev t;
   t.map = dmap;
   t.inv = dinv;
+  t.cols = set_columns(g, inv);
   t.scale = dscale;
   t.cw = dcw;
   void* tcs = nullptr;
-  if ((st = chi0_launch(ctx, g, n_b, n_occ, psi, n, scales, n_chi, prec, rb, t, cw32, cv, chi_w, s, &tcs))) return st;
+  if ((st = chi0_launch(ctx, g, n_b, n_occ, psi, n, scales, n_chi, prec, rb, t, cv, chi_w, s, &tcs))) return st;
   return tc ? tc_check(ctx, tcs, s) : GW_OK;
 }
 
@@ -406,18 +408,18 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
     for (int part = 0; part < 2; ++part) {
       char* m = part ? mu_ : mo;
       char* t = part ? tu : to;
-      if ((st = launch_col_line(ctx, g, prec, +1, 1, m, n_pw, t, n_pw, n_pw, dinv_pw, 1.0, s))) return st;
-      if ((st = launch_col_plane(ctx, g, prec, +1, t, n_pw, n_pw, 1.0, s))) return st;
+      if ((st = launch_col_line(ctx, g, prec, +1, 1, m, n_pw, t, n_pw, n_pw, dinv_pw, pw_cols, 1.0, s))) return st;
+      if ((st = launch_col_plane(ctx, g, prec, +1, t, n_pw, n_pw, 1.0, dinv_pw, pw_cols, s))) return st;
     }
     // chi(r, G', tau_j) for every row r: expand, multiply (Eq. chi_rr), transform (Eq. FFTX1)
     char* slab_j = slabs + (size_t)j * slab * es;
     if ((st = launch_row_pw_chi(ctx, g, prec, tu, to, n_pw, slab_j, n_chi, dinv_pw, n_pw, pw_cols, dinv, n_chi,
                                 chi_cols, g.nr, -2.0, rwork, s, 0)))
       return st;
-    if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, n_chi, n_chi, 1.0, s))) return st;
+    if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, n_chi, n_chi, 1.0, dinv, chi_cols, s))) return st;
   }
-  if ((st = launch_col_line_ct(ctx, g, prec, slabs, (long)slab, n_chi, n, dcw, n, chi_w, (long)n_chi * n_chi, n_chi,
-                               dinv, n_chi, s, cw32.empty() ? nullptr : cw32.data())))
+  if ((st = launch_col_line_ct(ctx, g, prec, slabs, (long)slab, n_chi, n, dcw, chi_w, (long)n_chi * n_chi, n_chi,
+                               dinv, chi_cols, n_chi, s)))
     return st;
   if ((st = launch_hermitize(ctx, prec, n, n_chi, chi_w, s))) return st;
   return tc ? tc_check(ctx, tcs, s) : GW_OK;
@@ -505,6 +507,7 @@ extern "C" gw_status gw_chi0_plan_create(gw_ctx* ctx, const gw_grid* grid, int n
   char* d = static_cast<char*>(p->dev);
   p->t.map = reinterpret_cast<const int*>(d + o_map);
   p->t.inv = reinterpret_cast<const int*>(d + o_inv);
+  p->t.cols = set_columns(g, inv);
   p->t.scale = d + o_scale;
   p->t.sk = reinterpret_cast<const float*>(d + o_sk);
   p->t.cw = d + o_cw;
@@ -525,7 +528,7 @@ extern "C" gw_status gw_chi0_plan_launch(gw_chi0_plan* p, const void* psi, void*
   if (!psi || !chi_w) return fail(ctx, GW_ERR_ARG, "NULL pointer");
   if (ctx->arena_bytes < p->work) return fail(ctx, GW_ERR_ARG, "the context arena is smaller than the plan's");
   Carver cv(ctx->arena);
-  return chi0_launch(ctx, p->g, p->n_b, p->n_occ, psi, p->n, p->scales, p->n_chi, p->prec, p->rb, p->t, p->cw32, cv,
+  return chi0_launch(ctx, p->g, p->n_b, p->n_occ, psi, p->n, p->scales, p->n_chi, p->prec, p->rb, p->t, cv,
                      chi_w, as_stream(stream), nullptr);
 }
 

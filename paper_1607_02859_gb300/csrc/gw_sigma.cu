@@ -578,11 +578,12 @@ size_t sigma_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_chi, in
   return probe.off;
 }
 
-gw_status sigma_upload_tables(gw_ctx* ctx, const SigmaTables& t, const GridInfo& g, int n_b, int n, int n_chi,
+gw_status sigma_upload_tables(gw_ctx* ctx, SigmaTables& t, const GridInfo& g, int n_b, int n, int n_chi,
                               const std::vector<int>& map, const std::vector<int>& inv, const int32_t* bands_h, int n_n,
                               const std::vector<GreenScales>& scales, const double* C_h, const double* S_h,
                               const double* omega_h, const double* w_real_h, int n_real, gw_prec prec, cudaStream_t s) {
   gw_status st;
+  t.cols = set_columns(g, inv);
   if ((st = upload(ctx, t.map, map.data(), sizeof(int) * n_chi, s))) return st;
   if ((st = upload(ctx, t.inv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if ((st = upload(ctx, t.bands, bands_h, sizeof(int) * n_n, s))) return st;
@@ -624,8 +625,8 @@ gw_status sigma_kernels(gw_ctx* ctx, const GridInfo& g, gw_prec prec, bool full,
   for (int j = 0; j < n; ++j) {
     const char* wj = static_cast<const char*>(w_tau) + (size_t)j * n_chi * n_chi * es;
     const char* sj = t.scale + (size_t)j * n_b * 8;
-    if ((st = launch_col_line(ctx, g, prec, +1, 1, wj, n_chi, w.wrg, n_chi, n_chi, t.inv, 1.0, s))) return st;
-    if ((st = launch_col_plane(ctx, g, prec, +1, w.wrg, n_chi, n_chi, 1.0, s))) return st;
+    if ((st = launch_col_line(ctx, g, prec, +1, 1, wj, n_chi, w.wrg, n_chi, n_chi, t.inv, t.cols, 1.0, s))) return st;
+    if ((st = launch_col_plane(ctx, g, prec, +1, w.wrg, n_chi, n_chi, 1.0, t.inv, t.cols, s))) return st;
     for (int r0 = 0; r0 < g.nr; r0 += rb) {
       const int rows = std::min(rb, g.nr - r0);
       if (w.fused) {
@@ -845,6 +846,7 @@ extern "C" gw_status gw_sigma_diag_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   std::vector<int> map_neg = map_nat, inv_neg = inv_nat;
   pw_negate(g, map_neg, inv_neg);
   if ((st = check_row_pw_sigma(ctx, g, prec, n_pw, n_chi))) return st;
+  const int pw_cols = set_columns(g, inv_neg);
   cudaStream_t s = as_stream(stream);
   const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
   const size_t es = csize(prec);
@@ -913,12 +915,12 @@ extern "C" gw_status gw_sigma_diag_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
     for (int part = 0; part < 2; ++part) {
       char* m = part ? mu_ : mo;
       char* tt = part ? tu : to;
-      if ((st = launch_col_line(ctx, g, prec, +1, 1, m, n_pw, tt, n_pw, n_pw, dinv_neg, 1.0, s))) return st;
-      if ((st = launch_col_plane(ctx, g, prec, +1, tt, n_pw, n_pw, 1.0, s))) return st;
+      if ((st = launch_col_line(ctx, g, prec, +1, 1, m, n_pw, tt, n_pw, n_pw, dinv_neg, pw_cols, 1.0, s))) return st;
+      if ((st = launch_col_plane(ctx, g, prec, +1, tt, n_pw, n_pw, 1.0, dinv_neg, pw_cols, s))) return st;
     }
     const char* wj = static_cast<const char*>(w_tau) + (size_t)j * n_chi * n_chi * es;
-    if ((st = launch_col_line(ctx, g, prec, +1, 1, wj, n_chi, wg, n_chi, n_chi, t.inv, 1.0, s))) return st;
-    if ((st = launch_col_plane(ctx, g, prec, +1, wg, n_chi, n_chi, 1.0, s))) return st;
+    if ((st = launch_col_line(ctx, g, prec, +1, 1, wj, n_chi, wg, n_chi, n_chi, t.inv, t.cols, 1.0, s))) return st;
+    if ((st = launch_col_plane(ctx, g, prec, +1, wg, n_chi, n_chi, 1.0, t.inv, t.cols, s))) return st;
     if ((st = launch_row_pw_sigma(ctx, g, prec, tu, to, n_pw, wg, n_chi, hu, ho, n_pw, dinv_neg, dinv_nat, n_pw, t.inv,
                                   n_chi, g.nr, s)))
       return st;
@@ -1073,8 +1075,8 @@ extern "C" gw_status gw_sigma_to_tau(gw_ctx* ctx, int n_n, int n, int matrix, co
   sigma_split_kernel<<<(unsigned)((E + 127) / 128), 128, 0, s>>>(dsig, n_n, n, matrix, herm, anti);
   if ((st = launch_check(ctx, "sigma_split_kernel"))) return st;
   // Eq. INV_CT_FFT on the cosine part, Eq. INV_ST_FFT (-i zeta sin) on the sine part, in FP64
-  if ((st = launch_ct(ctx, GW_FP64, false, n, dM, (size_t)E, herm, sc, s, nullptr))) return st;
-  if ((st = launch_ct(ctx, GW_FP64, true, n, dM + (size_t)n * n, (size_t)E, anti, ss, s, nullptr))) return st;
+  if ((st = launch_ct(ctx, GW_FP64, false, n, dM, (size_t)E, herm, sc, s))) return st;
+  if ((st = launch_ct(ctx, GW_FP64, true, n, dM + (size_t)n * n, (size_t)E, anti, ss, s))) return st;
   sigma_combine_kernel<<<(unsigned)((cplx + 255) / 256), 256, 0, s>>>(sc, ss, E, n, matrix,
                                                                       reinterpret_cast<double*>(dout));
   if ((st = launch_check(ctx, "sigma_combine_kernel"))) return st;
