@@ -33,6 +33,7 @@
 
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "gw_tc.h"
 #include "gw_tcgen05.cuh"
@@ -113,6 +114,13 @@ struct Params {
 // producer loads the tile's psi_n operand behind it, and the MMA warp
 // accumulates V for each half of the tile's columns in the free half of
 // tensor memory; unoccupied first, then occupied in the same shared memory.
+// The epilogue is not overlapped with MMAs, so its length counts: W~ is read
+// once, in 64-byte pieces into the place its own H will take, for both products
+// (H_occ waits in tensor memory), and the band sums are reduced by exchange.  With
+// one row of W~ per lane straight from global memory, twice, and five shuffles
+// and a double atomic per band, a tile's epilogue took 90 (4 bands) to 154
+// (32 bands) thousand cycles, now 38 and 50; sigma at 20^3 with 512 bands 14.9 ->
+// 10.4 ms, at 36^3 with 4224 bands and 2 tau 207 -> 170 ms.
 template <int MODE, uint32_t FMT>
 __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_constant__ CUtensorMap mA_hi,
                                                               const __grid_constant__ CUtensorMap mA_lo,
@@ -137,7 +145,7 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
   uint64_t* psi_full = vready + 2;       // psi_n operand of the tile landed
   uint64_t* redbar = psi_full + 1;       // the epilogue warps' band sums are in shared memory
   uint64_t* done2 = redbar + 1;          // every MMA of the self-energy phase done
-  double* red = reinterpret_cast<double*>(epi);   // [2][32] band sums of the CTA (MODE 2 only)
+  float* red = reinterpret_cast<float*>(epi);     // [8 warps][32][2] band sums of the warps (MODE 2 only)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // tiles in groups of kGroupRows row tiles: the CTAs that run together walk a group's rows for
@@ -181,7 +189,6 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
       mbar_init(psi_full, 1);
       mbar_init(redbar, EPI_WARPS);
       mbar_init(done2, 1);
-      for (int i = 0; i < 64; ++i) red[i] = 0.0;
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -378,48 +385,90 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
         const int row = q * 32 + lane;               // tensor-memory lane = tile row
         const int gm = m0 + row;
         const bool rvalid = gm < p.m_rows;
-        const float2* wrow = p.wrr + (long)(rvalid ? gm : 0) * p.ldw;
         const int c0 = n0 + h * 64;                   // first complex column of this warp's half
-        const bool vec = (p.ldw % 2 == 0) && ((reinterpret_cast<uintptr_t>(p.wrr) & 15) == 0);
-        // H = g tot o W~ in place; returns the power of two that puts the row's max below 2^15
         const long grow = grow0 + row;             // grid row r of this thread
-        auto times_w = [&](float g) -> int {
-          float m = 0.f;
-#pragma unroll
-          for (int c = 0; c < 64; c += 2) {
-            const int gn = c0 + c;
-            float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
-            // weight of (r, R'): 2 below the diagonal, 1 on it, 0 above (lower-triangle mode)
-            float wa = 1.f, wb = 1.f;
-            if (p.lower) {
-              wa = gn < grow ? 2.f : (gn == grow ? 1.f : 0.f);
-              wb = gn + 1 < grow ? 2.f : (gn + 1 == grow ? 1.f : 0.f);
+        const int swz = (row >> 1) & 3;
+        // The warp's 32 x 64 block of W~ goes through the shared memory that its own H will take:
+        // piece k (8 columns, 64 bytes a row) in the place of the warp's rows of K chunk 4h + k % 4,
+        // hi for k < 4 and lo above, 16-byte segments swizzled as H's.  Row r lies where row r of H
+        // will, so a thread only overwrites what it has read itself.
+        auto piece = [&](int k) -> uint8_t* {
+          return (k < 4 ? h_hi : h_lo) + (4 * h + (k & 3)) * A_BYTES + q * 2048;
+        };
+        {
+          const bool vec = (p.ldw % 2 == 0) && ((reinterpret_cast<uintptr_t>(p.wrr) & 15) == 0);
+#pragma unroll 4
+          for (int i = 0; i < 32; ++i) {              // eight rows of a piece per step, 64 bytes each
+            const int k = i >> 2, r = (i & 3) * 8 + (lane >> 2), sg = lane & 3;
+            const int gr = m0 + q * 32 + r, gn = c0 + 8 * k + 2 * sg;
+            uint8_t* dst = piece(k) + r * 64 + ((sg ^ ((r >> 1) & 3)) << 4);
+            const int have = gr < p.m_rows ? min(max(p.n_cols - gn, 0), 2) : 0;   // columns of the pair in range
+            const float2* src = have ? p.wrr + (long)gr * p.ldw + gn : p.wrr;
+            if (vec) {
+              cp_async16(dst, src, 8 * have);
+            } else {
+              cp_async8(dst, src, have > 0 ? 8 : 0);
+              cp_async8(dst + 8, have > 1 ? src + 1 : p.wrr, have > 1 ? 8 : 0);
             }
-            if (rvalid) {
-              if (vec && gn + 1 < p.n_cols) {
-                w = __ldg(reinterpret_cast<const float4*>(wrow + gn));
-              } else {
-                if (gn < p.n_cols) {
-                  const float2 a = wrow[gn];
-                  w.x = a.x;
-                  w.y = a.y;
-                }
-                if (gn + 1 < p.n_cols) {
-                  const float2 b = wrow[gn + 1];
-                  w.z = b.x;
-                  w.w = b.y;
-                }
+          }
+          cp_async_wait();
+          __syncwarp();
+        }
+        // H = w G o W~ for G_unocc in registers and for G_occ in tensor memory (in place); returns the
+        // powers of two that put the rows' maxima below 2^15
+        const uint32_t occ = tmem + lane_addr + (uint32_t)(bo * 256 + h * 128);
+        float mu = 0.f, mo = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const uint8_t* wp = piece(k) + lane * 64;
+#pragma unroll
+          for (int hs = 0; hs < 2; ++hs) {
+            uint32_t x[8];
+            tmem_ld8(occ + 16 * k + 8 * hs, x);
+            float4 w2[2];
+#pragma unroll
+            for (int s = 0; s < 2; ++s) w2[s] = *reinterpret_cast<const float4*>(wp + (((2 * hs + s) ^ swz) << 4));
+            tmem_wait_ld();
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+              const float4 w = w2[s];
+              const int c = 8 * k + 4 * hs + 2 * s;
+              const int gn = c0 + c;
+              // weight of (r, R'): 2 below the diagonal, 1 on it, 0 above (lower-triangle mode)
+              float wa = 1.f, wb = 1.f;
+              if (p.lower) {
+                wa = gn < grow ? 2.f : (gn == grow ? 1.f : 0.f);
+                wb = gn + 1 < grow ? 2.f : (gn + 1 == grow ? 1.f : 0.f);
+              }
+              {
+                const float ar = tot[2 * c] * au * wa, ai = tot[2 * c + 1] * au * wa;
+                const float br = tot[2 * c + 2] * au * wb, bi = tot[2 * c + 3] * au * wb;
+                tot[2 * c] = ar * w.x - ai * w.y;
+                tot[2 * c + 1] = ar * w.y + ai * w.x;
+                tot[2 * c + 2] = br * w.z - bi * w.w;
+                tot[2 * c + 3] = br * w.w + bi * w.z;
+                mu = fmaxf(mu, fmaxf(fmaxf(fabsf(tot[2 * c]), fabsf(tot[2 * c + 1])),
+                                     fmaxf(fabsf(tot[2 * c + 2]), fabsf(tot[2 * c + 3]))));
+              }
+              {
+                const float g0 = __uint_as_float(x[4 * s]), g1 = __uint_as_float(x[4 * s + 1]);
+                const float g2 = __uint_as_float(x[4 * s + 2]), g3 = __uint_as_float(x[4 * s + 3]);
+                const float ar = g0 * ao * wa, ai = g1 * ao * wa;
+                const float br = g2 * ao * wb, bi = g3 * ao * wb;
+                const float y0 = ar * w.x - ai * w.y, y1 = ar * w.y + ai * w.x;
+                const float y2 = br * w.z - bi * w.w, y3 = br * w.w + bi * w.z;
+                mo = fmaxf(mo, fmaxf(fmaxf(fabsf(y0), fabsf(y1)), fmaxf(fabsf(y2), fabsf(y3))));
+                x[4 * s] = __float_as_uint(y0);
+                x[4 * s + 1] = __float_as_uint(y1);
+                x[4 * s + 2] = __float_as_uint(y2);
+                x[4 * s + 3] = __float_as_uint(y3);
               }
             }
-            const float ar = tot[2 * c] * g * wa, ai = tot[2 * c + 1] * g * wa;
-            const float br = tot[2 * c + 2] * g * wb, bi = tot[2 * c + 3] * g * wb;
-            tot[2 * c] = ar * w.x - ai * w.y;
-            tot[2 * c + 1] = ar * w.y + ai * w.x;
-            tot[2 * c + 2] = br * w.z - bi * w.w;
-            tot[2 * c + 3] = br * w.w + bi * w.z;
-            m = fmaxf(m, fmaxf(fmaxf(fabsf(tot[2 * c]), fabsf(tot[2 * c + 1])),
-                               fmaxf(fabsf(tot[2 * c + 2]), fabsf(tot[2 * c + 3]))));
+            tmem_st8(occ + 16 * k + 8 * hs, x);
           }
+        }
+        tmem_wait_st();
+        auto exponent = [](float m) -> int {
           int ex = 0;
           if (m > 0.f) frexpf(m, &ex);
           return m > 0.f ? 14 - ex : 0;
@@ -440,13 +489,9 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
 #pragma unroll
               for (int t = 0; t < 4; ++t) {
                 const int c = 16 * j + 4 * sg + t;
-                uint16_t h0, l0, h1, l1;
-                split<FMT>(tot[2 * c] * s1 * s2, h0, l0);
-                split<FMT>(tot[2 * c + 1] * s1 * s2, h1, l1);
-                hw[t] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-                lw[t] = (uint32_t)l0 | ((uint32_t)l1 << 16);
+                split2<FMT>(tot[2 * c] * s1 * s2, tot[2 * c + 1] * s1 * s2, hw[t], lw[t]);
               }
-              const int off = base + ((sg ^ ((row >> 1) & 3)) << 4);
+              const int off = base + ((sg ^ swz) << 4);
               *reinterpret_cast<uint4*>(h_hi + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
               *reinterpret_cast<uint4*>(h_lo + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
             }
@@ -454,19 +499,18 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor cores
           __syncwarp();
         };
-        const int shu = times_w(au);
+        const int shu = exponent(mu), sho = exponent(mo);
         store_h(shu);
         if (lane == 0) mbar_arrive(&hready[h]);
-        // G_occ of this row and half from tensor memory
+        // H_occ of this row and half from tensor memory
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           uint32_t x[16];
-          tmem_ld16(tmem + lane_addr + (uint32_t)(bo * 256 + h * 128 + 16 * u), x);
+          tmem_ld16(occ + 16 * u, x);
           tmem_wait_ld();
 #pragma unroll
           for (int i = 0; i < 16; ++i) tot[16 * u + i] = __uint_as_float(x[i]);
         }
-        const int sho = times_w(ao);
         bool fine = wait_or_abort(&hfree[h], 0);     // the unoccupied MMAs have read this half
         if (__all_sync(0xffffffffu, fine)) {
           tc_fence_after();
@@ -496,24 +540,60 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
           const int e = *p.dexp, ku = shu + e, ko = sho + e;
           const float fu1 = ldexpf(1.0f, -(ku >> 1)), fu2 = ldexpf(1.0f, -(ku - (ku >> 1)));
           const float fo1 = ldexpf(1.0f, -(ko >> 1)), fo2 = ldexpf(1.0f, -(ko - (ko >> 1)));
+          // Re(conj(psi_n) V_n) of the row for NB >= n_n bands, then the sums over the warp's rows: at
+          // each of the five exchange steps a lane keeps half of its sums and hands over the other
+          // half, so that 62 shuffles leave lane l with sums l-th of 2 NB (the pairs added are those
+          // of a butterfly over each sum)
+          const int my_band = lane < p.n_n ? __ldg(p.bands + lane) : 0;
+          auto bands = [&](auto nb_c) {
+            constexpr int NB = decltype(nb_c)::value;
 #pragma unroll
-          for (int n = 0; n < 32; ++n) {
-            if (n < p.n_n) {
-              float2 ps = make_float2(0.f, 0.f);
-              if (rvalid) ps = __ldg(p.psi + (long)p.bands[n] * p.ldpsi + grow);
-              float su = (ps.x * tot[2 * n] + ps.y * tot[2 * n + 1]) * fu1 * fu2;    // Re(conj(psi_n) V_n)
-              float so = (ps.x * tot[64 + 2 * n] + ps.y * tot[64 + 2 * n + 1]) * fo1 * fo2;
+            for (int b0 = 0; b0 < NB; b0 += 8) {
+              float2 ps[8];
 #pragma unroll
-              for (int o = 16; o > 0; o >>= 1) {
-                su += __shfl_xor_sync(0xffffffffu, su, o);
-                so += __shfl_xor_sync(0xffffffffu, so, o);
+              for (int i = 0; i < 8 && b0 + i < NB; ++i) {
+                const int n = b0 + i;
+                const long at = (long)__shfl_sync(0xffffffffu, my_band, n) * p.ldpsi + grow;
+                ps[i] = rvalid && n < p.n_n ? __ldg(p.psi + at) : make_float2(0.f, 0.f);
               }
-              if (lane == 0) {
-                atomicAdd(&red[n], (double)su);
-                atomicAdd(&red[32 + n], (double)so);
+#pragma unroll
+              for (int i = 0; i < 8 && b0 + i < NB; ++i) {
+                const int n = b0 + i;
+                const float su = (ps[i].x * tot[2 * n] + ps[i].y * tot[2 * n + 1]) * fu1 * fu2;
+                const float so = (ps[i].x * tot[64 + 2 * n] + ps[i].y * tot[64 + 2 * n + 1]) * fo1 * fo2;
+                tot[2 * n] = su;
+                tot[2 * n + 1] = so;
               }
             }
-          }
+            int nv = 2 * NB;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+              if (nv > 1) {
+                nv >>= 1;
+                const bool up = (lane & off) != 0;
+#pragma unroll
+                for (int i = 0; i < NB; ++i)
+                  if (i < nv) {
+                    const float keep = up ? tot[i + nv] : tot[i], send = up ? tot[i] : tot[i + nv];
+                    tot[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+                  }
+              } else {
+                tot[0] += __shfl_xor_sync(0xffffffffu, tot[0], off);
+              }
+            }
+            // lane l: sums (l * 2 NB) / 32 .. of [su_0, so_0, su_1, ...]
+            float* rw = red + ew * 64;
+            if (NB == 32) {
+              rw[2 * lane] = tot[0];
+              rw[2 * lane + 1] = tot[1];
+            } else if (lane % (NB < 16 ? 16 / NB : 1) == 0) {
+              rw[lane * NB / 16] = tot[0];
+            }
+          };
+          if (p.n_n <= 4) bands(std::integral_constant<int, 4>{});
+          else if (p.n_n <= 8) bands(std::integral_constant<int, 8>{});
+          else if (p.n_n <= 16) bands(std::integral_constant<int, 16>{});
+          else bands(std::integral_constant<int, 32>{});
           __syncwarp();
           if (lane == 0) mbar_arrive(redbar);
         } else if (lane == 0 && !*abort_flag) {
@@ -523,8 +603,14 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
         if (ew == 0) {
           const bool got = wait_or_abort(redbar, 0);
           if (got && lane < p.n_n) {
-            atomicAdd(&p.acc_u[(long)lane * p.acc_stride], p.coef * red[lane]);
-            atomicAdd(&p.acc_o[(long)lane * p.acc_stride], -p.coef * red[32 + lane]);
+            double su = 0.0, so = 0.0;
+#pragma unroll
+            for (int w = 0; w < EPI_WARPS; ++w) {
+              su += (double)red[w * 64 + 2 * lane];
+              so += (double)red[w * 64 + 2 * lane + 1];
+            }
+            atomicAdd(&p.acc_u[(long)lane * p.acc_stride], p.coef * su);
+            atomicAdd(&p.acc_o[(long)lane * p.acc_stride], -p.coef * so);
           } else if (!got && lane == 0 && !*abort_flag) {
             timed_out(11);
           }
