@@ -910,8 +910,7 @@ extern "C" gw_status gw_workspace_size(const gw_grid* grid, int n_b, int n_occ, 
   if (!valid_prec(prec)) return fail(nullptr, GW_ERR_ARG, "bad precision");
   if (n_b < 2 || n_occ < 1 || n_occ >= n_b || n < 1 || n_chi < 1 || n_chi > g.nr || n_n < 1)
     return fail(nullptr, GW_ERR_SHAPE, "bad sizes");
-  const int rb = r_block > 0 ? std::min(r_block, g.nr) : std::min(g.nr, 2048);
-  if (chi0_bytes) *chi0_bytes = chi0_omega_scratch(g, n_b, n_occ, n, n_chi, prec, rb);
+  if (chi0_bytes) *chi0_bytes = chi0_omega_scratch(g, n_b, n_occ, n, n_chi, prec, r_block);
   if (screen_bytes) *screen_bytes = screen_scratch(n_chi, n, prec, nullptr, nullptr);
   if (sigma_bytes) *sigma_bytes = sigma_scratch(g, n_b, n_occ, n, n_chi, n_n, 64, prec);
   return GW_OK;

@@ -169,6 +169,7 @@ struct SigmaTables {
 // stack, tensor-core scratch).
 struct SigmaWork {
   bool fused;
+  int rb;             // rows per block
   double2* vout;
   char* wrg;
   char* gob;

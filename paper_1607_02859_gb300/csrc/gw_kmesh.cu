@@ -323,7 +323,7 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   probe.take<char>((size_t)n_k * rb * g.nr * es);
   probe.take<char>((size_t)rb * gs.nr * es);
   if (two_pass) probe.take<char>((size_t)rb * gs.nr * es);
-  if (tc) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false));
+  if (tc) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, n_k, n_k == 1));
   if ((st = reserve(ctx, probe.off))) return st;
   Carver cv(ctx->arena);
   int* dmap = cv.take<int>(n_chi);
@@ -339,7 +339,7 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   char* guk = cv.take<char>((size_t)n_k * rb * g.nr * es);
   char* rows_s = cv.take<char>((size_t)rb * gs.nr * es);
   char* tmp_s = two_pass ? cv.take<char>((size_t)rb * gs.nr * es) : nullptr;
-  void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false)) : nullptr;
+  void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, n_k, n_k == 1)) : nullptr;
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
   if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if ((st = upload(ctx, dsmap, smap.data(), sizeof(int) * n_k * n_chi, s))) return st;
@@ -363,17 +363,28 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
       scales[k] = green_scales(eps_k_h + (size_t)k * n_b, n_b, n_occ, mu, tau_h[j]);
       if (!tc && (st = upload_scales(ctx, dscale + (size_t)k * n_b * 8, scales[k], prec, s))) return st;
     }
+    if (tc) {
+      std::vector<float> f;
+      for (int k = 0; k < n_k; ++k) f.insert(f.end(), scales[k].s.begin(), scales[k].s.end());
+      if ((st = upload(ctx, dscale, f.data(), sizeof(float) * f.size(), s))) return st;
+    }
     char* slab_j = slabs + (size_t)j * slab * es;
     for (int r0 = 0; r0 < g.nr; r0 += rb) {
       const int rows = std::min(rb, g.nr - r0);
-      for (int k = 0; k < n_k; ++k) {
+      if (tc) {                    // every k in one launch; their psi-only operands are prepared once
+        TcEntries en;
+        en.n = n_k;
+        en.psi_stride = n_k > 1 ? (long)n_b * g.nr : 0;
+        en.out_stride = kstr;
+        if ((st = tc_green_rows(ctx, g, n_b, n_occ, psi_k, scales.data(), r0, rows, prec, gok, guk, tcs,
+                                j == 0 && r0 == 0, s, reinterpret_cast<const float*>(dscale), en)))
+          return st;
+      }
+      for (int k = 0; k < n_k && !tc; ++k) {
         const char* pk = static_cast<const char*>(psi_k) + (size_t)k * n_b * g.nr * es;
-        char* ok = gok + (size_t)k * kstr * es;
-        char* uk = guk + (size_t)k * kstr * es;
-        if (tc) st = tc_green_rows(ctx, g, n_b, n_occ, pk, scales[k], r0, rows, prec, ok, uk, tcs, true, s);
-        else st = green_rows(ctx, g, n_b, n_occ, pk, dscale + (size_t)k * n_b * 8, scales[k], r0, rows, prec, ok,
-                             uk, s);
-        if (st) return st;
+        if ((st = green_rows(ctx, g, n_b, n_occ, pk, dscale + (size_t)k * n_b * 8, scales[k], r0, rows, prec,
+                             gok + (size_t)k * kstr * es, guk + (size_t)k * kstr * es, s)))
+          return st;
       }
       if ((st = launch_stripe<true>(ctx, prec, g, nk, gok, guk, kstr, dph, rows, rows_s, nullptr, gs.nr, s)))
         return st;
@@ -533,7 +544,7 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
       const GreenScales sc = green_scales(eps_k_h + (size_t)k * n_b, n_b, n_occ, mu, tau_h[j]);
       const char* dck = dc + (size_t)k * n_b * n_pw * es;
       if (tc) {
-        st = tc_green_rows(ctx, gp, n_b, n_occ, dck, sc, 0, n_pw, prec, mo, mu_, tcs, true, s);
+        st = tc_green_rows(ctx, gp, n_b, n_occ, dck, &sc, 0, n_pw, prec, mo, mu_, tcs, true, s);
       } else {
         if ((st = upload_scales(ctx, dscale + (size_t)k * n_b * 8, sc, prec, s))) return st;
         st = green_rows(ctx, gp, n_b, n_occ, dck, dscale + (size_t)k * n_b * 8, sc, 0, n_pw, prec, mo, mu_, s);
@@ -627,7 +638,7 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   probe.take<char>((size_t)n_k * rb * g.nr * es);
   probe.take<char>(3 * (size_t)rb * gs.nr * es);
   probe.take<char>((size_t)n_n * (gs.nr + g.nr) * es);
-  if (tc) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false));
+  if (tc) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, n_k, n_k == 1));
   if ((st = reserve(ctx, probe.off))) return st;
   Carver cv(ctx->arena);
   int* dmap = cv.take<int>(n_chi);
@@ -651,7 +662,7 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   char* w_s = gu_s + (size_t)rb * gs.nr * es;
   char* ext = cv.take<char>((size_t)n_n * (gs.nr + g.nr) * es);
   char* prow = ext + (size_t)n_n * gs.nr * es;
-  void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false)) : nullptr;
+  void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, n_k, n_k == 1)) : nullptr;
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
   if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if ((st = upload(ctx, dsmap, smap.data(), sizeof(int) * n_k * n_chi, s))) return st;
@@ -688,6 +699,11 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
       scales[k] = green_scales(eps_k_h + (size_t)k * n_b, n_b, n_occ, mu, tau_h[j]);
       if (!tc && (st = upload_scales(ctx, dscale + (size_t)k * n_b * 8, scales[k], prec, s))) return st;
     }
+    if (tc) {
+      std::vector<float> f;
+      for (int k = 0; k < n_k; ++k) f.insert(f.end(), scales[k].s.begin(), scales[k].s.end());
+      if ((st = upload(ctx, dscale, f.data(), sizeof(float) * f.size(), s))) return st;
+    }
     for (int q = 0; q < n_k; ++q) {
       const char* wq = static_cast<const char*>(w_tau) + ((size_t)q * n + j) * n_chi * n_chi * es;
       char* blk = wrg + (size_t)q * n_chi * es;
@@ -697,14 +713,20 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
     if ((st = launch_q_phase(ctx, prec, g, nk, dqph, wrg, ld, n_chi, +1.0, s))) return st;
     for (int r0 = 0; r0 < g.nr; r0 += rb) {
       const int rows = std::min(rb, g.nr - r0);
-      for (int k = 0; k < n_k; ++k) {
+      if (tc) {                    // every k in one launch; their psi-only operands are prepared once
+        TcEntries en;
+        en.n = n_k;
+        en.psi_stride = n_k > 1 ? (long)n_b * g.nr : 0;
+        en.out_stride = kstr;
+        if ((st = tc_green_rows(ctx, g, n_b, n_occ, psi_k, scales.data(), r0, rows, prec, gok, guk, tcs,
+                                j == 0 && r0 == 0, s, reinterpret_cast<const float*>(dscale), en)))
+          return st;
+      }
+      for (int k = 0; k < n_k && !tc; ++k) {
         const char* pk = static_cast<const char*>(psi_k) + (size_t)k * n_b * g.nr * es;
-        char* ok = gok + (size_t)k * kstr * es;
-        char* uk = guk + (size_t)k * kstr * es;
-        if (tc) st = tc_green_rows(ctx, g, n_b, n_occ, pk, scales[k], r0, rows, prec, ok, uk, tcs, true, s);
-        else st = green_rows(ctx, g, n_b, n_occ, pk, dscale + (size_t)k * n_b * 8, scales[k], r0, rows, prec, ok,
-                             uk, s);
-        if (st) return st;
+        if ((st = green_rows(ctx, g, n_b, n_occ, pk, dscale + (size_t)k * n_b * 8, scales[k], r0, rows, prec,
+                             gok + (size_t)k * kstr * es, guk + (size_t)k * kstr * es, s)))
+          return st;
       }
       if ((st = launch_stripe<false>(ctx, prec, g, nk, gok, guk, kstr, dph, rows, go_s, gu_s, gs.nr, s))) return st;
       if ((st = launch_row_fft(ctx, gs, prec, 2, wrg + (size_t)r0 * ld * es, nullptr, ld, w_s, gs.nr, dsmap,

@@ -17,18 +17,44 @@
 
 namespace gw {
 
-size_t chi0_omega_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_chi, gw_prec prec, int rb) {
+// Rows per r-block and times per launch of the chi pass.  The tensor-core G
+// formation walks its tiles with one CTA per SM: where a block's triangle has fewer
+// than six rounds of tiles (grids up to 16^3 by default) several times go in one
+// launch, within 512 MB of chi rows.  At 12^3 a time has 105 tiles for 152 SMs.
+struct ChiShape {
+  int rb, nt;
+};
+static ChiShape chi_shape(const GridInfo& g, int n, gw_prec prec, int r_block) {
+  const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
+  ChiShape c;
+  c.rb = r_block > 0 ? std::min(r_block, g.nr) : std::min(g.nr, tc ? 4096 : 2048);
+  c.nt = 1;
+  if (tc) {
+    const double t = (g.nr + 127) / 128, blocks = (g.nr + c.rb - 1) / c.rb;
+    const double tiles = 0.5 * t * (t + 1) / blocks;
+    const double most = (512.0 * 1048576.0) / ((double)c.rb * g.nr * csize(prec));
+    c.nt = std::max(1, std::min({n, (int)std::ceil(6 * 152 / tiles), (int)most}));
+  }
+  return c;
+}
+// elements of the chi rows of a launch: nt blocks (tensor cores), or G_occ and G_unocc
+static size_t chi_rows_elems(const GridInfo& g, gw_prec prec, const ChiShape& c) {
+  const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
+  return (size_t)(tc ? c.nt : 2) * c.rb * g.nr;
+}
+
+size_t chi0_omega_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_chi, gw_prec prec, int r_block) {
   const size_t es = csize(prec);
   const size_t slab = (size_t)g.nr * n_chi;
+  const ChiShape c = chi_shape(g, n, prec, r_block);
   Carver probe(nullptr);
   probe.take<int>(n_chi);
   probe.take<int>(inv_ints(g));
   probe.take<double>((size_t)n * n_b);
   probe.take<double>((size_t)n * n);
   probe.take<char>(slab * n * es);
-  probe.take<char>((size_t)rb * g.nr * es);
-  probe.take<char>((size_t)rb * g.nr * es);
-  if (prec == GW_F16X3 || prec == GW_BF16X3) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false));
+  probe.take<char>(chi_rows_elems(g, prec, c) * es);
+  if (prec == GW_F16X3 || prec == GW_BF16X3) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, c.rb, false, 0, c.nt));
   return probe.off;
 }
 
@@ -77,7 +103,7 @@ struct Chi0Dev {
   const int* inv = nullptr;      // [N_r] position -> G index or -1, and the set's lists
   int cols = 0;                  // (i2,i3) columns that the set touches
   const char* scale = nullptr;   // CUDA-core path: [n][n_b] per-band factors in 8-byte slots
-  const float* sk = nullptr;     // tensor path: [n][n_b] FP32 factors, or NULL to copy them per call
+  const float* sk = nullptr;     // tensor path: [n][n_b] FP32 factors
   const void* cw = nullptr;      // transform weights, dV^2/Omega folded in (FP32 hi/lo or FP64)
   int* status = nullptr;         // tensor path: time-out status words owned by the caller, or NULL (in the scratch)
 };
@@ -112,44 +138,52 @@ static void chi0_tables(const GridInfo& g, int n_b, int n_occ, const double* eps
   }
 }
 
-// The kernels of the chain, launched on s with no host-device copy when t.sk
-// (tensor path) is given; scratch carved from cv.  *tcs_out: the tensor-core
-// status region for tc_check.
+// The kernels of the chain, launched on s with no host-device copy; scratch
+// carved from cv.  *tcs_out: the tensor-core status region for tc_check.
 static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, int n,
-                             const std::vector<GreenScales>& scales, int n_chi, gw_prec prec, int rb,
+                             const std::vector<GreenScales>& scales, int n_chi, gw_prec prec, const ChiShape& sh,
                              const Chi0Dev& t, Carver& cv, void* chi_w,
                              cudaStream_t s, void** tcs_out) {
   gw_status st;
   const size_t es = csize(prec);
   const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
   const size_t slab = (size_t)g.nr * n_chi;
+  const int rb = sh.rb;
   char* slabs = cv.take<char>(slab * n * es);
-  char* ga = cv.take<char>((size_t)rb * g.nr * es);
-  char* gb = cv.take<char>((size_t)rb * g.nr * es);
-  void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false)) : nullptr;
+  char* ga = cv.take<char>(chi_rows_elems(g, prec, sh) * es);
+  char* gb = ga + (size_t)rb * g.nr * es;
+  void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, sh.nt)) : nullptr;
   if (tcs_out) *tcs_out = tcs;
   bool first = true;
-  for (int j = 0; j < n; ++j) {
-    const GreenScales& gs = scales[j];
-    const char* sj = t.scale + (size_t)j * n_b * 8;
-    char* slab_j = slabs + (size_t)j * slab * es;
+  for (int j0 = 0; j0 < n; j0 += sh.nt) {
+    const int nt = std::min(sh.nt, n - j0);
     for (int r0 = 0; r0 < g.nr; r0 += rb) {
       const int rows = std::min(rb, g.nr - r0);
       if (tc) {
-        if ((st = tc_chi_rows(ctx, g, n_b, n_occ, psi, gs, r0, rows, prec, ga, tcs, first, s,
-                              t.sk ? t.sk + (size_t)j * n_b : nullptr, t.status, true)))
+        TcEntries en;
+        en.n = nt;
+        en.out_stride = (long)rb * g.nr;
+        if ((st = tc_chi_rows(ctx, g, n_b, n_occ, psi, &scales[j0], r0, rows, prec, ga, tcs, first, s,
+                              t.sk + (size_t)j0 * n_b, t.status, true, en)))
           return st;
         first = false;
-        st = launch_row_fft(ctx, g, prec, 1, ga, nullptr, g.nr, slab_j + (size_t)r0 * n_chi * es, n_chi, t.map, n_chi,
-                            rows, 1.0, s, t.inv, gb, r0);
+        for (int z = 0; z < nt; ++z) {
+          char* x = ga + (size_t)z * rb * g.nr * es;
+          if ((st = launch_row_fft(ctx, g, prec, 1, x, nullptr, g.nr, slabs + ((size_t)(j0 + z) * slab + (size_t)r0 * n_chi) * es,
+                                   n_chi, t.map, n_chi, rows, 1.0, s, t.inv, x, r0)))
+            return st;
+        }
       } else {
-        if ((st = green_rows(ctx, g, n_b, n_occ, psi, sj, gs, r0, rows, prec, ga, gb, s, r0))) return st;
-        st = launch_row_fft(ctx, g, prec, 0, ga, gb, g.nr, slab_j + (size_t)r0 * n_chi * es, n_chi, t.map, n_chi,
-                            rows, -2.0, s, t.inv, ga, r0);
+        const char* sj = t.scale + (size_t)j0 * n_b * 8;
+        if ((st = green_rows(ctx, g, n_b, n_occ, psi, sj, scales[j0], r0, rows, prec, ga, gb, s, r0))) return st;
+        if ((st = launch_row_fft(ctx, g, prec, 0, ga, gb, g.nr, slabs + ((size_t)j0 * slab + (size_t)r0 * n_chi) * es,
+                                 n_chi, t.map, n_chi, rows, -2.0, s, t.inv, ga, r0)))
+          return st;
       }
-      if (st) return st;
     }
-    if ((st = launch_col_plane(ctx, g, prec, -1, slab_j, n_chi, n_chi, 1.0, t.inv, t.cols, s))) return st;
+    for (int z = 0; z < nt; ++z)
+      if ((st = launch_col_plane(ctx, g, prec, -1, slabs + (size_t)(j0 + z) * slab * es, n_chi, n_chi, 1.0, t.inv, t.cols, s)))
+        return st;
   }
   if ((st = launch_col_line_ct(ctx, g, prec, slabs, (long)slab, n_chi, n, t.cw, chi_w, (long)n_chi * n_chi, n_chi,
                                t.inv, t.cols, n_chi, s)))
@@ -173,9 +207,9 @@ extern "C" gw_status gw_chi0_omega(gw_ctx* ctx, const gw_grid* grid, int n_b, in
   std::vector<int> map, inv;
   if ((st = index_maps(ctx, g, fft_index_h, n_chi, map, inv))) return st;
   cudaStream_t s = as_stream(stream);
-  const int rb = r_block > 0 ? std::min(r_block, g.nr) : std::min(g.nr, 2048);
+  const ChiShape sh = chi_shape(g, n, prec, r_block);
   const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
-  if ((st = reserve(ctx, chi0_omega_scratch(g, n_b, n_occ, n, n_chi, prec, rb)))) return st;
+  if ((st = reserve(ctx, chi0_omega_scratch(g, n_b, n_occ, n, n_chi, prec, r_block)))) return st;
   std::vector<GreenScales> scales;
   std::vector<double> cw64;
   std::vector<float> cw32;
@@ -190,17 +224,24 @@ extern "C" gw_status gw_chi0_omega(gw_ctx* ctx, const gw_grid* grid, int n_b, in
   if (is_fp64(prec)) st = upload(ctx, dcw, cw64.data(), sizeof(double) * n * n, s);
   else st = upload(ctx, dcw, cw32.data(), sizeof(float) * 2 * n * n, s);
   if (st) return st;
-  if (!tc)
+  if (tc) {                       // the factors of all times in one copy
+    std::vector<float> f;
+    f.reserve((size_t)n * n_b);
+    for (int j = 0; j < n; ++j) f.insert(f.end(), scales[j].s.begin(), scales[j].s.end());
+    if ((st = upload(ctx, dscale, f.data(), sizeof(float) * f.size(), s))) return st;
+  } else {
     for (int j = 0; j < n; ++j)
       if ((st = upload_scales(ctx, dscale + (size_t)j * n_b * 8, scales[j], prec, s))) return st;
+  }
   Chi0Dev t;
   t.map = dmap;
   t.inv = dinv;
   t.cols = set_columns(g, inv);
   t.scale = dscale;
+  t.sk = reinterpret_cast<const float*>(dscale);
   t.cw = dcw;
   void* tcs = nullptr;
-  if ((st = chi0_launch(ctx, g, n_b, n_occ, psi, n, scales, n_chi, prec, rb, t, cv, chi_w, s, &tcs))) return st;
+  if ((st = chi0_launch(ctx, g, n_b, n_occ, psi, n, scales, n_chi, prec, sh, t, cv, chi_w, s, &tcs))) return st;
   return tc ? tc_check(ctx, tcs, s) : GW_OK;
 }
 
@@ -399,7 +440,7 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   for (int j = 0; j < n; ++j) {
     // Mc_occ, Mc_unocc over the plane-wave set, then their column transforms T(r, g')
     if (tc) {
-      st = tc_green_rows(ctx, gp, n_b, n_occ, dc, scales[j], 0, n_pw, prec, mo, mu_, tcs, first, s);
+      st = tc_green_rows(ctx, gp, n_b, n_occ, dc, &scales[j], 0, n_pw, prec, mo, mu_, tcs, first, s);
       first = false;
     } else {
       st = green_rows(ctx, gp, n_b, n_occ, dc, dscale + (size_t)j * n_b * 8, scales[j], 0, n_pw, prec, mo, mu_, s);
@@ -430,7 +471,8 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
 struct gw_chi0_plan {
   gw_ctx* ctx = nullptr;
   GridInfo g{};
-  int n_b = 0, n_occ = 0, n = 0, n_chi = 0, rb = 0;
+  int n_b = 0, n_occ = 0, n = 0, n_chi = 0;
+  ChiShape sh{};
   gw_prec prec = GW_FP32;
   std::vector<GreenScales> scales;
   std::vector<float> cw32;
@@ -458,7 +500,7 @@ extern "C" gw_status gw_chi0_plan_create(gw_ctx* ctx, const gw_grid* grid, int n
   p->n = n;
   p->n_chi = n_chi;
   p->prec = prec;
-  p->rb = r_block > 0 ? std::min(r_block, g.nr) : std::min(g.nr, 2048);
+  p->sh = chi_shape(g, n, prec, r_block);
   std::vector<double> cw64;
   chi0_tables(g, n_b, n_occ, eps_h, mu, n, tau_h, C_h, prec, p->scales, cw64, p->cw32);
   // table layout
@@ -512,7 +554,7 @@ extern "C" gw_status gw_chi0_plan_create(gw_ctx* ctx, const gw_grid* grid, int n
   p->t.sk = reinterpret_cast<const float*>(d + o_sk);
   p->t.cw = d + o_cw;
   p->t.status = reinterpret_cast<int*>(d + o_status);
-  p->work = chi0_omega_scratch(g, n_b, n_occ, n, n_chi, prec, p->rb);
+  p->work = chi0_omega_scratch(g, n_b, n_occ, n, n_chi, prec, r_block);
   if ((st = reserve(ctx, p->work))) {
     cudaFree(p->dev);
     delete p;
@@ -528,7 +570,7 @@ extern "C" gw_status gw_chi0_plan_launch(gw_chi0_plan* p, const void* psi, void*
   if (!psi || !chi_w) return fail(ctx, GW_ERR_ARG, "NULL pointer");
   if (ctx->arena_bytes < p->work) return fail(ctx, GW_ERR_ARG, "the context arena is smaller than the plan's");
   Carver cv(ctx->arena);
-  return chi0_launch(ctx, p->g, p->n_b, p->n_occ, psi, p->n, p->scales, p->n_chi, p->prec, p->rb, p->t, cv,
+  return chi0_launch(ctx, p->g, p->n_b, p->n_occ, psi, p->n, p->scales, p->n_chi, p->prec, p->sh, p->t, cv,
                      chi_w, as_stream(stream), nullptr);
 }
 

@@ -563,8 +563,11 @@ void sigma_carve_work(Carver& cv, const GridInfo& g, int n_b, int n_occ, int n_c
   w.gob = cv.take<char>((size_t)rb * g.nr * es);
   w.gub = cv.take<char>((size_t)rb * g.nr * es);
   w.wrr = cv.take<char>((size_t)rb * g.nr * es);
+  // the fused contraction forms no G rows: W~ rows take all three blocks
+  w.rb = w.fused ? std::min(g.nr, 3 * rb) : rb;
+  if (w.fused) w.wrr = w.gob;
   w.tcs = (prec == GW_F16X3 || prec == GW_BF16X3)
-              ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, w.fused ? n_n : 0))
+              ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, w.rb, false, w.fused ? n_n : 0))
               : nullptr;
 }
 
@@ -610,7 +613,7 @@ gw_status sigma_kernels(gw_ctx* ctx, const GridInfo& g, gw_prec prec, bool full,
                         const SigmaTables& t, const SigmaWork& w, const void* w_tau, cudaStream_t s) {
   gw_status st;
   const size_t es = csize(prec);
-  const int rb = std::min(g.nr, 2048);
+  const int rb = w.rb;
   const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
   const size_t nnm = full ? (size_t)n_n * n_n : (size_t)n_n;
   const size_t acc_elems = (full ? 2 : 1) * nnm * n;
@@ -650,7 +653,7 @@ gw_status sigma_kernels(gw_ctx* ctx, const GridInfo& g, gw_prec prec, bool full,
         continue;
       }
       if (tc) {
-        st = tc_green_rows(ctx, g, n_b, n_occ, psi, scales[j], r0, rows, prec, w.gob, w.gub, w.tcs, first, s,
+        st = tc_green_rows(ctx, g, n_b, n_occ, psi, &scales[j], r0, rows, prec, w.gob, w.gub, w.tcs, first, s,
                            reinterpret_cast<const float*>(sj));
         first = false;
       }
@@ -905,7 +908,7 @@ extern "C" gw_status gw_sigma_diag_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   for (int j = 0; j < n; ++j) {
     const char* sj = t.scale + (size_t)j * n_b * 8;
     if (tc) {
-      st = tc_green_rows(ctx, gp, n_b, n_occ, dc, scales[j], 0, n_pw, prec, mo, mu_, tcs, first, s,
+      st = tc_green_rows(ctx, gp, n_b, n_occ, dc, &scales[j], 0, n_pw, prec, mo, mu_, tcs, first, s,
                          reinterpret_cast<const float*>(sj));
       first = false;
     } else {

@@ -58,6 +58,8 @@ constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 256;
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
 
+constexpr int kMaxEntries = 64;
+
 struct Params {
   int m_rows;             // valid output rows
   int n_cols;             // valid complex output columns (N_r)
@@ -67,9 +69,14 @@ struct Params {
   float2* out0;           // chi, or G_occ
   float2* out1;           // G_unocc (green mode)
   long ldo;
-  float alpha_occ;        // A_occ (FP64 max exponential, rounded) times 2^{-2e}
-  float alpha_un;
-  const int* dexp;        // device: e of the 2^e operand scaling
+  // independent products (k points, or times of one set of orbitals): entry z has its own A operand,
+  // factors and output, and its own B operand and scaling unless shared
+  int nb, b_shared;
+  long so;                // elements between the entries' outputs
+  float alpha_occ[kMaxEntries];   // A_occ (FP64 max exponential, rounded)
+  float alpha_un[kMaxEntries];
+  const int* dexp;        // device [nb] (or one, shared): e of the 2^e operand scaling
+  int gx, gy, tiles;      // column and row tiles, tiles in use per entry
   int* status;            // device: [0] time-out flag, [1] where
   // MODE 2 (self-energy): contraction of G o W~ with psi_n on the tensor cores
   const float2* wrr;      // W~(r, R') rows of the block, [m_rows][ldw]
@@ -145,27 +152,44 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
   uint64_t* psi_full = vready + 2;       // psi_n operand of the tile landed
   uint64_t* redbar = psi_full + 1;       // the epilogue warps' band sums are in shared memory
   uint64_t* done2 = redbar + 1;          // every MMA of the self-energy phase done
+  uint64_t* last_mma = done2 + 1;
   float* red = reinterpret_cast<float*>(epi);     // [8 warps][32][2] band sums of the warps (MODE 2 only)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // tiles in groups of kGroupRows row tiles: the CTAs that run together walk a group's rows for
-  // each column tile, so they share B (and A) tiles in L2 instead of each reading its B from DRAM
-  int m0, n0;
-  {
+  // Tile t: its entry, row tile and column tile.  Only tiles with some R' <= r are counted in
+  // lower-triangle mode.  They go in groups of eight row tiles, column by column: the CTAs that run
+  // together share B (and A) tiles in L2 instead of each reading its B from DRAM.
+  struct Tile {
+    int z, m0, n0;
+  };
+  auto cols_of = [&](int i) { return p.lower ? min(p.gx, (p.r0 + i * BM + BM - 1) / BNC + 1) : p.gx; };
+  auto tile_at = [&](int t) -> Tile {
     constexpr int kGroupRows = 8;
-    const int gx = gridDim.x, gy = gridDim.y;
-    const int id = blockIdx.y * gx + blockIdx.x;
-    const int per = kGroupRows * gx, grp = id / per, first = grp * kGroupRows;
-    const int rows = min(kGroupRows, gy - first), r = id - grp * per;
-    m0 = (first + r % rows) * BM;
-    n0 = (r / rows) * BNC;
-  }
-  const long grow0 = (long)p.r0 + m0;                 // grid row of the tile's first row
-  if (MODE != 1 && p.lower && n0 >= grow0 + BM) {
-    // every R' of the tile is above every r: nothing to do (the row transform takes them as zero)
-    return;
-  }
-  const bool diag_tile = MODE != 1 && p.lower && n0 + BNC > grow0;   // the tile meets the diagonal
+    Tile o;
+    o.z = t / p.tiles;
+    int r = t - o.z * p.tiles, first = 0, rows;
+    for (;; first += kGroupRows) {
+      rows = min(kGroupRows, p.gy - first);
+      int count = 0;
+      for (int i = 0; i < rows; ++i) count += cols_of(first + i);
+      if (r < count) break;
+      r -= count;
+    }
+    const int all = cols_of(first);                     // columns that every row of the group has
+    int i, c;
+    if (r < rows * all) {
+      i = r % rows;
+      c = r / rows;
+    } else {
+      r -= rows * all;
+      for (i = 0; r >= cols_of(first + i) - all; ++i) r -= cols_of(first + i) - all;
+      c = all + r;
+    }
+    o.m0 = (first + i) * BM;
+    o.n0 = c * BNC;
+    return o;
+  };
+  const int n_tiles = p.tiles * p.nb;
   const int total = p.k_occ_steps + p.k_un_steps;
   const int n_un_blocks = (p.k_un_steps + CH - 1) / CH;
   const bool have_occ = p.k_occ_steps > 0;
@@ -180,6 +204,7 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
       mbar_init(&tempty[b], EPI_WARPS);
     }
     mbar_init(done, 1);
+    mbar_init(last_mma, 1);
     if (MODE == 2) {
       for (int b = 0; b < 2; ++b) {
         mbar_init(&hready[b], 4);
@@ -226,409 +251,446 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
 
   if (warp == 0 && lane == 0) {
     // ---------------------------------------------------------- TMA producer (unoccupied K first)
-    int issued = 0;
-    for (int it = 0; it < total && !*abort_flag; ++it) {
-      const int s = it % STAGES;
-      if (it >= STAGES && !mbar_wait(&empty[s], ((it / STAGES) & 1) ^ 1)) {
-        timed_out(1);
+    int kit = 0, ti = 0;                               // stages issued, tiles of this CTA
+    for (int t = blockIdx.x; t < n_tiles && !*abort_flag; t += gridDim.x, ++ti) {
+      const Tile tl = tile_at(t);
+      const int zb = p.b_shared ? 0 : tl.z;
+      // MODE 2: the stages of the last tile held H and psi_n until its last MMA
+      if (MODE == 2 && ti > 0 && !wait_or_abort(done2, (uint32_t)((ti - 1) & 1))) {
+        if (!*abort_flag) timed_out(12);
         break;
       }
-      uint8_t* st = smem + s * STAGE_BYTES;
-      const int x = it < p.k_un_steps ? p.k_un_x + it * BK : (it - p.k_un_steps) * BK;
-      mbar_expect_tx(&full[s], STAGE_BYTES);
-      tma_load_3d(st, &mA_hi, &full[s], x, m0, 0);
-      tma_load_3d(st + A_BYTES, &mA_lo, &full[s], x, m0, 0);
-      tma_load_3d(st + 2 * A_BYTES, &mB_hi, &full[s], x, 2 * n0, 0);
-      tma_load_3d(st + 2 * A_BYTES + B_BYTES, &mB_lo, &full[s], x, 2 * n0, 0);
-      issued = it + 1;
-    }
-    if (*abort_flag) {
-      // let our own copies land before the CTA exits
-      for (int it = issued - STAGES < 0 ? 0 : issued - STAGES; it < issued; ++it)
-        mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
-    } else if constexpr (MODE == 2) {
-      // the tile's psi_n operand, once every MMA of the G formation has read its stages
-      if (wait_or_abort(done, 0)) {
-        mbar_expect_tx(psi_full, (uint32_t)(16 * p_chunk));
-        for (int cc = 0; cc < 8; ++cc) {
-          tma_load_3d(p_hi + cc * p_chunk, &mP_hi, psi_full, 2 * n0 + cc * BK, 0, 0);
-          tma_load_3d(p_lo + cc * p_chunk, &mP_lo, psi_full, 2 * n0 + cc * BK, 0, 0);
+      for (int it = 0; it < total; ++it, ++kit) {
+        const int s = kit % STAGES;
+        if (kit >= STAGES && !wait_or_abort(&empty[s], (uint32_t)(((kit / STAGES) & 1) ^ 1))) {
+          if (!*abort_flag) timed_out(1);
+          break;
         }
-        mbar_wait(psi_full, 0);    // our copies land before the CTA can exit
-      } else if (!*abort_flag) {
-        timed_out(6);
+        uint8_t* st = smem + s * STAGE_BYTES;
+        const int x = it < p.k_un_steps ? p.k_un_x + it * BK : (it - p.k_un_steps) * BK;
+        mbar_expect_tx(&full[s], STAGE_BYTES);
+        tma_load_3d(st, &mA_hi, &full[s], x, tl.m0, tl.z);
+        tma_load_3d(st + A_BYTES, &mA_lo, &full[s], x, tl.m0, tl.z);
+        tma_load_3d(st + 2 * A_BYTES, &mB_hi, &full[s], x, 2 * tl.n0, zb);
+        tma_load_3d(st + 2 * A_BYTES + B_BYTES, &mB_lo, &full[s], x, 2 * tl.n0, zb);
+      }
+      if (*abort_flag) break;
+      if constexpr (MODE == 2) {
+        // the tile's psi_n operand, once every MMA of the G formation has read its stages
+        if (wait_or_abort(done, (uint32_t)(ti & 1))) {
+          mbar_expect_tx(psi_full, (uint32_t)(16 * p_chunk));
+          for (int cc = 0; cc < 8; ++cc) {
+            tma_load_3d(p_hi + cc * p_chunk, &mP_hi, psi_full, 2 * tl.n0 + cc * BK, 0, 0);
+            tma_load_3d(p_lo + cc * p_chunk, &mP_lo, psi_full, 2 * tl.n0 + cc * BK, 0, 0);
+          }
+          mbar_wait(psi_full, (uint32_t)(ti & 1));    // our copies land before the CTA can exit
+        } else if (!*abort_flag) {
+          timed_out(6);
+        }
       }
     }
+    if (*abort_flag)
+      // let our own copies land before the CTA exits
+      for (int it = kit - STAGES < 0 ? 0 : kit - STAGES; it < kit; ++it)
+        mbar_wait(&full[it % STAGES], (uint32_t)((it / STAGES) & 1));
   } else if (warp == 1 && lane == 0) {
     // ---------------------------------------------------------- MMA issuer
     constexpr uint32_t idesc = make_idesc(FMT, 2 * BNC, BM);
     const int n_blocks = n_un_blocks + (have_occ ? 1 : 0);
-    int it = 0;
+    int kit = 0, bc = 0, ti = 0;                       // stages used, accumulation blocks, tiles
     bool ok = true;
-    for (int c = 0; c < n_blocks && ok; ++c) {
-      const int b = c & 1, use = c >> 1;
-      const int first = c < n_un_blocks ? c * CH : p.k_un_steps;
-      const int last = c < n_un_blocks ? min(p.k_un_steps, (c + 1) * CH) : total;
-      if (use > 0 && !wait_or_abort(&tempty[b], (use - 1) & 1)) {
-        if (!*abort_flag) timed_out(4);
+    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++ti) {
+      // MODE 2: the last tile's V sums have been read from tensor memory
+      if (MODE == 2 && ti > 0 && !wait_or_abort(redbar, (uint32_t)((ti - 1) & 1))) {
+        if (!*abort_flag) timed_out(13);
         ok = false;
         break;
       }
-      tc_fence_after();
-      const uint32_t d = tmem + (uint32_t)(b * 256);
-      for (; it < last; ++it) {
-        const int s = it % STAGES;
-        if (!wait_or_abort(&full[s], (it / STAGES) & 1)) {
-          if (!*abort_flag) timed_out(2);
+      int it = 0;
+      for (int c = 0; c < n_blocks && ok; ++c, ++bc) {
+        const int b = bc & 1, use = bc >> 1;
+        const int first = c < n_un_blocks ? c * CH : p.k_un_steps;
+        const int last = c < n_un_blocks ? min(p.k_un_steps, (c + 1) * CH) : total;
+        if (use > 0 && !wait_or_abort(&tempty[b], (uint32_t)((use - 1) & 1))) {
+          if (!*abort_flag) timed_out(4);
           ok = false;
           break;
         }
         tc_fence_after();
-        uint8_t* st = smem + s * STAGE_BYTES;
-        const uint64_t ah = sw64_desc(st), al = sw64_desc(st + A_BYTES);
-        const uint64_t bh = sw64_desc(st + 2 * A_BYTES), bl = sw64_desc(st + 2 * A_BYTES + B_BYTES);
-#pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk) {
-          const uint64_t off = (uint64_t)(kk * 32) >> 4;    // 16 elements = 32 bytes along K
-          umma(d, ah + off, bh + off, idesc, (it > first || kk > 0) ? 1u : 0u);
-          umma(d, ah + off, bl + off, idesc, 1u);
-          umma(d, al + off, bh + off, idesc, 1u);
-        }
-        umma_commit(&empty[s]);
-      }
-      if (ok) umma_commit(&tfull[b]);
-    }
-    umma_commit(done);     // arrives once every MMA issued above has completed
-    if (!mbar_wait(done, 0)) timed_out(5);
-    if constexpr (MODE == 2) {
-      // V accumulators [occ][half] of np columns each in the tensor-memory half the
-      // last G_unocc block used (drained before the epilogue signals hready)
-      const uint32_t vbase = tmem + (uint32_t)((1 - (n_un_blocks & 1)) * 256);
-      const uint32_t idesc2 = make_idesc(FMT, p.np, BM);
-      bool go = ok && wait_or_abort(psi_full, 0);
-      if (!go && !*abort_flag) timed_out(7);
-      for (int o = 0; o < 2 && go; ++o) {
-        for (int h = 0; h < 2 && go; ++h) {
-          if (!wait_or_abort(&hready[h], (uint32_t)o)) {
-            if (!*abort_flag) timed_out(8);
-            go = false;
+        const uint32_t d = tmem + (uint32_t)(b * 256);
+        for (; it < last; ++it, ++kit) {
+          const int s = kit % STAGES;
+          if (!wait_or_abort(&full[s], (uint32_t)((kit / STAGES) & 1))) {
+            if (!*abort_flag) timed_out(2);
+            ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t d = vbase + (uint32_t)((2 * o + h) * p.np);
-#pragma unroll 1
-          for (int cc = 4 * h; cc < 4 * h + 4; ++cc) {
-            const uint64_t ah = sw64_desc(h_hi + cc * A_BYTES), al = sw64_desc(h_lo + cc * A_BYTES);
-            const uint64_t bh = sw64_desc(p_hi + cc * p_chunk), bl = sw64_desc(p_lo + cc * p_chunk);
+          uint8_t* st = smem + s * STAGE_BYTES;
+          const uint64_t ah = sw64_desc(st), al = sw64_desc(st + A_BYTES);
+          const uint64_t bh = sw64_desc(st + 2 * A_BYTES), bl = sw64_desc(st + 2 * A_BYTES + B_BYTES);
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk) {
-              const uint64_t off = (uint64_t)(kk * 32) >> 4;
-              umma(d, ah + off, bh + off, idesc2, (cc > 4 * h || kk > 0) ? 1u : 0u);
-              umma(d, ah + off, bl + off, idesc2, 1u);
-              umma(d, al + off, bh + off, idesc2, 1u);
-            }
+          for (int kk = 0; kk < BK / 16; ++kk) {
+            const uint64_t off = (uint64_t)(kk * 32) >> 4;    // 16 elements = 32 bytes along K
+            umma(d, ah + off, bh + off, idesc, (it > first || kk > 0) ? 1u : 0u);
+            umma(d, ah + off, bl + off, idesc, 1u);
+            umma(d, al + off, bh + off, idesc, 1u);
           }
-          umma_commit(o == 0 ? &hfree[h] : &vready[h]);
+          umma_commit(&empty[s]);
         }
+        if (ok) umma_commit(&tfull[b]);
       }
-      umma_commit(done2);
-      if (!mbar_wait(done2, 0)) timed_out(9);
+      if constexpr (MODE == 2) {
+        umma_commit(done);     // arrives once every MMA issued above has completed
+        // V accumulators [occ][half] of np columns each in the half that G_occ does not hold (the last
+        // G_unocc block's, drained before the epilogue signals hready)
+        const uint32_t vbase = tmem + (uint32_t)((bc & 1) * 256);
+        const uint32_t idesc2 = make_idesc(FMT, p.np, BM);
+        bool go = ok && wait_or_abort(psi_full, (uint32_t)(ti & 1));
+        if (!go && !*abort_flag) timed_out(7);
+        for (int o = 0; o < 2 && go; ++o) {
+          for (int h = 0; h < 2 && go; ++h) {
+            if (!wait_or_abort(&hready[h], (uint32_t)o)) {
+              if (!*abort_flag) timed_out(8);
+              go = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t d = vbase + (uint32_t)((2 * o + h) * p.np);
+#pragma unroll 1
+            for (int cc = 4 * h; cc < 4 * h + 4; ++cc) {
+              const uint64_t ah = sw64_desc(h_hi + cc * A_BYTES), al = sw64_desc(h_lo + cc * A_BYTES);
+              const uint64_t bh = sw64_desc(p_hi + cc * p_chunk), bl = sw64_desc(p_lo + cc * p_chunk);
+#pragma unroll
+              for (int kk = 0; kk < BK / 16; ++kk) {
+                const uint64_t off = (uint64_t)(kk * 32) >> 4;
+                umma(d, ah + off, bh + off, idesc2, (cc > 4 * h || kk > 0) ? 1u : 0u);
+                umma(d, ah + off, bl + off, idesc2, 1u);
+                umma(d, al + off, bh + off, idesc2, 1u);
+              }
+            }
+            umma_commit(o == 0 ? &hfree[h] : &vready[h]);
+          }
+        }
+        ok = ok && go;
+        umma_commit(done2);
+      }
     }
+    umma_commit(last_mma);     // every MMA of this CTA has completed before tensor memory is freed
+    if (!mbar_wait(last_mma, 0)) timed_out(5);
   } else if (warp >= 2) {
     // ---------------------------------------------------------- epilogue
     const int ew = warp - 2;
     const int q = warp & 3;                       // tensor-memory lane quarter of this warp
     const int h = ew >> 2;                        // column half: real columns h*128 .. h*128+127
     const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
-    float tot[128];                               // this thread's row of G_unocc, FP32 round-to-nearest sums
-#pragma unroll
-    for (int i = 0; i < 128; ++i) tot[i] = 0.f;
+    int bc = 0, ti = 0;
     bool ok = true;
-    for (int c = 0; c < n_un_blocks; ++c) {
-      const int b = c & 1;
-      const bool got = wait_or_abort(&tfull[b], (c >> 1) & 1);
-      if (!__all_sync(0xffffffffu, got)) {
-        if (lane == 0 && !*abort_flag) timed_out(3);
-        ok = false;
-        break;
+    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++ti) {
+      const Tile tl = tile_at(t);
+      const int m0 = tl.m0, n0 = tl.n0;
+      const long grow0 = (long)p.r0 + m0;           // grid row of the tile's first row
+      const bool diag_tile = MODE != 1 && p.lower && n0 + BNC > grow0;   // the tile meets the diagonal
+      if (MODE == 2 && p.ldw % 2 == 0 && (reinterpret_cast<uintptr_t>(p.wrr) & 15) == 0) {
+        // this warp's block of W~ on its way into L2 while the K loop runs
+        const int gr = m0 + q * 32 + lane, gc = n0 + h * 64;
+        const int bytes = gr < p.m_rows ? min(64, p.n_cols - gc) * 8 & ~15 : 0;
+        if (bytes > 0) prefetch_l2(p.wrr + (long)gr * p.ldw + gc, bytes);
       }
-      tc_fence_after();
-      const uint32_t base = tmem + lane_addr + (uint32_t)(b * 256 + h * 128);
+      float tot[128];                               // this thread's row of G_unocc, FP32 round-to-nearest sums
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        uint32_t x[16];
-        tmem_ld16(base + 16 * u, x);
-        tmem_wait_ld();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) tot[16 * u + i] += __uint_as_float(x[i]);
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty[b]);
-    }
-    const int bo = n_un_blocks & 1;
-    if (ok && have_occ) {
-      const bool got = wait_or_abort(&tfull[bo], (n_un_blocks >> 1) & 1);
-      if (!__all_sync(0xffffffffu, got)) {
-        if (lane == 0 && !*abort_flag) timed_out(3);
-        ok = false;
-      }
-      tc_fence_after();
-    }
-    // tcgen05.ld is warp-collective: the whole warp takes the same branch
-    if (__all_sync(0xffffffffu, ok && !*abort_flag)) {
-      const int r0 = m0 + q * 32;                   // first output row of this warp
-      const float sc = ldexpf(1.0f, -2 * (*p.dexp));
-      const float ao = p.alpha_occ * sc, au = p.alpha_un * sc;
-      if constexpr (MODE == 2) {
-        // ---------------------------------------------- self-energy contraction of the tile
-        const int row = q * 32 + lane;               // tensor-memory lane = tile row
-        const int gm = m0 + row;
-        const bool rvalid = gm < p.m_rows;
-        const int c0 = n0 + h * 64;                   // first complex column of this warp's half
-        const long grow = grow0 + row;             // grid row r of this thread
-        const int swz = (row >> 1) & 3;
-        // The warp's 32 x 64 block of W~ goes through the shared memory that its own H will take:
-        // piece k (8 columns, 64 bytes a row) in the place of the warp's rows of K chunk 4h + k % 4,
-        // hi for k < 4 and lo above, 16-byte segments swizzled as H's.  Row r lies where row r of H
-        // will, so a thread only overwrites what it has read itself.
-        auto piece = [&](int k) -> uint8_t* {
-          return (k < 4 ? h_hi : h_lo) + (4 * h + (k & 3)) * A_BYTES + q * 2048;
-        };
-        {
-          const bool vec = (p.ldw % 2 == 0) && ((reinterpret_cast<uintptr_t>(p.wrr) & 15) == 0);
-#pragma unroll 4
-          for (int i = 0; i < 32; ++i) {              // eight rows of a piece per step, 64 bytes each
-            const int k = i >> 2, r = (i & 3) * 8 + (lane >> 2), sg = lane & 3;
-            const int gr = m0 + q * 32 + r, gn = c0 + 8 * k + 2 * sg;
-            uint8_t* dst = piece(k) + r * 64 + ((sg ^ ((r >> 1) & 3)) << 4);
-            const int have = gr < p.m_rows ? min(max(p.n_cols - gn, 0), 2) : 0;   // columns of the pair in range
-            const float2* src = have ? p.wrr + (long)gr * p.ldw + gn : p.wrr;
-            if (vec) {
-              cp_async16(dst, src, 8 * have);
-            } else {
-              cp_async8(dst, src, have > 0 ? 8 : 0);
-              cp_async8(dst + 8, have > 1 ? src + 1 : p.wrr, have > 1 ? 8 : 0);
-            }
-          }
-          cp_async_wait();
-          __syncwarp();
+      for (int i = 0; i < 128; ++i) tot[i] = 0.f;
+      for (int c = 0; c < n_un_blocks; ++c, ++bc) {
+        const int b = bc & 1;
+        const bool got = wait_or_abort(&tfull[b], (uint32_t)((bc >> 1) & 1));
+        if (!__all_sync(0xffffffffu, got)) {
+          if (lane == 0 && !*abort_flag) timed_out(3);
+          ok = false;
+          break;
         }
-        // H = w G o W~ for G_unocc in registers and for G_occ in tensor memory (in place); returns the
-        // powers of two that put the rows' maxima below 2^15
-        const uint32_t occ = tmem + lane_addr + (uint32_t)(bo * 256 + h * 128);
-        float mu = 0.f, mo = 0.f;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const uint8_t* wp = piece(k) + lane * 64;
-#pragma unroll
-          for (int hs = 0; hs < 2; ++hs) {
-            uint32_t x[8];
-            tmem_ld8(occ + 16 * k + 8 * hs, x);
-            float4 w2[2];
-#pragma unroll
-            for (int s = 0; s < 2; ++s) w2[s] = *reinterpret_cast<const float4*>(wp + (((2 * hs + s) ^ swz) << 4));
-            tmem_wait_ld();
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-              const float4 w = w2[s];
-              const int c = 8 * k + 4 * hs + 2 * s;
-              const int gn = c0 + c;
-              // weight of (r, R'): 2 below the diagonal, 1 on it, 0 above (lower-triangle mode)
-              float wa = 1.f, wb = 1.f;
-              if (p.lower) {
-                wa = gn < grow ? 2.f : (gn == grow ? 1.f : 0.f);
-                wb = gn + 1 < grow ? 2.f : (gn + 1 == grow ? 1.f : 0.f);
-              }
-              {
-                const float ar = tot[2 * c] * au * wa, ai = tot[2 * c + 1] * au * wa;
-                const float br = tot[2 * c + 2] * au * wb, bi = tot[2 * c + 3] * au * wb;
-                tot[2 * c] = ar * w.x - ai * w.y;
-                tot[2 * c + 1] = ar * w.y + ai * w.x;
-                tot[2 * c + 2] = br * w.z - bi * w.w;
-                tot[2 * c + 3] = br * w.w + bi * w.z;
-                mu = fmaxf(mu, fmaxf(fmaxf(fabsf(tot[2 * c]), fabsf(tot[2 * c + 1])),
-                                     fmaxf(fabsf(tot[2 * c + 2]), fabsf(tot[2 * c + 3]))));
-              }
-              {
-                const float g0 = __uint_as_float(x[4 * s]), g1 = __uint_as_float(x[4 * s + 1]);
-                const float g2 = __uint_as_float(x[4 * s + 2]), g3 = __uint_as_float(x[4 * s + 3]);
-                const float ar = g0 * ao * wa, ai = g1 * ao * wa;
-                const float br = g2 * ao * wb, bi = g3 * ao * wb;
-                const float y0 = ar * w.x - ai * w.y, y1 = ar * w.y + ai * w.x;
-                const float y2 = br * w.z - bi * w.w, y3 = br * w.w + bi * w.z;
-                mo = fmaxf(mo, fmaxf(fmaxf(fabsf(y0), fabsf(y1)), fmaxf(fabsf(y2), fabsf(y3))));
-                x[4 * s] = __float_as_uint(y0);
-                x[4 * s + 1] = __float_as_uint(y1);
-                x[4 * s + 2] = __float_as_uint(y2);
-                x[4 * s + 3] = __float_as_uint(y3);
-              }
-            }
-            tmem_st8(occ + 16 * k + 8 * hs, x);
-          }
-        }
-        tmem_wait_st();
-        auto exponent = [](float m) -> int {
-          int ex = 0;
-          if (m > 0.f) frexpf(m, &ex);
-          return m > 0.f ? 14 - ex : 0;
-        };
-        // this row of H, scaled by 2^sh and split in two 16-bit parts, into K chunks
-        // 4h..4h+3: row `row` of a chunk is 64 bytes at (row/8)*512 + (row%8)*64, its
-        // 16-byte segment s stored at s ^ ((row/2) % 4) (the 64-byte swizzle of TMA)
-        auto store_h = [&](int sh) {
-          // 2^sh in two factors: a row of tiny H (W~ of a large tau decays like exp(-omega tau))
-          // can need sh above 127, where one FP32 power of two would overflow
-          const float s1 = ldexpf(1.0f, sh >> 1), s2 = ldexpf(1.0f, sh - (sh >> 1));
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int base = (4 * h + j) * A_BYTES + (row >> 3) * 512 + (row & 7) * 64;
-#pragma unroll
-            for (int sg = 0; sg < 4; ++sg) {
-              uint32_t hw[4], lw[4];
-#pragma unroll
-              for (int t = 0; t < 4; ++t) {
-                const int c = 16 * j + 4 * sg + t;
-                split2<FMT>(tot[2 * c] * s1 * s2, tot[2 * c + 1] * s1 * s2, hw[t], lw[t]);
-              }
-              const int off = base + ((sg ^ swz) << 4);
-              *reinterpret_cast<uint4*>(h_hi + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-              *reinterpret_cast<uint4*>(h_lo + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-            }
-          }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor cores
-          __syncwarp();
-        };
-        const int shu = exponent(mu), sho = exponent(mo);
-        store_h(shu);
-        if (lane == 0) mbar_arrive(&hready[h]);
-        // H_occ of this row and half from tensor memory
+        tc_fence_after();
+        const uint32_t base = tmem + lane_addr + (uint32_t)(b * 256 + h * 128);
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           uint32_t x[16];
-          tmem_ld16(occ + 16 * u, x);
+          tmem_ld16(base + 16 * u, x);
           tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 16; ++i) tot[16 * u + i] = __uint_as_float(x[i]);
+          for (int i = 0; i < 16; ++i) tot[16 * u + i] += __uint_as_float(x[i]);
         }
-        bool fine = wait_or_abort(&hfree[h], 0);     // the unoccupied MMAs have read this half
-        if (__all_sync(0xffffffffu, fine)) {
-          tc_fence_after();
-          store_h(sho);
-          if (lane == 0) mbar_arrive(&hready[h]);
-          fine = wait_or_abort(&vready[h], 0);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[b]);
+      }
+      const int bo = bc & 1;
+      if (ok && have_occ) {
+        const bool got = wait_or_abort(&tfull[bo], (uint32_t)((bc >> 1) & 1));
+        if (!__all_sync(0xffffffffu, got)) {
+          if (lane == 0 && !*abort_flag) timed_out(3);
+          ok = false;
         }
-        if (__all_sync(0xffffffffu, fine)) {
-          tc_fence_after();
-          const uint32_t vb = tmem + lane_addr + (uint32_t)((1 - bo) * 256);
+        tc_fence_after();
+      }
+      // tcgen05.ld is warp-collective: the whole warp takes the same branch
+      ok = __all_sync(0xffffffffu, ok && !*abort_flag);
+      if (ok) {
+        const int r0 = m0 + q * 32;                   // first output row of this warp
+        const float sc = ldexpf(1.0f, -2 * p.dexp[p.b_shared ? 0 : tl.z]);
+        const float ao = p.alpha_occ[tl.z] * sc, au = p.alpha_un[tl.z] * sc;
+        // the half that G_occ holds may take the next tile's sums
+        auto free_occ = [&]() {
+          tc_fence_before();
+          __syncwarp();
+          if (have_occ && lane == 0) mbar_arrive(&tempty[bo]);
+        };
+        if constexpr (MODE == 2) {
+          // ---------------------------------------------- self-energy contraction of the tile
+          const int row = q * 32 + lane;               // tensor-memory lane = tile row
+          const int gm = m0 + row;
+          const bool rvalid = gm < p.m_rows;
+          const int c0 = n0 + h * 64;                   // first complex column of this warp's half
+          const long grow = grow0 + row;             // grid row r of this thread
+          const int swz = (row >> 1) & 3;
+          // The warp's 32 x 64 block of W~ goes through the shared memory that its own H will take:
+          // piece k (8 columns, 64 bytes a row) in the place of the warp's rows of K chunk 4h + k % 4,
+          // hi for k < 4 and lo above, 16-byte segments swizzled as H's.  Row r lies where row r of H
+          // will, so a thread only overwrites what it has read itself.
+          auto piece = [&](int k) -> uint8_t* {
+            return (k < 4 ? h_hi : h_lo) + (4 * h + (k & 3)) * A_BYTES + q * 2048;
+          };
+          {
+            const bool vec = (p.ldw % 2 == 0) && ((reinterpret_cast<uintptr_t>(p.wrr) & 15) == 0);
+#pragma unroll 4
+            for (int i = 0; i < 32; ++i) {              // eight rows of a piece per step, 64 bytes each
+              const int k = i >> 2, r = (i & 3) * 8 + (lane >> 2), sg = lane & 3;
+              const int gr = m0 + q * 32 + r, gn = c0 + 8 * k + 2 * sg;
+              uint8_t* dst = piece(k) + r * 64 + ((sg ^ ((r >> 1) & 3)) << 4);
+              const int have = gr < p.m_rows ? min(max(p.n_cols - gn, 0), 2) : 0;   // columns of the pair in range
+              const float2* src = have ? p.wrr + (long)gr * p.ldw + gn : p.wrr;
+              if (vec) {
+                cp_async16(dst, src, 8 * have);
+              } else {
+                cp_async8(dst, src, have > 0 ? 8 : 0);
+                cp_async8(dst + 8, have > 1 ? src + 1 : p.wrr, have > 1 ? 8 : 0);
+              }
+            }
+            cp_async_wait();
+            __syncwarp();
+          }
+          // H = w G o W~ for G_unocc in registers and for G_occ in tensor memory (in place); returns the
+          // powers of two that put the rows' maxima below 2^15
+          const uint32_t occ = tmem + lane_addr + (uint32_t)(bo * 256 + h * 128);
+          const int dr = (int)(grow - c0);              // column of the row's diagonal element
+          float mu = 0.f, mo = 0.f;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            if (16 * u < p.np) {                      // np is the same for the whole warp
-              uint32_t x[16], y[16];
-              tmem_ld16(vb + (uint32_t)(h * p.np + 16 * u), x);
-              tmem_ld16(vb + (uint32_t)((2 + h) * p.np + 16 * u), y);
+          for (int k = 0; k < 8; ++k) {
+            const uint8_t* wp = piece(k) + lane * 64;
+#pragma unroll
+            for (int hs = 0; hs < 2; ++hs) {
+              uint32_t x[8];
+              tmem_ld8(occ + 16 * k + 8 * hs, x);
+              float4 w2[2];
+#pragma unroll
+              for (int s = 0; s < 2; ++s) w2[s] = *reinterpret_cast<const float4*>(wp + (((2 * hs + s) ^ swz) << 4));
               tmem_wait_ld();
 #pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                tot[16 * u + i] = __uint_as_float(x[i]);
-                tot[64 + 16 * u + i] = __uint_as_float(y[i]);
+              for (int s = 0; s < 2; ++s) {
+                const float4 w = w2[s];
+                const int c = 8 * k + 4 * hs + 2 * s;
+                // weight of (r, R'): 2 below the diagonal, 1 on it, 0 above (lower-triangle mode)
+                float wa = 1.f, wb = 1.f;
+                if (p.lower) {
+                  wa = c < dr ? 2.f : (c == dr ? 1.f : 0.f);
+                  wb = c + 1 < dr ? 2.f : (c + 1 == dr ? 1.f : 0.f);
+                }
+                {
+                  const float ar = tot[2 * c] * au * wa, ai = tot[2 * c + 1] * au * wa;
+                  const float br = tot[2 * c + 2] * au * wb, bi = tot[2 * c + 3] * au * wb;
+                  tot[2 * c] = ar * w.x - ai * w.y;
+                  tot[2 * c + 1] = ar * w.y + ai * w.x;
+                  tot[2 * c + 2] = br * w.z - bi * w.w;
+                  tot[2 * c + 3] = br * w.w + bi * w.z;
+                  mu = fmaxf(mu, fmaxf(fmaxf(fabsf(tot[2 * c]), fabsf(tot[2 * c + 1])),
+                                       fmaxf(fabsf(tot[2 * c + 2]), fabsf(tot[2 * c + 3]))));
+                }
+                {
+                  const float g0 = __uint_as_float(x[4 * s]), g1 = __uint_as_float(x[4 * s + 1]);
+                  const float g2 = __uint_as_float(x[4 * s + 2]), g3 = __uint_as_float(x[4 * s + 3]);
+                  const float ar = g0 * ao * wa, ai = g1 * ao * wa;
+                  const float br = g2 * ao * wb, bi = g3 * ao * wb;
+                  const float y0 = ar * w.x - ai * w.y, y1 = ar * w.y + ai * w.x;
+                  const float y2 = br * w.z - bi * w.w, y3 = br * w.w + bi * w.z;
+                  mo = fmaxf(mo, fmaxf(fmaxf(fabsf(y0), fabsf(y1)), fmaxf(fabsf(y2), fabsf(y3))));
+                  x[4 * s] = __float_as_uint(y0);
+                  x[4 * s + 1] = __float_as_uint(y1);
+                  x[4 * s + 2] = __float_as_uint(y2);
+                  x[4 * s + 3] = __float_as_uint(y3);
+                }
               }
+              tmem_st8(occ + 16 * k + 8 * hs, x);
             }
           }
-          // 2^-(sh + e) in two factors as well, applied one after the other, so that the
-          // tiny rows come back as normal FP32 numbers where they are representable
-          const int e = *p.dexp, ku = shu + e, ko = sho + e;
-          const float fu1 = ldexpf(1.0f, -(ku >> 1)), fu2 = ldexpf(1.0f, -(ku - (ku >> 1)));
-          const float fo1 = ldexpf(1.0f, -(ko >> 1)), fo2 = ldexpf(1.0f, -(ko - (ko >> 1)));
-          // Re(conj(psi_n) V_n) of the row for NB >= n_n bands, then the sums over the warp's rows: at
-          // each of the five exchange steps a lane keeps half of its sums and hands over the other
-          // half, so that 62 shuffles leave lane l with sums l-th of 2 NB (the pairs added are those
-          // of a butterfly over each sum)
-          const int my_band = lane < p.n_n ? __ldg(p.bands + lane) : 0;
-          auto bands = [&](auto nb_c) {
-            constexpr int NB = decltype(nb_c)::value;
-#pragma unroll
-            for (int b0 = 0; b0 < NB; b0 += 8) {
-              float2 ps[8];
-#pragma unroll
-              for (int i = 0; i < 8 && b0 + i < NB; ++i) {
-                const int n = b0 + i;
-                const long at = (long)__shfl_sync(0xffffffffu, my_band, n) * p.ldpsi + grow;
-                ps[i] = rvalid && n < p.n_n ? __ldg(p.psi + at) : make_float2(0.f, 0.f);
-              }
-#pragma unroll
-              for (int i = 0; i < 8 && b0 + i < NB; ++i) {
-                const int n = b0 + i;
-                const float su = (ps[i].x * tot[2 * n] + ps[i].y * tot[2 * n + 1]) * fu1 * fu2;
-                const float so = (ps[i].x * tot[64 + 2 * n] + ps[i].y * tot[64 + 2 * n + 1]) * fo1 * fo2;
-                tot[2 * n] = su;
-                tot[2 * n + 1] = so;
-              }
-            }
-            int nv = 2 * NB;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-              if (nv > 1) {
-                nv >>= 1;
-                const bool up = (lane & off) != 0;
-#pragma unroll
-                for (int i = 0; i < NB; ++i)
-                  if (i < nv) {
-                    const float keep = up ? tot[i + nv] : tot[i], send = up ? tot[i] : tot[i + nv];
-                    tot[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-                  }
-              } else {
-                tot[0] += __shfl_xor_sync(0xffffffffu, tot[0], off);
-              }
-            }
-            // lane l: sums (l * 2 NB) / 32 .. of [su_0, so_0, su_1, ...]
-            float* rw = red + ew * 64;
-            if (NB == 32) {
-              rw[2 * lane] = tot[0];
-              rw[2 * lane + 1] = tot[1];
-            } else if (lane % (NB < 16 ? 16 / NB : 1) == 0) {
-              rw[lane * NB / 16] = tot[0];
-            }
+          tmem_wait_st();
+          auto exponent = [](float m) -> int {
+            int ex = 0;
+            if (m > 0.f) frexpf(m, &ex);
+            return m > 0.f ? 14 - ex : 0;
           };
-          if (p.n_n <= 4) bands(std::integral_constant<int, 4>{});
-          else if (p.n_n <= 8) bands(std::integral_constant<int, 8>{});
-          else if (p.n_n <= 16) bands(std::integral_constant<int, 16>{});
-          else bands(std::integral_constant<int, 32>{});
-          __syncwarp();
-          if (lane == 0) mbar_arrive(redbar);
-        } else if (lane == 0 && !*abort_flag) {
-          timed_out(10);
-        }
-        // one warp adds the CTA's band sums into Sigma_unocc_nn(tau_j), Sigma_occ_nn(-tau_j)
-        if (ew == 0) {
-          const bool got = wait_or_abort(redbar, 0);
-          if (got && lane < p.n_n) {
-            double su = 0.0, so = 0.0;
+          // this row of H, scaled by 2^sh and split in two 16-bit parts, into K chunks
+          // 4h..4h+3: row `row` of a chunk is 64 bytes at (row/8)*512 + (row%8)*64, its
+          // 16-byte segment s stored at s ^ ((row/2) % 4) (the 64-byte swizzle of TMA)
+          auto store_h = [&](int sh) {
+            // 2^sh in two factors: a row of tiny H (W~ of a large tau decays like exp(-omega tau))
+            // can need sh above 127, where one FP32 power of two would overflow
+            const float s1 = ldexpf(1.0f, sh >> 1), s2 = ldexpf(1.0f, sh - (sh >> 1));
 #pragma unroll
-            for (int w = 0; w < EPI_WARPS; ++w) {
-              su += (double)red[w * 64 + 2 * lane];
-              so += (double)red[w * 64 + 2 * lane + 1];
+            for (int j = 0; j < 4; ++j) {
+              const int base = (4 * h + j) * A_BYTES + (row >> 3) * 512 + (row & 7) * 64;
+#pragma unroll
+              for (int sg = 0; sg < 4; ++sg) {
+                uint32_t hw[4], lw[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                  const int c = 16 * j + 4 * sg + t;
+                  split2<FMT>(tot[2 * c] * s1 * s2, tot[2 * c + 1] * s1 * s2, hw[t], lw[t]);
+                }
+                const int off = base + ((sg ^ swz) << 4);
+                *reinterpret_cast<uint4*>(h_hi + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+                *reinterpret_cast<uint4*>(h_lo + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+              }
             }
-            atomicAdd(&p.acc_u[(long)lane * p.acc_stride], p.coef * su);
-            atomicAdd(&p.acc_o[(long)lane * p.acc_stride], -p.coef * so);
-          } else if (!got && lane == 0 && !*abort_flag) {
-            timed_out(11);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor cores
+            __syncwarp();
+          };
+          const int shu = exponent(mu), sho = exponent(mo);
+          store_h(shu);
+          if (lane == 0) mbar_arrive(&hready[h]);
+          // H_occ of this row and half from tensor memory
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            uint32_t x[16];
+            tmem_ld16(occ + 16 * u, x);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) tot[16 * u + i] = __uint_as_float(x[i]);
           }
-        }
-      } else {
-        float2* stg = epi + ew * 32 * EPI_COLS;
+          free_occ();
+          bool fine = wait_or_abort(&hfree[h], (uint32_t)(ti & 1));   // the unoccupied MMAs have read this half
+          if (__all_sync(0xffffffffu, fine)) {
+            tc_fence_after();
+            store_h(sho);
+            if (lane == 0) mbar_arrive(&hready[h]);
+            fine = wait_or_abort(&vready[h], (uint32_t)(ti & 1));
+          }
+          if (__all_sync(0xffffffffu, fine)) {
+            tc_fence_after();
+            const uint32_t vb = tmem + lane_addr + (uint32_t)((1 - bo) * 256);
 #pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-          const int nc0 = n0 + h * 64 + cc * 16;
+            for (int u = 0; u < 4; ++u) {
+              if (16 * u < p.np) {                      // np is the same for the whole warp
+                uint32_t x[16], y[16];
+                tmem_ld16(vb + (uint32_t)(h * p.np + 16 * u), x);
+                tmem_ld16(vb + (uint32_t)((2 + h) * p.np + 16 * u), y);
+                tmem_wait_ld();
 #pragma unroll
-          for (int pass = 0; pass < (MODE == 0 ? 1 : 2); ++pass) {
-            // row `lane` of the chunk to shared memory (rotated), then 128-byte row segments out
+                for (int i = 0; i < 16; ++i) {
+                  tot[16 * u + i] = __uint_as_float(x[i]);
+                  tot[64 + 16 * u + i] = __uint_as_float(y[i]);
+                }
+              }
+            }
+            // 2^-(sh + e) in two factors as well, applied one after the other, so that the
+            // tiny rows come back as normal FP32 numbers where they are representable
+            const int e = p.dexp[0], ku = shu + e, ko = sho + e;
+            const float fu1 = ldexpf(1.0f, -(ku >> 1)), fu2 = ldexpf(1.0f, -(ku - (ku >> 1)));
+            const float fo1 = ldexpf(1.0f, -(ko >> 1)), fo2 = ldexpf(1.0f, -(ko - (ko >> 1)));
+            // Re(conj(psi_n) V_n) of the row for NB >= n_n bands, then the sums over the warp's rows: at
+            // each of the five exchange steps a lane keeps half of its sums and hands over the other
+            // half, so that 62 shuffles leave lane l with sums l-th of 2 NB (the pairs added are those
+            // of a butterfly over each sum)
+            const int my_band = lane < p.n_n ? __ldg(p.bands + lane) : 0;
+            tc_fence_before();                          // V is read: the next tile may sum over it (redbar)
+            auto bands = [&](auto nb_c) {
+              constexpr int NB = decltype(nb_c)::value;
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
+              for (int b0 = 0; b0 < NB; b0 += 8) {
+                float2 ps[8];
+#pragma unroll
+                for (int i = 0; i < 8 && b0 + i < NB; ++i) {
+                  const int n = b0 + i;
+                  const long at = (long)__shfl_sync(0xffffffffu, my_band, n) * p.ldpsi + grow;
+                  ps[i] = rvalid && n < p.n_n ? __ldg(p.psi + at) : make_float2(0.f, 0.f);
+                }
+#pragma unroll
+                for (int i = 0; i < 8 && b0 + i < NB; ++i) {
+                  const int n = b0 + i;
+                  const float su = (ps[i].x * tot[2 * n] + ps[i].y * tot[2 * n + 1]) * fu1 * fu2;
+                  const float so = (ps[i].x * tot[64 + 2 * n] + ps[i].y * tot[64 + 2 * n + 1]) * fo1 * fo2;
+                  tot[2 * n] = su;
+                  tot[2 * n + 1] = so;
+                }
+              }
+              int nv = 2 * NB;
+#pragma unroll
+              for (int off = 16; off > 0; off >>= 1) {
+                if (nv > 1) {
+                  nv >>= 1;
+                  const bool up = (lane & off) != 0;
+#pragma unroll
+                  for (int i = 0; i < NB; ++i)
+                    if (i < nv) {
+                      const float keep = up ? tot[i + nv] : tot[i], send = up ? tot[i] : tot[i + nv];
+                      tot[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+                    }
+                } else {
+                  tot[0] += __shfl_xor_sync(0xffffffffu, tot[0], off);
+                }
+              }
+              // lane l: sums (l * 2 NB) / 32 .. of [su_0, so_0, su_1, ...]
+              float* rw = red + ew * 64;
+              if (NB == 32) {
+                rw[2 * lane] = tot[0];
+                rw[2 * lane + 1] = tot[1];
+              } else if (lane % (NB < 16 ? 16 / NB : 1) == 0) {
+                rw[lane * NB / 16] = tot[0];
+              }
+            };
+            if (p.n_n <= 4) bands(std::integral_constant<int, 4>{});
+            else if (p.n_n <= 8) bands(std::integral_constant<int, 8>{});
+            else if (p.n_n <= 16) bands(std::integral_constant<int, 16>{});
+            else bands(std::integral_constant<int, 32>{});
+            __syncwarp();
+            if (lane == 0) mbar_arrive(redbar);
+          } else {
+            if (lane == 0 && !*abort_flag) timed_out(10);
+            ok = false;
+          }
+          // one warp adds the CTA's band sums into Sigma_unocc_nn(tau_j), Sigma_occ_nn(-tau_j)
+          if (ew == 0) {
+            const bool got = wait_or_abort(redbar, (uint32_t)(ti & 1));
+            if (got && lane < p.n_n) {
+              double su = 0.0, so = 0.0;
+#pragma unroll
+              for (int w = 0; w < EPI_WARPS; ++w) {
+                su += (double)red[w * 64 + 2 * lane];
+                so += (double)red[w * 64 + 2 * lane + 1];
+              }
+              atomicAdd(&p.acc_u[(long)lane * p.acc_stride], p.coef * su);
+              atomicAdd(&p.acc_o[(long)lane * p.acc_stride], -p.coef * so);
+            } else if (!got && lane == 0 && !*abort_flag) {
+              timed_out(11);
+            }
+          }
+        } else {
+          // MODE 0 forms chi over G_unocc in registers at once, which frees G_occ's tensor memory: the
+          // MMAs of the next tile run while this one is written.  MODE 1 writes G_occ first.
+          if (MODE == 0) {
+            const int dr = (int)(grow0 - n0) + q * 32 + lane - h * 64;   // column of the row's diagonal element
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
               uint32_t ro[16];
-              const bool need_occ = MODE == 0 || pass == 0;
-              if (need_occ && have_occ) {
-                tmem_ld16(tmem + lane_addr + (uint32_t)(bo * 256 + h * 128 + 32 * cc + 16 * u), ro);
+              if (have_occ) {
+                tmem_ld16(tmem + lane_addr + (uint32_t)(bo * 256 + h * 128 + 16 * u), ro);
                 tmem_wait_ld();
               } else {
 #pragma unroll
@@ -637,44 +699,77 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
                 const float gor = __uint_as_float(ro[2 * j]) * ao, goi = __uint_as_float(ro[2 * j + 1]) * ao;
-                const float gur = tot[32 * cc + 16 * u + 2 * j] * au, gui = tot[32 * cc + 16 * u + 2 * j + 1] * au;
-                float2 v;
-                if (MODE == 0) {
-                  v = make_float2(-2.0f * (gor * gur + goi * gui), -2.0f * (goi * gur - gor * gui));
-                  if (diag_tile) {
-                    const long rr = grow0 + q * 32 + lane, cn = nc0 + u * 8 + j;
-                    const float f = cn < rr ? 1.f : (cn == rr ? 0.5f : 0.f);
-                    v.x *= f;
-                    v.y *= f;
-                  }
-                } else {
-                  v = pass == 0 ? make_float2(gor, goi) : make_float2(gur, gui);
+                const float gur = tot[16 * u + 2 * j] * au, gui = tot[16 * u + 2 * j + 1] * au;
+                float2 v = make_float2(-2.0f * (gor * gur + goi * gui), -2.0f * (goi * gur - gor * gui));
+                if (diag_tile) {
+                  const float f = 8 * u + j < dr ? 1.f : (8 * u + j == dr ? 0.5f : 0.f);
+                  v.x *= f;
+                  v.y *= f;
                 }
-                stg[lane * EPI_COLS + ((u * 8 + j + lane) & (EPI_COLS - 1))] = v;
+                tot[16 * u + 2 * j] = v.x;
+                tot[16 * u + 2 * j + 1] = v.y;
               }
             }
-            __syncwarp();
-            float2* outp = (MODE == 0 || pass == 0) ? p.out0 : p.out1;
+            free_occ();
+          }
+          float2* stg = epi + ew * 32 * EPI_COLS;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int idx = i * 32 + lane;
-              const int rr = idx >> 3, pc = (idx & 7) * 2;
-              const int gm = r0 + rr, gn = nc0 + pc;
-              if (gm >= p.m_rows || gn >= p.n_cols) continue;
-              const float2 v0 = stg[rr * EPI_COLS + ((pc + rr) & (EPI_COLS - 1))];
-              const float2 v1 = stg[rr * EPI_COLS + ((pc + 1 + rr) & (EPI_COLS - 1))];
-              float2* o = outp + (long)gm * p.ldo + gn;
-              if (gn + 1 < p.n_cols && ((reinterpret_cast<uintptr_t>(o) & 15) == 0)) {
-                *reinterpret_cast<float4*>(o) = make_float4(v0.x, v0.y, v1.x, v1.y);
-              } else {
-                o[0] = v0;
-                if (gn + 1 < p.n_cols) o[1] = v1;
+          for (int pass = 0; pass < (MODE == 0 ? 1 : 2); ++pass) {
+            // the warp's 32 x 64 block of the output; offsets within it are 32-bit
+            const int ldo = (int)p.ldo;
+            float2* outp = (MODE == 0 || pass == 0 ? p.out0 : p.out1) + tl.z * p.so + (long)r0 * ldo + n0 + h * 64 +
+                           (lane >> 3) * ldo + (lane & 7) * 2;
+            const int rows_left = p.m_rows - r0 - (lane >> 3), cols_left = p.n_cols - n0 - h * 64 - (lane & 7) * 2;
+            const bool vec = (ldo & 1) == 0 && (reinterpret_cast<uintptr_t>(outp) & 15) == 0;
+#pragma unroll
+            for (int cc = 0; cc < 4; ++cc) {
+              // row `lane` of the chunk to shared memory (rotated), then 128-byte row segments out
+#pragma unroll
+              for (int u = 0; u < 2; ++u) {
+                if (MODE == 1 && pass == 0) {
+                  uint32_t ro[16];
+                  if (have_occ) {
+                    tmem_ld16(tmem + lane_addr + (uint32_t)(bo * 256 + h * 128 + 32 * cc + 16 * u), ro);
+                    tmem_wait_ld();
+                  } else {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) ro[i] = 0u;
+                  }
+#pragma unroll
+                  for (int j = 0; j < 8; ++j)
+                    stg[lane * EPI_COLS + ((u * 8 + j + lane) & (EPI_COLS - 1))] =
+                        make_float2(__uint_as_float(ro[2 * j]) * ao, __uint_as_float(ro[2 * j + 1]) * ao);
+                } else {
+#pragma unroll
+                  for (int j = 0; j < 8; ++j) {
+                    const int c = 32 * cc + 16 * u + 2 * j;
+                    stg[lane * EPI_COLS + ((u * 8 + j + lane) & (EPI_COLS - 1))] =
+                        MODE == 0 ? make_float2(tot[c], tot[c + 1]) : make_float2(tot[c] * au, tot[c + 1] * au);
+                  }
+                }
               }
+              __syncwarp();
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                if (4 * i >= rows_left || 16 * cc >= cols_left) continue;
+                const int rr = 4 * i + (lane >> 3), pc = (lane & 7) * 2;
+                const float2 v0 = stg[rr * EPI_COLS + ((pc + rr) & (EPI_COLS - 1))];
+                const float2 v1 = stg[rr * EPI_COLS + ((pc + 1 + rr) & (EPI_COLS - 1))];
+                float2* o = outp + (4 * i * ldo + 16 * cc);
+                if (vec && 16 * cc + 1 < cols_left) {
+                  *reinterpret_cast<float4*>(o) = make_float4(v0.x, v0.y, v1.x, v1.y);
+                } else {
+                  o[0] = v0;
+                  if (16 * cc + 1 < cols_left) o[1] = v1;
+                }
+              }
+              __syncwarp();
             }
-            __syncwarp();
+            if (MODE == 1 && pass == 0) free_occ();
           }
         }
       }
+      if (have_occ) ++bc;
     }
   }
   tc_fence_before();
@@ -688,7 +783,10 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
 
 // ---------------------------------------------------------------------- operand preparation
 
-__global__ void maxabs_kernel(const float2* __restrict__ x, size_t n, unsigned int* __restrict__ out) {
+// max |component| of the n elements of entry blockIdx.y (stride sx)
+__global__ void maxabs_kernel(const float2* __restrict__ x, size_t n, long sx, unsigned int* __restrict__ out) {
+  x += blockIdx.y * sx;
+  out += blockIdx.y;
   float m = 0.f;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     m = fmaxf(m, fmaxf(fabsf(x[i].x), fabsf(x[i].y)));
@@ -696,15 +794,15 @@ __global__ void maxabs_kernel(const float2* __restrict__ x, size_t n, unsigned i
   if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));   // non-negative floats order as uints
 }
 
-// e such that max|x| * 2^e lies in [2^14, 2^15)
+// e such that max|x| * 2^e lies in [2^14, 2^15), one thread per entry
 __global__ void exponent_kernel(const unsigned int* __restrict__ maxbits, int* __restrict__ e) {
-  const float m = __uint_as_float(*maxbits);
+  const float m = __uint_as_float(maxbits[threadIdx.x]);
   int ex = 0;
   if (m > 0.f) {
     frexpf(m, &ex);        // m = f * 2^ex, f in [0.5, 1)
-    *e = 15 - ex;
+    e[threadIdx.x] = 15 - ex;
   } else {
-    *e = 0;
+    e[threadIdx.x] = 0;
   }
 }
 
@@ -713,15 +811,23 @@ __global__ void exponent_kernel(const unsigned int* __restrict__ maxbits, int* _
 // k_un_x + 2(k - n_occ) (unoccupied); padding columns are written as zero.
 //  A: row r (rows r0..r0+rows-1):  (ar, ai) * s_k * 2^e
 //  B: rows 2R', 2R'+1:             (br, -bi) and (bi, br) of conj(psi) * 2^e
+// Entry blockIdx.z: orbitals sx elements apart, its own factors s_k, scaling (unless
+// e_shared) and operand.
 template <bool IS_B, uint32_t FMT>
 __global__ void __launch_bounds__(256) prep_kernel(const float2* __restrict__ psi, int n_b, int n_occ, int nr, int r0,
                                                    int rows, const float* __restrict__ sk,
                                                    const int* __restrict__ dexp, int k_occ_pad, int k_un_x,
-                                                   int kpad, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo) {
+                                                   int kpad, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
+                                                   long sx, int e_shared) {
   __shared__ float2 t[32][33];
+  const int z = blockIdx.z;
+  psi += z * sx;
+  sk += (long)z * n_b;
+  hi += (long)z * (IS_B ? 2 : 1) * rows * kpad;
+  lo += (long)z * (IS_B ? 2 : 1) * rows * kpad;
   const int kb = blockIdx.y * 32;       // band tile (covers padded band slots)
   const int rb = blockIdx.x * 32;       // row tile
-  const float sc = ldexpf(1.0f, *dexp);
+  const float sc = ldexpf(1.0f, dexp[e_shared ? 0 : z]);
   // band slot -> band index (or -1 for padding)
   const int occ_slots = k_occ_pad / 2, un_slots = (kpad - k_un_x) / 2;
   auto band_of = [&](int slot) -> int {
@@ -882,19 +988,24 @@ static Layout layout(int n_b, int n_occ) {
 static int sig_np(int n_sig) { return (2 * n_sig + 15) / 16 * 16; }
 static int sig_kp(const GridInfo& g) { return (2 * g.nr + BK - 1) / BK * BK; }
 
-static size_t scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, bool with_tmp, int n_sig = 0) {
+// Words at the start of the scratch: [2..3] time-out status, then the entries' maxima and exponents.
+constexpr int kWords = 64 + 2 * kMaxEntries;
+
+static size_t scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, bool with_tmp, int n_sig, int nb,
+                            bool b_shared) {
   const Layout L = layout(n_b, n_occ);
+  const size_t nbb = b_shared ? 1 : nb;
   Carver probe(nullptr);
-  probe.take<unsigned int>(64);
-  probe.take<float>(n_b);
-  probe.take<uint16_t>((size_t)2 * g.nr * L.kpad);
-  probe.take<uint16_t>((size_t)2 * g.nr * L.kpad);
+  probe.take<unsigned int>(kWords);
+  probe.take<uint16_t>(nbb * 2 * g.nr * L.kpad);
+  probe.take<uint16_t>(nbb * 2 * g.nr * L.kpad);
   if (n_sig > 0) {
     probe.take<uint16_t>((size_t)sig_np(n_sig) * sig_kp(g));
     probe.take<uint16_t>((size_t)sig_np(n_sig) * sig_kp(g));
   }
-  probe.take<uint16_t>((size_t)n_rows * L.kpad);
-  probe.take<uint16_t>((size_t)n_rows * L.kpad);
+  probe.take<float>((size_t)nb * n_b);
+  probe.take<uint16_t>((size_t)nb * n_rows * L.kpad);
+  probe.take<uint16_t>((size_t)nb * n_rows * L.kpad);
   if (with_tmp) probe.take<float2>((size_t)n_rows * g.nr);
   return Carver::round(probe.off);
 }
@@ -904,29 +1015,34 @@ static size_t scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, b
 // into out1 (a NULL one goes to scratch).  prep_b = false reuses the B operand
 // and the operand scaling left in the same scratch by an earlier call for the
 // same psi.
-static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales& gs,
+static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales* gs,
                      int r0, int n_rows, gw_prec prec, int mode, void* out0, void* out1, void* scratch, bool prep_b,
                      cudaStream_t st, const float* sk_dev = nullptr, int* status_dev = nullptr,
-                     const TcSigma* sig = nullptr, bool lower = false) {
+                     const TcSigma* sig = nullptr, bool lower = false, const TcEntries& en = TcEntries{}) {
   const uint32_t fmt = prec == GW_BF16X3 ? 1u : 0u;
   const Layout L = layout(n_b, n_occ);
   gw_status rc;
+  const int nb = en.n;
+  const bool b_shared = en.psi_stride == 0;
+  const size_t nbb = b_shared ? 1 : nb;
+  if (nb < 1 || nb > kMaxEntries) return fail(ctx, GW_ERR_SHAPE, "1 to 64 entries per G formation");
   const bool need_tmp = mode == 1 && (!out0 || !out1);
   Carver cv(scratch);
-  unsigned int* dmax = cv.take<unsigned int>(64);
-  int* dexp = reinterpret_cast<int*>(dmax + 1);
+  unsigned int* words = cv.take<unsigned int>(kWords);
+  unsigned int* dmax = words + 64;
+  int* dexp = reinterpret_cast<int*>(words + 64 + kMaxEntries);
   // time-out status: in the scratch, or in a word the caller owns (kept past later uses of the scratch)
-  int* status = status_dev ? status_dev : reinterpret_cast<int*>(dmax + 2);
-  float* dsk = cv.take<float>(n_b);
-  uint16_t* bhi = cv.take<uint16_t>((size_t)2 * g.nr * L.kpad);
-  uint16_t* blo = cv.take<uint16_t>((size_t)2 * g.nr * L.kpad);
-  // the psi_n operand is prepared by the first call and read by later ones: its place must
-  // not depend on this call's number of rows, so it comes before the A operand
+  int* status = status_dev ? status_dev : reinterpret_cast<int*>(words + 2);
+  uint16_t* bhi = cv.take<uint16_t>(nbb * 2 * g.nr * L.kpad);
+  uint16_t* blo = cv.take<uint16_t>(nbb * 2 * g.nr * L.kpad);
+  // these operands are prepared by the first call and read by later ones: their place must not
+  // depend on this call's number of rows or entries, so they come before what does
   const int np = mode == 2 ? sig_np(sig->n_n) : 0, kps = sig_kp(g);
   uint16_t* phi = mode == 2 ? cv.take<uint16_t>((size_t)np * kps) : nullptr;
   uint16_t* plo = mode == 2 ? cv.take<uint16_t>((size_t)np * kps) : nullptr;
-  uint16_t* ahi = cv.take<uint16_t>((size_t)n_rows * L.kpad);
-  uint16_t* alo = cv.take<uint16_t>((size_t)n_rows * L.kpad);
+  float* dsk = cv.take<float>((size_t)nb * n_b);
+  uint16_t* ahi = cv.take<uint16_t>((size_t)nb * n_rows * L.kpad);
+  uint16_t* alo = cv.take<uint16_t>((size_t)nb * n_rows * L.kpad);
   float2* tmp = need_tmp ? cv.take<float2>((size_t)n_rows * g.nr) : nullptr;
   if (mode == 1) {
     if (!out0) out0 = tmp;
@@ -935,29 +1051,30 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
   // per-band factors: uploaded here, or already on the device (sk_dev: no host-to-device copy in this call)
   const float* sk = sk_dev;
   if (!sk) {
-    std::vector<float> skf(gs.s.begin(), gs.s.end());
-    if ((rc = upload(ctx, dsk, skf.data(), sizeof(float) * n_b, st))) return rc;
+    std::vector<float> skf;
+    for (int z = 0; z < nb; ++z) skf.insert(skf.end(), gs[z].s.begin(), gs[z].s.end());
+    if ((rc = upload(ctx, dsk, skf.data(), sizeof(float) * skf.size(), st))) return rc;
     sk = dsk;
   }
   const dim3 tb(32, 8);
   const int slots = L.kpad / 2;
   if (prep_b) {
-    if ((rc = cuda_check(ctx, cudaMemsetAsync(dmax, 0, 64 * sizeof(unsigned int), st), "memset"))) return rc;
+    if ((rc = cuda_check(ctx, cudaMemsetAsync(words, 0, kWords * sizeof(unsigned int), st), "memset"))) return rc;
     if (status_dev && (rc = cuda_check(ctx, cudaMemsetAsync(status_dev, 0, 2 * sizeof(int), st), "memset")))
       return rc;
     const size_t nel = (size_t)n_b * g.nr;
-    maxabs_kernel<<<std::min<size_t>((nel + 255) / 256, (size_t)ctx->num_sms * 8), 256, 0, st>>>(
-        static_cast<const float2*>(psi), nel, dmax);
+    maxabs_kernel<<<dim3((unsigned)std::min<size_t>((nel + 255) / 256, (size_t)ctx->num_sms * 8 / nbb + 1), nbb), 256, 0,
+                    st>>>(static_cast<const float2*>(psi), nel, en.psi_stride, dmax);
     if ((rc = launch_check(ctx, "maxabs_kernel"))) return rc;
-    exponent_kernel<<<1, 1, 0, st>>>(dmax, dexp);
+    exponent_kernel<<<1, (unsigned)nbb, 0, st>>>(dmax, dexp);
     if ((rc = launch_check(ctx, "exponent_kernel"))) return rc;
-    const dim3 gbB((g.nr + 31) / 32, (slots + 31) / 32);
+    const dim3 gbB((g.nr + 31) / 32, (slots + 31) / 32, nbb);
     if (fmt == 0)
       prep_kernel<true, 0><<<gbB, tb, 0, st>>>((const float2*)psi, n_b, n_occ, g.nr, 0, g.nr, sk, dexp,
-                                                L.k_occ_pad, L.k_un_x, L.kpad, bhi, blo);
+                                                L.k_occ_pad, L.k_un_x, L.kpad, bhi, blo, en.psi_stride, b_shared);
     else
       prep_kernel<true, 1><<<gbB, tb, 0, st>>>((const float2*)psi, n_b, n_occ, g.nr, 0, g.nr, sk, dexp,
-                                                L.k_occ_pad, L.k_un_x, L.kpad, bhi, blo);
+                                                L.k_occ_pad, L.k_un_x, L.kpad, bhi, blo, en.psi_stride, b_shared);
     if ((rc = launch_check(ctx, "prep_kernel(B)"))) return rc;
     if (mode == 2) {
       const dim3 gp((kps / 2 + 255) / 256, np / 2);
@@ -967,22 +1084,20 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
         prep_psin_kernel<1><<<gp, 256, 0, st>>>((const float2*)psi, g.nr, sig->bands, sig->n_n, kps, dexp, phi, plo);
       if ((rc = launch_check(ctx, "prep_psin_kernel"))) return rc;
     }
-  } else {
-    if ((rc = cuda_check(ctx, cudaMemsetAsync(status, 0, 2 * sizeof(int), st), "memset"))) return rc;
   }
-  const dim3 gbA((n_rows + 31) / 32, (slots + 31) / 32);
+  const dim3 gbA((n_rows + 31) / 32, (slots + 31) / 32, nb);
   if (fmt == 0)
     prep_kernel<false, 0><<<gbA, tb, 0, st>>>((const float2*)psi, n_b, n_occ, g.nr, r0, n_rows, sk, dexp,
-                                               L.k_occ_pad, L.k_un_x, L.kpad, ahi, alo);
+                                               L.k_occ_pad, L.k_un_x, L.kpad, ahi, alo, en.psi_stride, b_shared);
   else
     prep_kernel<false, 1><<<gbA, tb, 0, st>>>((const float2*)psi, n_b, n_occ, g.nr, r0, n_rows, sk, dexp,
-                                               L.k_occ_pad, L.k_un_x, L.kpad, ahi, alo);
+                                               L.k_occ_pad, L.k_un_x, L.kpad, ahi, alo, en.psi_stride, b_shared);
   if ((rc = launch_check(ctx, "prep_kernel(A)"))) return rc;
   CUtensorMap mah, mal, mbh, mbl, mph, mpl;
-  if ((rc = tc_make_map3(ctx, &mah, ahi, L.kpad, n_rows, 1, BM, fmt, BK))) return rc;
-  if ((rc = tc_make_map3(ctx, &mal, alo, L.kpad, n_rows, 1, BM, fmt, BK))) return rc;
-  if ((rc = tc_make_map3(ctx, &mbh, bhi, L.kpad, 2L * g.nr, 1, 2 * BNC, fmt, BK))) return rc;
-  if ((rc = tc_make_map3(ctx, &mbl, blo, L.kpad, 2L * g.nr, 1, 2 * BNC, fmt, BK))) return rc;
+  if ((rc = tc_make_map3(ctx, &mah, ahi, L.kpad, n_rows, nb, BM, fmt, BK))) return rc;
+  if ((rc = tc_make_map3(ctx, &mal, alo, L.kpad, n_rows, nb, BM, fmt, BK))) return rc;
+  if ((rc = tc_make_map3(ctx, &mbh, bhi, L.kpad, 2L * g.nr, (int)nbb, 2 * BNC, fmt, BK))) return rc;
+  if ((rc = tc_make_map3(ctx, &mbl, blo, L.kpad, 2L * g.nr, (int)nbb, 2 * BNC, fmt, BK))) return rc;
   if (mode == 2) {
     if ((rc = tc_make_map3(ctx, &mph, phi, kps, np, 1, np, fmt, BK))) return rc;
     if ((rc = tc_make_map3(ctx, &mpl, plo, kps, np, 1, np, fmt, BK))) return rc;
@@ -999,8 +1114,13 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
   P.out0 = static_cast<float2*>(out0);
   P.out1 = static_cast<float2*>(mode == 1 ? out1 : out0);
   P.ldo = g.nr;
-  P.alpha_occ = (float)gs.amax_occ;
-  P.alpha_un = (float)gs.amax_unocc;
+  for (int z = 0; z < nb; ++z) {
+    P.alpha_occ[z] = (float)gs[z].amax_occ;
+    P.alpha_un[z] = (float)gs[z].amax_unocc;
+  }
+  P.nb = nb;
+  P.b_shared = b_shared ? 1 : 0;
+  P.so = en.out_stride;
   P.dexp = dexp;
   P.status = status;
   P.wrr = nullptr;
@@ -1025,19 +1145,15 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
     P.acc_o = sig->acc_o;
     P.acc_stride = sig->acc_stride;
   }
-  // the column tiles past the block's last row hold no R' <= r
-  const int col_end = P.lower ? std::min(g.nr, r0 + n_rows) : g.nr;
-  const dim3 grid((col_end + BNC - 1) / BNC, (n_rows + BM - 1) / BM);
-  // multiply-adds the launch performs: full tiles, or those meeting R' <= r
-  double tiles = (double)grid.x * grid.y;
-  if (P.lower) {
-    tiles = 0;
-    for (unsigned by = 0; by < grid.y; ++by) {
-      const long last_row = (long)r0 + by * BM + BM - 1;
-      tiles += std::min<double>(grid.x, (double)(last_row / BNC + 1));
-    }
-  }
-  const double tile_frac = tiles / ((double)((g.nr + BNC - 1) / BNC) * grid.y);
+  // tiles per entry: all, or those meeting R' <= r
+  P.gx = (g.nr + BNC - 1) / BNC;
+  P.gy = (n_rows + BM - 1) / BM;
+  P.tiles = 0;
+  for (int i = 0; i < P.gy; ++i) P.tiles += P.lower ? std::min(P.gx, (r0 + i * BM + BM - 1) / BNC + 1) : P.gx;
+  const double tile_frac = nb * (double)P.tiles / ((double)P.gx * P.gy);
+  // persistent: one CTA per SM walks the tiles, so that the TMA loads and MMAs of a tile start while the
+  // last one's epilogue runs (modes 0 and 1) and no tile pays for a CTA's set-up
+  const unsigned grid = (unsigned)std::min<long>((long)P.tiles * nb, ctx->num_sms);
   auto go = [&](auto kernel) -> gw_status {
     gw_status r = cuda_check(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES),
                              "cudaFuncSetAttribute");
@@ -1067,29 +1183,31 @@ static gw_status check_status(gw_ctx* ctx, void* scratch, cudaStream_t st) {
 
 }  // namespace tc
 
-size_t tc_scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, bool with_tmp, int n_sig) {
-  return tc::scratch_bytes(g, n_b, n_occ, n_rows, with_tmp, n_sig);
+size_t tc_scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, bool with_tmp, int n_sig, int n_entries,
+                        bool one_psi) {
+  return tc::scratch_bytes(g, n_b, n_occ, n_rows, with_tmp, n_sig, n_entries, one_psi);
 }
 
 gw_status tc_sigma_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales& gs,
                         int r0, int n_rows, gw_prec prec, const TcSigma& sig, void* scratch, bool prep_b,
                         cudaStream_t st) {
   if (sig.n_n < 1 || sig.n_n > 32) return fail(ctx, GW_ERR_SHAPE, "fused self-energy contraction takes 1..32 bands");
-  return tc::run(ctx, g, n_b, n_occ, psi, gs, r0, n_rows, prec, 2, nullptr, nullptr, scratch, prep_b, st, sig.sk,
+  return tc::run(ctx, g, n_b, n_occ, psi, &gs, r0, n_rows, prec, 2, nullptr, nullptr, scratch, prep_b, st, sig.sk,
                  nullptr, &sig, true);
 }
 
-gw_status tc_green_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales& gs,
+gw_status tc_green_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales* gs,
                         int r0, int n_rows, gw_prec prec, void* g_occ, void* g_unocc, void* scratch, bool prep_b,
-                        cudaStream_t st, const float* sk_dev) {
-  return tc::run(ctx, g, n_b, n_occ, psi, gs, r0, n_rows, prec, 1, g_occ, g_unocc, scratch, prep_b, st, sk_dev);
+                        cudaStream_t st, const float* sk_dev, const TcEntries& en) {
+  return tc::run(ctx, g, n_b, n_occ, psi, gs, r0, n_rows, prec, 1, g_occ, g_unocc, scratch, prep_b, st, sk_dev, nullptr,
+                 nullptr, false, en);
 }
 
-gw_status tc_chi_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales& gs,
+gw_status tc_chi_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales* gs,
                       int r0, int n_rows, gw_prec prec, void* chi, void* scratch, bool prep_b, cudaStream_t st,
-                      const float* sk_dev, int* status_dev, bool lower) {
+                      const float* sk_dev, int* status_dev, bool lower, const TcEntries& en) {
   return tc::run(ctx, g, n_b, n_occ, psi, gs, r0, n_rows, prec, 0, chi, nullptr, scratch, prep_b, st, sk_dev,
-                 status_dev, nullptr, lower);
+                 status_dev, nullptr, lower, en);
 }
 
 gw_status tc_check_status(gw_ctx* ctx, const int* status_dev, cudaStream_t st) {

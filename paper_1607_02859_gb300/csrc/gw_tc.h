@@ -7,24 +7,34 @@
 
 namespace gw {
 
-// Scratch the two calls below need for n_rows rows (with_tmp: room for an
-// output the caller did not supply).
-size_t tc_scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, bool with_tmp, int n_sig = 0);
+// Entries of one launch: products that share the grid, the bands and the rows.
+// Entry z takes the orbitals psi + z psi_stride (elements; 0: the same for all, which
+// then share their psi-only operand), the factors gs[z] and the outputs
+// out + z out_stride.
+struct TcEntries {
+  int n = 1;
+  long psi_stride = 0, out_stride = 0;
+};
+// Scratch the calls below need for n_rows rows (with_tmp: room for an output the
+// caller did not supply; one_psi: psi_stride 0).
+size_t tc_scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, bool with_tmp, int n_sig = 0,
+                        int n_entries = 1, bool one_psi = true);
 // G_occ / G_unocc rows as 3 fp16 (or bf16) split products on tcgen05 with FP32
-// accumulation in tensor memory.  Either output may be NULL.  prep_b = false
-// reuses the psi-only operand an earlier call left in the same scratch.
-gw_status tc_green_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi,
-                        const GreenScales& gs, int r0, int n_rows, gw_prec prec, void* g_occ, void* g_unocc,
-                        void* scratch, bool prep_b, cudaStream_t st, const float* sk_dev = nullptr);
+// accumulation in tensor memory.  Either output may be NULL (one entry only).
+// prep_b = false reuses the psi-only operand an earlier call left in the same scratch.
+gw_status tc_green_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales* gs,
+                        int r0, int n_rows, gw_prec prec, void* g_occ, void* g_unocc, void* scratch, bool prep_b,
+                        cudaStream_t st, const float* sk_dev = nullptr, const TcEntries& en = TcEntries{});
 // chi rows = -2 G_occ o conj(G_unocc) with both tiles accumulated in tensor memory.
-// sk_dev: the per-band factors gs.s already on the device as FP32 (then the
-// call copies nothing from the host).
+// sk_dev: the per-band factors gs[z].s, entry after entry, already on the device as
+// FP32 (then the call copies nothing from the host).
 // lower: only R' <= r (grid rows r0 ..), with the diagonal halved; what lies above is not
 // all written (launch_row_fft with low takes it as zero).  Its transform X gives
 // chi(G,G') = X + X^H (chi is Hermitian in (r, R')).
-gw_status tc_chi_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales& gs,
+gw_status tc_chi_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales* gs,
                       int r0, int n_rows, gw_prec prec, void* chi, void* scratch, bool prep_b, cudaStream_t st,
-                      const float* sk_dev = nullptr, int* status_dev = nullptr, bool lower = false);
+                      const float* sk_dev = nullptr, int* status_dev = nullptr, bool lower = false,
+                      const TcEntries& en = TcEntries{});
 // The self-energy contraction fused into the G formation of rows r0 .. r0+n_rows-1
 // (first term of Eq. Sigma_occ_reduce): for every 128 x 128 tile with R' <= r
 // (G o W~ is Hermitian in (r, R'), so the real quadratic form is twice its
