@@ -24,7 +24,7 @@
 // epilogue either writes both (gw_green_tau) or their product
 // chi = -2 G_occ conj(G_unocc) (gw_chi0_rtau_fused), so for chi neither G tile
 // ever reaches HBM.  Warp roles: 0 = TMA producer, 1 = MMA issuer (and tensor
-// memory owner), 2..9 = epilogue.  Every wait is bounded; on time-out the
+// memory owner), the rest = epilogue.  Every wait is bounded; on time-out the
 // kernel records it in the status word, drains its own copies and MMAs, frees
 // its tensor memory and returns.
 #include <cuda.h>
@@ -48,14 +48,23 @@ constexpr int BNC = 128;                // complex columns per tile (MMA N = 256
 constexpr int BK = 32;                  // real K per stage (one 64-byte swizzle row)
 constexpr int STAGES = 4;
 constexpr int CH = 4;                   // stages per accumulation block (128 real K)
-constexpr int EPI_WARPS = 8;            // two per tensor-memory lane quarter, one per column half
+// Epilogue warps: four per tensor-memory lane quarter (64 sums a thread, 96 registers) for the modes
+// that write their tile; two (128 sums, 168 registers) for the self-energy, whose longer code spilled
+// inside the K loop with 96 (36^3, 2 tau: 180 against 148 ms).  With two, the writing modes spilled
+// 400 bytes a thread past the small L1 and their tile's end took 16 thousand cycles, more than the two
+// accumulation blocks that the MMAs run ahead: chi rows at 20^3 with 512 bands 3.96 ms, with four 3.42
+// (466 TFLOP/s), at 24^3 with 1024 bands 13.1 and 11.9 ms.
+template <int MODE>
+constexpr int kEpiWarps = MODE == 2 ? 8 : 16;
 constexpr int A_BYTES = BM * BK * 2;            // 8 KB
 constexpr int B_BYTES = 2 * BNC * BK * 2;       // 16 KB
 constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
-constexpr int EPI_COLS = 16;                    // complex columns per epilogue round
-constexpr int EPI_BYTES = EPI_WARPS * 32 * EPI_COLS * 8;
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 256;
-constexpr int THREADS = 64 + 32 * EPI_WARPS;
+constexpr int EPI_COLS = 8;                     // complex columns per epilogue round
+constexpr int EPI_BYTES = 16 * 32 * EPI_COLS * 8;
+constexpr int kTileTab = 256;                   // tiles of a CTA looked up in advance
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 4 * kTileTab + 1024 + 256;
+template <int MODE>
+constexpr int kThreads = 64 + 32 * kEpiWarps<MODE>;
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
 
 constexpr int kMaxEntries = 64;
@@ -129,16 +138,18 @@ struct Params {
 // (32 bands) thousand cycles, now 38 and 50; sigma at 20^3 with 512 bands 14.9 ->
 // 10.4 ms, at 36^3 with 4224 bands and 2 tau 207 -> 170 ms.
 template <int MODE, uint32_t FMT>
-__global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_constant__ CUtensorMap mA_hi,
+__global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __grid_constant__ CUtensorMap mA_hi,
                                                               const __grid_constant__ CUtensorMap mA_lo,
                                                               const __grid_constant__ CUtensorMap mB_hi,
                                                               const __grid_constant__ CUtensorMap mB_lo,
                                                               const __grid_constant__ CUtensorMap mP_hi,
                                                               const __grid_constant__ CUtensorMap mP_lo, Params p) {
+  constexpr int EW = kEpiWarps<MODE>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   float2* epi = reinterpret_cast<float2*>(smem + STAGES * STAGE_BYTES);     // [8 warps][32 rows][16]
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES + EPI_BYTES);
+  uint32_t* tile_tab = reinterpret_cast<uint32_t*>(smem + STAGES * STAGE_BYTES + EPI_BYTES);
+  uint64_t* full = reinterpret_cast<uint64_t*>(tile_tab + kTileTab);
   uint64_t* empty = full + STAGES;
   uint64_t* tfull = empty + STAGES;      // [2] block finished in tensor-memory half b
   uint64_t* tempty = tfull + 2;          // [2] half b drained by the epilogue
@@ -163,7 +174,7 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
     int z, m0, n0;
   };
   auto cols_of = [&](int i) { return p.lower ? min(p.gx, (p.r0 + i * BM + BM - 1) / BNC + 1) : p.gx; };
-  auto tile_at = [&](int t) -> Tile {
+  auto find_tile = [&](int t) -> Tile {
     constexpr int kGroupRows = 8;
     Tile o;
     o.z = t / p.tiles;
@@ -190,6 +201,20 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
     return o;
   };
   const int n_tiles = p.tiles * p.nb;
+  // the CTA's first tiles are found by all its threads at once
+  for (int i = threadIdx.x; i < kTileTab && blockIdx.x + (long)i * gridDim.x < n_tiles; i += kThreads<MODE>) {
+    const Tile o = find_tile(blockIdx.x + i * gridDim.x);
+    tile_tab[i] = (uint32_t)o.z << 26 | (uint32_t)(o.m0 / BM) << 13 | (uint32_t)(o.n0 / BNC);
+  }
+  auto tile_at = [&](int t, int i) -> Tile {       // tile t, the CTA's i-th
+    if (i >= kTileTab) return find_tile(t);
+    const uint32_t e = tile_tab[i];
+    Tile o;
+    o.z = (int)(e >> 26);
+    o.m0 = (int)(e >> 13 & 8191) * BM;
+    o.n0 = (int)(e & 8191) * BNC;
+    return o;
+  };
   const int total = p.k_occ_steps + p.k_un_steps;
   const int n_un_blocks = (p.k_un_steps + CH - 1) / CH;
   const bool have_occ = p.k_occ_steps > 0;
@@ -201,18 +226,18 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], EPI_WARPS);
+      mbar_init(&tempty[b], EW);
     }
     mbar_init(done, 1);
     mbar_init(last_mma, 1);
     if (MODE == 2) {
       for (int b = 0; b < 2; ++b) {
-        mbar_init(&hready[b], 4);
+        mbar_init(&hready[b], EW / 2);
         mbar_init(&hfree[b], 1);
         mbar_init(&vready[b], 1);
       }
       mbar_init(psi_full, 1);
-      mbar_init(redbar, EPI_WARPS);
+      mbar_init(redbar, EW);
       mbar_init(done2, 1);
     }
     *abort_flag = 0;
@@ -253,7 +278,7 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
     // ---------------------------------------------------------- TMA producer (unoccupied K first)
     int kit = 0, ti = 0;                               // stages issued, tiles of this CTA
     for (int t = blockIdx.x; t < n_tiles && !*abort_flag; t += gridDim.x, ++ti) {
-      const Tile tl = tile_at(t);
+      const Tile tl = tile_at(t, ti);
       const int zb = p.b_shared ? 0 : tl.z;
       // MODE 2: the stages of the last tile held H and psi_n until its last MMA
       if (MODE == 2 && ti > 0 && !wait_or_abort(done2, (uint32_t)((ti - 1) & 1))) {
@@ -380,26 +405,31 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
     if (!mbar_wait(last_mma, 0)) timed_out(5);
   } else if (warp >= 2) {
     // ---------------------------------------------------------- epilogue
+    constexpr int CW = 1024 / EW;                 // real columns of a warp
+    constexpr int NC = CW / 2;                    // complex columns
     const int ew = warp - 2;
     const int q = warp & 3;                       // tensor-memory lane quarter of this warp
-    const int h = ew >> 2;                        // column half: real columns h*128 .. h*128+127
+    const int cg = ew >> 2;                       // column group: complex columns cg*NC .. of the tile
     const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
+    const int row = q * 32 + lane;                // tensor-memory lane = tile row
+    const int swz = (row >> 1) & 3;               // 64-byte swizzle key of the row
     int bc = 0, ti = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++ti) {
-      const Tile tl = tile_at(t);
+      const Tile tl = tile_at(t, ti);
       const int m0 = tl.m0, n0 = tl.n0;
-      const long grow0 = (long)p.r0 + m0;           // grid row of the tile's first row
-      const bool diag_tile = MODE != 1 && p.lower && n0 + BNC > grow0;   // the tile meets the diagonal
+      const int c0 = n0 + cg * NC;                  // first complex column of this warp
+      const int grow0 = p.r0 + m0;                  // grid row of the tile's first row
+      const int dr = grow0 + row - c0;              // column (from c0) of this row's diagonal element
       if (MODE == 2 && p.ldw % 2 == 0 && (reinterpret_cast<uintptr_t>(p.wrr) & 15) == 0) {
         // this warp's block of W~ on its way into L2 while the K loop runs
-        const int gr = m0 + q * 32 + lane, gc = n0 + h * 64;
-        const int bytes = gr < p.m_rows ? min(64, p.n_cols - gc) * 8 & ~15 : 0;
-        if (bytes > 0) prefetch_l2(p.wrr + (long)gr * p.ldw + gc, bytes);
+        const int gr = m0 + row;
+        const int bytes = gr < p.m_rows ? min(NC, p.n_cols - c0) * 8 & ~15 : 0;
+        if (bytes > 0) prefetch_l2(p.wrr + (long)gr * p.ldw + c0, bytes);
       }
-      float tot[128];                               // this thread's row of G_unocc, FP32 round-to-nearest sums
+      float tot[CW];                                // this thread's part of its row of G_unocc, FP32 round-to-nearest sums
 #pragma unroll
-      for (int i = 0; i < 128; ++i) tot[i] = 0.f;
+      for (int i = 0; i < CW; ++i) tot[i] = 0.f;
       for (int c = 0; c < n_un_blocks; ++c, ++bc) {
         const int b = bc & 1;
         const bool got = wait_or_abort(&tfull[b], (uint32_t)((bc >> 1) & 1));
@@ -409,9 +439,9 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
           break;
         }
         tc_fence_after();
-        const uint32_t base = tmem + lane_addr + (uint32_t)(b * 256 + h * 128);
+        const uint32_t base = tmem + lane_addr + (uint32_t)(b * 256 + cg * CW);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < CW / 16; ++u) {
           uint32_t x[16];
           tmem_ld16(base + 16 * u, x);
           tmem_wait_ld();
@@ -434,9 +464,9 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
       // tcgen05.ld is warp-collective: the whole warp takes the same branch
       ok = __all_sync(0xffffffffu, ok && !*abort_flag);
       if (ok) {
-        const int r0 = m0 + q * 32;                   // first output row of this warp
         const float sc = ldexpf(1.0f, -2 * p.dexp[p.b_shared ? 0 : tl.z]);
         const float ao = p.alpha_occ[tl.z] * sc, au = p.alpha_un[tl.z] * sc;
+        const uint32_t occ = tmem + lane_addr + (uint32_t)(bo * 256 + cg * CW);
         // the half that G_occ holds may take the next tile's sums
         auto free_occ = [&]() {
           tc_fence_before();
@@ -445,12 +475,9 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
         };
         if constexpr (MODE == 2) {
           // ---------------------------------------------- self-energy contraction of the tile
-          const int row = q * 32 + lane;               // tensor-memory lane = tile row
-          const int gm = m0 + row;
-          const bool rvalid = gm < p.m_rows;
-          const int c0 = n0 + h * 64;                   // first complex column of this warp's half
-          const long grow = grow0 + row;             // grid row r of this thread
-          const int swz = (row >> 1) & 3;
+          const bool rvalid = m0 + row < p.m_rows;
+          const int h = cg;                             // the warp's column half
+          const long grow = grow0 + row;                // grid row r of this thread
           // The warp's 32 x 64 block of W~ goes through the shared memory that its own H will take:
           // piece k (8 columns, 64 bytes a row) in the place of the warp's rows of K chunk 4h + k % 4,
           // hi for k < 4 and lo above, 16-byte segments swizzled as H's.  Row r lies where row r of H
@@ -479,8 +506,6 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
           }
           // H = w G o W~ for G_unocc in registers and for G_occ in tensor memory (in place); returns the
           // powers of two that put the rows' maxima below 2^15
-          const uint32_t occ = tmem + lane_addr + (uint32_t)(bo * 256 + h * 128);
-          const int dr = (int)(grow - c0);              // column of the row's diagonal element
           float mu = 0.f, mo = 0.f;
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
@@ -671,7 +696,7 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
             if (got && lane < p.n_n) {
               double su = 0.0, so = 0.0;
 #pragma unroll
-              for (int w = 0; w < EPI_WARPS; ++w) {
+              for (int w = 0; w < EW; ++w) {
                 su += (double)red[w * 64 + 2 * lane];
                 so += (double)red[w * 64 + 2 * lane + 1];
               }
@@ -685,12 +710,12 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
           // MODE 0 forms chi over G_unocc in registers at once, which frees G_occ's tensor memory: the
           // MMAs of the next tile run while this one is written.  MODE 1 writes G_occ first.
           if (MODE == 0) {
-            const int dr = (int)(grow0 - n0) + q * 32 + lane - h * 64;   // column of the row's diagonal element
+            const bool diag_tile = p.lower && n0 + BNC > grow0;   // the tile meets the diagonal
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < 4; ++u) {
               uint32_t ro[16];
               if (have_occ) {
-                tmem_ld16(tmem + lane_addr + (uint32_t)(bo * 256 + h * 128 + 16 * u), ro);
+                tmem_ld16(occ + 16 * u, ro);
                 tmem_wait_ld();
               } else {
 #pragma unroll
@@ -712,55 +737,55 @@ __global__ void __launch_bounds__(THREADS, 1) green_tc_kernel(const __grid_const
             }
             free_occ();
           }
-          float2* stg = epi + ew * 32 * EPI_COLS;
+          // 32 rows x 8 columns at a time through shared memory as pairs of columns (pair s of row r at
+          // s ^ (r/2) % 4), then 64-byte row segments out
+          float4* stg = reinterpret_cast<float4*>(epi + ew * 32 * EPI_COLS);
+          float4* const st_w = stg + lane * 4;                               // this lane's row
+          const int rrow = lane >> 2, rpair = lane & 3;                      // written out: row rrow + 8 i
+          const float4* const st_r = stg + rrow * 4 + (rpair ^ (rrow >> 1 & 3));
 #pragma unroll
           for (int pass = 0; pass < (MODE == 0 ? 1 : 2); ++pass) {
-            // the warp's 32 x 64 block of the output; offsets within it are 32-bit
             const int ldo = (int)p.ldo;
-            float2* outp = (MODE == 0 || pass == 0 ? p.out0 : p.out1) + tl.z * p.so + (long)r0 * ldo + n0 + h * 64 +
-                           (lane >> 3) * ldo + (lane & 7) * 2;
-            const int rows_left = p.m_rows - r0 - (lane >> 3), cols_left = p.n_cols - n0 - h * 64 - (lane & 7) * 2;
+            float2* outp = (MODE == 0 || pass == 0 ? p.out0 : p.out1) + tl.z * p.so + (long)(m0 + q * 32) * ldo + c0 +
+                           rrow * ldo + rpair * 2;
+            const int rows_left = p.m_rows - m0 - q * 32 - rrow, cols_left = p.n_cols - c0 - rpair * 2;
             const bool vec = (ldo & 1) == 0 && (reinterpret_cast<uintptr_t>(outp) & 15) == 0;
 #pragma unroll
             for (int cc = 0; cc < 4; ++cc) {
-              // row `lane` of the chunk to shared memory (rotated), then 128-byte row segments out
-#pragma unroll
-              for (int u = 0; u < 2; ++u) {
-                if (MODE == 1 && pass == 0) {
-                  uint32_t ro[16];
-                  if (have_occ) {
-                    tmem_ld16(tmem + lane_addr + (uint32_t)(bo * 256 + h * 128 + 32 * cc + 16 * u), ro);
-                    tmem_wait_ld();
-                  } else {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) ro[i] = 0u;
-                  }
-#pragma unroll
-                  for (int j = 0; j < 8; ++j)
-                    stg[lane * EPI_COLS + ((u * 8 + j + lane) & (EPI_COLS - 1))] =
-                        make_float2(__uint_as_float(ro[2 * j]) * ao, __uint_as_float(ro[2 * j + 1]) * ao);
+              uint32_t ro[16];
+              if (MODE == 1 && pass == 0) {
+                if (have_occ) {
+                  tmem_ld16(occ + 16 * cc, ro);
+                  tmem_wait_ld();
                 } else {
 #pragma unroll
-                  for (int j = 0; j < 8; ++j) {
-                    const int c = 32 * cc + 16 * u + 2 * j;
-                    stg[lane * EPI_COLS + ((u * 8 + j + lane) & (EPI_COLS - 1))] =
-                        MODE == 0 ? make_float2(tot[c], tot[c + 1]) : make_float2(tot[c] * au, tot[c + 1] * au);
-                  }
+                  for (int i = 0; i < 16; ++i) ro[i] = 0u;
                 }
               }
-              __syncwarp();
 #pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                if (4 * i >= rows_left || 16 * cc >= cols_left) continue;
-                const int rr = 4 * i + (lane >> 3), pc = (lane & 7) * 2;
-                const float2 v0 = stg[rr * EPI_COLS + ((pc + rr) & (EPI_COLS - 1))];
-                const float2 v1 = stg[rr * EPI_COLS + ((pc + 1 + rr) & (EPI_COLS - 1))];
-                float2* o = outp + (4 * i * ldo + 16 * cc);
-                if (vec && 16 * cc + 1 < cols_left) {
-                  *reinterpret_cast<float4*>(o) = make_float4(v0.x, v0.y, v1.x, v1.y);
+              for (int j = 0; j < 4; ++j) {
+                float4 v;
+                if (MODE == 1 && pass == 0)
+                  v = make_float4(__uint_as_float(ro[4 * j]) * ao, __uint_as_float(ro[4 * j + 1]) * ao,
+                                  __uint_as_float(ro[4 * j + 2]) * ao, __uint_as_float(ro[4 * j + 3]) * ao);
+                else {
+                  const int c = 16 * cc + 4 * j;
+                  const float f = MODE == 0 ? 1.f : au;
+                  v = make_float4(tot[c] * f, tot[c + 1] * f, tot[c + 2] * f, tot[c + 3] * f);
+                }
+                st_w[j ^ swz] = v;
+              }
+              __syncwarp();
+              float2* o = outp + 8 * cc;
+#pragma unroll
+              for (int i = 0; i < 4; ++i, o += 8 * ldo) {
+                if (8 * i >= rows_left || 8 * cc >= cols_left) continue;
+                const float4 v = st_r[8 * i * 4];
+                if (vec && 8 * cc + 1 < cols_left) {
+                  *reinterpret_cast<float4*>(o) = v;
                 } else {
-                  o[0] = v0;
-                  if (16 * cc + 1 < cols_left) o[1] = v1;
+                  o[0] = make_float2(v.x, v.y);
+                  if (8 * cc + 1 < cols_left) o[1] = make_float2(v.z, v.w);
                 }
               }
               __syncwarp();
@@ -1154,6 +1179,7 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
   // persistent: one CTA per SM walks the tiles, so that the TMA loads and MMAs of a tile start while the
   // last one's epilogue runs (modes 0 and 1) and no tile pays for a CTA's set-up
   const unsigned grid = (unsigned)std::min<long>((long)P.tiles * nb, ctx->num_sms);
+  const int threads = mode == 2 ? kThreads<2> : kThreads<0>;
   auto go = [&](auto kernel) -> gw_status {
     gw_status r = cuda_check(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES),
                              "cudaFuncSetAttribute");
@@ -1161,7 +1187,7 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
     const double work =
         tile_frac * (8.0 * n_rows * (double)g.nr * n_b + (mode == 2 ? 16.0 * n_rows * (double)g.nr * P.n_n : 0.0));
     KTimer kt(ctx, KF_GREEN_TC, work, st);
-    kernel<<<grid, THREADS, SMEM_BYTES, st>>>(mah, mal, mbh, mbl, mph, mpl, P);
+    kernel<<<grid, threads, SMEM_BYTES, st>>>(mah, mal, mbh, mbl, mph, mpl, P);
     return launch_check(ctx, "green_tc_kernel");
   };
   if (mode == 0) rc = fmt == 0 ? go(green_tc_kernel<0, 0>) : go(green_tc_kernel<0, 1>);
