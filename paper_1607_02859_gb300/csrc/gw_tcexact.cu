@@ -29,11 +29,21 @@
 //
 // Complex-to-real mapping as in the other tensor-core GEMMs: A is a real
 // [M][2K] operand with (re, im) interleaved along K, B holds two real rows per
-// complex column, (br, -bi) and (bi, br).  Tile 128 rows x 128 complex columns
-// (MMA 128 x 256 x 16), one slice of A and one of B per 32-wide K stage, six
+// complex column, (br, -bi) and (bi, br).  A pair of CTAs (cta_group::2) takes a
+// tile of 256 rows x 128 complex columns (MMA 256 x 256 x 16): each holds its 128
+// rows of A and half of B's rows, one slice of each per 64-wide K stage, six
 // stages in flight; two 256-column accumulators in tensor memory so that one
-// pass's epilogue overlaps the next pass's MMAs; the FP64 output tile (256 KB)
-// stays in L2 across a tile's passes.  Persistent CTAs, bounded waits.
+// pass's epilogue overlaps the next pass's MMAs; the FP64 output tile (256 KB a
+// CTA) stays in L2 across a tile's passes.  Persistent pairs, bounded waits.
+//
+// Every slice pair uses its stage once, so a single CTA asks 24 KB written to and
+// read from shared memory per 256 cycles of MMAs, 188 of its 128 bytes a cycle; in
+// the pair B's rows are read once for both tiles, 125 bytes a cycle.  And the TMA
+// loads want 128-byte rows (64 real K): with 64-byte rows the pair was no faster than
+// the single CTA.  8192^3, 15 pairs: single CTA 55.5 ms (79 TFLOP/s), pair with
+// 64-byte rows 54.5, pair with 128-byte rows 41.6 (106; 110 at 4096^3).  What is left
+// is operand traffic from L2 (14 TB/s) and the passes of a single pair, whose MMAs
+// take less time than the epilogue of the pass before.
 #include <algorithm>
 #include <climits>
 
@@ -45,26 +55,26 @@ namespace tx {
 
 using namespace tcx;
 
-constexpr int BM = 128, BNC = 128, BK = 32, STAGES = 6;
+constexpr int BM = 128, BNC = 128, BK = 64, STAGES = 6;   // rows of a CTA (a pair takes 2 BM)
 constexpr int BETA = 6;                          // bits per slice
 constexpr int KB_REAL = 1 << (24 - 2 * BETA);    // real K per exact block: 4096
 constexpr int KB_STEPS = KB_REAL / BK;
 constexpr int MAX_LEVELS = 7;
 constexpr int MAX_PAIRS = (MAX_LEVELS + 1) * (MAX_LEVELS + 2) / 2;
 constexpr int MAX_GROUPS = MAX_PAIRS;
-constexpr int A_BYTES = BM * BK * 2;             // 8 KB
-constexpr int B_BYTES = 2 * BNC * BK * 2;        // 16 KB
+constexpr int A_BYTES = BM * BK * 2;             // 16 KB, 128-byte swizzled rows
+constexpr int B_BYTES = BNC * BK * 2;            // 16 KB: half of the pair's 2 BNC rows
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int EPI_CPX = 16;                      // complex columns per epilogue round
 constexpr int EPI_WARPS = 8;                     // two per tensor-memory lane quarter, one per column half
 constexpr int EPI_BYTES = EPI_WARPS * 32 * EPI_CPX * 8;   // per epilogue warp: 32 rows x 16 complex (FP32)
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 256;
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
-constexpr int kGroupM = 8;                       // row tiles per group of the tile order
+constexpr int kGroupM = 4;                       // pairs' row tiles per group of the tile order
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
 
-// tile t of the persistent order -> (row tile, column tile): kGroupM row tiles are
-// walked down each column before moving on, so ~152 consecutive tiles span
+// tile t of the persistent order -> (pair's row tile, column tile): kGroupM row tiles
+// are walked down each column before moving on, so ~76 consecutive tiles span
 // kGroupM row tiles and ~19 column tiles of operands
 __device__ __forceinline__ void tile_of(long t, int tm, int tn, int& bm, int& bn) {
   const long per_group = (long)kGroupM * tn;
@@ -91,7 +101,7 @@ struct XParams {
   int k_steps;            // BK stages over the padded real K
   int n_kb;               // K blocks (KB_STEPS stages each, the last one shorter)
   int n_groups;           // groups of pairs summed in one accumulator
-  int tm, tn;
+  int tm, tn;             // pairs' row tiles (2 BM rows), column tiles
   int gstart[MAX_GROUPS + 1];          // pairs gstart[g] .. gstart[g+1]-1 form group g
   int glevel[MAX_GROUPS];              // a + b of the group's pairs
   int pa[MAX_PAIRS], pb[MAX_PAIRS];    // slice indices of each pair
@@ -102,7 +112,6 @@ struct XParams {
   int* status;
 };
 
-template <int DUMMY>
 __global__ void __launch_bounds__(THREADS, 1) cgemm_sliced_kernel(const __grid_constant__ CUtensorMap mA,
                                                                   const __grid_constant__ CUtensorMap mB, XParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -116,6 +125,8 @@ __global__ void __launch_bounds__(THREADS, 1) cgemm_sliced_kernel(const __grid_c
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+  const long pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const long ntiles = (long)p.tm * p.tn;
   const int passes = p.n_groups * p.n_kb;
 
@@ -126,19 +137,20 @@ __global__ void __launch_bounds__(THREADS, 1) cgemm_sliced_kernel(const __grid_c
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], EPI_WARPS);
+      mbar_init(&tempty[b], 2 * EPI_WARPS);      // the leader's: both CTAs' epilogues
     }
     mbar_init(done, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(512));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();                                  // both CTAs' barriers are initialised
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   auto timed_out = [&](int where) {
@@ -149,9 +161,9 @@ __global__ void __launch_bounds__(THREADS, 1) cgemm_sliced_kernel(const __grid_c
   auto k_last = [&](int kb) { return min((kb + 1) * KB_STEPS, p.k_steps); };
 
   if (warp == 0 && lane == 0) {
-    // ---------------------------------------------------------- TMA producer
+    // ---------------------------------------------------------- TMA producer (its CTA's operand rows)
     long kit = 0;
-    for (long t = blockIdx.x; t < ntiles && !*abort_flag; t += gridDim.x) {
+    for (long t = pair; t < ntiles && !*abort_flag; t += n_pairs) {
       int bm, bn;
       tile_of(t, p.tm, p.tn, bm, bn);
       for (int q = 0; q < passes && !*abort_flag; ++q) {
@@ -164,22 +176,34 @@ __global__ void __launch_bounds__(THREADS, 1) cgemm_sliced_kernel(const __grid_c
               break;
             }
             uint8_t* st = smem + s * STAGE_BYTES;
-            mbar_expect_tx(&full[s], STAGE_BYTES);
-            tma_load_3d(st, &mA, &full[s], ks * BK, bm * BM, p.pa[pr]);
-            tma_load_3d(st + A_BYTES, &mB, &full[s], ks * BK, 2 * bn * BNC, p.pb[pr]);
+            // the leader's barrier counts both CTAs' bytes; this CTA's empty barrier has told that the
+            // leader's has moved on
+            const uint32_t bar = peer_addr(&full[s], 0);
+            if (rank == 0) mbar_expect_tx(&full[s], 2 * STAGE_BYTES);
+            tma_load_3d_pair(st, &mA, bar, ks * BK, (2 * bm + (int)rank) * BM, p.pa[pr]);
+            tma_load_3d_pair(st + A_BYTES, &mB, bar, ks * BK, (2 * bn + (int)rank) * BNC, p.pb[pr]);
           }
       }
     }
-    if (*abort_flag)
-      for (long it = kit - STAGES < 0 ? 0 : kit - STAGES; it < kit; ++it)
-        mbar_wait(&full[it % STAGES], (uint32_t)((it / STAGES) & 1));
-  } else if (warp == 1 && lane == 0) {
-    // ---------------------------------------------------------- MMA issuer
-    constexpr uint32_t idesc = make_idesc(0u, 2 * BNC, BM);
+    // before this CTA ends: the last stages' MMAs have reported here (their copies have landed then);
+    // after a time-out, the copies of both CTAs as the leader's barriers count them
+    const long tail = kit - STAGES < 0 ? 0 : kit - STAGES;
+    if (!*abort_flag) {
+      for (long it = tail; it < kit; ++it)
+        if (!mbar_wait(&empty[it % STAGES], (uint32_t)((it / STAGES) & 1))) {
+          timed_out(36);
+          break;
+        }
+    } else if (rank == 0) {
+      for (long it = tail; it < kit; ++it) mbar_wait(&full[it % STAGES], (uint32_t)((it / STAGES) & 1));
+    }
+  } else if (warp == 1 && lane == 0 && rank == 0) {
+    // ---------------------------------------------------------- MMA issuer (the leader's, for both)
+    constexpr uint32_t idesc = make_idesc(0u, 2 * BNC, 2 * BM);
     long kit = 0;
     long pc = 0;                                   // passes issued by this CTA
     bool ok = true;
-    for (long t = blockIdx.x; t < ntiles && ok && !*abort_flag; t += gridDim.x) {
+    for (long t = pair; t < ntiles && ok && !*abort_flag; t += n_pairs) {
       for (int q = 0; q < passes && ok; ++q, ++pc) {
         const int g = q / p.n_kb, kb = q - g * p.n_kb;
         const int b = (int)(pc & 1);
@@ -201,20 +225,20 @@ __global__ void __launch_bounds__(THREADS, 1) cgemm_sliced_kernel(const __grid_c
             }
             tc_fence_after();
             uint8_t* st = smem + s * STAGE_BYTES;
-            const uint64_t ad = sw64_desc(st), bd = sw64_desc(st + A_BYTES);
+            const uint64_t ad = sw128_desc(st), bd = sw128_desc(st + A_BYTES);
             const bool fresh = pr == p.gstart[g] && ks == f;      // first stage of the group's sum
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {
               const uint64_t off = (uint64_t)(kk * 32) >> 4;
-              umma(d, ad + off, bd + off, idesc, (fresh && kk == 0) ? 0u : 1u);
+              umma_pair(d, ad + off, bd + off, idesc, (fresh && kk == 0) ? 0u : 1u);
             }
-            umma_commit(&empty[s]);
+            umma_commit_pair(&empty[s]);
           }
-        umma_commit(&tfull[b]);
+        umma_commit_pair(&tfull[b]);
       }
     }
-    umma_commit(done);
-    mbar_wait(done, 0);
+    umma_commit_own(done);
+    if (!mbar_wait(done, 0)) timed_out(35);
   } else if (warp >= 2) {
     // ---------------------------------------------------------- epilogue
     const int ew = warp - 2;
@@ -224,10 +248,10 @@ __global__ void __launch_bounds__(THREADS, 1) cgemm_sliced_kernel(const __grid_c
     float2* stg = epi + ew * 32 * EPI_CPX;
     long pc = 0;
     bool go = true;
-    for (long t = blockIdx.x; t < ntiles && go; t += gridDim.x) {
+    for (long t = pair; t < ntiles && go; t += n_pairs) {
       int bm, bn;
       tile_of(t, p.tm, p.tn, bm, bn);
-      const int r0 = bm * BM + qw * 32;
+      const int r0 = (2 * bm + (int)rank) * BM + qw * 32;
       const int n0 = bn * BNC;
       for (int q = 0; q < passes; ++q, ++pc) {
         const int g = q / p.n_kb;
@@ -289,16 +313,18 @@ __global__ void __launch_bounds__(THREADS, 1) cgemm_sliced_kernel(const __grid_c
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty[b]);
+        if (lane == 0) mbar_arrive_peer(peer_addr(&tempty[b], 0));
       }
     }
   }
+  // no CTA of the pair frees tensor memory or ends while MMAs or copies of the other may touch it
   tc_fence_before();
   __syncthreads();
+  cluster_sync();
   tc_fence_after();
   if (warp == 1) {
     __syncwarp();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
   }
 }
 
@@ -475,7 +501,7 @@ gw_status tc_zgemm_sliced(gw_ctx* ctx, int M, int N, int K, const double2* A, lo
   if (rc) return rc;
   CUtensorMap ma, mb;
   if ((rc = tc_make_map3(ctx, &ma, As, kp, M, S, BM, 0, BK))) return rc;
-  if ((rc = tc_make_map3(ctx, &mb, Bs, kp, 2L * N, S, 2 * BNC, 0, BK))) return rc;
+  if ((rc = tc_make_map3(ctx, &mb, Bs, kp, 2L * N, S, BNC, 0, BK))) return rc;
   XParams P;
   P.M = M;
   P.N = N;
@@ -503,7 +529,7 @@ gw_status tc_zgemm_sliced(gw_ctx* ctx, int M, int N, int K, const double2* A, lo
     }
   }
   P.gstart[P.n_groups] = n_pairs;
-  P.tm = (M + BM - 1) / BM;
+  P.tm = (M + 2 * BM - 1) / (2 * BM);
   P.tn = (N + BNC - 1) / BNC;
   P.rexp = rexp;
   P.cexp = cexp;
@@ -511,13 +537,25 @@ gw_status tc_zgemm_sliced(gw_ctx* ctx, int M, int N, int K, const double2* A, lo
   P.ldc = ldc;
   P.status = status;
   const long tiles = (long)P.tm * P.tn;
-  const dim3 grid((unsigned)std::max<long>(1, std::min<long>(tiles, ctx->num_sms)));
-  auto kernel = cgemm_sliced_kernel<0>;
+  auto kernel = cgemm_sliced_kernel;
   if ((rc = cuda_check(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES),
                        "cudaFuncSetAttribute")))
     return rc;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(2 * std::min<long>(tiles, std::max(1, ctx->num_sms / 2))));
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
   KTimer kt(ctx, KF_CGEMM_EXACT, 8.0 * M * (double)N * K, st);
-  kernel<<<grid, THREADS, SMEM_BYTES, st>>>(ma, mb, P);
+  if ((rc = cuda_check(ctx, cudaLaunchKernelEx(&cfg, kernel, ma, mb, P), "cudaLaunchKernelEx(cgemm_sliced_kernel)")))
+    return rc;
   return launch_check(ctx, "cgemm_sliced_kernel");
 }
 
