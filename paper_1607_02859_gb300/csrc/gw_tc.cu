@@ -17,8 +17,10 @@
 // the same code with a coarser 2 x 8-bit representation.
 //
 // Tile: 128 rows r x 128 complex columns R' (MMA 128 x 256 x 16), K staged 32
-// real elements (64 B, SWIZZLE_64B) at a time through a 4-stage TMA/mbarrier
-// pipeline; the epilogue stages rows in shared memory and writes 128-byte row
+// real elements at a time through a 4-stage TMA/mbarrier pipeline.  The 32 hi and
+// 32 lo values of a row lie side by side (128 B, SWIZZLE_128B), one load for A and
+// one for B: with hi and lo apart in 64-byte rows the loads lagged the MMAs (36^3, 4224
+// bands: 133 to 138 ms for 2 tau, now 130.5, 564 TFLOP/s); the epilogue stages rows in shared memory and writes 128-byte row
 // segments.  G_unocc is summed blockwise through the two 256-column halves of
 // tensor memory into registers, G_occ accumulates last in one half; the
 // epilogue either writes both (gw_green_tau) or their product
@@ -45,7 +47,7 @@ using namespace tcx;
 
 constexpr int BM = 128;                 // rows per tile
 constexpr int BNC = 128;                // complex columns per tile (MMA N = 256)
-constexpr int BK = 32;                  // real K per stage (one 64-byte swizzle row)
+constexpr int BK = 32;                  // real K per stage: its hi and lo values make one 128-byte operand row
 constexpr int STAGES = 4;
 constexpr int CH = 4;                   // stages per accumulation block (128 real K)
 // Epilogue warps: four per tensor-memory lane quarter (64 sums a thread, 96 registers) for the modes
@@ -56,9 +58,10 @@ constexpr int CH = 4;                   // stages per accumulation block (128 re
 // (466 TFLOP/s), at 24^3 with 1024 bands 13.1 and 11.9 ms.
 template <int MODE>
 constexpr int kEpiWarps = MODE == 2 ? 8 : 16;
-constexpr int A_BYTES = BM * BK * 2;            // 8 KB
-constexpr int B_BYTES = 2 * BNC * BK * 2;       // 16 KB
-constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
+constexpr int A_BYTES = BM * BK * 4;            // 16 KB
+constexpr int B_BYTES = 2 * BNC * BK * 4;       // 32 KB
+constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+constexpr int H_BYTES = BM * BK * 2;            // a 32-wide K chunk of H, hi or lo (64-byte rows)
 constexpr int EPI_COLS = 8;                     // complex columns per epilogue round
 constexpr int EPI_BYTES = 16 * 32 * EPI_COLS * 8;
 constexpr int kTileTab = 256;                   // tiles of a CTA looked up in advance
@@ -138,12 +141,11 @@ struct Params {
 // (32 bands) thousand cycles, now 38 and 50; sigma at 20^3 with 512 bands 14.9 ->
 // 10.4 ms, at 36^3 with 4224 bands and 2 tau 207 -> 170 ms.
 template <int MODE, uint32_t FMT>
-__global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __grid_constant__ CUtensorMap mA_hi,
-                                                              const __grid_constant__ CUtensorMap mA_lo,
-                                                              const __grid_constant__ CUtensorMap mB_hi,
-                                                              const __grid_constant__ CUtensorMap mB_lo,
-                                                              const __grid_constant__ CUtensorMap mP_hi,
-                                                              const __grid_constant__ CUtensorMap mP_lo, Params p) {
+__global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __grid_constant__ CUtensorMap mA,
+                                                                     const __grid_constant__ CUtensorMap mB,
+                                                                     const __grid_constant__ CUtensorMap mP_hi,
+                                                                     const __grid_constant__ CUtensorMap mP_lo,
+                                                                     Params p) {
   constexpr int EW = kEpiWarps<MODE>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -255,8 +257,8 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
   // MODE 2 operands in the freed pipeline stages: H hi [0, 64 KB), H lo [64, 128 KB) as eight
   // 32-wide K chunks of 128 rows; psi_n hi and lo from 128 KB, chunks of np rows.
   uint8_t* const h_hi = smem;
-  uint8_t* const h_lo = smem + 8 * A_BYTES;
-  uint8_t* const p_hi = smem + 16 * A_BYTES;
+  uint8_t* const h_lo = smem + 8 * H_BYTES;
+  uint8_t* const p_hi = smem + 16 * H_BYTES;
   const int p_chunk = MODE == 2 ? p.np * BK * 2 : 0;
   uint8_t* const p_lo = p_hi + 8 * p_chunk;
 
@@ -294,10 +296,8 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
         uint8_t* st = smem + s * STAGE_BYTES;
         const int x = it < p.k_un_steps ? p.k_un_x + it * BK : (it - p.k_un_steps) * BK;
         mbar_expect_tx(&full[s], STAGE_BYTES);
-        tma_load_3d(st, &mA_hi, &full[s], x, tl.m0, tl.z);
-        tma_load_3d(st + A_BYTES, &mA_lo, &full[s], x, tl.m0, tl.z);
-        tma_load_3d(st + 2 * A_BYTES, &mB_hi, &full[s], x, 2 * tl.n0, zb);
-        tma_load_3d(st + 2 * A_BYTES + B_BYTES, &mB_lo, &full[s], x, 2 * tl.n0, zb);
+        tma_load_3d(st, &mA, &full[s], 2 * x, tl.m0, tl.z);
+        tma_load_3d(st + A_BYTES, &mB, &full[s], 2 * x, 2 * tl.n0, zb);
       }
       if (*abort_flag) break;
       if constexpr (MODE == 2) {
@@ -352,8 +352,8 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
           }
           tc_fence_after();
           uint8_t* st = smem + s * STAGE_BYTES;
-          const uint64_t ah = sw64_desc(st), al = sw64_desc(st + A_BYTES);
-          const uint64_t bh = sw64_desc(st + 2 * A_BYTES), bl = sw64_desc(st + 2 * A_BYTES + B_BYTES);
+          const uint64_t ah = sw128_desc(st), al = ah + (64 >> 4);      // lo: 64 bytes along the row
+          const uint64_t bh = sw128_desc(st + A_BYTES), bl = bh + (64 >> 4);
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk) {
             const uint64_t off = (uint64_t)(kk * 32) >> 4;    // 16 elements = 32 bytes along K
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
             const uint32_t d = vbase + (uint32_t)((2 * o + h) * p.np);
 #pragma unroll 1
             for (int cc = 4 * h; cc < 4 * h + 4; ++cc) {
-              const uint64_t ah = sw64_desc(h_hi + cc * A_BYTES), al = sw64_desc(h_lo + cc * A_BYTES);
+              const uint64_t ah = sw64_desc(h_hi + cc * H_BYTES), al = sw64_desc(h_lo + cc * H_BYTES);
               const uint64_t bh = sw64_desc(p_hi + cc * p_chunk), bl = sw64_desc(p_lo + cc * p_chunk);
 #pragma unroll
               for (int kk = 0; kk < BK / 16; ++kk) {
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
           // hi for k < 4 and lo above, 16-byte segments swizzled as H's.  Row r lies where row r of H
           // will, so a thread only overwrites what it has read itself.
           auto piece = [&](int k) -> uint8_t* {
-            return (k < 4 ? h_hi : h_lo) + (4 * h + (k & 3)) * A_BYTES + q * 2048;
+            return (k < 4 ? h_hi : h_lo) + (4 * h + (k & 3)) * H_BYTES + q * 2048;
           };
           {
             const bool vec = (p.ldw % 2 == 0) && ((reinterpret_cast<uintptr_t>(p.wrr) & 15) == 0);
@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
             const float s1 = ldexpf(1.0f, sh >> 1), s2 = ldexpf(1.0f, sh - (sh >> 1));
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              const int base = (4 * h + j) * A_BYTES + (row >> 3) * 512 + (row & 7) * 64;
+              const int base = (4 * h + j) * H_BYTES + (row >> 3) * 512 + (row & 7) * 64;
 #pragma unroll
               for (int sg = 0; sg < 4; ++sg) {
                 uint32_t hw[4], lw[4];
@@ -842,14 +842,12 @@ template <bool IS_B, uint32_t FMT>
 __global__ void __launch_bounds__(256) prep_kernel(const float2* __restrict__ psi, int n_b, int n_occ, int nr, int r0,
                                                    int rows, const float* __restrict__ sk,
                                                    const int* __restrict__ dexp, int k_occ_pad, int k_un_x,
-                                                   int kpad, uint16_t* __restrict__ hi, uint16_t* __restrict__ lo,
-                                                   long sx, int e_shared) {
+                                                   int kpad, uint16_t* __restrict__ op, long sx, int e_shared) {
   __shared__ float2 t[32][33];
   const int z = blockIdx.z;
   psi += z * sx;
   sk += (long)z * n_b;
-  hi += (long)z * (IS_B ? 2 : 1) * rows * kpad;
-  lo += (long)z * (IS_B ? 2 : 1) * rows * kpad;
+  op += (long)z * (IS_B ? 2 : 1) * rows * 2 * kpad;
   const int kb = blockIdx.y * 32;       // band tile (covers padded band slots)
   const int rb = blockIdx.x * 32;       // row tile
   const float sc = ldexpf(1.0f, dexp[e_shared ? 0 : z]);
@@ -879,26 +877,24 @@ __global__ void __launch_bounds__(256) prep_kernel(const float2* __restrict__ ps
     const int slot = kb + threadIdx.x;
     const int col = slot < occ_slots ? 2 * slot : k_un_x + 2 * (slot - occ_slots);
     if (col >= kpad) continue;
+    const int at = col / BK * (2 * BK) + col % BK;      // hi of the stage's 32 values, lo 32 further
     const float2 v = t[threadIdx.x][i];
-    uint16_t h0, l0, h1, l1;
+    uint32_t h, l;
     if (!IS_B) {
-      split<FMT>(v.x, h0, l0);
-      split<FMT>(v.y, h1, l1);
-      const long o = (long)rr * kpad + col;
-      reinterpret_cast<uint32_t*>(hi + o)[0] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-      reinterpret_cast<uint32_t*>(lo + o)[0] = (uint32_t)l0 | ((uint32_t)l1 << 16);
+      split2<FMT>(v.x, v.y, h, l);
+      uint16_t* o = op + (long)rr * 2 * kpad + at;
+      *reinterpret_cast<uint32_t*>(o) = h;
+      *reinterpret_cast<uint32_t*>(o + BK) = l;
     } else {
       // b = conj(psi): br = v.x, bi = -v.y;  row 2R': (br, -bi) = (v.x, v.y); row 2R'+1: (bi, br) = (-v.y, v.x)
-      split<FMT>(v.x, h0, l0);
-      split<FMT>(v.y, h1, l1);
-      const long o0 = (long)(2 * rr) * kpad + col;
-      reinterpret_cast<uint32_t*>(hi + o0)[0] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-      reinterpret_cast<uint32_t*>(lo + o0)[0] = (uint32_t)l0 | ((uint32_t)l1 << 16);
-      uint16_t h2, l2;
-      split<FMT>(-v.y, h2, l2);
-      const long o1 = o0 + kpad;
-      reinterpret_cast<uint32_t*>(hi + o1)[0] = (uint32_t)h2 | ((uint32_t)h0 << 16);
-      reinterpret_cast<uint32_t*>(lo + o1)[0] = (uint32_t)l2 | ((uint32_t)l0 << 16);
+      split2<FMT>(v.x, v.y, h, l);
+      uint16_t* o = op + (long)(2 * rr) * 2 * kpad + at;
+      *reinterpret_cast<uint32_t*>(o) = h;
+      *reinterpret_cast<uint32_t*>(o + BK) = l;
+      split2<FMT>(-v.y, v.x, h, l);
+      o += 2 * kpad;
+      *reinterpret_cast<uint32_t*>(o) = h;
+      *reinterpret_cast<uint32_t*>(o + BK) = l;
     }
   }
 }
@@ -1022,15 +1018,13 @@ static size_t scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, b
   const size_t nbb = b_shared ? 1 : nb;
   Carver probe(nullptr);
   probe.take<unsigned int>(kWords);
-  probe.take<uint16_t>(nbb * 2 * g.nr * L.kpad);
-  probe.take<uint16_t>(nbb * 2 * g.nr * L.kpad);
+  probe.take<uint16_t>(nbb * 2 * g.nr * 2 * L.kpad);
   if (n_sig > 0) {
     probe.take<uint16_t>((size_t)sig_np(n_sig) * sig_kp(g));
     probe.take<uint16_t>((size_t)sig_np(n_sig) * sig_kp(g));
   }
   probe.take<float>((size_t)nb * n_b);
-  probe.take<uint16_t>((size_t)nb * n_rows * L.kpad);
-  probe.take<uint16_t>((size_t)nb * n_rows * L.kpad);
+  probe.take<uint16_t>((size_t)nb * n_rows * 2 * L.kpad);
   if (with_tmp) probe.take<float2>((size_t)n_rows * g.nr);
   return Carver::round(probe.off);
 }
@@ -1058,16 +1052,14 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
   int* dexp = reinterpret_cast<int*>(words + 64 + kMaxEntries);
   // time-out status: in the scratch, or in a word the caller owns (kept past later uses of the scratch)
   int* status = status_dev ? status_dev : reinterpret_cast<int*>(words + 2);
-  uint16_t* bhi = cv.take<uint16_t>(nbb * 2 * g.nr * L.kpad);
-  uint16_t* blo = cv.take<uint16_t>(nbb * 2 * g.nr * L.kpad);
+  uint16_t* bop = cv.take<uint16_t>(nbb * 2 * g.nr * 2 * L.kpad);
   // these operands are prepared by the first call and read by later ones: their place must not
   // depend on this call's number of rows or entries, so they come before what does
   const int np = mode == 2 ? sig_np(sig->n_n) : 0, kps = sig_kp(g);
   uint16_t* phi = mode == 2 ? cv.take<uint16_t>((size_t)np * kps) : nullptr;
   uint16_t* plo = mode == 2 ? cv.take<uint16_t>((size_t)np * kps) : nullptr;
   float* dsk = cv.take<float>((size_t)nb * n_b);
-  uint16_t* ahi = cv.take<uint16_t>((size_t)nb * n_rows * L.kpad);
-  uint16_t* alo = cv.take<uint16_t>((size_t)nb * n_rows * L.kpad);
+  uint16_t* aop = cv.take<uint16_t>((size_t)nb * n_rows * 2 * L.kpad);
   float2* tmp = need_tmp ? cv.take<float2>((size_t)n_rows * g.nr) : nullptr;
   if (mode == 1) {
     if (!out0) out0 = tmp;
@@ -1096,10 +1088,10 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
     const dim3 gbB((g.nr + 31) / 32, (slots + 31) / 32, nbb);
     if (fmt == 0)
       prep_kernel<true, 0><<<gbB, tb, 0, st>>>((const float2*)psi, n_b, n_occ, g.nr, 0, g.nr, sk, dexp,
-                                                L.k_occ_pad, L.k_un_x, L.kpad, bhi, blo, en.psi_stride, b_shared);
+                                                L.k_occ_pad, L.k_un_x, L.kpad, bop, en.psi_stride, b_shared);
     else
       prep_kernel<true, 1><<<gbB, tb, 0, st>>>((const float2*)psi, n_b, n_occ, g.nr, 0, g.nr, sk, dexp,
-                                                L.k_occ_pad, L.k_un_x, L.kpad, bhi, blo, en.psi_stride, b_shared);
+                                                L.k_occ_pad, L.k_un_x, L.kpad, bop, en.psi_stride, b_shared);
     if ((rc = launch_check(ctx, "prep_kernel(B)"))) return rc;
     if (mode == 2) {
       const dim3 gp((kps / 2 + 255) / 256, np / 2);
@@ -1113,22 +1105,20 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
   const dim3 gbA((n_rows + 31) / 32, (slots + 31) / 32, nb);
   if (fmt == 0)
     prep_kernel<false, 0><<<gbA, tb, 0, st>>>((const float2*)psi, n_b, n_occ, g.nr, r0, n_rows, sk, dexp,
-                                               L.k_occ_pad, L.k_un_x, L.kpad, ahi, alo, en.psi_stride, b_shared);
+                                               L.k_occ_pad, L.k_un_x, L.kpad, aop, en.psi_stride, b_shared);
   else
     prep_kernel<false, 1><<<gbA, tb, 0, st>>>((const float2*)psi, n_b, n_occ, g.nr, r0, n_rows, sk, dexp,
-                                               L.k_occ_pad, L.k_un_x, L.kpad, ahi, alo, en.psi_stride, b_shared);
+                                               L.k_occ_pad, L.k_un_x, L.kpad, aop, en.psi_stride, b_shared);
   if ((rc = launch_check(ctx, "prep_kernel(A)"))) return rc;
-  CUtensorMap mah, mal, mbh, mbl, mph, mpl;
-  if ((rc = tc_make_map3(ctx, &mah, ahi, L.kpad, n_rows, nb, BM, fmt, BK))) return rc;
-  if ((rc = tc_make_map3(ctx, &mal, alo, L.kpad, n_rows, nb, BM, fmt, BK))) return rc;
-  if ((rc = tc_make_map3(ctx, &mbh, bhi, L.kpad, 2L * g.nr, (int)nbb, 2 * BNC, fmt, BK))) return rc;
-  if ((rc = tc_make_map3(ctx, &mbl, blo, L.kpad, 2L * g.nr, (int)nbb, 2 * BNC, fmt, BK))) return rc;
+  CUtensorMap ma, mb, mph, mpl;
+  if ((rc = tc_make_map3(ctx, &ma, aop, 2 * L.kpad, n_rows, nb, BM, fmt, 2 * BK))) return rc;
+  if ((rc = tc_make_map3(ctx, &mb, bop, 2 * L.kpad, 2L * g.nr, (int)nbb, 2 * BNC, fmt, 2 * BK))) return rc;
   if (mode == 2) {
     if ((rc = tc_make_map3(ctx, &mph, phi, kps, np, 1, np, fmt, BK))) return rc;
     if ((rc = tc_make_map3(ctx, &mpl, plo, kps, np, 1, np, fmt, BK))) return rc;
   } else {
-    mph = mah;                                   // unused outside the self-energy mode
-    mpl = mal;
+    mph = ma;                                    // unused outside the self-energy mode
+    mpl = ma;
   }
   Params P;
   P.m_rows = n_rows;
@@ -1187,7 +1177,7 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
     const double work =
         tile_frac * (8.0 * n_rows * (double)g.nr * n_b + (mode == 2 ? 16.0 * n_rows * (double)g.nr * P.n_n : 0.0));
     KTimer kt(ctx, KF_GREEN_TC, work, st);
-    kernel<<<grid, threads, SMEM_BYTES, st>>>(mah, mal, mbh, mbl, mph, mpl, P);
+    kernel<<<grid, threads, SMEM_BYTES, st>>>(ma, mb, mph, mpl, P);
     return launch_check(ctx, "green_tc_kernel");
   };
   if (mode == 0) rc = fmt == 0 ? go(green_tc_kernel<0, 0>) : go(green_tc_kernel<0, 1>);

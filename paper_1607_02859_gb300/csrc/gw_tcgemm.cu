@@ -21,9 +21,9 @@ namespace tg {
 using namespace tcx;
 
 constexpr int BM = 128, BNC = 128, BK = 32, STAGES = 4;
-constexpr int A_BYTES = BM * BK * 2;            // 8 KB
-constexpr int B_BYTES = 2 * BNC * BK * 2;       // 16 KB
-constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
+constexpr int A_BYTES = BM * BK * 4;            // 16 KB: 32 hi and 32 lo values per 128-byte row
+constexpr int B_BYTES = 2 * BNC * BK * 4;       // 32 KB
+constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int EPI_COLS = 32;                     // complex columns per epilogue round
 constexpr int EPI_BYTES = 4 * 32 * EPI_COLS * 8; // per epilogue warp: 32 rows x 32 complex
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 256;
@@ -53,13 +53,12 @@ __device__ __forceinline__ int scale_exp(unsigned int bits) {
 // Persistent: CTA c takes tiles c, c + gridDim.x, ... (row tiles ascending, so
 // the longest tiles of a triangular product go first).  Two 256-column
 // accumulators in tensor memory let the epilogue of one tile run while the
-// MMAs of the next one issue.  Stages are 32 real K (64-byte swizzled rows),
-// four in flight.
+// MMAs of the next one issue.  Stages are 32 real K, hi and lo side by side in
+// 128-byte swizzled rows, four in flight (in separate 64-byte rows the products of
+// two 8192 screenings with refinement took 28.7 ms, so 25.1).
 template <uint32_t FMT, int TRI>
-__global__ void __launch_bounds__(THREADS, 1) cgemm_tc_kernel(const __grid_constant__ CUtensorMap mA_hi,
-                                                              const __grid_constant__ CUtensorMap mA_lo,
-                                                              const __grid_constant__ CUtensorMap mB_hi,
-                                                              const __grid_constant__ CUtensorMap mB_lo, KParams p) {
+__global__ void __launch_bounds__(THREADS, 1) cgemm_tc_kernel(const __grid_constant__ CUtensorMap mA,
+                                                              const __grid_constant__ CUtensorMap mB, KParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   float2* epi = reinterpret_cast<float2*>(smem + STAGES * STAGE_BYTES);     // [4 warps][32 rows][32]
@@ -125,10 +124,8 @@ __global__ void __launch_bounds__(THREADS, 1) cgemm_tc_kernel(const __grid_const
         uint8_t* st = smem + s * STAGE_BYTES;
         const int x = ks * BK;
         mbar_expect_tx(&full[s], STAGE_BYTES);
-        tma_load_3d(st, &mA_hi, &full[s], x, bm * BM, bz);
-        tma_load_3d(st + A_BYTES, &mA_lo, &full[s], x, bm * BM, bz);
-        tma_load_3d(st + 2 * A_BYTES, &mB_hi, &full[s], x, 2 * bn * BNC, bz);
-        tma_load_3d(st + 2 * A_BYTES + B_BYTES, &mB_lo, &full[s], x, 2 * bn * BNC, bz);
+        tma_load_3d(st, &mA, &full[s], 2 * x, bm * BM, bz);
+        tma_load_3d(st + A_BYTES, &mB, &full[s], 2 * x, 2 * bn * BNC, bz);
       }
     }
     if (*abort_flag)
@@ -158,8 +155,8 @@ __global__ void __launch_bounds__(THREADS, 1) cgemm_tc_kernel(const __grid_const
         }
         tc_fence_after();
         uint8_t* st = smem + s * STAGE_BYTES;
-        const uint64_t ah = sw64_desc(st), al = sw64_desc(st + A_BYTES);
-        const uint64_t bh = sw64_desc(st + 2 * A_BYTES), bl = sw64_desc(st + 2 * A_BYTES + B_BYTES);
+        const uint64_t ah = sw128_desc(st), al = ah + (64 >> 4);        // lo: 64 bytes along the row
+        const uint64_t bh = sw128_desc(st + A_BYTES), bl = bh + (64 >> 4);
 #pragma unroll
         for (int kk = 0; kk < BK / 16; ++kk) {
           const uint64_t off = (uint64_t)(kk * 32) >> 4;    // 16 elements = 32 bytes along K
@@ -314,13 +311,11 @@ template <bool IS_B, uint32_t FMT>
 __global__ void __launch_bounds__(256) prep_op_kernel(const float2* __restrict__ X, long ld, long sx, int trans,
                                                       int conj, int rows, int K, int kp,
                                                       const unsigned int* __restrict__ maxbits,
-                                                      uint16_t* __restrict__ hi, uint16_t* __restrict__ lo) {
+                                                      uint16_t* __restrict__ op) {
   __shared__ float2 t[32][33];                  // t[i][k]
   const int i0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
   X += blockIdx.z * sx;
-  const long ob = (long)blockIdx.z * (IS_B ? 2 : 1) * rows * kp;
-  hi += ob;
-  lo += ob;
+  op += (long)blockIdx.z * (IS_B ? 2 : 1) * rows * 2 * kp;
   const float sc = ldexpf(1.0f, scale_exp(maxbits[blockIdx.z]));
   for (int y = threadIdx.y; y < 32; y += blockDim.y) {
     // trans: X[k][i] is contiguous in i -> thread x walks i; else walks k
@@ -341,22 +336,23 @@ __global__ void __launch_bounds__(256) prep_op_kernel(const float2* __restrict__
     const int i = i0 + y, k = k0 + threadIdx.x;
     if (i >= rows || 2 * k >= kp) continue;
     const float2 v = t[y][threadIdx.x];
-    uint16_t h0, l0, h1, l1;
-    split<FMT>(v.x, h0, l0);
-    split<FMT>(v.y, h1, l1);
+    const int at = 2 * k / BK * (2 * BK) + 2 * k % BK;      // hi of the stage's 32 values, lo 32 further
+    uint32_t h, l;
     if (!IS_B) {
-      const long o = (long)i * kp + 2 * k;
-      reinterpret_cast<uint32_t*>(hi + o)[0] = (uint32_t)h0 | ((uint32_t)h1 << 16);
-      reinterpret_cast<uint32_t*>(lo + o)[0] = (uint32_t)l0 | ((uint32_t)l1 << 16);
+      split2<FMT>(v.x, v.y, h, l);
+      uint16_t* o = op + (long)i * 2 * kp + at;
+      *reinterpret_cast<uint32_t*>(o) = h;
+      *reinterpret_cast<uint32_t*>(o + BK) = l;
     } else {
       // rows 2i: (br, -bi); 2i+1: (bi, br)
-      uint16_t h2, l2;
-      split<FMT>(-v.y, h2, l2);
-      const long o0 = (long)(2 * i) * kp + 2 * k, o1 = o0 + kp;
-      reinterpret_cast<uint32_t*>(hi + o0)[0] = (uint32_t)h0 | ((uint32_t)h2 << 16);
-      reinterpret_cast<uint32_t*>(lo + o0)[0] = (uint32_t)l0 | ((uint32_t)l2 << 16);
-      reinterpret_cast<uint32_t*>(hi + o1)[0] = (uint32_t)h1 | ((uint32_t)h0 << 16);
-      reinterpret_cast<uint32_t*>(lo + o1)[0] = (uint32_t)l1 | ((uint32_t)l0 << 16);
+      split2<FMT>(v.x, -v.y, h, l);
+      uint16_t* o = op + (long)(2 * i) * 2 * kp + at;
+      *reinterpret_cast<uint32_t*>(o) = h;
+      *reinterpret_cast<uint32_t*>(o + BK) = l;
+      split2<FMT>(v.y, v.x, h, l);
+      o += 2 * kp;
+      *reinterpret_cast<uint32_t*>(o) = h;
+      *reinterpret_cast<uint32_t*>(o + BK) = l;
     }
   }
 }
@@ -367,10 +363,8 @@ size_t tc_gemm_scratch(int M, int N, int K, int batch) {
   const size_t kp = (size_t)(2 * std::max(K, 1) + tg::BK - 1) / tg::BK * tg::BK;
   Carver probe(nullptr);
   probe.take<unsigned int>(256);
-  probe.take<uint16_t>((size_t)batch * M * kp);
-  probe.take<uint16_t>((size_t)batch * M * kp);
-  probe.take<uint16_t>((size_t)batch * 2 * N * kp);
-  probe.take<uint16_t>((size_t)batch * 2 * N * kp);
+  probe.take<uint16_t>((size_t)batch * M * 2 * kp);
+  probe.take<uint16_t>((size_t)batch * 2 * N * 2 * kp);
   return Carver::round(probe.off);
 }
 
@@ -384,10 +378,8 @@ gw_status tc_gemm(gw_ctx* ctx, gw_prec prec, const TcGemm& g, void* scratch, cud
   const int kp = (2 * K + BK - 1) / BK * BK;
   Carver cv(scratch);
   unsigned int* words = cv.take<unsigned int>(256);    // [b] max A, [batch + b] max B
-  uint16_t* ahi = cv.take<uint16_t>((size_t)batch * g.M * kp);
-  uint16_t* alo = cv.take<uint16_t>((size_t)batch * g.M * kp);
-  uint16_t* bhi = cv.take<uint16_t>((size_t)batch * 2 * g.N * kp);
-  uint16_t* blo = cv.take<uint16_t>((size_t)batch * 2 * g.N * kp);
+  uint16_t* aop = cv.take<uint16_t>((size_t)batch * g.M * 2 * kp);
+  uint16_t* bop = cv.take<uint16_t>((size_t)batch * 2 * g.N * 2 * kp);
   gw_status rc;
   if ((rc = cuda_check(ctx, cudaMemsetAsync(words, 0, 2 * batch * sizeof(unsigned int), st), "memset"))) return rc;
   // A is [M][K] (or [K][M] if transposed); B's op is [K][N]: stored [K][N], or [N][K] if transposed
@@ -411,21 +403,17 @@ gw_status tc_gemm(gw_ctx* ctx, gw_prec prec, const TcGemm& g, void* scratch, cud
   // B operand rows are indexed by n with k along the row: element (n, k) = opB(k, n), i.e.
   // B[k][n] (stored [K][N]: read transposed) or B[n][k] (b_trans: read as is).
   if (fmt == 0) {
-    prep_op_kernel<false, 0><<<ga, tb, 0, st>>>(g.A, g.lda, g.sA, g.a_trans, g.a_conj, g.M, g.K, kp, words, ahi, alo);
-    prep_op_kernel<true, 0><<<gb, tb, 0, st>>>(g.B, g.ldb, g.sB, !g.b_trans, g.b_conj, g.N, g.K, kp, words + batch,
-                                                bhi, blo);
+    prep_op_kernel<false, 0><<<ga, tb, 0, st>>>(g.A, g.lda, g.sA, g.a_trans, g.a_conj, g.M, g.K, kp, words, aop);
+    prep_op_kernel<true, 0><<<gb, tb, 0, st>>>(g.B, g.ldb, g.sB, !g.b_trans, g.b_conj, g.N, g.K, kp, words + batch, bop);
   } else {
-    prep_op_kernel<false, 1><<<ga, tb, 0, st>>>(g.A, g.lda, g.sA, g.a_trans, g.a_conj, g.M, g.K, kp, words, ahi, alo);
-    prep_op_kernel<true, 1><<<gb, tb, 0, st>>>(g.B, g.ldb, g.sB, !g.b_trans, g.b_conj, g.N, g.K, kp, words + batch,
-                                                bhi, blo);
+    prep_op_kernel<false, 1><<<ga, tb, 0, st>>>(g.A, g.lda, g.sA, g.a_trans, g.a_conj, g.M, g.K, kp, words, aop);
+    prep_op_kernel<true, 1><<<gb, tb, 0, st>>>(g.B, g.ldb, g.sB, !g.b_trans, g.b_conj, g.N, g.K, kp, words + batch, bop);
   }
   if ((rc = launch_check(ctx, "prep_op_kernel"))) return rc;
   ctx->launches++;
-  CUtensorMap mah, mal, mbh, mbl;
-  if ((rc = tc_make_map3(ctx, &mah, ahi, kp, g.M, batch, BM, fmt, BK))) return rc;
-  if ((rc = tc_make_map3(ctx, &mal, alo, kp, g.M, batch, BM, fmt, BK))) return rc;
-  if ((rc = tc_make_map3(ctx, &mbh, bhi, kp, 2L * g.N, batch, 2 * BNC, fmt, BK))) return rc;
-  if ((rc = tc_make_map3(ctx, &mbl, blo, kp, 2L * g.N, batch, 2 * BNC, fmt, BK))) return rc;
+  CUtensorMap ma, mb;
+  if ((rc = tc_make_map3(ctx, &ma, aop, 2 * kp, g.M, batch, BM, fmt, 2 * BK))) return rc;
+  if ((rc = tc_make_map3(ctx, &mb, bop, 2 * kp, 2L * g.N, batch, 2 * BNC, fmt, 2 * BK))) return rc;
   KParams P;
   P.M = g.M;
   P.N = g.N;
@@ -449,7 +437,7 @@ gw_status tc_gemm(gw_ctx* ctx, gw_prec prec, const TcGemm& g, void* scratch, cud
                              "cudaFuncSetAttribute");
     if (r) return r;
     KTimer kt(ctx, KF_CGEMM_TC, batch * gemm_flops(g.M, g.N, g.K, g.tri), st);
-    kernel<<<grid, THREADS, SMEM_BYTES, st>>>(mah, mal, mbh, mbl, P);
+    kernel<<<grid, THREADS, SMEM_BYTES, st>>>(ma, mb, P);
     return launch_check(ctx, "cgemm_tc_kernel");
   };
   if (fmt == 0) rc = g.tri == 0 ? go(cgemm_tc_kernel<0, 0>) : g.tri == 1 ? go(cgemm_tc_kernel<0, 1>) : go(cgemm_tc_kernel<0, 2>);
