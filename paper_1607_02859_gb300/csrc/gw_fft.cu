@@ -84,25 +84,23 @@ struct RowCfg {
   static constexpr int MINB = F32 ? (NR >= 13824 ? 2 : (NR >= 4096 ? 3 : 4)) : 1;
 };
 
-// MODE 0: x = scale * a * conj(b) (Eq. chi_rr), forward (+i), gather the G' set.
-// MODE 1: x = a, forward (+i), gather.            (Eq. FFTX1)
+// MODE 1: x = a, forward (+i), gather the G' set.  (Eq. FFTX1)
 // MODE 2: scatter a[j] to fft positions, backward (-i), times scale.   (Eq. FFTW, 2nd step)
-// VI / VO: the grid side / the G-set side (modes 0, 1) moves as 16-byte pairs of
+// VI / VO: the grid side / the G-set side (mode 1) moves as 16-byte pairs of
 // elements (aligned rows of even length), four pairs in flight per thread.
 //
 // The three passes over the row do only what the G set (lists) and the triangle
 // (low) need: forward the planes i1 <= i1(r), of them the i3 of the set in the i2
 // pass, and the set's (i2, i3) columns in the i1 pass; backward the set's (i1, i2)
 // pencils, then its i1 planes, and of the i1 pass the planes up to the last one
-// read.  A MODE 0 row of the triangle takes half of its diagonal element.
+// read.
 // That is 0.44 of a whole row's pencils at 24^3 with n_chi = 4097; the rows of one
 // tau went from 790 to 560 us there (scalar loads for the odd n_chi before), from
 // 250 to 172 us at 20^3 with n_chi = 1536.  Bound by instruction issue.
 template <typename T, int N1, int N2, int N3, int MODE, bool VI, bool VO>
 __global__ void __launch_bounds__(RowCfg<T, N1, N2, N3>::TH, RowCfg<T, N1, N2, N3>::MINB)
-    row_fft_kernel(const typename cpx<T>::t* __restrict__ a, const typename cpx<T>::t* __restrict__ b, long lda,
-                   typename cpx<T>::t* __restrict__ out, long ldo, const int* __restrict__ map,
-                   const int* __restrict__ inv, int n_chi, T scale, int low) {
+    row_fft_kernel(const typename cpx<T>::t* __restrict__ a, long lda, typename cpx<T>::t* __restrict__ out, long ldo,
+                   const int* __restrict__ map, const int* __restrict__ inv, int n_chi, T scale, int low) {
   using C = typename cpx<T>::t;
   using L = RowLayout<N1, N2, N3>;
   constexpr int THREADS = RowCfg<T, N1, N2, N3>::TH;
@@ -176,45 +174,28 @@ __global__ void __launch_bounds__(RowCfg<T, N1, N2, N3>::TH, RowCfg<T, N1, N2, N
   }
   const int last = low_last_fwd(low, row, L::NR);
   const int i1m = last / PL + 1;                                 // planes with an element R' <= r
-  const int half = MODE == 0 && low >= 0 ? last : -1;
   const C* pa = a + row * lda;
-  const C* pb = b + row * lda;
-  auto value = [&](C v, C w, int r) -> C {
-    if (r > last) return mk(T(0), T(0));
-    if (MODE != 0) return v;
-    return cscale(cmulc(v, w), r == half ? scale * T(0.5) : scale);
-  };
   if (VI) {
     const int np = i1m * PL / 2;
     for (int q0 = threadIdx.x; q0 < np; q0 += 4 * THREADS) {
-      C v[4][2], w[4][2];
+      C v[4][2];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int q = q0 + u * THREADS;
-        v[u][0] = v[u][1] = w[u][0] = w[u][1] = mk(T(0), T(0));
-        if (q < np && 2 * q <= last) {
-          ld_pair(pa + 2 * q, v[u][0], v[u][1]);
-          if (MODE == 0) ld_pair(pb + 2 * q, w[u][0], w[u][1]);
-        }
+        v[u][0] = v[u][1] = mk(T(0), T(0));
+        if (q < np && 2 * q <= last) ld_pair(pa + 2 * q, v[u][0], v[u][1]);
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int q = q0 + u * THREADS;
         if (q >= np) continue;
         const int p = L::pos(2 * q);           // 2q and 2q+1 share an i3 pencil (N3 even)
-        s[p] = value(v[u][0], w[u][0], 2 * q);
-        s[p + 1] = value(v[u][1], w[u][1], 2 * q + 1);
+        s[p] = v[u][0];
+        s[p + 1] = 2 * q + 1 <= last ? v[u][1] : mk(T(0), T(0));
       }
     }
   } else {
-    for (int r = threadIdx.x; r < i1m * PL; r += THREADS) {
-      C v = mk(T(0), T(0)), w = v;
-      if (r <= last) {
-        v = pa[r];
-        if (MODE == 0) w = pb[r];
-      }
-      s[L::pos(r)] = value(v, w, r);
-    }
+    for (int r = threadIdx.x; r < i1m * PL; r += THREADS) s[L::pos(r)] = r <= last ? pa[r] : mk(T(0), T(0));
   }
   __syncthreads();
   for (int e = threadIdx.x; e < i1m * N2; e += THREADS) {
@@ -288,13 +269,12 @@ struct PlaneCfg {
   static constexpr size_t kStage = 110 * 1024;
 };
 
-// MODE 0 / 1 as for row_fft_kernel: planes of x = scale a conj(b) or a, (+i) over
-// i3 and the set's i3 of i2, the set's columns to t.  MODE 2: the columns from t,
+// MODE 1 as for row_fft_kernel: planes of a, (+i) over i3 and the set's i3 of i2,
+// the set's columns to t.  MODE 2: the columns from t,
 // (-i) over the set's i2 of i3 and i2, times scale, to the planes of out.
 template <typename T, int N1, int N2, int N3, int MODE, bool VEC>
 __global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::TH, PlaneCfg<T, N1, N2, N3>::MINB)
-    row_plane_kernel(const typename cpx<T>::t* a, const typename cpx<T>::t* b, long lda, typename cpx<T>::t* t,
-                     long t_row, long t_plane, typename cpx<T>::t* out, long ldo, const int* __restrict__ inv, T scale,
+    row_plane_kernel(const typename cpx<T>::t* a, long lda, typename cpx<T>::t* t, long t_row, long t_plane, typename cpx<T>::t* out, long ldo, const int* __restrict__ inv, T scale,
                      int low) {
   using C = typename cpx<T>::t;
   using R = PlaneCfg<T, N1, N2, N3>;
@@ -348,45 +328,28 @@ __global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::TH, PlaneCfg<T, N1, N
     return;
   }
   const int last0 = last - p0 * PL;                                // the last element in use, from the CTA's first
-  const int half = MODE == 0 && low >= 0 ? last0 : -1;
   const C* pa = a + row * lda + (long)p0 * PL;
-  const C* pb = b + row * lda + (long)p0 * PL;
-  auto value = [&](C v, C w, int e) -> C {
-    if (e > last0) return mk(T(0), T(0));
-    if (MODE != 0) return v;
-    return cscale(cmulc(v, w), e == half ? scale * T(0.5) : scale);
-  };
   if (VEC) {
-    constexpr int LB = MODE == 0 ? 4 : 8;                          // 16-byte loads in flight per thread
+    constexpr int LB = 8;                                          // 16-byte loads in flight per thread
     for (int q0 = threadIdx.x; q0 < np * PL / 2; q0 += LB * TH) {
-      C v[LB][2], w[LB][2];
+      C v[LB][2];
 #pragma unroll
       for (int u = 0; u < LB; ++u) {
         const int q = q0 + u * TH;
-        v[u][0] = v[u][1] = w[u][0] = w[u][1] = mk(T(0), T(0));
-        if (q < np * PL / 2 && 2 * q <= last0) {
-          ld_pair_rw(pa + 2 * q, v[u][0], v[u][1]);
-          if (MODE == 0) ld_pair_rw(pb + 2 * q, w[u][0], w[u][1]);
-        }
+        v[u][0] = v[u][1] = mk(T(0), T(0));
+        if (q < np * PL / 2 && 2 * q <= last0) ld_pair_rw(pa + 2 * q, v[u][0], v[u][1]);
       }
 #pragma unroll
       for (int u = 0; u < LB; ++u) {
         const int q = q0 + u * TH;
         if (q >= np * PL / 2) continue;
         const int o = pos(2 * q);
-        s[o] = value(v[u][0], w[u][0], 2 * q);
-        s[o + 1] = value(v[u][1], w[u][1], 2 * q + 1);
+        s[o] = v[u][0];
+        s[o + 1] = 2 * q + 1 <= last0 ? v[u][1] : mk(T(0), T(0));
       }
     }
   } else {
-    for (int e = threadIdx.x; e < np * PL; e += TH) {
-      C v = mk(T(0), T(0)), w = v;
-      if (e <= last0) {
-        v = pa[e];
-        if (MODE == 0) w = pb[e];
-      }
-      s[pos(e)] = value(v, w, e);
-    }
+    for (int e = threadIdx.x; e < np * PL; e += TH) s[pos(e)] = e <= last0 ? pa[e] : mk(T(0), T(0));
   }
   __syncthreads();
   pencil_pass<N3, +1>(s, np * N2, 1, [](int q) { return q * S2; });
@@ -1195,7 +1158,7 @@ struct GridOps {
     const int last = bwd ? (g0 + 127) / 128 * 128 + 127 : low + n_rows - 1;
     return std::min(N1, last / PC::PL + 1);
   }
-  static gw_status row_two_pass(gw_ctx* ctx, int mode, const void* a, const void* b, long lda, void* out, long ldo,
+  static gw_status row_two_pass(gw_ctx* ctx, int mode, const void* a, long lda, void* out, long ldo,
                                 const int* inv, void* tmp, int n_chi, int n_rows, double scale, cudaStream_t st,
                                 bool vec, int low, double work) {
     constexpr int NR = N1 * N2 * N3;
@@ -1208,7 +1171,7 @@ struct GridOps {
       gw_status r = set_smem(ctx, kernel, PC::bytes);
       if (r) return r;
       KTimer kt(ctx, KF_ROW_FFT, work, st);
-      kernel<<<pgrid, PC::TH, PC::bytes, st>>>((const C*)a, (const C*)b, lda, (C*)t, t_row, (long)PC::PL, (C*)out, ldo,
+      kernel<<<pgrid, PC::TH, PC::bytes, st>>>((const C*)a, lda, (C*)t, t_row, (long)PC::PL, (C*)out, ldo,
                                                inv, (T)scale, low);
       return launch_check(ctx, "row_plane_kernel");
     };
@@ -1220,54 +1183,43 @@ struct GridOps {
       return vec ? plane(row_plane_kernel<T, N1, N2, N3, 2, E>, out, ldo)
                  : plane(row_plane_kernel<T, N1, N2, N3, 2, false>, out, ldo);
     }
-    if (mode == 0)
-      rc = vec ? plane(row_plane_kernel<T, N1, N2, N3, 0, E>, tmp, NR)
-               : plane(row_plane_kernel<T, N1, N2, N3, 0, false>, tmp, NR);
-    else
-      rc = vec ? plane(row_plane_kernel<T, N1, N2, N3, 1, E>, tmp, NR)
-               : plane(row_plane_kernel<T, N1, N2, N3, 1, false>, tmp, NR);
+    rc = vec ? plane(row_plane_kernel<T, N1, N2, N3, 1, E>, tmp, NR)
+             : plane(row_plane_kernel<T, N1, N2, N3, 1, false>, tmp, NR);
     if (rc) return rc;
     return line_fwd(ctx, tmp, NR, PC::PL, out, ldo, inv, n_chi, n_rows, low, 0.0, KF_ROW_FFT, st);
   }
-  static gw_status row(gw_ctx* ctx, int mode, const void* a, const void* b, long lda, void* out, long ldo,
+  static gw_status row(gw_ctx* ctx, int mode, const void* a, long lda, void* out, long ldo,
                        const int* map, int n_chi, int n_rows, double scale, cudaStream_t st, const int* inv,
                        void* tmp, int low) {
     using L = RowLayout<N1, N2, N3>;
     const size_t bytes = L::TOT * sizeof(C);
-    const double rd = mode == 0 ? 2.0 * L::NR : (mode == 1 ? L::NR : n_chi);
-    const double wr = mode == 2 ? L::NR : n_chi;
     // HBM bytes of the launch: whole rows, or the triangle's share of the grid side
     double grid_el = (double)n_rows * L::NR;
     if (low >= 0) {
       grid_el = 0;
       for (int r = 0; r < n_rows; ++r) grid_el += std::min(L::NR, low + r + 1);
     }
-    const double work = (grid_el * (mode == 0 ? 2.0 : 1.0) + (double)n_rows * n_chi) * sizeof(C);
+    const double work = (grid_el + (double)n_rows * n_chi) * sizeof(C);
     auto al = [](const void* p) { return p == nullptr || reinterpret_cast<uintptr_t>(p) % 16 == 0; };
-    // 16-byte pairs on the grid side (rows of a and b, or of out for mode 2) and on the G-set side
-    const bool vi = mode == 2 ? al(out) && ldo % 2 == 0 && N3 % 2 == 0 : al(a) && al(b) && lda % 2 == 0 && N3 % 2 == 0;
+    // 16-byte pairs on the grid side (rows of a, or of out for mode 2) and on the G-set side
+    const bool vi = mode == 2 ? al(out) && ldo % 2 == 0 && N3 % 2 == 0 : al(a) && lda % 2 == 0 && N3 % 2 == 0;
     const bool vo = mode != 2 && al(out) && ldo % 2 == 0 && n_chi % 2 == 0;
     if (!inv) return fail(ctx, GW_ERR_ARG, "row transform without the G set's inverse map");
     if constexpr (L::TOT * sizeof(C) > kRowSmemMax)
-      return row_two_pass(ctx, mode, a, b, lda, out, ldo, inv, tmp, n_chi, n_rows, scale, st, vi, low, work);
+      return row_two_pass(ctx, mode, a, lda, out, ldo, inv, tmp, n_chi, n_rows, scale, st, vi, low, work);
     if constexpr (L::TOT * sizeof(C) <= kRowSmemMax) {
       auto go = [&](auto kernel) -> gw_status {
         gw_status s = set_smem(ctx, kernel, bytes);
         if (s) return s;
         KTimer kt(ctx, KF_ROW_FFT, work, st);
-        kernel<<<n_rows, RowCfg<T, N1, N2, N3>::TH, bytes, st>>>((const C*)a, (const C*)b, lda, (C*)out, ldo, map, inv,
+        kernel<<<n_rows, RowCfg<T, N1, N2, N3>::TH, bytes, st>>>((const C*)a, lda, (C*)out, ldo, map, inv,
                                                                  n_chi, (T)scale, low);
         return launch_check(ctx, "row_fft_kernel");
       };
       constexpr bool E = N3 % 2 == 0;
-#define GW_ROW_GO(M)                                                        \
-      if (mode == M)                                                        \
-        return vi ? (vo ? go(row_fft_kernel<T, N1, N2, N3, M, E, true>)     \
-                        : go(row_fft_kernel<T, N1, N2, N3, M, E, false>))   \
-                  : go(row_fft_kernel<T, N1, N2, N3, M, false, false>);
-      GW_ROW_GO(0)
-      GW_ROW_GO(1)
-#undef GW_ROW_GO
+      if (mode == 1)
+        return vi ? (vo ? go(row_fft_kernel<T, N1, N2, N3, 1, E, true>) : go(row_fft_kernel<T, N1, N2, N3, 1, E, false>))
+                  : go(row_fft_kernel<T, N1, N2, N3, 1, false, false>);
       if (mode == 2) return vi ? go(row_fft_kernel<T, N1, N2, N3, 2, E, false>)
                                : go(row_fft_kernel<T, N1, N2, N3, 2, false, false>);
     }
@@ -1444,11 +1396,11 @@ static bool with_grid(const GridInfo& g, F&& f) {
   if (!found) return fail(ctx, GW_ERR_UNSUPPORTED, "no FFT kernels compiled for this grid");     \
   return rc;
 
-gw_status launch_row_fft(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int mode, const void* a, const void* b,
-                         long lda, void* out, long ldo, const int* map, int n_chi, int n_rows, double scale,
+gw_status launch_row_fft(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int mode, const void* a, long lda, void* out,
+                         long ldo, const int* map, int n_chi, int n_rows, double scale,
                          cudaStream_t st, const int* inv, void* tmp, int low) {
   if (n_rows <= 0) return GW_OK;
-  GW_DISPATCH(prec, g, rc = O::row(ctx, mode, a, b, lda, out, ldo, map, n_chi, n_rows, scale, st, inv, tmp, low))
+  GW_DISPATCH(prec, g, rc = O::row(ctx, mode, a, lda, out, ldo, map, n_chi, n_rows, scale, st, inv, tmp, low))
 }
 
 gw_status launch_row_pw_chi(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* a, const void* b, long lda,
@@ -1655,8 +1607,8 @@ extern "C" gw_status gw_rr_to_GG_fft(gw_ctx* ctx, const gw_grid* grid, int direc
   if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if (stage == 1) {
     if (direction > 0)
-      return launch_row_fft(ctx, g, prec, 1, in, nullptr, g.nr, out, n_chi, dmap, n_chi, n_rows, 1.0, s, dinv, tmp);
-    return launch_row_fft(ctx, g, prec, 2, in, nullptr, n_chi, out, g.nr, dmap, n_chi, n_rows, 1.0 / g.volume, s,
+      return launch_row_fft(ctx, g, prec, 1, in, g.nr, out, n_chi, dmap, n_chi, n_rows, 1.0, s, dinv, tmp);
+    return launch_row_fft(ctx, g, prec, 2, in, n_chi, out, g.nr, dmap, n_chi, n_rows, 1.0 / g.volume, s,
                           dinv);
   }
   if (direction > 0) {
@@ -1786,8 +1738,8 @@ extern "C" gw_status gw_rr_to_GG_fft_noalloc(const gw_grid* grid, int direction,
   if ((st = upload(&local, dmap, map.data(), sizeof(int) * n_chi, s))) return done(st);
   if ((st = upload(&local, dinv, inv.data(), sizeof(int) * inv.size(), s))) return done(st);
   if (stage == 1) {
-    if (direction > 0) st = launch_row_fft(&local, g, prec, 1, in, nullptr, g.nr, out, n_chi, dmap, n_chi, n_rows, 1.0, s, dinv);
-    else st = launch_row_fft(&local, g, prec, 2, in, nullptr, n_chi, out, g.nr, dmap, n_chi, n_rows, 1.0 / g.volume, s, dinv);
+    if (direction > 0) st = launch_row_fft(&local, g, prec, 1, in, g.nr, out, n_chi, dmap, n_chi, n_rows, 1.0, s, dinv);
+    else st = launch_row_fft(&local, g, prec, 2, in, n_chi, out, g.nr, dmap, n_chi, n_rows, 1.0 / g.volume, s, dinv);
     return done(st);
   }
   if (direction > 0) {

@@ -30,7 +30,7 @@ GreenScales green_scales(const double* eps, int n_b, int n_occ, double mu, doubl
 
 gw_status green_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const void* dscale,
                      const GreenScales& gs, int r0, int n_rows, gw_prec prec, void* g_occ, void* g_unocc,
-                     cudaStream_t st, int low) {
+                     cudaStream_t st) {
   const size_t es = csize(prec);
   const size_t ss = is_fp64(prec) ? 8 : 4;
   const char* p = static_cast<const char*>(psi);
@@ -60,7 +60,6 @@ gw_status green_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
     a.ldc = g.nr;
     a.kscale = sc + (size_t)k0 * ss;
     a.tri = 0;
-    a.low = low;
     if ((rc = launch_gemm(ctx, prec, a, st))) return rc;
   }
   return GW_OK;

@@ -10,12 +10,13 @@ namespace gw {
 // copy exceeds kRowSmemMax take two kernels (row_two_pass(g, prec)); forward,
 // those need a [n_rows][N_r] workspace tmp (which may be a itself).
 constexpr size_t kRowSmemMax = 227 * 1024;
-gw_status launch_row_fft(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int mode, const void* a, const void* b,
-                         long lda, void* out, long ldo, const int* map, int n_chi, int n_rows, double scale,
+// mode 1: rows x(r, R') -> the G set; mode 2: rows over the G set -> x(r, R').
+gw_status launch_row_fft(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int mode, const void* a, long lda, void* out,
+                         long ldo, const int* map, int n_chi, int n_rows, double scale,
                          cudaStream_t st, const int* inv, void* tmp = nullptr,
                          int low = -1);
 // low >= 0: the rows are rows low .. of a Hermitian matrix used only for R' <= r
-// (forward: elements past r count as zero and mode 0 halves the diagonal; backward:
+// (forward: elements past r count as zero; backward:
 // only what the fused self-energy reads is written).
 // A G set's inverse map on the device: inv [N_r] (grid position -> G index or -1)
 // followed by what of the grid the set touches (set_lists appends it; index_maps
@@ -117,8 +118,6 @@ struct GemmArgs {
   int tri;
   int batch = 1;              // grid z: independent problems sA/sB/sC elements apart
   long sA = 0, sB = 0, sC = 0;
-  int low = -1;               // >= 0: row m is row low + m of a matrix of which only the columns n <= low + m
-                              // are needed: tiles wholly above that line are left as they are
 };
 gw_status launch_gemm(gw_ctx* ctx, gw_prec prec, const GemmArgs& a, cudaStream_t st);
 
@@ -130,7 +129,12 @@ struct GreenScales {
 GreenScales green_scales(const double* eps, int n_b, int n_occ, double mu, double tau);
 gw_status green_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const void* dscale,
                      const GreenScales& gs, int r0, int n_rows, gw_prec prec, void* g_occ, void* g_unocc,
-                     cudaStream_t st, int low = -1);
+                     cudaStream_t st);
+// chi rows r0 .. of nt times (<= 32), the triangle R' <= r as tc_chi_rows' lower; scale: the band
+// factors on the device, n_b 8-byte slots per time, packed in the working precision.
+gw_status launch_chi_simt(gw_ctx* ctx, gw_prec prec, const GridInfo& g, int n_b, int n_occ, const void* psi,
+                          const void* scale, const GreenScales* gs, int nt, int r0, int rows, void* out, long s_out,
+                          cudaStream_t st);
 
 }  // namespace gw
 

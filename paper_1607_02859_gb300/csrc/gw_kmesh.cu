@@ -388,7 +388,7 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
       }
       if ((st = launch_stripe<true>(ctx, prec, g, nk, gok, guk, kstr, dph, rows, rows_s, nullptr, gs.nr, s)))
         return st;
-      if ((st = launch_row_fft(ctx, gs, prec, 1, rows_s, nullptr, gs.nr, slab_j + (size_t)r0 * ld * es, ld, dsmap,
+      if ((st = launch_row_fft(ctx, gs, prec, 1, rows_s, gs.nr, slab_j + (size_t)r0 * ld * es, ld, dsmap,
                                n_k * n_chi, rows, 1.0, s, dsinv, tmp_s)))
         return st;
     }
@@ -729,7 +729,7 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
           return st;
       }
       if ((st = launch_stripe<false>(ctx, prec, g, nk, gok, guk, kstr, dph, rows, go_s, gu_s, gs.nr, s))) return st;
-      if ((st = launch_row_fft(ctx, gs, prec, 2, wrg + (size_t)r0 * ld * es, nullptr, ld, w_s, gs.nr, dsmap,
+      if ((st = launch_row_fft(ctx, gs, prec, 2, wrg + (size_t)r0 * ld * es, ld, w_s, gs.nr, dsmap,
                                n_k * n_chi, rows, 1.0, s, dsinv)))
         return st;
       if ((st = launch_sigma_contract(ctx, prec, w_s, go_s, gu_s, gs.nr, gs.nr, rows, ext, dbid, n_n, r0, coef,

@@ -17,10 +17,10 @@
 
 namespace gw {
 
-// Rows per r-block and times per launch of the chi pass.  The tensor-core G
-// formation walks its tiles with one CTA per SM: where a block's triangle has fewer
-// than six rounds of tiles (grids up to 16^3 by default) several times go in one
-// launch, within 512 MB of chi rows.  At 12^3 a time has 105 tiles for 152 SMs.
+// Rows per r-block and times per launch of the chi pass.  Where a block's triangle
+// has fewer than a few rounds of tiles for the SMs (grids up to 16^3 by default)
+// several times go in one launch, within 512 MB of chi rows: at 12^3 a time has 105
+// tensor-core tiles (one CTA per SM) or 378 CUDA-core ones (two) for 152 SMs.
 struct ChiShape {
   int rb, nt;
 };
@@ -28,20 +28,14 @@ static ChiShape chi_shape(const GridInfo& g, int n, gw_prec prec, int r_block) {
   const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
   ChiShape c;
   c.rb = r_block > 0 ? std::min(r_block, g.nr) : std::min(g.nr, tc ? 4096 : 2048);
-  c.nt = 1;
-  if (tc) {
-    const double t = (g.nr + 127) / 128, blocks = (g.nr + c.rb - 1) / c.rb;
-    const double tiles = 0.5 * t * (t + 1) / blocks;
-    const double most = (512.0 * 1048576.0) / ((double)c.rb * g.nr * csize(prec));
-    c.nt = std::max(1, std::min({n, (int)std::ceil(6 * 152 / tiles), (int)most}));
-  }
+  const int edge = tc ? 128 : 64;
+  const double t = (g.nr + edge - 1) / edge, blocks = (g.nr + c.rb - 1) / c.rb;
+  const double tiles = 0.5 * t * (t + 1) / blocks;
+  const double most = (512.0 * 1048576.0) / ((double)c.rb * g.nr * csize(prec));
+  c.nt = std::max(1, std::min({n, (int)std::ceil((tc ? 6 : 12) * 152 / tiles), (int)most}));
   return c;
 }
-// elements of the chi rows of a launch: nt blocks (tensor cores), or G_occ and G_unocc
-static size_t chi_rows_elems(const GridInfo& g, gw_prec prec, const ChiShape& c) {
-  const bool tc = prec == GW_F16X3 || prec == GW_BF16X3;
-  return (size_t)(tc ? c.nt : 2) * c.rb * g.nr;
-}
+static size_t chi_rows_elems(const GridInfo& g, const ChiShape& c) { return (size_t)c.nt * c.rb * g.nr; }
 
 size_t chi0_omega_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_chi, gw_prec prec, int r_block) {
   const size_t es = csize(prec);
@@ -53,7 +47,7 @@ size_t chi0_omega_scratch(const GridInfo& g, int n_b, int n_occ, int n, int n_ch
   probe.take<double>((size_t)n * n_b);
   probe.take<double>((size_t)n * n);
   probe.take<char>(slab * n * es);
-  probe.take<char>(chi_rows_elems(g, prec, c) * es);
+  probe.take<char>(chi_rows_elems(g, c) * es);
   if (prec == GW_F16X3 || prec == GW_BF16X3) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, c.rb, false, 0, c.nt));
   return probe.off;
 }
@@ -150,8 +144,7 @@ static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ,
   const size_t slab = (size_t)g.nr * n_chi;
   const int rb = sh.rb;
   char* slabs = cv.take<char>(slab * n * es);
-  char* ga = cv.take<char>(chi_rows_elems(g, prec, sh) * es);
-  char* gb = ga + (size_t)rb * g.nr * es;
+  char* ga = cv.take<char>(chi_rows_elems(g, sh) * es);
   void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, sh.nt)) : nullptr;
   if (tcs_out) *tcs_out = tcs;
   bool first = true;
@@ -163,21 +156,19 @@ static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ,
         TcEntries en;
         en.n = nt;
         en.out_stride = (long)rb * g.nr;
-        if ((st = tc_chi_rows(ctx, g, n_b, n_occ, psi, &scales[j0], r0, rows, prec, ga, tcs, first, s,
-                              t.sk + (size_t)j0 * n_b, t.status, true, en)))
-          return st;
+        st = tc_chi_rows(ctx, g, n_b, n_occ, psi, &scales[j0], r0, rows, prec, ga, tcs, first, s,
+                         t.sk + (size_t)j0 * n_b, t.status, true, en);
         first = false;
-        for (int z = 0; z < nt; ++z) {
-          char* x = ga + (size_t)z * rb * g.nr * es;
-          if ((st = launch_row_fft(ctx, g, prec, 1, x, nullptr, g.nr, slabs + ((size_t)(j0 + z) * slab + (size_t)r0 * n_chi) * es,
-                                   n_chi, t.map, n_chi, rows, 1.0, s, t.inv, x, r0)))
-            return st;
-        }
       } else {
-        const char* sj = t.scale + (size_t)j0 * n_b * 8;
-        if ((st = green_rows(ctx, g, n_b, n_occ, psi, sj, scales[j0], r0, rows, prec, ga, gb, s, r0))) return st;
-        if ((st = launch_row_fft(ctx, g, prec, 0, ga, gb, g.nr, slabs + ((size_t)j0 * slab + (size_t)r0 * n_chi) * es,
-                                 n_chi, t.map, n_chi, rows, -2.0, s, t.inv, ga, r0)))
+        st = launch_chi_simt(ctx, prec, g, n_b, n_occ, psi, t.scale + (size_t)j0 * n_b * 8, &scales[j0], nt, r0, rows,
+                             ga, (long)rb * g.nr, s);
+      }
+      if (st) return st;
+      for (int z = 0; z < nt; ++z) {
+        char* x = ga + (size_t)z * rb * g.nr * es;
+        if ((st = launch_row_fft(ctx, g, prec, 1, x, g.nr,
+                                 slabs + ((size_t)(j0 + z) * slab + (size_t)r0 * n_chi) * es, n_chi, t.map, n_chi, rows,
+                                 1.0, s, t.inv, x, r0)))
           return st;
       }
     }
@@ -328,7 +319,7 @@ gw_status pw_coefficients(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const vo
   const size_t es = csize(prec);
   const int step = row_two_pass(g, prec) ? tmp_rows : n_b;
   for (int b = 0; b < n_b; b += step)
-    if ((st = launch_row_fft(ctx, g, prec, 1, static_cast<const char*>(psi) + (size_t)b * g.nr * es, nullptr, g.nr,
+    if ((st = launch_row_fft(ctx, g, prec, 1, static_cast<const char*>(psi) + (size_t)b * g.nr * es, g.nr,
                              static_cast<char*>(dc) + (size_t)b * n_pw * es, n_pw, dmap_neg, n_pw,
                              std::min(step, n_b - b), 1.0, s, dinv_neg, tmp)))
       return st;

@@ -635,7 +635,7 @@ gw_status sigma_kernels(gw_ctx* ctx, const GridInfo& g, gw_prec prec, bool full,
       if (w.fused) {
         // W~(r,R') of the block (as far as the tiles with R' <= r reach), then G formation with the
         // contraction in its epilogue
-        if ((st = launch_row_fft(ctx, g, prec, 2, w.wrg + (size_t)r0 * n_chi * es, nullptr, n_chi, w.wrr, g.nr, t.map,
+        if ((st = launch_row_fft(ctx, g, prec, 2, w.wrg + (size_t)r0 * n_chi * es, n_chi, w.wrr, g.nr, t.map,
                                  n_chi, rows, 1.0, s, t.inv, nullptr, r0)))
           return st;
         TcSigma sg;
@@ -660,7 +660,7 @@ gw_status sigma_kernels(gw_ctx* ctx, const GridInfo& g, gw_prec prec, bool full,
       else st = green_rows(ctx, g, n_b, n_occ, psi, sj, scales[j], r0, rows, prec, w.gob, w.gub, s);
       if (st) return st;
       // W~(r,R') of the block (second step of Eq. FFTW), then the contraction
-      if ((st = launch_row_fft(ctx, g, prec, 2, w.wrg + (size_t)r0 * n_chi * es, nullptr, n_chi, w.wrr, g.nr, t.map,
+      if ((st = launch_row_fft(ctx, g, prec, 2, w.wrg + (size_t)r0 * n_chi * es, n_chi, w.wrr, g.nr, t.map,
                                n_chi, rows, 1.0, s, t.inv)))
         return st;
       if (!full) {
