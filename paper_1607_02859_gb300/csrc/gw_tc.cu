@@ -133,8 +133,8 @@ struct Params {
 // producer loads the tile's psi_n operand behind it, and the MMA warp
 // accumulates V for each half of the tile's columns in the free half of
 // tensor memory; unoccupied first, then occupied in the same shared memory.
-// The epilogue is not overlapped with MMAs, so its length counts: W~ is read
-// once, in 64-byte pieces into the place its own H will take, for both products
+// The epilogue is not overlapped with MMAs, so its length counts: W~ is loaded
+// once, by TMA into the place its own H will take, for both products
 // (H_occ waits in tensor memory), and the band sums are reduced by exchange.  With
 // one row of W~ per lane straight from global memory, twice, and five shuffles
 // and a double atomic per band, a tile's epilogue took 90 (4 bands) to 154
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
                                                                      const __grid_constant__ CUtensorMap mB,
                                                                      const __grid_constant__ CUtensorMap mP_hi,
                                                                      const __grid_constant__ CUtensorMap mP_lo,
-                                                                     Params p) {
+                                                                     const __grid_constant__ CUtensorMap mW, Params p) {
   constexpr int EW = kEpiWarps<MODE>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -166,6 +166,7 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
   uint64_t* redbar = psi_full + 1;       // the epilogue warps' band sums are in shared memory
   uint64_t* done2 = redbar + 1;          // every MMA of the self-energy phase done
   uint64_t* last_mma = done2 + 1;
+  uint64_t* w_full = last_mma + 1;       // W~ of the tile landed
   float* red = reinterpret_cast<float*>(epi);     // [8 warps][32][2] band sums of the warps (MODE 2 only)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -241,6 +242,7 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
       mbar_init(psi_full, 1);
       mbar_init(redbar, EW);
       mbar_init(done2, 1);
+      mbar_init(w_full, 1);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -261,6 +263,10 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
   uint8_t* const p_hi = smem + 16 * H_BYTES;
   const int p_chunk = MODE == 2 ? p.np * BK * 2 : 0;
   uint8_t* const p_lo = p_hi + 8 * p_chunk;
+  // W~ columns 64 h + 8 k .. + 7 of the tile lie where K chunk 4 h + k % 4 of H will, hi for k < 4 and
+  // lo above, swizzled alike: row r of W~ is where row r of that chunk will be, so the thread that owns
+  // row r and half h overwrites only what it has read itself
+  auto w_piece = [&](int h, int k) -> uint8_t* { return (k < 4 ? h_hi : h_lo) + (4 * h + (k & 3)) * H_BYTES; };
 
   auto timed_out = [&](int where) {
     *abort_flag = 1;
@@ -301,14 +307,19 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
       }
       if (*abort_flag) break;
       if constexpr (MODE == 2) {
-        // the tile's psi_n operand, once every MMA of the G formation has read its stages
+        // once every MMA of the G formation has read its stages: the tile's W~, 8 columns (64 bytes a row)
+        // per load, each in the place of an H chunk, then its psi_n operand
         if (wait_or_abort(done, (uint32_t)(ti & 1))) {
+          mbar_expect_tx(w_full, 16 * H_BYTES);
+          for (int k = 0; k < 16; ++k)
+            tma_load_3d(w_piece(k >> 3, k & 7), &mW, w_full, 2 * tl.n0 + 16 * k, tl.m0, 0);
           mbar_expect_tx(psi_full, (uint32_t)(16 * p_chunk));
           for (int cc = 0; cc < 8; ++cc) {
             tma_load_3d(p_hi + cc * p_chunk, &mP_hi, psi_full, 2 * tl.n0 + cc * BK, 0, 0);
             tma_load_3d(p_lo + cc * p_chunk, &mP_lo, psi_full, 2 * tl.n0 + cc * BK, 0, 0);
           }
-          mbar_wait(psi_full, (uint32_t)(ti & 1));    // our copies land before the CTA can exit
+          mbar_wait(w_full, (uint32_t)(ti & 1));      // our copies land before the CTA can exit
+          mbar_wait(psi_full, (uint32_t)(ti & 1));
         } else if (!*abort_flag) {
           timed_out(6);
         }
@@ -478,38 +489,18 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
           const bool rvalid = m0 + row < p.m_rows;
           const int h = cg;                             // the warp's column half
           const long grow = grow0 + row;                // grid row r of this thread
-          // The warp's 32 x 64 block of W~ goes through the shared memory that its own H will take:
-          // piece k (8 columns, 64 bytes a row) in the place of the warp's rows of K chunk 4h + k % 4,
-          // hi for k < 4 and lo above, 16-byte segments swizzled as H's.  Row r lies where row r of H
-          // will, so a thread only overwrites what it has read itself.
-          auto piece = [&](int k) -> uint8_t* {
-            return (k < 4 ? h_hi : h_lo) + (4 * h + (k & 3)) * H_BYTES + q * 2048;
-          };
-          {
-            const bool vec = (p.ldw % 2 == 0) && ((reinterpret_cast<uintptr_t>(p.wrr) & 15) == 0);
-#pragma unroll 4
-            for (int i = 0; i < 32; ++i) {              // eight rows of a piece per step, 64 bytes each
-              const int k = i >> 2, r = (i & 3) * 8 + (lane >> 2), sg = lane & 3;
-              const int gr = m0 + q * 32 + r, gn = c0 + 8 * k + 2 * sg;
-              uint8_t* dst = piece(k) + r * 64 + ((sg ^ ((r >> 1) & 3)) << 4);
-              const int have = gr < p.m_rows ? min(max(p.n_cols - gn, 0), 2) : 0;   // columns of the pair in range
-              const float2* src = have ? p.wrr + (long)gr * p.ldw + gn : p.wrr;
-              if (vec) {
-                cp_async16(dst, src, 8 * have);
-              } else {
-                cp_async8(dst, src, have > 0 ? 8 : 0);
-                cp_async8(dst + 8, have > 1 ? src + 1 : p.wrr, have > 1 ? 8 : 0);
-              }
-            }
-            cp_async_wait();
-            __syncwarp();
+          bool fine = wait_or_abort(w_full, (uint32_t)(ti & 1));
+          ok = __all_sync(0xffffffffu, fine);
+          if (!ok) {
+            if (lane == 0 && !*abort_flag) timed_out(14);
+            break;
           }
           // H = w G o W~ for G_unocc in registers and for G_occ in tensor memory (in place); returns the
           // powers of two that put the rows' maxima below 2^15
           float mu = 0.f, mo = 0.f;
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
-            const uint8_t* wp = piece(k) + lane * 64;
+            const uint8_t* wp = w_piece(h, k) + row * 64;
 #pragma unroll
             for (int hs = 0; hs < 2; ++hs) {
               uint32_t x[8];
@@ -600,7 +591,7 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
             for (int i = 0; i < 16; ++i) tot[16 * u + i] = __uint_as_float(x[i]);
           }
           free_occ();
-          bool fine = wait_or_abort(&hfree[h], (uint32_t)(ti & 1));   // the unoccupied MMAs have read this half
+          fine = wait_or_abort(&hfree[h], (uint32_t)(ti & 1));   // the unoccupied MMAs have read this half
           if (__all_sync(0xffffffffu, fine)) {
             tc_fence_after();
             store_h(sho);
@@ -993,6 +984,25 @@ gw_status tc_make_map3(gw_ctx* ctx, CUtensorMap* m, const void* base, int kpad, 
 
 namespace tc {
 
+// Map over W~ rows [rows][ldw] as FP32 pairs, box 8 complex x 128 rows, 64-byte swizzle; what lies
+// past the grid or the block reads as zero.
+static gw_status w_map(gw_ctx* ctx, CUtensorMap* m, const float2* base, int nr, long ldw, int rows) {
+  gw_status st;
+  EncodeFn enc = encoder(ctx, &st);
+  if (!enc) return st;
+  if (ldw % 2 || reinterpret_cast<uintptr_t>(base) % 16)
+    return fail(ctx, GW_ERR_UNSUPPORTED, "fused self-energy: W~ rows must be 16-byte aligned");
+  cuuint64_t dims[3] = {(cuuint64_t)2 * nr, (cuuint64_t)rows, 1};
+  cuuint64_t strides[2] = {(cuuint64_t)ldw * 8, (cuuint64_t)ldw * 8 * (cuuint64_t)rows};
+  cuuint32_t box[3] = {16, BM, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float2*>(base), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(ctx, GW_ERR_CUDA, "cuTensorMapEncodeTiled (W~) failed (" + std::to_string((int)r) + ")");
+  return GW_OK;
+}
+
 struct Layout {
   int k_occ_pad, k_un_pad, k_un_x, kpad;
 };
@@ -1110,15 +1120,17 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
     prep_kernel<false, 1><<<gbA, tb, 0, st>>>((const float2*)psi, n_b, n_occ, g.nr, r0, n_rows, sk, dexp,
                                                L.k_occ_pad, L.k_un_x, L.kpad, aop, en.psi_stride, b_shared);
   if ((rc = launch_check(ctx, "prep_kernel(A)"))) return rc;
-  CUtensorMap ma, mb, mph, mpl;
+  CUtensorMap ma, mb, mph, mpl, mw;
   if ((rc = tc_make_map3(ctx, &ma, aop, 2 * L.kpad, n_rows, nb, BM, fmt, 2 * BK))) return rc;
   if ((rc = tc_make_map3(ctx, &mb, bop, 2 * L.kpad, 2L * g.nr, (int)nbb, 2 * BNC, fmt, 2 * BK))) return rc;
   if (mode == 2) {
     if ((rc = tc_make_map3(ctx, &mph, phi, kps, np, 1, np, fmt, BK))) return rc;
     if ((rc = tc_make_map3(ctx, &mpl, plo, kps, np, 1, np, fmt, BK))) return rc;
+    if ((rc = w_map(ctx, &mw, sig->wrr, g.nr, sig->ldw, n_rows))) return rc;
   } else {
     mph = ma;                                    // unused outside the self-energy mode
     mpl = ma;
+    mw = ma;
   }
   Params P;
   P.m_rows = n_rows;
@@ -1177,7 +1189,7 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
     const double work =
         tile_frac * (8.0 * n_rows * (double)g.nr * n_b + (mode == 2 ? 16.0 * n_rows * (double)g.nr * P.n_n : 0.0));
     KTimer kt(ctx, KF_GREEN_TC, work, st);
-    kernel<<<grid, threads, SMEM_BYTES, st>>>(ma, mb, mph, mpl, P);
+    kernel<<<grid, threads, SMEM_BYTES, st>>>(ma, mb, mph, mpl, mw, P);
     return launch_check(ctx, "green_tc_kernel");
   };
   if (mode == 0) rc = fmt == 0 ? go(green_tc_kernel<0, 0>) : go(green_tc_kernel<0, 1>);
