@@ -55,6 +55,17 @@ struct SetLists {
   }
 };
 
+// Bit i of the result: index i is in the list of n indices below 64 (whole warps call it).
+__device__ __forceinline__ unsigned long long set_mask(const int* __restrict__ list, int n) {
+  unsigned lo = 0, hi = 0;
+  for (int e = threadIdx.x & 31; e < n; e += 32) {
+    const int v = __ldg(list + e);
+    if (v < 32) lo |= 1u << v;
+    else hi |= 1u << (v - 32);
+  }
+  return (unsigned long long)__reduce_or_sync(~0u, hi) << 32 | __reduce_or_sync(~0u, lo);
+}
+
 // Rows of a Hermitian matrix x(r, R') of which only R' <= r is used: the row kernels
 // take the grid index low of the launch's first row (-1: whole rows).
 // Forward: elements past r are taken as zero without being read (the tensor-core
@@ -251,8 +262,10 @@ __global__ void __launch_bounds__(RowCfg<T, N1, N2, N3>::TH, RowCfg<T, N1, N2, N
 // plane).  Both kernels keep many small CTAs on an SM.  A thread-block cluster
 // holding the whole row in distributed shared memory (one pass over HBM, but 76
 // rows in flight, three cluster barriers and scattered remote accesses) took
-// 204 ns a row of the triangle at 36^3 with n_chi = 8192, these take 152 ns
-// forward and 128 ns backward; with all pencils of whole rows it was 340 ns.
+// 204 ns a row of the triangle at 36^3 with n_chi = 8192, these take 118 ns
+// either way; with all pencils of whole rows it was 340 ns.  With the plane filled
+// into (or read from) shared memory around the i2 pass, and 128 threads per line
+// CTA (12 warps per SM in flight), it was 152 ns forward and 128 ns backward.
 template <typename T, int N1, int N2, int N3>
 struct PlaneCfg {
   using C = typename cpx<T>::t;
@@ -263,19 +276,73 @@ struct PlaneCfg {
   static constexpr int TH = (PP * N2 + 31) / 32 * 32;              // one pencil per thread and pass
   static constexpr int MINB = sizeof(T) == 4 ? (N2 >= 30 ? 4 : 6) : 2;
   static constexpr size_t bytes = (size_t)PP * S1 * sizeof(C);
-  static constexpr int LT = 128;                                    // threads of the line kernels
-  static constexpr int LMINB = sizeof(T) == 4 ? 4 : 2;
+  // threads and CTAs per SM of the line kernels (forward, backward)
+  static constexpr int LF = sizeof(T) == 4 ? 160 : 128, LFB = sizeof(T) == 4 ? 3 : 2;
+  static constexpr int LB = sizeof(T) == 4 ? 256 : 128, LBB = 2;
   // the longest G-set row that the line kernels stage in shared memory (two CTAs per SM)
   static constexpr size_t kStage = 110 * 1024;
 };
 
-// MODE 1 as for row_fft_kernel: planes of a, (+i) over i3 and the set's i3 of i2,
+// One i3 pencil of a plane in shared memory, transformed in place; the elements of mask are written.
+template <int N, int DIR, typename C>
+__device__ __forceinline__ void plane_pencil(C* s, unsigned long long mask) {
+  C x[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) x[k] = s[k];
+  RegFFT<N, DIR>::run(x);
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+    if (mask >> k & 1) s[k] = x[k];
+}
+
+// The set's columns of up to PP planes of each of ROWS rows into the zeroed pencils of its i2, and out again.
+template <int N2, int N3, int PP, int ROWS, typename G, typename C, typename F>
+__device__ __forceinline__ void plane_scatter(const G& g, C* s, int s1, int s2, int np, F load) {
+  const int n = np * g.n2;
+  for (int t = threadIdx.x; t < ROWS * n; t += blockDim.x) {
+    const int r = t / n, e = t - r * n, p = e / g.n2;
+    C* z = s + (r * PP + p) * s1 + __ldg(g.l2 + (e - p * g.n2)) * s2;
+#pragma unroll
+    for (int k = 0; k < N3; ++k) z[k] = C{};
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < g.n23; e += blockDim.x) {
+    const int q = __ldg(g.l23 + e);
+    const int o = q / N3 * s2 + q % N3;
+    C v[ROWS][PP];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+      for (int p = 0; p < PP; ++p)
+        if (p < np) v[r][p] = load(r, p, e);
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+      for (int p = 0; p < PP; ++p)
+        if (p < np) s[(r * PP + p) * s1 + o] = v[r][p];
+  }
+  __syncthreads();
+}
+template <int N2, int N3, int PP, typename G, typename C, typename F>
+__device__ __forceinline__ void plane_gather(const G& g, const C* s, int s1, int s2, int np, F store) {
+  for (int e = threadIdx.x; e < g.n23; e += blockDim.x) {
+    const int q = __ldg(g.l23 + e);
+    const int o = q / N3 * s2 + q % N3;
+#pragma unroll
+    for (int p = 0; p < PP; ++p)
+      if (p < np) store(p, e, s[p * s1 + o]);
+  }
+}
+
+// MODE 1 as for row_fft_kernel: planes of a, (+i) over i2 and the set's i2 of i3,
 // the set's columns to t.  MODE 2: the columns from t,
 // (-i) over the set's i2 of i3 and i2, times scale, to the planes of out.
-template <typename T, int N1, int N2, int N3, int MODE, bool VEC>
+// The i2 pass meets global memory in registers (a warp's elements of one i2 lie
+// side by side there), and shared memory holds the set's i2 only.
+template <typename T, int N1, int N2, int N3, int MODE>
 __global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::TH, PlaneCfg<T, N1, N2, N3>::MINB)
-    row_plane_kernel(const typename cpx<T>::t* a, long lda, typename cpx<T>::t* t, long t_row, long t_plane, typename cpx<T>::t* out, long ldo, const int* __restrict__ inv, T scale,
-                     int low) {
+    row_plane_kernel(const typename cpx<T>::t* a, long lda, typename cpx<T>::t* t, long t_row, long t_plane,
+                     typename cpx<T>::t* out, long ldo, const int* __restrict__ inv, T scale, int low) {
   using C = typename cpx<T>::t;
   using R = PlaneCfg<T, N1, N2, N3>;
   constexpr int PL = R::PL, S1 = R::S1, S2 = R::S2, TH = R::TH;
@@ -287,101 +354,59 @@ __global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::TH, PlaneCfg<T, N1, N
   const int np = min(R::PP, last / PL + 1 - p0);                   // planes of this CTA in use
   if (np <= 0) return;
   const SetLists<N1, N2, N3> g(inv);
-  auto pos = [](int e) {                                           // e = p PL + i2 N3 + i3
-    const int p = e / PL, rem = e - p * PL, i2 = rem / N3;
-    return p * S1 + i2 * S2 + (rem - i2 * N3);
-  };
+  const unsigned long long m2 = set_mask(g.l2, g.n2);
   C* tp = t + row * t_row + (long)p0 * t_plane;
   if constexpr (MODE == 2) {
-    for (int e = threadIdx.x; e < np * S1; e += TH) s[e] = mk(T(0), T(0));
-    __syncthreads();
-    for (int e = threadIdx.x; e < g.n23; e += TH) {
-      const int q = __ldg(g.l23 + e);
-      const int o = q / N3 * S2 + q % N3;
-#pragma unroll
-      for (int p = 0; p < R::PP; ++p)
-        if (p < np) s[p * S1 + o] = tp[p * t_plane + e];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < np * g.n2; e += TH) {            // pencils outside the set's i2 are zero
-      const int p = e / g.n2;
-      const int o = p * S1 + __ldg(g.l2 + (e - p * g.n2)) * S2;
-      C x[N3];
-#pragma unroll
-      for (int k = 0; k < N3; ++k) x[k] = s[o + k];
-      RegFFT<N3, -1>::run(x);
-#pragma unroll
-      for (int k = 0; k < N3; ++k) s[o + k] = x[k];
-    }
-    __syncthreads();
-    pencil_pass<N2, -1>(s, np * N3, S2, [](int q) { return (q / N3) * S1 + (q % N3); });
+    plane_scatter<N2, N3, R::PP, 1>(g, s, S1, S2, np, [&](int, int p, int e) { return tp[p * t_plane + e]; });
+    for (int e = threadIdx.x; e < np * g.n2; e += TH)              // pencils outside the set's i2 are zero
+      plane_pencil<N3, -1>(s + e / g.n2 * S1 + __ldg(g.l2 + e % g.n2) * S2, ~0ull);
     __syncthreads();
     C* dst = out + row * ldo + (long)p0 * PL;
-    if (VEC) {
-      for (int q = threadIdx.x; q < np * PL / 2; q += TH) {
-        const int o = pos(2 * q);
-        st_pair(dst + 2 * q, cscale(s[o], scale), cscale(s[o + 1], scale));
+    for (int e = threadIdx.x; e < np * N3; e += TH) {
+      const int p = e / N3, i3 = e - p * N3;
+      C x[N2];
+#pragma unroll
+      for (int k = 0; k < N2; ++k) {
+        x[k] = mk(T(0), T(0));
+        if (m2 >> k & 1) x[k] = s[p * S1 + i3 + k * S2];
       }
-    } else {
-      for (int e = threadIdx.x; e < np * PL; e += TH) dst[e] = cscale(s[pos(e)], scale);
+      RegFFT<N2, -1>::run(x);
+#pragma unroll
+      for (int k = 0; k < N2; ++k) dst[p * PL + i3 + k * N3] = cscale(x[k], scale);
     }
     return;
   }
   const int last0 = last - p0 * PL;                                // the last element in use, from the CTA's first
   const C* pa = a + row * lda + (long)p0 * PL;
-  if (VEC) {
-    constexpr int LB = 8;                                          // 16-byte loads in flight per thread
-    for (int q0 = threadIdx.x; q0 < np * PL / 2; q0 += LB * TH) {
-      C v[LB][2];
-#pragma unroll
-      for (int u = 0; u < LB; ++u) {
-        const int q = q0 + u * TH;
-        v[u][0] = v[u][1] = mk(T(0), T(0));
-        if (q < np * PL / 2 && 2 * q <= last0) ld_pair_rw(pa + 2 * q, v[u][0], v[u][1]);
-      }
-#pragma unroll
-      for (int u = 0; u < LB; ++u) {
-        const int q = q0 + u * TH;
-        if (q >= np * PL / 2) continue;
-        const int o = pos(2 * q);
-        s[o] = v[u][0];
-        s[o + 1] = 2 * q + 1 <= last0 ? v[u][1] : mk(T(0), T(0));
-      }
-    }
-  } else {
-    for (int e = threadIdx.x; e < np * PL; e += TH) s[pos(e)] = e <= last0 ? pa[e] : mk(T(0), T(0));
-  }
-  __syncthreads();
-  pencil_pass<N3, +1>(s, np * N2, 1, [](int q) { return q * S2; });
-  __syncthreads();
-  for (int e = threadIdx.x; e < np * g.n3; e += TH) {
-    const int p = e / g.n3;
-    const int o = p * S1 + __ldg(g.l3 + (e - p * g.n3));
+  for (int e = threadIdx.x; e < np * N3; e += TH) {
+    const int p = e / N3, i3 = e - p * N3, r0 = p * PL + i3;
     C x[N2];
 #pragma unroll
-    for (int k = 0; k < N2; ++k) x[k] = s[o + k * S2];
+    for (int k = 0; k < N2; ++k) {
+      x[k] = mk(T(0), T(0));
+      if (r0 + k * N3 <= last0) x[k] = pa[r0 + k * N3];
+    }
     RegFFT<N2, +1>::run(x);
 #pragma unroll
-    for (int k = 0; k < N2; ++k) s[o + k * S2] = x[k];
+    for (int k = 0; k < N2; ++k)
+      if (m2 >> k & 1) s[p * S1 + i3 + k * S2] = x[k];
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < g.n23; e += TH) {
-    const int q = __ldg(g.l23 + e);
-    const int o = q / N3 * S2 + q % N3;
-#pragma unroll
-    for (int p = 0; p < R::PP; ++p)
-      if (p < np) tp[p * t_plane + e] = s[p * S1 + o];
-  }
+  const unsigned long long m3 = set_mask(g.l3, g.n3);
+  for (int e = threadIdx.x; e < np * g.n2; e += TH)
+    plane_pencil<N3, +1>(s + e / g.n2 * S1 + __ldg(g.l2 + e % g.n2) * S2, m3);
+  __syncthreads();
+  plane_gather<N2, N3, R::PP>(g, s, S1, S2, np, [&](int p, int e, C v) { tp[p * t_plane + e] = v; });
 }
 
 // Forward line pass of one row per CTA: i1 transforms (+i) of the set's columns,
 // the results to out[row][inv], in order through shared memory where STAGE.
 template <typename T, int N1, int N2, int N3, bool STAGE>
-__global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::LT, PlaneCfg<T, N1, N2, N3>::LMINB)
+__global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::LF, PlaneCfg<T, N1, N2, N3>::LFB)
     row_line_fwd_kernel(const typename cpx<T>::t* t, long t_row, long t_plane, typename cpx<T>::t* __restrict__ out,
                         long ldo, const int* __restrict__ inv, int n_chi, int low) {
   using C = typename cpx<T>::t;
-  constexpr int PL = N2 * N3, LT = PlaneCfg<T, N1, N2, N3>::LT;
+  constexpr int PL = N2 * N3, LT = PlaneCfg<T, N1, N2, N3>::LF;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* so = reinterpret_cast<C*>(smem_raw);                          // [n_chi]
   const long row = blockIdx.x;
@@ -408,11 +433,11 @@ __global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::LT, PlaneCfg<T, N1, N
 // Backward line pass: the row's n_chi values (through shared memory where STAGE)
 // gathered through inv, i1 transforms (-i) of the set's columns, the planes in use to t.
 template <typename T, int N1, int N2, int N3, bool STAGE>
-__global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::LT, PlaneCfg<T, N1, N2, N3>::LMINB)
+__global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::LB, PlaneCfg<T, N1, N2, N3>::LBB)
     row_line_bwd_kernel(const typename cpx<T>::t* __restrict__ a, long lda, typename cpx<T>::t* __restrict__ t,
                         long t_row, long t_plane, const int* __restrict__ inv, int n_chi, int low, int fwd_rows) {
   using C = typename cpx<T>::t;
-  constexpr int PL = N2 * N3, LT = PlaneCfg<T, N1, N2, N3>::LT;
+  constexpr int PL = N2 * N3, LT = PlaneCfg<T, N1, N2, N3>::LB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* si = reinterpret_cast<C*>(smem_raw);                          // [n_chi]
   const long row = blockIdx.x;
@@ -462,8 +487,8 @@ struct PwPlane {
   using C = typename cpx<T>::t;
   using R = PlaneCfg<T, N1, N2, N3>;
   static constexpr int PP = N2 >= 30 ? 2 : 4;
-  static constexpr int TH = (2 * PP * N2 + 31) / 32 * 32;          // one pencil of the two rows per thread
-  static constexpr int MINB = sizeof(T) == 4 ? (N2 >= 30 ? 4 : 3) : 1;
+  static constexpr int TH = (2 * PP * (N2 > N3 ? N2 : N3) + 31) / 32 * 32;   // one pencil of the two rows per thread
+  static constexpr int MINB = sizeof(T) == 4 ? (N2 >= 40 ? 2 : N2 >= 30 ? 4 : 3) : 1;
   static constexpr size_t bytes = 2 * (size_t)PP * R::S1 * sizeof(C);
 };
 
@@ -485,86 +510,60 @@ __global__ void __launch_bounds__(PwPlane<T, N1, N2, N3>::TH, PwPlane<T, N1, N2,
   if (np <= 0) return;
   const int last0 = last - p0 * PL;
   const SetLists<N1, N2, N3> gp(inv_pw), gx(inv_chi);
-  for (int e = threadIdx.x; e < 2 * PP * S1; e += TH) sa[e] = mk(T(0), T(0));
-  __syncthreads();
   {
     const C* pa = ta + row * ta_row + (long)p0 * ta_plane;
     const C* pb = tb + row * ta_row + (long)p0 * ta_plane;
-    for (int e = threadIdx.x; e < gp.n23; e += TH) {
-      const int q = __ldg(gp.l23 + e);
-      const int o = q / N3 * S2 + q % N3;
-#pragma unroll
-      for (int p = 0; p < PP; ++p)
-        if (p < np) {
-          sa[p * S1 + o] = pa[p * ta_plane + e];
-          sb[p * S1 + o] = pb[p * ta_plane + e];
-        }
-    }
+    plane_scatter<N2, N3, PP, 2>(gp, sa, S1, S2, np,
+                                 [&](int r, int p, int e) { return (r ? pb : pa)[p * ta_plane + e]; });
   }
-  __syncthreads();
   {                                                                // pencils outside the set's i2 are zero
     const int n = np * gp.n2;
     for (int t = threadIdx.x; t < 2 * n; t += TH) {
-      const int e = t >= n ? t - n : t, p = e / gp.n2;
-      C* s = (t >= n ? sb : sa) + p * S1 + __ldg(gp.l2 + (e - p * gp.n2)) * S2;
-      C x[N3];
-#pragma unroll
-      for (int k = 0; k < N3; ++k) x[k] = s[k];
-      RegFFT<N3, -1>::run(x);
-#pragma unroll
-      for (int k = 0; k < N3; ++k) s[k] = x[k];
+      const int e = t >= n ? t - n : t;
+      plane_pencil<N3, -1>((t >= n ? sb : sa) + e / gp.n2 * S1 + __ldg(gp.l2 + e % gp.n2) * S2, ~0ull);
     }
   }
   __syncthreads();
   {
-    const int n = np * N3;
-    for (int t = threadIdx.x; t < 2 * n; t += TH) {
-      const int e = t >= n ? t - n : t;
-      C* s = (t >= n ? sb : sa) + e / N3 * S1 + e % N3;
-      C x[N2];
-#pragma unroll
-      for (int k = 0; k < N2; ++k) x[k] = s[k * S2];
-      RegFFT<N2, -1>::run(x);
-#pragma unroll
-      for (int k = 0; k < N2; ++k) s[k * S2] = x[k];
-    }
-  }
-  __syncthreads();
-  // the product of Eq. chi_rr as the input of the forward i2 pass, then the i3 pass of the set's pencils
-  for (int e = threadIdx.x; e < np * N3; e += TH) {
-    const int p = e / N3, i3 = e - p * N3, o = p * S1 + i3, r0 = p * PL + i3;
+    // i2 of both rows, a column per thread; those of a stay in registers for the product of Eq. chi_rr and i2 of x
+    const unsigned long long m2 = set_mask(gp.l2, gp.n2), mx = set_mask(gx.l2, gx.n2);
+    const int n = np * N3, t = threadIdx.x;
+    const int e = t >= n ? t - n : t, p = e / N3, i3 = e - p * N3, o = p * S1 + i3, r0 = p * PL + i3;
     C x[N2];
+    if (t < 2 * n) {
+      C* s = (t >= n ? sb : sa) + o;
 #pragma unroll
-    for (int k = 0; k < N2; ++k) {
-      const int r = r0 + k * N3;
-      x[k] = mk(T(0), T(0));
-      if (r <= last0)
-        x[k] = cscale(cmulc(sa[o + k * S2], sb[o + k * S2]), low >= 0 && r == last0 ? scale * T(0.5) : scale);
+      for (int k = 0; k < N2; ++k) {
+        x[k] = mk(T(0), T(0));
+        if (m2 >> k & 1) x[k] = s[k * S2];
+      }
+      RegFFT<N2, -1>::run(x);
+      if (t >= n) {
+#pragma unroll
+        for (int k = 0; k < N2; ++k) s[k * S2] = x[k];
+      }
     }
-    RegFFT<N2, +1>::run(x);
+    __syncthreads();
+    if (t < n) {
 #pragma unroll
-    for (int k = 0; k < N2; ++k) sa[o + k * S2] = x[k];
+      for (int k = 0; k < N2; ++k) {
+        const int r = r0 + k * N3;
+        if (r <= last0) x[k] = cscale(cmulc(x[k], sb[o + k * S2]), low >= 0 && r == last0 ? scale * T(0.5) : scale);
+        else x[k] = mk(T(0), T(0));
+      }
+      RegFFT<N2, +1>::run(x);
+#pragma unroll
+      for (int k = 0; k < N2; ++k)
+        if (mx >> k & 1) sa[o + k * S2] = x[k];
+    }
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < np * gx.n2; e += TH) {
-    const int p = e / gx.n2;
-    C* s = sa + p * S1 + __ldg(gx.l2 + (e - p * gx.n2)) * S2;
-    C x[N3];
-#pragma unroll
-    for (int k = 0; k < N3; ++k) x[k] = s[k];
-    RegFFT<N3, +1>::run(x);
-#pragma unroll
-    for (int k = 0; k < N3; ++k) s[k] = x[k];
-  }
+  const unsigned long long m3 = set_mask(gx.l3, gx.n3);
+  for (int e = threadIdx.x; e < np * gx.n2; e += TH)
+    plane_pencil<N3, +1>(sa + e / gx.n2 * S1 + __ldg(gx.l2 + e % gx.n2) * S2, m3);
   __syncthreads();
   C* px = tx + row * tx_row + (long)p0 * tx_plane;
-  for (int e = threadIdx.x; e < gx.n23; e += TH) {
-    const int q = __ldg(gx.l23 + e);
-    const int o = q / N3 * S2 + q % N3;
-#pragma unroll
-    for (int p = 0; p < PP; ++p)
-      if (p < np) px[p * tx_plane + e] = sa[p * S1 + o];
-  }
+  plane_gather<N2, N3, PP>(gx, sa, S1, S2, np, [&](int p, int e, C v) { px[p * tx_plane + e] = v; });
 }
 
 // Rows too long for one CTA in the plane-wave self-energy: the CL CTAs of a
@@ -1132,7 +1131,7 @@ struct GridOps {
       gw_status r = set_smem(ctx, kernel, sm);
       if (r) return r;
       KTimer kt(ctx, fam, work, st);
-      kernel<<<n_rows, PC::LT, sm, st>>>((const C*)t, t_row, t_plane, (C*)out, ldo, inv, n_chi, low);
+      kernel<<<n_rows, PC::LF, sm, st>>>((const C*)t, t_row, t_plane, (C*)out, ldo, inv, n_chi, low);
       return launch_check(ctx, "row_line_fwd_kernel");
     };
     return bytes <= PC::kStage ? go(row_line_fwd_kernel<T, N1, N2, N3, true>, bytes)
@@ -1145,7 +1144,7 @@ struct GridOps {
       gw_status r = set_smem(ctx, kernel, sm);
       if (r) return r;
       KTimer kt(ctx, fam, work, st);
-      kernel<<<n_rows, PC::LT, sm, st>>>((const C*)a, lda, (C*)t, t_row, t_plane, inv, n_chi, low, fwd_rows ? 1 : 0);
+      kernel<<<n_rows, PC::LB, sm, st>>>((const C*)a, lda, (C*)t, t_row, t_plane, inv, n_chi, low, fwd_rows ? 1 : 0);
       return launch_check(ctx, "row_line_bwd_kernel");
     };
     return bytes <= PC::kStage ? go(row_line_bwd_kernel<T, N1, N2, N3, true>, bytes)
@@ -1160,7 +1159,7 @@ struct GridOps {
   }
   static gw_status row_two_pass(gw_ctx* ctx, int mode, const void* a, long lda, void* out, long ldo,
                                 const int* inv, void* tmp, int n_chi, int n_rows, double scale, cudaStream_t st,
-                                bool vec, int low, double work) {
+                                int low, double work) {
     constexpr int NR = N1 * N2 * N3;
     if (mode != 2 && !tmp)
       return fail(ctx, GW_ERR_UNSUPPORTED, "this grid's rows need the two-pass transform (index map and workspace)");
@@ -1175,17 +1174,13 @@ struct GridOps {
                                                inv, (T)scale, low);
       return launch_check(ctx, "row_plane_kernel");
     };
-    constexpr bool E = N3 % 2 == 0;
     gw_status rc;
     if (mode == 2) {
       // the columns lie in out itself, at the start of each plane
       if ((rc = line_bwd(ctx, a, lda, out, ldo, PC::PL, inv, n_chi, n_rows, low, false, 0.0, KF_ROW_FFT, st))) return rc;
-      return vec ? plane(row_plane_kernel<T, N1, N2, N3, 2, E>, out, ldo)
-                 : plane(row_plane_kernel<T, N1, N2, N3, 2, false>, out, ldo);
+      return plane(row_plane_kernel<T, N1, N2, N3, 2>, out, ldo);
     }
-    rc = vec ? plane(row_plane_kernel<T, N1, N2, N3, 1, E>, tmp, NR)
-             : plane(row_plane_kernel<T, N1, N2, N3, 1, false>, tmp, NR);
-    if (rc) return rc;
+    if ((rc = plane(row_plane_kernel<T, N1, N2, N3, 1>, tmp, NR))) return rc;
     return line_fwd(ctx, tmp, NR, PC::PL, out, ldo, inv, n_chi, n_rows, low, 0.0, KF_ROW_FFT, st);
   }
   static gw_status row(gw_ctx* ctx, int mode, const void* a, long lda, void* out, long ldo,
@@ -1206,7 +1201,7 @@ struct GridOps {
     const bool vo = mode != 2 && al(out) && ldo % 2 == 0 && n_chi % 2 == 0;
     if (!inv) return fail(ctx, GW_ERR_ARG, "row transform without the G set's inverse map");
     if constexpr (L::TOT * sizeof(C) > kRowSmemMax)
-      return row_two_pass(ctx, mode, a, lda, out, ldo, inv, tmp, n_chi, n_rows, scale, st, vi, low, work);
+      return row_two_pass(ctx, mode, a, lda, out, ldo, inv, tmp, n_chi, n_rows, scale, st, low, work);
     if constexpr (L::TOT * sizeof(C) <= kRowSmemMax) {
       auto go = [&](auto kernel) -> gw_status {
         gw_status s = set_smem(ctx, kernel, bytes);
