@@ -409,7 +409,8 @@ gw_status gw_chi0_omega(gw_ctx* ctx, const gw_grid* grid, int n_b, int n_occ,
  * (Eq. chi_rr) and transforms it onto the G set (Eq. FFTX1); then Eqs. FFTX2
  * and CTX as in gw_chi0_omega.  Scratch (context arena): the slabs
  * (N_r n_chi n elements) plus 2 N_r n_pw + 2 n_pw^2 + N_b n_pw elements (8 or 16
- * bytes each) and the tensor-core operands.  GW_ERR_UNSUPPORTED where two
+ * bytes each), the columns between the row kernels (at most 1024 rows of 3 N_r
+ * elements) and the tensor-core operands.  GW_ERR_UNSUPPORTED where two
  * expanded rows of the grid do not fit a thread-block cluster's shared memory
  * (GW_FP64 at 36^3, every precision at 48^3).  Synchronises the stream once
  * (the norm check). */
@@ -475,7 +476,8 @@ gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const int* nk, i
  * functions over R', forms -2 G_occ conj(G_unocc) and transforms it onto the
  * supercell G set {q + g}; the rest as gw_chi0_omega_kmesh.  Scratch (context
  * arena): the slabs (N_r N_k n_chi n elements) plus 2 N_r N_k n_pw + 2 n_pw^2 +
- * N_k N_b n_pw + N_b N_r elements and the tensor-core operands.
+ * N_k N_b n_pw + N_b N_r elements, the columns between the row kernels (as
+ * gw_chi0_omega_pw, of the supercell) and the tensor-core operands.
  * GW_ERR_UNSUPPORTED where two expanded supercell rows do not fit a
  * thread-block cluster (supercells beyond 36^3, GW_FP64 at 36^3).  Synchronises
  * the stream once per k (the norm check). */

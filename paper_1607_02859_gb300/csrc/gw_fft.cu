@@ -1,5 +1,5 @@
-// Spatial transforms within the cell (Eqs. FFTX1, FFTX2, FFTW), the
-// real-space product of Eq. chi_rr fused into the row transform, and the
+// Spatial transforms within the cell (Eqs. FFTX1, FFTX2, FFTW), the product of
+// Eq. chi_rr of plane-wave Green's functions fused into the row transform, and the
 // nonuniform time/frequency transforms (Eqs. CTX, CT_W, ST_FFT).
 //
 // Data stay in HBM as row-major complex matrices whose row index is a grid
@@ -7,7 +7,9 @@
 // point R' or a G' of the set.
 //  * row kernels: one CTA per row; the N_r-point row is staged in shared memory
 //    (odd-padded pencil stride, so every pencil pass is bank-conflict free) and
-//    transformed by three passes of fully unrolled register FFTs.
+//    transformed by three passes of fully unrolled register FFTs, over the pencils
+//    that the G set and the used part of the row touch; a row too long for one CTA
+//    takes a plane and a line kernel.
 //  * column kernels: the transform runs over the row index for a chunk of
 //    contiguous columns, so every HBM access is a coalesced row segment:
 //    a "plane" kernel does the (i2,i3) 2-D FFT through shared memory and a
@@ -1165,6 +1167,13 @@ struct GridOps {
       return fail(ctx, GW_ERR_UNSUPPORTED, "this grid's rows need the two-pass transform (index map and workspace)");
     if (sizeof(T) == 8 && (size_t)n_chi * sizeof(C) > 200 * 1024)
       return fail(ctx, GW_ERR_UNSUPPORTED, "G set too large for the two-pass row transform");
+    constexpr int kMost = 32768;                                   // rows are the grid's y: whole 128-row tiles at a time
+    for (int r = 0; n_rows > kMost && r < n_rows; r += kMost) {
+      const int rows = std::min(kMost, n_rows - r);
+      gw_status rc = row_two_pass(ctx, mode, (const C*)a + (long)r * lda, lda, (C*)out + (long)r * ldo, ldo, inv, tmp,
+                                  n_chi, rows, scale, st, low >= 0 ? low + r : -1, work * rows / n_rows);
+      if (rc || r + rows == n_rows) return rc;
+    }
     const dim3 pgrid((row_planes(low, n_rows, mode == 2) + PC::PP - 1) / PC::PP, n_rows);
     auto plane = [&](auto kernel, void* t, long t_row) -> gw_status {
       gw_status r = set_smem(ctx, kernel, PC::bytes);
@@ -1587,20 +1596,28 @@ extern "C" gw_status gw_rr_to_GG_fft(gw_ctx* ctx, const gw_grid* grid, int direc
   if (stage == 1 && (n_rows < 0 || r0 < 0 || r0 + n_rows > g.nr)) return fail(ctx, GW_ERR_SHAPE, "rows out of range");
   cudaStream_t s = as_stream(stream);
   const int cols = set_columns(g, inv);
-  // rows too long for shared memory need a [n_rows][N_r] workspace forward
+  // rows too long for shared memory need a [rows][N_r] workspace forward: so many rows at a time
   const bool work_rows = stage == 1 && direction > 0 && row_two_pass(g, prec);
+  const int chunk = std::min(n_rows, 1024);
   Carver probe(nullptr);
   probe.take<int>(n_chi);
   probe.take<int>(inv_ints(g));
-  if (work_rows) probe.take<char>((size_t)n_rows * g.nr * csize(prec));
+  if (work_rows) probe.take<char>((size_t)chunk * g.nr * csize(prec));
   if ((st = reserve(ctx, probe.off))) return st;
   Carver cv(ctx->arena);
   int* dmap = cv.take<int>(n_chi);
   int* dinv = cv.take<int>(inv_ints(g));
-  void* tmp = work_rows ? cv.take<char>((size_t)n_rows * g.nr * csize(prec)) : nullptr;
+  void* tmp = work_rows ? cv.take<char>((size_t)chunk * g.nr * csize(prec)) : nullptr;
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
   if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if (stage == 1) {
+    const size_t es = csize(prec);
+    for (int r = 0; work_rows && r < n_rows; r += chunk)
+      if ((st = launch_row_fft(ctx, g, prec, 1, static_cast<const char*>(in) + (size_t)r * g.nr * es, g.nr,
+                               static_cast<char*>(out) + (size_t)r * n_chi * es, n_chi, dmap, n_chi,
+                               std::min(chunk, n_rows - r), 1.0, s, dinv, tmp)))
+        return st;
+    if (work_rows) return GW_OK;
     if (direction > 0)
       return launch_row_fft(ctx, g, prec, 1, in, g.nr, out, n_chi, dmap, n_chi, n_rows, 1.0, s, dinv, tmp);
     return launch_row_fft(ctx, g, prec, 2, in, n_chi, out, g.nr, dmap, n_chi, n_rows, 1.0 / g.volume, s,

@@ -1,4 +1,4 @@
-// Shared-memory 3-D FFT of one grid row (internal).
+// Shared-memory pencils of one grid row (internal).
 #pragma once
 
 #include "gw_common.cuh"
@@ -59,17 +59,6 @@ __device__ __forceinline__ void pencil_pass(C* s, int count, int stride, BaseF b
 #pragma unroll
     for (int k = 0; k < N; ++k) s[b + k * stride] = x[k];
   }
-}
-
-template <int N1, int N2, int N3, int DIR, typename C>
-__device__ __forceinline__ void fft3_smem(C* s) {
-  using L = RowLayout<N1, N2, N3>;
-  pencil_pass<N3, DIR>(s, N1 * N2, 1, [](int p) { return p * L::S2; });
-  __syncthreads();
-  pencil_pass<N2, DIR>(s, N1 * N3, L::S2, [](int p) { return (p / N3) * L::S1 + (p % N3); });
-  __syncthreads();
-  pencil_pass<N1, DIR>(s, N2 * N3, L::S1, [](int p) { return (p / N3) * L::S2 + (p % N3); });
-  __syncthreads();
 }
 
 }  // namespace gw
