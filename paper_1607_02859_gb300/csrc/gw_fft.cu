@@ -1533,6 +1533,7 @@ gw_status index_maps(gw_ctx* ctx, const GridInfo& g, const int32_t* fft_index_h,
   if (!fft_index_h) return fail(ctx, GW_ERR_ARG, "fft_index_h is NULL");
   if (n_chi < 1 || n_chi > g.nr) return fail(ctx, GW_ERR_SHAPE, "need 1 <= n_chi <= N_r");
   map.assign(fft_index_h, fft_index_h + n_chi);
+  inv.reserve(inv_ints(g));
   inv.assign(g.nr, -1);
   for (int j = 0; j < n_chi; ++j) {
     if (map[j] < 0 || map[j] >= g.nr) return fail(ctx, GW_ERR_ARG, "fft_index out of range");
@@ -1545,23 +1546,37 @@ gw_status index_maps(gw_ctx* ctx, const GridInfo& g, const int32_t* fft_index_h,
 
 void set_lists(const GridInfo& g, std::vector<int>& inv) {
   inv.resize(g.nr);
-  const int pl = g.n2 * g.n3;
-  std::vector<char> c23(pl, 0), c12((size_t)g.n1 * g.n2, 0), u1(g.n1, 0), u2(g.n2, 0), u3(g.n3, 0);
-  for (int p = 0; p < g.nr; ++p) {
-    if (inv[p] < 0) continue;
-    const int i1 = p / pl, i2 = p % pl / g.n3, i3 = p % g.n3;
-    c23[p % pl] = c12[i1 * g.n2 + i2] = u1[i1] = u2[i2] = u3[i3] = 1;
+  const int pl = g.n2 * g.n3, n12 = g.n1 * g.n2;
+  const int sizes[5] = {pl, n12, g.n1, g.n2, g.n3};
+  std::vector<char> marks((size_t)pl + n12 + g.n1 + g.n2 + g.n3, 0);
+  char *c23 = marks.data(), *c12 = c23 + pl, *u1 = c12 + n12, *u2 = u1 + g.n1, *u3 = u2 + g.n2;
+  // Every entry point with a G set pays for this walk over the grid, so no division and no branch per
+  // point: with three of the former and five marks a call with the whole set of 24^3 took 0.09 ms longer.
+  const int* at_p = inv.data();
+  for (int e = 0; e < n12; ++e) {
+    char* c = c23 + e % g.n2 * g.n3;
+    char any = 0;
+    for (int i3 = 0; i3 < g.n3; ++i3) {
+      const char in = *at_p++ >= 0;
+      c[i3] |= in;
+      any |= in;
+    }
+    c12[e] = any;
+    u1[e / g.n2] |= any;
+  }
+  for (int e = 0; e < pl; ++e) {
+    u2[e / g.n3] |= c23[e];
+    u3[e % g.n3] |= c23[e];
   }
   inv.resize(inv_ints(g), 0);
   int* x = inv.data() + g.nr;
   int* at = x + kSetHead;
-  int head = 0;
-  for (const std::vector<char>* v : {&c23, &c12, &u1, &u2, &u3}) {
+  const char* m = c23;
+  for (int v = 0; v < 5; m += sizes[v], at += sizes[v], ++v) {
     int count = 0;
-    for (size_t i = 0; i < v->size(); ++i)
-      if ((*v)[i]) at[count++] = (int)i;
-    x[head++] = count;
-    at += v->size();
+    for (int i = 0; i < sizes[v]; ++i)
+      if (m[i]) at[count++] = i;
+    x[v] = count;
   }
 }
 
