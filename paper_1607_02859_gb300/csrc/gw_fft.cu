@@ -83,16 +83,20 @@ __device__ __forceinline__ int low_last_bwd(int low, long row, int nr) {
   return min(nr - 1, (g0 + 127) / 128 * 128 + 127);
 }
 
-// Threads and CTAs per SM of the one-CTA rows: two rounds of pencils (N1 N2 per
-// pass) for the larger grids, so that the registers of two or three CTAs fit an SM
-// and one row's loads overlap another's arithmetic.  FP64 is bound by its ALU.
+// Threads and CTAs per SM of the one-CTA rows (FP32): two or three CTAs on an SM, so
+// that one row's loads overlap another's arithmetic.  Two rounds of pencils (N1 N2 per
+// pass) for the middle grids; from 24^3, where two rows fill an SM's shared memory, as
+// many threads as the registers of two CTAs allow, which hides more latency than even
+// rounds: 4096 rows onto 4097 G vectors 222 -> 203 us, from them 203 -> 189, the
+// triangle rows of 4 times 2.18 -> 1.90 ms.  At 20^3 and 16^3 512 threads are slower
+// (triangle rows 0.91 -> 0.94, 0.24 -> 0.29 ms).  FP64 is bound by its ALU.
 template <typename T, int N1, int N2, int N3>
 struct RowCfg {
   static constexpr int PC = N1 * N2;
   static constexpr bool F32 = sizeof(T) == 4;
   static constexpr int NR = N1 * N2 * N3;
-  static constexpr int TH = F32 ? (NR >= 4096 ? ((PC / 2 + 31) / 32 * 32 < 64 ? 64 : (PC / 2 + 31) / 32 * 32)
-                                              : ((PC + 31) / 32 * 32))
+  static constexpr int TH = F32 ? (NR >= 13824 ? 512 : NR >= 4096 ? ((PC / 2 + 31) / 32 * 32 < 64 ? 64 : (PC / 2 + 31) / 32 * 32)
+                                                           : ((PC + 31) / 32 * 32))
                                 : (NR >= 4096 ? 512 : 256);
   static constexpr int MINB = F32 ? (NR >= 13824 ? 2 : (NR >= 4096 ? 3 : 4)) : 1;
 };
@@ -101,6 +105,7 @@ struct RowCfg {
 // MODE 2: scatter a[j] to fft positions, backward (-i), times scale.   (Eq. FFTW, 2nd step)
 // VI / VO: the grid side / the G-set side (mode 1) moves as 16-byte pairs of
 // elements (aligned rows of even length), four pairs in flight per thread.
+// LOW: rows of a triangle (low >= 0); whole rows are compiled without its checks.
 //
 // The three passes over the row do only what the G set (lists) and the triangle
 // (low) need: forward the planes i1 <= i1(r), of them the i3 of the set in the i2
@@ -110,7 +115,7 @@ struct RowCfg {
 // That is 0.44 of a whole row's pencils at 24^3 with n_chi = 4097; the rows of one
 // tau went from 790 to 560 us there (scalar loads for the odd n_chi before), from
 // 250 to 172 us at 20^3 with n_chi = 1536.  Bound by instruction issue.
-template <typename T, int N1, int N2, int N3, int MODE, bool VI, bool VO>
+template <typename T, int N1, int N2, int N3, int MODE, bool VI, bool VO, bool LOW>
 __global__ void __launch_bounds__(RowCfg<T, N1, N2, N3>::TH, RowCfg<T, N1, N2, N3>::MINB)
     row_fft_kernel(const typename cpx<T>::t* __restrict__ a, long lda, typename cpx<T>::t* __restrict__ out, long ldo,
                    const int* __restrict__ map, const int* __restrict__ inv, int n_chi, T scale, int low) {
@@ -123,7 +128,7 @@ __global__ void __launch_bounds__(RowCfg<T, N1, N2, N3>::TH, RowCfg<T, N1, N2, N
   const long row = blockIdx.x;
   const SetLists<N1, N2, N3> g(inv);
   if constexpr (MODE == 2) {
-    const int i1m = low_last_bwd(low, row, L::NR) / PL + 1;      // planes to deliver
+    const int i1m = LOW ? low_last_bwd(low, row, L::NR) / PL + 1 : N1;   // planes to deliver
     for (int e = threadIdx.x; e < L::TOT; e += THREADS) s[e] = mk(T(0), T(0));
     __syncthreads();
     const C* src = a + row * lda;
@@ -185,7 +190,7 @@ __global__ void __launch_bounds__(RowCfg<T, N1, N2, N3>::TH, RowCfg<T, N1, N2, N
     }
     return;
   }
-  const int last = low_last_fwd(low, row, L::NR);
+  const int last = LOW ? low_last_fwd(low, row, L::NR) : L::NR - 1;
   const int i1m = last / PL + 1;                                 // planes with an element R' <= r
   const C* pa = a + row * lda;
   if (VI) {
@@ -1221,11 +1226,16 @@ struct GridOps {
         return launch_check(ctx, "row_fft_kernel");
       };
       constexpr bool E = N3 % 2 == 0;
-      if (mode == 1)
-        return vi ? (vo ? go(row_fft_kernel<T, N1, N2, N3, 1, E, true>) : go(row_fft_kernel<T, N1, N2, N3, 1, E, false>))
-                  : go(row_fft_kernel<T, N1, N2, N3, 1, false, false>);
-      if (mode == 2) return vi ? go(row_fft_kernel<T, N1, N2, N3, 2, E, false>)
-                               : go(row_fft_kernel<T, N1, N2, N3, 2, false, false>);
+      auto with_low = [&](auto low_c) -> gw_status {
+        constexpr bool LOW = decltype(low_c)::value;
+        if (mode == 1)
+          return vi ? (vo ? go(row_fft_kernel<T, N1, N2, N3, 1, E, true, LOW>)
+                          : go(row_fft_kernel<T, N1, N2, N3, 1, E, false, LOW>))
+                    : go(row_fft_kernel<T, N1, N2, N3, 1, false, false, LOW>);
+        return vi ? go(row_fft_kernel<T, N1, N2, N3, 2, E, false, LOW>)
+                  : go(row_fft_kernel<T, N1, N2, N3, 2, false, false, LOW>);
+      };
+      if (mode == 1 || mode == 2) return low >= 0 ? with_low(std::true_type{}) : with_low(std::false_type{});
     }
     return fail(ctx, GW_ERR_ARG, "bad row transform mode");
   }
