@@ -288,6 +288,13 @@ struct PlaneCfg {
   static constexpr int LB = sizeof(T) == 4 ? 256 : 128, LBB = 2;
   // the longest G-set row that the line kernels stage in shared memory (two CTAs per SM)
   static constexpr size_t kStage = 110 * 1024;
+  // Beyond it the forward kernel scatters single values into the row in global memory, and L2 has to
+  // join the 8-byte ones of FP32 to sectors before they leave: one CTA per SM (kAlone bytes of shared
+  // memory keep a second one out), so that the rows in flight, 152 of 373 KB at 36^3, stay there.  1024
+  // rows at 36^3 with three CTAs per SM and with one: 20000 G vectors 458 and 351 us, all 46656 1059 and
+  // 680; FP64 keeps its two (512 rows, 7041 G vectors: 1700 us, 1747 with one).
+  static constexpr int LFU = sizeof(T) == 4 ? 3 * LF : LF, LFUB = sizeof(T) == 4 ? 1 : LFB;
+  static constexpr size_t kAlone = sizeof(T) == 4 ? 120 * 1024 : 0;
 };
 
 // One i3 pencil of a plane in shared memory, transformed in place; the elements of mask are written.
@@ -409,11 +416,12 @@ __global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::TH, PlaneCfg<T, N1, N
 // Forward line pass of one row per CTA: i1 transforms (+i) of the set's columns,
 // the results to out[row][inv], in order through shared memory where STAGE.
 template <typename T, int N1, int N2, int N3, bool STAGE>
-__global__ void __launch_bounds__(PlaneCfg<T, N1, N2, N3>::LF, PlaneCfg<T, N1, N2, N3>::LFB)
+__global__ void __launch_bounds__(STAGE ? PlaneCfg<T, N1, N2, N3>::LF : PlaneCfg<T, N1, N2, N3>::LFU,
+                                  STAGE ? PlaneCfg<T, N1, N2, N3>::LFB : PlaneCfg<T, N1, N2, N3>::LFUB)
     row_line_fwd_kernel(const typename cpx<T>::t* t, long t_row, long t_plane, typename cpx<T>::t* __restrict__ out,
                         long ldo, const int* __restrict__ inv, int n_chi, int low) {
   using C = typename cpx<T>::t;
-  constexpr int PL = N2 * N3, LT = PlaneCfg<T, N1, N2, N3>::LF;
+  constexpr int PL = N2 * N3, LT = STAGE ? PlaneCfg<T, N1, N2, N3>::LF : PlaneCfg<T, N1, N2, N3>::LFU;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* so = reinterpret_cast<C*>(smem_raw);                          // [n_chi]
   const long row = blockIdx.x;
@@ -1134,15 +1142,15 @@ struct GridOps {
   static gw_status line_fwd(gw_ctx* ctx, const void* t, long t_row, long t_plane, void* out, long ldo, const int* inv,
                             int n_chi, int n_rows, int low, double work, int fam, cudaStream_t st) {
     const size_t bytes = (size_t)n_chi * sizeof(C);
-    auto go = [&](auto kernel, size_t sm) -> gw_status {
+    auto go = [&](auto kernel, size_t sm, int threads) -> gw_status {
       gw_status r = set_smem(ctx, kernel, sm);
       if (r) return r;
       KTimer kt(ctx, fam, work, st);
-      kernel<<<n_rows, PC::LF, sm, st>>>((const C*)t, t_row, t_plane, (C*)out, ldo, inv, n_chi, low);
+      kernel<<<n_rows, threads, sm, st>>>((const C*)t, t_row, t_plane, (C*)out, ldo, inv, n_chi, low);
       return launch_check(ctx, "row_line_fwd_kernel");
     };
-    return bytes <= PC::kStage ? go(row_line_fwd_kernel<T, N1, N2, N3, true>, bytes)
-                               : go(row_line_fwd_kernel<T, N1, N2, N3, false>, 0);
+    return bytes <= PC::kStage ? go(row_line_fwd_kernel<T, N1, N2, N3, true>, bytes, PC::LF)
+                               : go(row_line_fwd_kernel<T, N1, N2, N3, false>, PC::kAlone, PC::LFU);
   }
   static gw_status line_bwd(gw_ctx* ctx, const void* a, long lda, void* t, long t_row, long t_plane, const int* inv,
                             int n_chi, int n_rows, int low, bool fwd_rows, double work, int fam, cudaStream_t st) {
