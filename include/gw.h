@@ -87,6 +87,11 @@ size_t gw_ctx_scratch_bytes(const gw_ctx* ctx);
  * synchronises the device; a smaller request does nothing.  GW_ERR_OOM if the
  * allocation fails (the arena is then empty). */
 gw_status gw_ctx_reserve(gw_ctx* ctx, size_t bytes);
+/* Failure injection on the host, for tests: after the product-th tensor-core G
+ * formation that ctx launches from now on (1: the next one; 0: none) the time-out
+ * words of that product's call are set as a bounded wait that gave up sets them,
+ * so that the call has to return GW_ERR_TIMEOUT.  Not while a stream is captured. */
+gw_status gw_ctx_inject_timeout(gw_ctx* ctx, int product);
 /* Per-kernel timing for benchmarks.  While enabled, the library brackets every
  * launch of its main kernels with CUDA events on the launch stream and records,
  * per kernel family, the number of launches, their summed device time and their

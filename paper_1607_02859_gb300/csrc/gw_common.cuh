@@ -28,6 +28,7 @@ struct gw_ctx {
   unsigned long long launches = 0;
   int* dflag = nullptr;        // device status word written by kernels
   int num_sms = 0;
+  int inject_timeout = 0;      // tests: G formations until one records a time-out (0: none)
   // opt-in per-launch timing of the main kernels
   bool timing = false;
   std::vector<gw_krec> pending;

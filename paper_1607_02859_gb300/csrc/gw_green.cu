@@ -101,6 +101,7 @@ extern "C" gw_status gw_green_tau(gw_ctx* ctx, const gw_grid* grid, int n_b, int
   GreenScales gs = green_scales(eps_h, n_b, n_occ, mu, tau);
   if (prec == GW_F16X3 || prec == GW_BF16X3) {
     if ((st = reserve(ctx, tc_scratch_bytes(g, n_b, n_occ, n_rows, !g_occ || !g_unocc)))) return st;
+    if ((st = tc_begin(ctx, ctx->arena, s))) return st;
     if ((st = tc_green_rows(ctx, g, n_b, n_occ, psi, &gs, r0, n_rows, prec, g_occ, g_unocc, ctx->arena, true, s)))
       return st;
     return tc_check(ctx, ctx->arena, s);
@@ -122,6 +123,7 @@ extern "C" gw_status gw_chi0_rtau_fused(gw_ctx* ctx, const gw_grid* grid, int n_
   GreenScales gs = green_scales(eps_h, n_b, n_occ, mu, tau);
   if (prec == GW_F16X3 || prec == GW_BF16X3) {
     if ((st = reserve(ctx, tc_scratch_bytes(g, n_b, n_occ, n_rows, false)))) return st;
+    if ((st = tc_begin(ctx, ctx->arena, s))) return st;
     if ((st = tc_chi_rows(ctx, g, n_b, n_occ, psi, &gs, r0, n_rows, prec, chi, ctx->arena, true, s))) return st;
     return tc_check(ctx, ctx->arena, s);
   }

@@ -212,6 +212,13 @@ extern "C" const char* gw_last_error(const gw_ctx* ctx) {
 extern "C" unsigned long long gw_ctx_launches(const gw_ctx* ctx) { return ctx ? ctx->launches : 0ull; }
 extern "C" size_t gw_ctx_scratch_bytes(const gw_ctx* ctx) { return ctx ? ctx->arena_bytes : 0; }
 
+extern "C" gw_status gw_ctx_inject_timeout(gw_ctx* ctx, int product) {
+  if (!ctx) return fail(nullptr, GW_ERR_ARG, "ctx is NULL");
+  if (product < 0) return fail(ctx, GW_ERR_ARG, "product must be >= 0");
+  ctx->inject_timeout = product;
+  return GW_OK;
+}
+
 extern "C" gw_status gw_ctx_reserve(gw_ctx* ctx, size_t bytes) {
   if (!ctx) return fail(nullptr, GW_ERR_ARG, "ctx is NULL");
   return reserve(ctx, bytes);

@@ -346,6 +346,7 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   if ((st = upload(ctx, dsinv, sinv.data(), sizeof(int) * sinv.size(), s))) return st;
   if ((st = upload_phases(ctx, dph, kl_phases(nk), prec, s))) return st;
   if ((st = fill_q_phases(ctx, prec, g, nk, dqph, s))) return st;
+  if (tc && (st = tc_begin(ctx, tcs, s))) return st;
   const double fac = g.dv * g.dv / g.volume;   // Eq. FFTX2 normalisation
   std::vector<float> cw32;
   if (is_fp64(prec)) {
@@ -522,6 +523,7 @@ extern "C" gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, co
     if ((st = upload(ctx, dcw, cw32.data(), sizeof(float) * 2 * n * n, s))) return st;
   }
   if ((st = fill_q_phases(ctx, prec, g, nk, dqph, s))) return st;
+  if (tc && (st = tc_begin(ctx, tcs, s))) return st;
   // the coefficients of u_ak over the set for every k (checked to span every band)
   for (int k = 0; k < n_k; ++k) {
     const int kv[3] = {k / (nk[1] * nk[2]), (k / nk[2]) % nk[1], k % nk[2]};
@@ -673,6 +675,7 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   if ((st = upload(ctx, dbk, bk.data(), sizeof(int) * 3 * n_n, s))) return st;
   if ((st = upload_phases(ctx, dph, kl_phases(nk), prec, s))) return st;
   if ((st = fill_q_phases(ctx, prec, g, nk, dqph, s))) return st;
+  if (tc && (st = tc_begin(ctx, tcs, s))) return st;
   if ((st = upload(ctx, tab, C_h, sizeof(double) * n * n, s))) return st;
   if ((st = upload(ctx, tab + (size_t)n * n, S_h, sizeof(double) * n * n, s))) return st;
   if ((st = upload(ctx, tab + 2 * (size_t)n * n, omega_h, sizeof(double) * n, s))) return st;

@@ -147,6 +147,7 @@ static gw_status chi0_launch(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ,
   char* ga = cv.take<char>(chi_rows_elems(g, sh) * es);
   void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, sh.nt)) : nullptr;
   if (tcs_out) *tcs_out = tcs;
+  if (tc && (st = tc_begin(ctx, tcs, s, t.status))) return st;
   bool first = true;
   for (int j0 = 0; j0 < n; j0 += sh.nt) {
     const int nt = std::min(sh.nt, n - j0);
@@ -427,6 +428,7 @@ extern "C" gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
     for (int j = 0; j < n; ++j)
       if ((st = upload_scales(ctx, dscale + (size_t)j * n_b * 8, scales[j], prec, s))) return st;
   if ((st = pw_coefficients(ctx, g, prec, psi, n_b, n_pw, dmap_pw, dinv_pw, dc, dnorm, to, n_pw, s))) return st;
+  if (tc && (st = tc_begin(ctx, tcs, s))) return st;
   bool first = true;
   for (int j = 0; j < n; ++j) {
     // Mc_occ, Mc_unocc over the plane-wave set, then their column transforms T(r, g')

@@ -624,6 +624,7 @@ gw_status sigma_kernels(gw_ctx* ctx, const GridInfo& g, gw_prec prec, bool full,
   double2* accm_u = t.acc2;
   double2* accm_o = t.acc2 + nnm * n;
   const double coef = g.dv * g.dv / g.volume;   // dV^2 and the 1/Omega of Eq. FFTW
+  if (tc && (st = tc_begin(ctx, w.tcs, s))) return st;
   bool first = true;
   for (int j = 0; j < n; ++j) {
     const char* wj = static_cast<const char*>(w_tau) + (size_t)j * n_chi * n_chi * es;
@@ -904,6 +905,7 @@ extern "C" gw_status gw_sigma_diag_pw(gw_ctx* ctx, const gw_grid* grid, int n_b,
   double* acc_u = reinterpret_cast<double*>(t.acc2);
   double* acc_o = acc_u + (size_t)n_n * n;
   const double coef = g.dv * g.dv / g.volume;   // dV^2 and the 1/Omega of Eq. FFTW
+  if (tc && (st = tc_begin(ctx, tcs, s))) return st;
   bool first = true;
   for (int j = 0; j < n; ++j) {
     const char* sj = t.scale + (size_t)j * n_b * 8;

@@ -1039,6 +1039,8 @@ static size_t scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, b
   return Carver::round(probe.off);
 }
 
+static int* status_words(void* scratch) { return static_cast<int*>(scratch) + 2; }
+
 // One G/chi formation for rows r0 .. r0+n_rows-1 using `scratch` (of at least
 // scratch_bytes()).  mode 0: chi into out0; mode 1: G_occ into out0 and G_unocc
 // into out1 (a NULL one goes to scratch).  prep_b = false reuses the B operand
@@ -1061,7 +1063,7 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
   unsigned int* dmax = words + 64;
   int* dexp = reinterpret_cast<int*>(words + 64 + kMaxEntries);
   // time-out status: in the scratch, or in a word the caller owns (kept past later uses of the scratch)
-  int* status = status_dev ? status_dev : reinterpret_cast<int*>(words + 2);
+  int* status = status_dev ? status_dev : status_words(scratch);
   uint16_t* bop = cv.take<uint16_t>(nbb * 2 * g.nr * 2 * L.kpad);
   // these operands are prepared by the first call and read by later ones: their place must not
   // depend on this call's number of rows or entries, so they come before what does
@@ -1086,9 +1088,7 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
   const dim3 tb(32, 8);
   const int slots = L.kpad / 2;
   if (prep_b) {
-    if ((rc = cuda_check(ctx, cudaMemsetAsync(words, 0, kWords * sizeof(unsigned int), st), "memset"))) return rc;
-    if (status_dev && (rc = cuda_check(ctx, cudaMemsetAsync(status_dev, 0, 2 * sizeof(int), st), "memset")))
-      return rc;
+    if ((rc = cuda_check(ctx, cudaMemsetAsync(dmax, 0, nbb * sizeof(unsigned int), st), "memset"))) return rc;
     const size_t nel = (size_t)n_b * g.nr;
     maxabs_kernel<<<dim3((unsigned)std::min<size_t>((nel + 255) / 256, (size_t)ctx->num_sms * 8 / nbb + 1), nbb), 256, 0,
                     st>>>(static_cast<const float2*>(psi), nel, en.psi_stride, dmax);
@@ -1195,13 +1195,15 @@ static gw_status run(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const v
   if (mode == 0) rc = fmt == 0 ? go(green_tc_kernel<0, 0>) : go(green_tc_kernel<0, 1>);
   else if (mode == 1) rc = fmt == 0 ? go(green_tc_kernel<1, 0>) : go(green_tc_kernel<1, 1>);
   else rc = fmt == 0 ? go(green_tc_kernel<2, 0>) : go(green_tc_kernel<2, 1>);
+  if (!rc && ctx->inject_timeout > 0 && --ctx->inject_timeout == 0)
+    rc = cuda_check(ctx, cudaMemsetAsync(status, 1, 2 * sizeof(int), st), "memset");
   return rc;
 }
 
 // Reads the status word the kernels' bounded waits write (synchronises the stream).
 static gw_status check_status(gw_ctx* ctx, void* scratch, cudaStream_t st) {
   int hs[2] = {0, 0};
-  const int* status = reinterpret_cast<const int*>(static_cast<const unsigned int*>(scratch) + 2);
+  const int* status = status_words(scratch);
   gw_status rc;
   if ((rc = cuda_check(ctx, cudaMemcpyAsync(hs, status, sizeof(hs), cudaMemcpyDeviceToHost, st), "status"))) return rc;
   if ((rc = cuda_check(ctx, cudaStreamSynchronize(st), "tensor-core GEMM"))) return rc;
@@ -1214,6 +1216,11 @@ static gw_status check_status(gw_ctx* ctx, void* scratch, cudaStream_t st) {
 size_t tc_scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, bool with_tmp, int n_sig, int n_entries,
                         bool one_psi) {
   return tc::scratch_bytes(g, n_b, n_occ, n_rows, with_tmp, n_sig, n_entries, one_psi);
+}
+
+gw_status tc_begin(gw_ctx* ctx, void* scratch, cudaStream_t st, int* status_dev) {
+  return cuda_check(ctx, cudaMemsetAsync(status_dev ? status_dev : tc::status_words(scratch), 0, 2 * sizeof(int), st),
+                    "memset");
 }
 
 gw_status tc_sigma_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi, const GreenScales& gs,

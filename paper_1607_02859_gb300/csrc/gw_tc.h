@@ -19,6 +19,10 @@ struct TcEntries {
 // caller did not supply; one_psi: psi_stride 0).
 size_t tc_scratch_bytes(const GridInfo& g, int n_b, int n_occ, int n_rows, bool with_tmp, int n_sig = 0,
                         int n_entries = 1, bool one_psi = true);
+// Clears the time-out words that the calls below record in `scratch` (or the caller's
+// own, status_dev), once per entry point before its first product: preparing an operand
+// leaves them alone, so that a time-out of any product is there for tc_check.
+gw_status tc_begin(gw_ctx* ctx, void* scratch, cudaStream_t st, int* status_dev = nullptr);
 // G_occ / G_unocc rows as 3 fp16 (or bf16) split products on tcgen05 with FP32
 // accumulation in tensor memory.  Either output may be NULL (one entry only).
 // prep_b = false reuses the psi-only operand an earlier call left in the same scratch.
@@ -62,7 +66,7 @@ gw_status tc_sigma_rows(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, cons
 // As tc_check for a status word the caller owns (status_dev of tc_chi_rows).
 gw_status tc_check_status(gw_ctx* ctx, const int* status_dev, cudaStream_t st);
 // Synchronises and reports a time-out of the tensor-core pipeline waits
-// (GW_ERR_TIMEOUT) recorded in `scratch` since its last prep_b call.
+// (GW_ERR_TIMEOUT) recorded in `scratch` since tc_begin.
 gw_status tc_check(gw_ctx* ctx, void* scratch, cudaStream_t st);
 
 // 2-D TMA map over a [rows][kpad] row-major 16-bit array (fmt 0: fp16, 1: bf16),

@@ -24,6 +24,7 @@ STATUS = {0: "GW_OK", 1: "GW_ERR_ARG", 2: "GW_ERR_SHAPE", 3: "GW_ERR_OOM", 4: "G
 
 # every symbol declared in include/gw.h
 EXPORTS = ["gw_ctx_create", "gw_ctx_destroy", "gw_last_error", "gw_ctx_launches", "gw_ctx_scratch_bytes", "gw_ctx_reserve",
+           "gw_ctx_inject_timeout",
            "gw_ctx_set_timing", "gw_ctx_kernel_stats", "gw_version", "gw_g_set", "gw_coulomb_sqrt", "gw_fit_transform", "gw_green_tau", "gw_chi0_rtau",
            "gw_chi0_rtau_fused", "gw_rr_to_GG_fft", "gw_tau_to_omega", "gw_screen_W", "gw_sigma_diag",
            "gw_chi0_omega", "gw_rr_to_GG_fft_noalloc", "gw_workspace_size", "gw_screen_W_refine", "gw_chi0_omega_kmesh", "gw_sigma_diag_kmesh",
@@ -68,6 +69,7 @@ _SIGS = {
     "gw_ctx_launches": (ct.c_ulonglong, [_P]),
     "gw_ctx_scratch_bytes": (ct.c_size_t, [_P]),
     "gw_ctx_reserve": (ct.c_int, [_P, ct.c_size_t]),
+    "gw_ctx_inject_timeout": (_I, [_P, _I]),
     "gw_version": (_I, []),
     "gw_ctx_set_timing": (_I, [_P, _I]),
     "gw_ctx_kernel_stats": (_I, [_P, ct.c_char_p, ct.POINTER(ct.c_ulonglong), _DP, _DP, ct.POINTER(ct.c_int)]),
@@ -201,6 +203,10 @@ class Context:
     def reserve(self, nbytes: int):
         """Grow the scratch arena to at least nbytes now (synchronises the device when it grows)."""
         _check(lib().gw_ctx_reserve(self.handle, int(nbytes)), self)
+
+    def inject_timeout(self, product: int):
+        """Have the product-th tensor-core G formation from now record a time-out (tests; 0: none)."""
+        _check(lib().gw_ctx_inject_timeout(self.handle, int(product)), self)
 
     FAMILIES = ("green_tc", "cgemm_tc", "cgemm_simt", "row_fft", "col_fft", "col_line_ct", "sigma_contract", "ct",
                 "cgemm_exact", "row_pw")
