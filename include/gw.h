@@ -461,7 +461,10 @@ gw_status gw_sigma_diag_pw(gw_ctx* ctx, const gw_grid* grid, int n_b, int n_occ,
  * ascending per k with mu in every gap.  gvec_h [n_chi][3]: the cell G set as
  * integer triples with g_d in [-n_d/2, n_d/2).  At most 64 k points; the
  * supercell grid nk[d] n_d must be one the library compiles.  r_block <= 0
- * picks a default.  The result is the q-diagonal block of the Gamma-point
+ * picks a default.  Scratch (context arena): the slabs (N_r N_k n_chi n elements),
+ * 2 N_k N_r r_block elements of G rows and r_block supercell rows; the tensor-core
+ * operands hold as many k points as fit in as much memory again (at least one).
+ * The result is the q-diagonal block of the Gamma-point
  * chi0 of the supercell holding the N_k cells. */
 gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const int* nk, int n_b, int n_occ,
                               const void* psi_k, const double* eps_k_h, double mu, int n,

@@ -259,6 +259,39 @@ static gw_status launch_stripe(gw_ctx* ctx, gw_prec prec, const GridInfo& g, con
   return go(stripe_chi_kernel<float, PRODUCT>, (float2*)nullptr);
 }
 
+// k points per launch of the tensor-core G formation: all, so that their psi-only
+// operands are prepared once per call, while the operands take no more than the rest of
+// the call's scratch (`rest` bytes); beyond that even groups, prepared anew for every
+// launch as with one k at a time.  A 12^3 cell on 4 x 4 x 4 with 500 bands: 1.2 GB for
+// all k, beside 4 GB of slabs and G rows by default, but 0.3 GB with 64-row blocks.
+static int k_group(const GridInfo& g, int n_b, int n_occ, int rb, int n_k, size_t rest) {
+  int m = n_k;
+  while (m > 1 && tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, m, false) > rest) --m;
+  const int groups = (n_k + m - 1) / m;
+  return (n_k + groups - 1) / groups;
+}
+
+// G_occ and G_unocc rows of every k, kg at a time; scale: the band factors of all k as
+// FP32.  first: the call's first rows, where the operands of a single group are prepared.
+static gw_status green_of_k(gw_ctx* ctx, const GridInfo& g, int n_b, int n_occ, const void* psi_k,
+                            const std::vector<GreenScales>& scales, int kg, int r0, int rows, gw_prec prec, char* gok,
+                            char* guk, long kstr, void* tcs, bool first, const char* scale, cudaStream_t s) {
+  const int n_k = (int)scales.size();
+  const size_t es = csize(prec);
+  for (int k = 0; k < n_k; k += kg) {
+    TcEntries en;
+    en.n = std::min(kg, n_k - k);
+    en.psi_stride = en.n > 1 ? (long)n_b * g.nr : 0;
+    en.out_stride = kstr;
+    const gw_status st = tc_green_rows(ctx, g, n_b, n_occ, static_cast<const char*>(psi_k) + (size_t)k * n_b * g.nr * es,
+                                       &scales[k], r0, rows, prec, gok + (size_t)k * kstr * es,
+                                       guk + (size_t)k * kstr * es, tcs, first || kg < n_k, s,
+                                       reinterpret_cast<const float*>(scale) + (size_t)k * n_b, en);
+    if (st) return st;
+  }
+  return GW_OK;
+}
+
 // The phase table of a call: N_r N_k complex numbers at tab.
 static gw_status fill_q_phases(gw_ctx* ctx, gw_prec prec, const GridInfo& g, const int* nk, void* tab, cudaStream_t s) {
   const int blocks = (g.nr * nk[0] * nk[1] * nk[2] + 127) / 128;
@@ -323,7 +356,8 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   probe.take<char>((size_t)n_k * rb * g.nr * es);
   probe.take<char>((size_t)rb * gs.nr * es);
   if (two_pass) probe.take<char>((size_t)rb * gs.nr * es);
-  if (tc) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, n_k, n_k == 1));
+  const int kg = tc ? k_group(g, n_b, n_occ, rb, n_k, probe.off) : n_k;
+  if (tc) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, kg, kg == 1));
   if ((st = reserve(ctx, probe.off))) return st;
   Carver cv(ctx->arena);
   int* dmap = cv.take<int>(n_chi);
@@ -339,7 +373,7 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   char* guk = cv.take<char>((size_t)n_k * rb * g.nr * es);
   char* rows_s = cv.take<char>((size_t)rb * gs.nr * es);
   char* tmp_s = two_pass ? cv.take<char>((size_t)rb * gs.nr * es) : nullptr;
-  void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, n_k, n_k == 1)) : nullptr;
+  void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, kg, kg == 1)) : nullptr;
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
   if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if ((st = upload(ctx, dsmap, smap.data(), sizeof(int) * n_k * n_chi, s))) return st;
@@ -372,15 +406,9 @@ extern "C" gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const
     char* slab_j = slabs + (size_t)j * slab * es;
     for (int r0 = 0; r0 < g.nr; r0 += rb) {
       const int rows = std::min(rb, g.nr - r0);
-      if (tc) {                    // every k in one launch; their psi-only operands are prepared once
-        TcEntries en;
-        en.n = n_k;
-        en.psi_stride = n_k > 1 ? (long)n_b * g.nr : 0;
-        en.out_stride = kstr;
-        if ((st = tc_green_rows(ctx, g, n_b, n_occ, psi_k, scales.data(), r0, rows, prec, gok, guk, tcs,
-                                j == 0 && r0 == 0, s, reinterpret_cast<const float*>(dscale), en)))
-          return st;
-      }
+      if (tc && (st = green_of_k(ctx, g, n_b, n_occ, psi_k, scales, kg, r0, rows, prec, gok, guk, kstr, tcs,
+                                 j == 0 && r0 == 0, dscale, s)))
+        return st;
       for (int k = 0; k < n_k && !tc; ++k) {
         const char* pk = static_cast<const char*>(psi_k) + (size_t)k * n_b * g.nr * es;
         if ((st = green_rows(ctx, g, n_b, n_occ, pk, dscale + (size_t)k * n_b * 8, scales[k], r0, rows, prec,
@@ -640,7 +668,8 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   probe.take<char>((size_t)n_k * rb * g.nr * es);
   probe.take<char>(3 * (size_t)rb * gs.nr * es);
   probe.take<char>((size_t)n_n * (gs.nr + g.nr) * es);
-  if (tc) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, n_k, n_k == 1));
+  const int kg = tc ? k_group(g, n_b, n_occ, rb, n_k, probe.off) : n_k;
+  if (tc) probe.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, kg, kg == 1));
   if ((st = reserve(ctx, probe.off))) return st;
   Carver cv(ctx->arena);
   int* dmap = cv.take<int>(n_chi);
@@ -664,7 +693,7 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
   char* w_s = gu_s + (size_t)rb * gs.nr * es;
   char* ext = cv.take<char>((size_t)n_n * (gs.nr + g.nr) * es);
   char* prow = ext + (size_t)n_n * gs.nr * es;
-  void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, n_k, n_k == 1)) : nullptr;
+  void* tcs = tc ? cv.take<char>(tc_scratch_bytes(g, n_b, n_occ, rb, false, 0, kg, kg == 1)) : nullptr;
   if ((st = upload(ctx, dmap, map.data(), sizeof(int) * n_chi, s))) return st;
   if ((st = upload(ctx, dinv, inv.data(), sizeof(int) * inv.size(), s))) return st;
   if ((st = upload(ctx, dsmap, smap.data(), sizeof(int) * n_k * n_chi, s))) return st;
@@ -716,15 +745,9 @@ extern "C" gw_status gw_sigma_diag_kmesh(gw_ctx* ctx, const gw_grid* grid, const
     if ((st = launch_q_phase(ctx, prec, g, nk, dqph, wrg, ld, n_chi, +1.0, s))) return st;
     for (int r0 = 0; r0 < g.nr; r0 += rb) {
       const int rows = std::min(rb, g.nr - r0);
-      if (tc) {                    // every k in one launch; their psi-only operands are prepared once
-        TcEntries en;
-        en.n = n_k;
-        en.psi_stride = n_k > 1 ? (long)n_b * g.nr : 0;
-        en.out_stride = kstr;
-        if ((st = tc_green_rows(ctx, g, n_b, n_occ, psi_k, scales.data(), r0, rows, prec, gok, guk, tcs,
-                                j == 0 && r0 == 0, s, reinterpret_cast<const float*>(dscale), en)))
-          return st;
-      }
+      if (tc && (st = green_of_k(ctx, g, n_b, n_occ, psi_k, scales, kg, r0, rows, prec, gok, guk, kstr, tcs,
+                                 j == 0 && r0 == 0, dscale, s)))
+        return st;
       for (int k = 0; k < n_k && !tc; ++k) {
         const char* pk = static_cast<const char*>(psi_k) + (size_t)k * n_b * g.nr * es;
         if ((st = green_rows(ctx, g, n_b, n_occ, pk, dscale + (size_t)k * n_b * 8, scales[k], r0, rows, prec,
