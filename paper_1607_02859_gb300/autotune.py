@@ -1,8 +1,9 @@
 """r-block autotuner for the chi0(i omega) pipeline.
 
 gw_chi0_omega walks the real-space rows r in blocks of r_block rows: each block
-holds 2 x r_block x N_r Green's-function slabs in the scratch arena (and, on the
-tensor-core path, the split operands).  Larger blocks feed the GEMMs and the row
+holds r_block x N_r values of chi(r,R') in the scratch arena, for several times
+where a block has few tiles (and, on the tensor-core path, the split operands).
+Larger blocks feed the GEMMs and the row
 FFTs bigger batches; smaller ones keep the working set in L2 and leave device
 memory to concurrent requests.  The tuner times chi0_omega for each candidate
 whose scratch fits the given budget (CUDA events on the launching stream, after

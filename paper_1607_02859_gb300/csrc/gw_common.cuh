@@ -46,6 +46,10 @@ gw_status cuda_check(gw_ctx* ctx, cudaError_t e, const char* what);
 gw_status launch_check(gw_ctx* ctx, const char* what);
 gw_status reserve(gw_ctx* ctx, size_t bytes);   // ensure arena >= bytes (syncs if it grows)
 
+// SMs of a GB300, for sizes that are fixed without a context (scratch figures on the
+// host); grids of kernels are sized by the device's own count.
+constexpr int kSms = 152;
+
 // Carves aligned pieces out of the context arena.
 struct Carver {
   char* base;

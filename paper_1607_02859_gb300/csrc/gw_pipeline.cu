@@ -32,7 +32,7 @@ static ChiShape chi_shape(const GridInfo& g, int n, gw_prec prec, int r_block) {
   const double t = (g.nr + edge - 1) / edge, blocks = (g.nr + c.rb - 1) / c.rb;
   const double tiles = 0.5 * t * (t + 1) / blocks;
   const double most = (512.0 * 1048576.0) / ((double)c.rb * g.nr * csize(prec));
-  c.nt = std::max(1, std::min({n, (int)std::ceil((tc ? 6 : 12) * 152 / tiles), (int)most}));
+  c.nt = std::max(1, std::min({n, (int)std::ceil((tc ? 6 : 12) * kSms / tiles), (int)most}));
   return c;
 }
 static size_t chi_rows_elems(const GridInfo& g, const ChiShape& c) { return (size_t)c.nt * c.rb * g.nr; }
