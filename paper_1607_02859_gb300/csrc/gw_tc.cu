@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kThreads<MODE>, 1) green_tc_kernel(const __gri
   constexpr int EW = kEpiWarps<MODE>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  float2* epi = reinterpret_cast<float2*>(smem + STAGES * STAGE_BYTES);     // [8 warps][32 rows][16]
+  float2* epi = reinterpret_cast<float2*>(smem + STAGES * STAGE_BYTES);     // [16 warps][32 rows][8]
   uint32_t* tile_tab = reinterpret_cast<uint32_t*>(smem + STAGES * STAGE_BYTES + EPI_BYTES);
   uint64_t* full = reinterpret_cast<uint64_t*>(tile_tab + kTileTab);
   uint64_t* empty = full + STAGES;
@@ -944,25 +944,7 @@ static EncodeFn encoder(gw_ctx* ctx, gw_status* st) {
   return fn;
 }
 
-// 2-D map over a [rows][kpad] 16-bit row-major array, box = 64 x box_rows, 128-byte swizzle.
 }  // namespace tc
-
-gw_status tc_make_map(gw_ctx* ctx, CUtensorMap* m, const void* base, int kpad, long rows, int box_rows,
-                      uint32_t fmt) {
-  using namespace tc;
-  gw_status st;
-  EncodeFn enc = encoder(ctx, &st);
-  if (!enc) return st;
-  cuuint64_t dims[2] = {(cuuint64_t)kpad, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)kpad * 2};
-  cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = enc(m, fmt == 0 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
-                   const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return fail(ctx, GW_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
-  return GW_OK;
-}
 
 gw_status tc_make_map3(gw_ctx* ctx, CUtensorMap* m, const void* base, int kpad, long rows, int batch, int box_rows,
                        uint32_t fmt, int box_k) {

@@ -69,12 +69,9 @@ gw_status tc_check_status(gw_ctx* ctx, const int* status_dev, cudaStream_t st);
 // (GW_ERR_TIMEOUT) recorded in `scratch` since tc_begin.
 gw_status tc_check(gw_ctx* ctx, void* scratch, cudaStream_t st);
 
-// 2-D TMA map over a [rows][kpad] row-major 16-bit array (fmt 0: fp16, 1: bf16),
-// box 64 x box_rows, 128-byte swizzle.
-gw_status tc_make_map(gw_ctx* ctx, CUtensorMap* m, const void* base, int kpad, long rows, int box_rows,
-                      uint32_t fmt);
-// Same over a [batch][rows][kpad] array (3-D map, box depth 1), with a box of
-// box_k elements along K and the matching swizzle (64 -> 128 B, 32 -> 64 B).
+// 3-D TMA map over a [batch][rows][kpad] row-major 16-bit array (fmt 0: fp16, 1: bf16),
+// box depth 1, box_rows rows and box_k elements along K, with the matching swizzle
+// (64 -> 128 B, 32 -> 64 B).
 gw_status tc_make_map3(gw_ctx* ctx, CUtensorMap* m, const void* base, int kpad, long rows, int batch, int box_rows,
                        uint32_t fmt, int box_k);
 
