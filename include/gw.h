@@ -415,10 +415,11 @@ gw_status gw_chi0_omega(gw_ctx* ctx, const gw_grid* grid, int n_b, int n_occ,
  * and CTX as in gw_chi0_omega.  Scratch (context arena): the slabs
  * (N_r n_chi n elements) plus 2 N_r n_pw + 2 n_pw^2 + N_b n_pw elements (8 or 16
  * bytes each), the columns between the row kernels (at most 1024 rows of 3 N_r
- * elements) and the tensor-core operands.  GW_ERR_UNSUPPORTED where two
- * expanded rows of the grid do not fit a thread-block cluster's shared memory
- * (GW_FP64 at 36^3, every precision at 48^3).  Synchronises the stream once
- * (the norm check). */
+ * elements) and the tensor-core operands.  GW_ERR_UNSUPPORTED beyond the sizes
+ * of the plane-wave route, those for which two expanded rows of the grid fit a
+ * thread-block cluster's shared memory as the rows of its self-energy need (not
+ * GW_FP64 at 36^3, no precision at 48^3).  Synchronises the stream once (the
+ * norm check). */
 gw_status gw_chi0_omega_pw(gw_ctx* ctx, const gw_grid* grid, int n_b, int n_occ, const void* psi,
                            const double* eps_h, double mu, int n, const double* tau_h, const double* C_h,
                            int n_chi, const int32_t* fft_index_h, int n_pw, const int32_t* pw_index_h,
@@ -486,9 +487,9 @@ gw_status gw_chi0_omega_kmesh(gw_ctx* ctx, const gw_grid* grid, const int* nk, i
  * arena): the slabs (N_r N_k n_chi n elements) plus 2 N_r N_k n_pw + 2 n_pw^2 +
  * N_k N_b n_pw + N_b N_r elements, the columns between the row kernels (as
  * gw_chi0_omega_pw, of the supercell) and the tensor-core operands.
- * GW_ERR_UNSUPPORTED where two expanded supercell rows do not fit a
- * thread-block cluster (supercells beyond 36^3, GW_FP64 at 36^3).  Synchronises
- * the stream once per k (the norm check). */
+ * GW_ERR_UNSUPPORTED beyond the sizes of gw_chi0_omega_pw for the supercell
+ * (beyond 36^3, GW_FP64 at 36^3).  Synchronises the stream once per k (the norm
+ * check). */
 gw_status gw_chi0_omega_kmesh_pw(gw_ctx* ctx, const gw_grid* grid, const int* nk, int n_b, int n_occ,
                                  const void* psi_k, const double* eps_k_h, double mu, int n,
                                  const double* tau_h, const double* C_h, int n_chi, const int32_t* gvec_h,

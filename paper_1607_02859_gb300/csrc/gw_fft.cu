@@ -113,8 +113,8 @@ struct RowCfg {
 // pencils, then its i1 planes, and of the i1 pass the planes up to the last one
 // read.
 // That is 0.44 of a whole row's pencils at 24^3 with n_chi = 4097; the rows of one
-// tau went from 790 to 560 us there (scalar loads for the odd n_chi before), from
-// 250 to 172 us at 20^3 with n_chi = 1536.  Bound by instruction issue.
+// tau went from 800 to 470 us there (scalar loads for the odd n_chi before), from
+// 250 to 150 us at 20^3 with n_chi = 1536.  Bound by instruction issue.
 template <typename T, int N1, int N2, int N3, int MODE, bool VI, bool VO, bool LOW>
 __global__ void __launch_bounds__(RowCfg<T, N1, N2, N3>::TH, RowCfg<T, N1, N2, N3>::MINB)
     row_fft_kernel(const typename cpx<T>::t* __restrict__ a, long lda, typename cpx<T>::t* __restrict__ out, long ldo,
@@ -279,9 +279,10 @@ struct PlaneCfg {
   static constexpr int S2 = N3 % 2 == 0 ? N3 + 1 : N3;
   static constexpr int S1 = N2 * S2;
   static constexpr int PL = N2 * N3;
-  static constexpr int PP = N2 >= 40 ? 2 : 4;                      // planes per CTA
+  // planes per CTA: four of 36 x 36 are 43 KB, so that MINB CTAs fit an SM; of 48 x 48, 75 KB, only two
+  static constexpr int PP = N2 >= 40 ? 2 : 4;
   static constexpr int TH = (PP * N2 + 31) / 32 * 32;              // one pencil per thread and pass
-  static constexpr int MINB = sizeof(T) == 4 ? (N2 >= 30 ? 4 : 6) : 2;
+  static constexpr int MINB = sizeof(T) == 4 ? (N2 >= 30 ? 4 : 6) : 2;   // a 36-point pencil takes 72 of 100 registers
   static constexpr size_t bytes = (size_t)PP * S1 * sizeof(C);
   // threads and CTAs per SM of the line kernels (forward, backward)
   static constexpr int LF = sizeof(T) == 4 ? 160 : 128, LFB = sizeof(T) == 4 ? 3 : 2;
@@ -501,6 +502,8 @@ template <typename T, int N1, int N2, int N3>
 struct PwPlane {
   using C = typename cpx<T>::t;
   using R = PlaneCfg<T, N1, N2, N3>;
+  // two rows of as many planes as leave MINB CTAs of registers and shared memory on an SM; at 36^3, 2 tau,
+  // three CTAs take 32.3 ms, one plane per CTA 35.6, as here 30.5
   static constexpr int PP = N2 >= 30 ? 2 : 4;
   static constexpr int TH = (2 * PP * (N2 > N3 ? N2 : N3) + 31) / 32 * 32;   // one pencil of the two rows per thread
   static constexpr int MINB = sizeof(T) == 4 ? (N2 >= 40 ? 2 : N2 >= 30 ? 4 : 3) : 1;
@@ -603,7 +606,8 @@ struct PwRow {
     const size_t in = 2 * (size_t)((n_pw + CL - 1) / CL), out = (size_t)((n_chi + CL - 1) / CL);
     return in > out ? in : out;
   }
-  // the sizes the plane-wave rows take: two expanded rows and their slices in a cluster's shared memory
+  // the sizes that the plane-wave route takes, chi and self-energy alike: two expanded rows and their
+  // slices in a cluster's shared memory (chi's own row kernels use no cluster)
   static size_t smem(int n_pw, int n_chi) { return 2 * plane_bytes(CL) + slice_elems(n_pw, n_chi) * sizeof(C); }
   // row_pw_sigma_kernel: [T_occ | T_unocc | W~] slices in, hu and ho out over the last two
   static size_t sig_smem(int n_pw, int n_chi) {
@@ -768,8 +772,10 @@ struct ColPlane {
 // Towards the G set (DIR -1) only the (i2, i3) rows that the set touches are
 // written (the i1 pass reads no others) and the i2 pass visits the set's i3;
 // from it (DIR +1) only those rows are read (the others are zero) and the i3
-// pass visits the set's i2.  HBM bounds it: one pass at 36^3, 8192 columns, takes
-// 1.29 ms (3.3 TB/s); with all rows and one 16-column CTA per SM it took 2.28 ms.
+// pass visits the set's i2.  The latency of its loads bounds it, with 18 warps on
+// an SM (of 12.3 cycles between a warp's issues 5.1 wait for memory; shared-memory
+// pipe 63%, DRAM 42%, issue 36%): one pass at 36^3, 8192 columns, takes 1.29 ms
+// (3.3 TB/s); with all rows and one 16-column CTA per SM it took 2.28 ms.
 template <typename T, int N1, int N2, int N3, int DIR, bool PAIRS>
 __global__ void __launch_bounds__(ColPlane<T, N2, N3>::TH, ColPlane<T, N2, N3>::MINB)
     col_plane_kernel(typename cpx<T>::t* __restrict__ buf, long ld, int ncols, T scale, const int* __restrict__ inv) {
@@ -1439,8 +1445,8 @@ size_t row_pw_work(const GridInfo& g, gw_prec prec, int pw_cols, int chi_cols) {
 
 gw_status check_row_pw(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int n_pw, int n_chi) {
   GW_DISPATCH(prec, g, rc = O::row_pw_ok(n_pw, n_chi) ? GW_OK : fail(ctx, GW_ERR_UNSUPPORTED,
-                                                                     "plane-wave chi rows: this grid, precision and "
-                                                                     "G sets do not fit a thread-block cluster"))
+                                                                     "plane-wave chi rows: grid, precision and G sets "
+                                                                     "beyond the sizes of the plane-wave route"))
 }
 
 gw_status launch_row_pw_sigma(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* tu, const void* to, long ldt,

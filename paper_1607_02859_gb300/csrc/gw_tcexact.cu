@@ -70,7 +70,7 @@ constexpr int EPI_WARPS = 8;                     // two per tensor-memory lane q
 constexpr int EPI_BYTES = EPI_WARPS * 32 * EPI_CPX * 8;   // per epilogue warp: 32 rows x 16 complex (FP32)
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 256;
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
-constexpr int kGroupM = 4;                       // pairs' row tiles per group of the tile order
+constexpr int kGroupM = 4;                       // pairs' row tiles per group of the tile order (1024 rows)
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
 
 // tile t of the persistent order -> (pair's row tile, column tile): kGroupM row tiles
