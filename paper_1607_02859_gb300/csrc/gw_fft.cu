@@ -584,6 +584,119 @@ __global__ void __launch_bounds__(PwPlane<T, N1, N2, N3>::TH, PwPlane<T, N1, N2,
   plane_gather<N2, N3, PP>(gx, sa, S1, S2, np, [&](int p, int e, C v) { px[p * tx_plane + e] = v; });
 }
 
+// Small grids: both rows of a grid point in one CTA's shared memory and the whole of
+// the above in one launch, while two or three such CTAs share an SM (kPwOneMax: up to
+// 16^3 in FP32, 12^3 in FP64).  The three kernels are bound by their launches and the
+// columns' way through L2 there: 6 tau of 16^3 with 600 plane waves and 2000 G vectors
+// took them 1.41 ms, this one 0.61 (a CTA per whole row 1.16); 12^3, 500 and 1728, FP32
+// 0.47 and 0.17 (0.29), FP64 2.88 and 2.34 (3.68).  At 20^3, where two rows leave one
+// CTA per SM, that whole-row form took 5.8 ms and the three kernels take 4.1.
+template <typename T, int N1, int N2, int N3>
+struct PwOne {
+  using L = RowLayout<N1, N2, N3>;
+  static constexpr size_t bytes = 2 * (size_t)L::TOT * sizeof(typename cpx<T>::t);
+  static constexpr bool use = bytes <= kPwOneMax;
+  static constexpr int PEN = N1 * (N2 > N3 ? N2 : N3);             // pencils of a pass over one row
+  static constexpr int TH = PEN >= 256 ? 256 : (PEN + 31) / 32 * 32;
+};
+
+template <typename T, int N1, int N2, int N3>
+__global__ void __launch_bounds__(PwOne<T, N1, N2, N3>::TH, 2)
+    row_pw_one_kernel(const typename cpx<T>::t* __restrict__ ta, const typename cpx<T>::t* __restrict__ tb, long lda,
+                      typename cpx<T>::t* __restrict__ out, long ldo, const int* __restrict__ inv_pw,
+                      const int* __restrict__ inv_chi, int n_chi, T scale, int low) {
+  using C = typename cpx<T>::t;
+  using L = RowLayout<N1, N2, N3>;
+  constexpr int PL = N2 * N3, S1 = L::S1, S2 = L::S2, TH = PwOne<T, N1, N2, N3>::TH;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* sa = reinterpret_cast<C*>(smem_raw);                          // [N1][N2][S2] a, then x
+  C* sb = sa + L::TOT;                                             // b, then the row of out
+  const long row = blockIdx.x;
+  const int last = low_last_fwd(low, row, N1 * PL), i1m = last / PL + 1;   // planes with an element R' <= r
+  const SetLists<N1, N2, N3> gp(inv_pw), gx(inv_chi);
+  auto pencils = [&](auto f) {                                     // the (i1, i2) pencils of both rows that hold plane waves
+    const int n = i1m * gp.n2;
+    for (int t = threadIdx.x; t < 2 * n; t += TH) {
+      const int e = t >= n ? t - n : t;
+      f((t >= n ? sb : sa) + e / gp.n2 * S1 + __ldg(gp.l2 + e % gp.n2) * S2);
+    }
+  };
+  pencils([](C* s) {
+#pragma unroll
+    for (int k = 0; k < N3; ++k) s[k] = C{};
+  });
+  __syncthreads();
+  for (int t = threadIdx.x; t < 2 * gp.n23; t += TH) {             // i1 (-i) of the set's columns
+    const bool second = t >= gp.n23;
+    const int q = __ldg(gp.l23 + (second ? t - gp.n23 : t));
+    const C* src = (second ? tb : ta) + row * lda;
+    C x[N1];
+#pragma unroll
+    for (int i1 = 0; i1 < N1; ++i1) {
+      const int j = __ldg(inv_pw + i1 * PL + q);
+      x[i1] = mk(T(0), T(0));
+      if (j >= 0) x[i1] = __ldg(src + j);
+    }
+    RegFFT<N1, -1>::run(x);
+    C* s = (second ? sb : sa) + q / N3 * S2 + q % N3;
+#pragma unroll
+    for (int i1 = 0; i1 < N1; ++i1)
+      if (i1 < i1m) s[i1 * S1] = x[i1];
+  }
+  __syncthreads();
+  pencils([](C* s) { plane_pencil<N3, -1>(s, ~0ull); });
+  __syncthreads();
+  {
+    // i2 of both rows, the product of Eq. chi_rr and i2 of x, a column per thread
+    const unsigned long long m2 = set_mask(gp.l2, gp.n2), mx = set_mask(gx.l2, gx.n2);
+    for (int e = threadIdx.x; e < i1m * N3; e += TH) {
+      const int i1 = e / N3, i3 = e - i1 * N3, o = i1 * S1 + i3, r0 = i1 * PL + i3;
+      C x[N2], y[N2];
+#pragma unroll
+      for (int k = 0; k < N2; ++k) {
+        x[k] = y[k] = mk(T(0), T(0));
+        if (m2 >> k & 1) {
+          x[k] = sa[o + k * S2];
+          y[k] = sb[o + k * S2];
+        }
+      }
+      RegFFT<N2, -1>::run(x);
+      RegFFT<N2, -1>::run(y);
+#pragma unroll
+      for (int k = 0; k < N2; ++k) {
+        const int r = r0 + k * N3;
+        if (r <= last) x[k] = cscale(cmulc(x[k], y[k]), low >= 0 && r == last ? scale * T(0.5) : scale);
+        else x[k] = mk(T(0), T(0));
+      }
+      RegFFT<N2, +1>::run(x);
+#pragma unroll
+      for (int k = 0; k < N2; ++k)
+        if (mx >> k & 1) sa[o + k * S2] = x[k];
+    }
+  }
+  __syncthreads();
+  {
+    const unsigned long long m3 = set_mask(gx.l3, gx.n3);
+    for (int e = threadIdx.x; e < i1m * gx.n2; e += TH)
+      plane_pencil<N3, +1>(sa + e / gx.n2 * S1 + __ldg(gx.l2 + e % gx.n2) * S2, m3);
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < gx.n23; e += TH) {                 // i1 (+i) of chi's columns, in order through sb
+    const int q = __ldg(gx.l23 + e), o = q / N3 * S2 + q % N3;
+    C x[N1];
+#pragma unroll
+    for (int i1 = 0; i1 < N1; ++i1) x[i1] = i1 < i1m ? sa[o + i1 * S1] : mk(T(0), T(0));
+    RegFFT<N1, +1>::run(x);
+#pragma unroll
+    for (int i1 = 0; i1 < N1; ++i1) {
+      const int j = __ldg(inv_chi + i1 * PL + q);
+      if (j >= 0) sb[j] = x[i1];
+    }
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < n_chi; j += TH) out[row * ldo + j] = sb[j];
+}
+
 // Rows too long for one CTA in the plane-wave self-energy: the CL CTAs of a
 // cluster share a row's planes and columns through distributed shared memory.
 template <typename T, int N1, int N2, int N3>
@@ -1263,34 +1376,46 @@ struct GridOps {
                           int n_rows, double scale, cudaStream_t st, int low, void* work) {
     if (!row_pw_ok(n_pw, n_chi))
       return fail(ctx, GW_ERR_UNSUPPORTED, "plane-wave chi rows: no cluster split fits this grid and precision");
-    using PP = PwPlane<T, N1, N2, N3>;
-    auto kernel = row_pw_plane_kernel<T, N1, N2, N3>;
-    gw_status s = set_smem(ctx, kernel, PP::bytes);
-    if (s) return s;
-    const int ch = std::min(n_rows, kPwChunk);
-    const long tp = pw_cols, tr = (long)N1 * tp, xp = chi_cols, xr = (long)N1 * xp;
-    C* ta = static_cast<C*>(work);
-    C* tb = ta + ch * tr;
-    C* tx = tb + ch * tr;
     const double nr = (double)N1 * N2 * N3;
-    for (int r = 0; r < n_rows; r += ch) {
-      const int rows = std::min(ch, n_rows - r), lo = low >= 0 ? low + r : -1;
-      // ALU work: three transforms of N_r points (5 N log2 N each) and the product per row, booked on the planes
-      const C* pa = static_cast<const C*>(a) + (long)r * lda;
-      const C* pb = static_cast<const C*>(b) + (long)r * lda;
-      if ((s = line_bwd(ctx, pa, lda, ta, tr, tp, inv_pw, n_pw, rows, lo, true, 0.0, KF_ROW_PW, st))) return s;
-      if ((s = line_bwd(ctx, pb, lda, tb, tr, tp, inv_pw, n_pw, rows, lo, true, 0.0, KF_ROW_PW, st))) return s;
-      {
-        const dim3 grid((row_planes(lo, rows, false) + PP::PP - 1) / PP::PP, rows);
-        KTimer kt(ctx, KF_ROW_PW, (double)rows * (3.0 * 5.0 * nr * std::log2(nr) + 6.0 * nr), st);
-        kernel<<<grid, PP::TH, PP::bytes, st>>>(ta, tb, tr, tp, tx, xr, xp, inv_pw, inv_chi, (T)scale, lo);
-        if ((s = launch_check(ctx, "row_pw_plane_kernel"))) return s;
+    // ALU work: three transforms of N_r points (5 N log2 N each) and the product per row
+    auto flops = [&](int rows) { return (double)rows * (3.0 * 5.0 * nr * std::log2(nr) + 6.0 * nr); };
+    using P1 = PwOne<T, N1, N2, N3>;
+    if constexpr (P1::use) {
+      auto one = row_pw_one_kernel<T, N1, N2, N3>;
+      gw_status s = set_smem(ctx, one, P1::bytes);
+      if (s) return s;
+      KTimer kt(ctx, KF_ROW_PW, flops(n_rows), st);
+      one<<<n_rows, P1::TH, P1::bytes, st>>>(static_cast<const C*>(a), static_cast<const C*>(b), lda,
+                                             static_cast<C*>(out), ldo, inv_pw, inv_chi, n_chi, (T)scale, low);
+      return launch_check(ctx, "row_pw_one_kernel");
+    } else {
+      using PP = PwPlane<T, N1, N2, N3>;
+      auto kernel = row_pw_plane_kernel<T, N1, N2, N3>;
+      gw_status s = set_smem(ctx, kernel, PP::bytes);
+      if (s) return s;
+      const int ch = std::min(n_rows, kPwChunk);
+      const long tp = pw_cols, tr = (long)N1 * tp, xp = chi_cols, xr = (long)N1 * xp;
+      C* ta = static_cast<C*>(work);
+      C* tb = ta + ch * tr;
+      C* tx = tb + ch * tr;
+      for (int r = 0; r < n_rows; r += ch) {
+        const int rows = std::min(ch, n_rows - r), lo = low >= 0 ? low + r : -1;
+        const C* pa = static_cast<const C*>(a) + (long)r * lda;
+        const C* pb = static_cast<const C*>(b) + (long)r * lda;
+        if ((s = line_bwd(ctx, pa, lda, ta, tr, tp, inv_pw, n_pw, rows, lo, true, 0.0, KF_ROW_PW, st))) return s;
+        if ((s = line_bwd(ctx, pb, lda, tb, tr, tp, inv_pw, n_pw, rows, lo, true, 0.0, KF_ROW_PW, st))) return s;
+        {
+          const dim3 grid((row_planes(lo, rows, false) + PP::PP - 1) / PP::PP, rows);
+          KTimer kt(ctx, KF_ROW_PW, flops(rows), st);             // booked on the planes
+          kernel<<<grid, PP::TH, PP::bytes, st>>>(ta, tb, tr, tp, tx, xr, xp, inv_pw, inv_chi, (T)scale, lo);
+          if ((s = launch_check(ctx, "row_pw_plane_kernel"))) return s;
+        }
+        if ((s = line_fwd(ctx, tx, xr, xp, static_cast<C*>(out) + (long)r * ldo, ldo, inv_chi, n_chi, rows, lo, 0.0,
+                          KF_ROW_PW, st)))
+          return s;
       }
-      if ((s = line_fwd(ctx, tx, xr, xp, static_cast<C*>(out) + (long)r * ldo, ldo, inv_chi, n_chi, rows, lo, 0.0,
-                        KF_ROW_PW, st)))
-        return s;
+      return GW_OK;
     }
-    return GW_OK;
   }
   static bool row_pw_sigma_ok(int n_pw, int n_chi) {
     using PR = PwRow<T, N1, N2, N3>;
@@ -1431,6 +1556,13 @@ gw_status launch_row_fft(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int mode,
   GW_DISPATCH(prec, g, rc = O::row(ctx, mode, a, lda, out, ldo, map, n_chi, n_rows, scale, st, inv, tmp, low))
 }
 
+// shared memory of one row (RowLayout)
+static size_t row_smem(const GridInfo& g, gw_prec prec) {
+  return (size_t)g.n1 * g.n2 * (g.n3 % 2 == 0 ? g.n3 + 1 : g.n3) * csize(prec);
+}
+
+bool row_two_pass(const GridInfo& g, gw_prec prec) { return row_smem(g, prec) > kRowSmemMax; }
+
 gw_status launch_row_pw_chi(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* a, const void* b, long lda,
                             void* out, long ldo, const int* inv_pw, int n_pw, int pw_cols, const int* inv_chi,
                             int n_chi, int chi_cols, int n_rows, double scale, void* work, cudaStream_t st, int low) {
@@ -1440,6 +1572,7 @@ gw_status launch_row_pw_chi(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const 
 }
 
 size_t row_pw_work(const GridInfo& g, gw_prec prec, int pw_cols, int chi_cols) {
+  if (2 * row_smem(g, prec) <= kPwOneMax) return 0;               // one CTA per row
   return (size_t)std::min(g.nr, kPwChunk) * g.n1 * (2 * (size_t)pw_cols + chi_cols) * csize(prec);
 }
 
@@ -1463,11 +1596,6 @@ gw_status check_row_pw_sigma(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int n
                                                                            "plane-wave Sigma rows: this grid, "
                                                                            "precision and G sets do not fit a "
                                                                            "thread-block cluster"))
-}
-
-bool row_two_pass(const GridInfo& g, gw_prec prec) {
-  const size_t s2 = g.n3 % 2 == 0 ? g.n3 + 1 : g.n3;
-  return (size_t)g.n1 * g.n2 * s2 * csize(prec) > kRowSmemMax;
 }
 
 gw_status launch_col_plane(gw_ctx* ctx, const GridInfo& g, gw_prec prec, int dir, void* buf, long ld, int ncols,

@@ -35,7 +35,9 @@ bool row_two_pass(const GridInfo& g, gw_prec prec);
 // pw_cols, chi_cols: the columns that the two sets touch (set_columns); work: row_pw_work
 // bytes, the columns of a chunk of kPwChunk rows (95 MB for the triangle at 36^3 with
 // 4224 plane waves: it stays in L2).
+// Small grids (two rows within kPwOneMax of shared memory) take one kernel and no columns.
 constexpr int kPwChunk = 1024;
+constexpr size_t kPwOneMax = 72 * 1024;
 size_t row_pw_work(const GridInfo& g, gw_prec prec, int pw_cols, int chi_cols);
 gw_status launch_row_pw_chi(gw_ctx* ctx, const GridInfo& g, gw_prec prec, const void* a, const void* b, long lda,
                             void* out, long ldo, const int* inv_pw, int n_pw, int pw_cols, const int* inv_chi,
