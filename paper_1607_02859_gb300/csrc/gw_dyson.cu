@@ -67,10 +67,12 @@ __device__ __forceinline__ double inv_sqrt(double x) { return 1.0 / sqrt(x); }
 // live in registers, a 4 x 4 cyclic block each per thread of a 16 x 16 grid,
 // and advance together: with the raw column j of the factor and the raw row j
 // of the inverse published in (double-buffered) shared memory behind one
-// barrier, every thread scales them by 1 / L_jj itself and applies
+// barrier, together with 1 / L_jj from the thread that holds the pivot (a square
+// root and a division of every thread would cost more FP64 issue than the updates of
+// a small block), every thread scales them itself and applies
 //   S -= l l^H,   X[i > j] -= l_i x_j.
-// Only the 16-wide register blocks that column j touches are updated.  The
-// inverse turns the triangular solves of the panel into products (below): one
+// Only the 16-wide register blocks that column j touches are updated, of a short
+// block only those that hold its rows.  The inverse turns the triangular solves of the panel into products (below): one
 // thread per row of a solve walked 64 columns serially (68 us a panel, and 74 us
 // for the inverse's rows, whatever the size).  Screening 12 frequencies of 1536
 // G vectors (fp16x3) went from 7.02 to 3.96 ms, 2 x 8192 with refinement from
@@ -82,6 +84,7 @@ __global__ void __launch_bounds__(256) potrf_inv_kernel(typename cpx<T>::t* A, l
   using C = typename cpx<T>::t;
   static_assert(kNB == 64, "4 x 4 blocks of a 16 x 16 thread grid");
   __shared__ C col[2][kNB], row[2][kNB];
+  __shared__ T piv[2];                         // 1 / L_jj
   A += blockIdx.z * s_a;
   P += blockIdx.z * s_p;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -107,11 +110,16 @@ __global__ void __launch_bounds__(256) potrf_inv_kernel(typename cpx<T>::t* A, l
       if (ty == jj)
 #pragma unroll
         for (int b = 0; b <= jb; ++b) row[buf][tx + 16 * b] = X[jb][b];
+      T d = T(0);
+      bool bad = false;
+      if (tx == jj && ty == jj) {
+        d = S[jb][jb].x;                       // eps~_jj - 1 after the updates
+        bad = !(T(1) + d > T(0));
+        if (bad) d = T(0);
+        piv[buf] = inv_sqrt(T(1) + d);
+      }
       __syncthreads();
-      T d = col[buf][j].x;                     // eps~_jj - 1 after the updates
-      const bool bad = !(T(1) + d > T(0));
-      if (bad) d = T(0);
-      const T inv = inv_sqrt(T(1) + d);
+      const T inv = piv[buf];
       C l[4], lc[4], xr[4];
 #pragma unroll
       for (int a = jb; a < 4; ++a) {
@@ -139,6 +147,7 @@ __global__ void __launch_bounds__(256) potrf_inv_kernel(typename cpx<T>::t* A, l
       if (tx <= jj) lc[jb] = mk(T(0), T(0));
 #pragma unroll
       for (int a = jb; a < 4; ++a) {
+        if (16 * a >= kb) break;                // rows past a short block
         const C nl = mk(-l[a].x, -l[a].y);
 #pragma unroll
         for (int b = jb; b <= a; ++b) S[a][b] = cfmac(nl, lc[b], S[a][b]);
