@@ -75,8 +75,8 @@ __device__ __forceinline__ double inv_sqrt(double x) { return 1.0 / sqrt(x); }
 // block only those that hold its rows.  The inverse turns the triangular solves of the panel into products (below): one
 // thread per row of a solve walked 64 columns serially (68 us a panel, and 74 us
 // for the inverse's rows, whatever the size).  Screening 12 frequencies of 1536
-// G vectors (fp16x3) went from 7.02 to 3.96 ms, 2 x 8192 with refinement from
-// 185 to 170 ms; FP64, 4 x 1024, from 41.8 to 32.1 ms, FP32, 8 x 1536, from 8.7 to 5.3.
+// G vectors (fp16x3) went from 7.02 to 3.79 ms, 2 x 8192 with refinement from
+// 185 to 170 ms; FP64, 4 x 513, from 18.1 to 13.1 ms, FP32, 8 x 300, from 1.05 to 0.46.
 template <typename T>
 __global__ void __launch_bounds__(256) potrf_inv_kernel(typename cpx<T>::t* A, long lda, long s_a,
                                                         typename cpx<T>::t* P, long ldp, long s_p, int kb, int* flag,
@@ -170,55 +170,111 @@ __global__ void __launch_bounds__(256) potrf_inv_kernel(typename cpx<T>::t* A, l
 
 constexpr int kPR = 32;     // rows (columns) of a panel product per CTA
 
-// Shared memory of the two panel products: the inverted diagonal block and the tile.
+// Shared memory of the two panel products: the inverted diagonal block and the tile;
+// for the right one also the diagonal block itself and the product.
 template <typename T>
-constexpr size_t panel_smem() {
-  return sizeof(typename cpx<T>::t) * (kNB * (kNB + 1) + kPR * (kNB + 1));
+constexpr size_t panel_smem(bool right) {
+  return (right ? 2 : 1) * sizeof(typename cpx<T>::t) * (kNB * (kNB + 1) + kPR * (kNB + 1));
 }
 
-// Rows below the diagonal block: L21 = A21 L11^{-H} = A21 + A21 P11^H, in place,
-// kPR rows per CTA and 2 x 4 outputs per thread; P11 is lower triangular, so
-// the sum of each group of 16 columns stops at its last column.
+// R x W elements of a row-major matrix on their way from memory, all in flight at
+// once (256 threads; 0 outside): in a loop of loads and stores each of them was waited
+// for, 13 of the 18 us of a panel.
+template <int R, int W, typename C>
+struct Tile {
+  static constexpr int N = R * W / 256, RQ = 256 / W;
+  C v[N];
+  template <typename In>
+  __device__ __forceinline__ void load(const C* src, long ld, In in) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const int i = RQ * q + (int)threadIdx.x / W, c = threadIdx.x % W;
+      v[q] = C{};
+      if (in(i, c)) v[q] = src[(long)i * ld + c];
+    }
+  }
+  __device__ __forceinline__ void store(C* dst, int ld) const {
+#pragma unroll
+    for (int q = 0; q < N; ++q) dst[(RQ * q + (int)threadIdx.x / W) * ld + threadIdx.x % W] = v[q];
+  }
+};
+
+// Rows below the diagonal block: L21 = A21 L11^{-H}, in place, kPR rows per CTA and
+// 2 x 4 outputs per thread, with P11 = L11^{-1} - 1 and K11 = L11 - 1 lower triangular,
+// so that the sum of each group of 16 columns stops at its last column:
+//   Y = A21 + A21 P11^H,   R = A21 - Y - Y K11^H,   L21 = Y + R + R P11^H.
+// The product alone leaves a residual of cond(L11) roundings of A21, which the updates
+// of all later columns take up; the correction brings it back to that of a solve.
+// eps~ with a largest eigenvalue of 1e5, 700 G vectors: W~ off by 3.1e-3 in FP32 with the
+// product, by 2.0e-4 with a solve of every row (FP64 6.3e-12 and 2.9e-12).
 template <typename T>
-__global__ void __launch_bounds__(256) panel_right_kernel(typename cpx<T>::t* A, long lda, long s_a,
-                                                          const typename cpx<T>::t* P, long ldp, long s_p, int kb,
-                                                          int rows) {
+__global__ void __launch_bounds__(256) panel_right_kernel(typename cpx<T>::t* A, const typename cpx<T>::t* L, long lda,
+                                                          long s_a, const typename cpx<T>::t* P, long ldp, long s_p,
+                                                          int kb, int rows) {
   using C = typename cpx<T>::t;
+  constexpr int LD = kNB + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* Ps = reinterpret_cast<C*>(smem_raw);          // [kNB][kNB + 1]
-  C* As = Ps + kNB * (kNB + 1);                     // [kPR][kNB + 1]
+  C* Ps = reinterpret_cast<C*>(smem_raw);          // [kNB][LD]
+  C* Ks = Ps + kNB * LD;                            // [kNB][LD]
+  C* As = Ks + kNB * LD;                            // [kPR][LD] A21, then R
+  C* Ys = As + kPR * LD;                            // [kPR][LD]
   A += blockIdx.z * s_a;
+  L += blockIdx.z * s_a;
   P += blockIdx.z * s_p;
   const int r0 = blockIdx.x * kPR;
-  for (int e = threadIdx.x; e < kNB * kNB; e += 256) {
-    const int i = e / kNB, c = e % kNB;
-    Ps[i * (kNB + 1) + c] = i < kb && c <= i ? P[(long)i * ldp + c] : mk(T(0), T(0));
-  }
-  for (int e = threadIdx.x; e < kPR * kNB; e += 256) {
-    const int i = e / kNB, c = e % kNB;
-    As[i * (kNB + 1) + c] = r0 + i < rows && c < kb ? A[(long)(r0 + i) * lda + c] : mk(T(0), T(0));
+  {
+    auto lower = [&](int i, int c) { return i < kb && c <= i; };
+    Tile<kNB, kNB, C> tp, tk;
+    Tile<kPR, kNB, C> ta;
+    tp.load(P, ldp, lower);
+    tk.load(L, lda, lower);
+    ta.load(A + (long)r0 * lda, lda, [&](int i, int c) { return r0 + i < rows && c < kb; });
+    tp.store(Ps, LD);
+    tk.store(Ks, LD);
+    ta.store(As, LD);
   }
   __syncthreads();
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  C acc[2][4];
+  C acc[2][4], y[2][4];
+  auto times = [&](const C* X, const C* W) {       // acc = this thread's elements of X W^H
 #pragma unroll
-  for (int b = 0; b < 4; ++b)
+    for (int b = 0; b < 4; ++b)
 #pragma unroll
-    for (int a = 0; a < 2; ++a) acc[a][b] = mk(T(0), T(0));
+      for (int a = 0; a < 2; ++a) acc[a][b] = mk(T(0), T(0));
 #pragma unroll
-  for (int pb = 0; pb < 4; ++pb) {
+    for (int pb = 0; pb < 4; ++pb) {
 #pragma unroll 4
-    for (int pp = 0; pp < 16; ++pp) {
-      const int p = 16 * pb + pp;
-      const C a0 = As[ty * (kNB + 1) + p], a1 = As[(ty + 16) * (kNB + 1) + p];
+      for (int pp = 0; pp < 16; ++pp) {
+        const int p = 16 * pb + pp;
+        const C a0 = X[ty * LD + p], a1 = X[(ty + 16) * LD + p];
 #pragma unroll
-      for (int b = pb; b < 4; ++b) {
-        const C w = Ps[(tx + 16 * b) * (kNB + 1) + p];
-        acc[0][b] = cfmac(a0, w, acc[0][b]);
-        acc[1][b] = cfmac(a1, w, acc[1][b]);
+        for (int b = pb; b < 4; ++b) {
+          const C w = W[(tx + 16 * b) * LD + p];
+          acc[0][b] = cfmac(a0, w, acc[0][b]);
+          acc[1][b] = cfmac(a1, w, acc[1][b]);
+        }
       }
     }
-  }
+  };
+  times(As, Ps);
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int at = (ty + 16 * a) * LD + tx + 16 * b;
+      y[a][b] = Ys[at] = cadd(As[at], acc[a][b]);
+    }
+  __syncthreads();
+  times(Ys, Ks);
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      C& r = As[(ty + 16 * a) * LD + tx + 16 * b];
+      r = csub(csub(r, y[a][b]), acc[a][b]);
+    }
+  __syncthreads();
+  times(As, Ps);
 #pragma unroll
   for (int a = 0; a < 2; ++a) {
     const int i = ty + 16 * a;
@@ -226,7 +282,7 @@ __global__ void __launch_bounds__(256) panel_right_kernel(typename cpx<T>::t* A,
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const int c = tx + 16 * b;
-      if (c < kb) A[(long)(r0 + i) * lda + c] = cadd(As[i * (kNB + 1) + c], acc[a][b]);
+      if (c < kb) A[(long)(r0 + i) * lda + c] = cadd(y[a][b], cadd(As[i * LD + c], acc[a][b]));
     }
   }
 }
@@ -260,13 +316,13 @@ __global__ void __launch_bounds__(256) panel_left_kernel(const typename cpx<T>::
   P += blockIdx.z * s_p;
   Y += blockIdx.z * s_p;
   const int c0 = blockIdx.x * kPR;
-  for (int e = threadIdx.x; e < kNB * kNB; e += 256) {
-    const int i = e / kNB, c = e % kNB;
-    Ps[i * (kNB + 1) + c] = i < kb && c <= i ? P[(long)i * ldp + c] : mk(T(0), T(0));
-  }
-  for (int e = threadIdx.x; e < kNB * kPR; e += 256) {
-    const int i = e / kPR, c = e % kPR;
-    Ys[i * kPR + c] = i < kb && c0 + c < ncols ? Y[(long)i * ldp + c0 + c] : mk(T(0), T(0));
+  {
+    Tile<kNB, kNB, C> tp;
+    Tile<kNB, kPR, C> ty;
+    tp.load(P, ldp, [&](int i, int c) { return i < kb && c <= i; });
+    ty.load(Y + c0, ldp, [&](int i, int c) { return i < kb && c0 + c < ncols; });
+    tp.store(Ps, kNB + 1);
+    ty.store(Ys, kPR);
   }
   __syncthreads();
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -421,16 +477,14 @@ struct Batch {
 
 template <typename T>
 static gw_status set_attrs(gw_ctx* ctx) {
-  gw_status rc = GW_OK;
-  if (panel_smem<T>() > 48 * 1024) {
-    rc = cuda_check(ctx, cudaFuncSetAttribute(panel_right_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)panel_smem<T>()),
+  gw_status rc = cuda_check(ctx, cudaFuncSetAttribute(panel_right_kernel<T>,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      (int)panel_smem<T>(true)),
+                            "cudaFuncSetAttribute");
+  if (!rc && panel_smem<T>(false) > 48 * 1024)
+    rc = cuda_check(ctx, cudaFuncSetAttribute(panel_left_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)panel_smem<T>(false)),
                     "cudaFuncSetAttribute");
-    if (!rc)
-      rc = cuda_check(ctx, cudaFuncSetAttribute(panel_left_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)panel_smem<T>()),
-                      "cudaFuncSetAttribute");
-  }
   return rc;
 }
 
@@ -452,8 +506,8 @@ static gw_status chol_simt(gw_ctx* ctx, gw_prec prec, typename cpx<T>::t* a, lon
     if ((rc = launch_check(ctx, "potrf_inv_kernel"))) return rc;
     const int rows = n - k0 - kb;
     if (rows <= 0) break;
-    panel_right_kernel<T><<<dim3((rows + kPR - 1) / kPR, 1, bt.B), 256, panel_smem<T>(), st>>>(
-        a + (long)(k0 + kb) * lda + k0, lda, bt.ms, pii, ldp, bt.ms, kb, rows);
+    panel_right_kernel<T><<<dim3((rows + kPR - 1) / kPR, 1, bt.B), 256, panel_smem<T>(true), st>>>(
+        a + (long)(k0 + kb) * lda + k0, a + (long)k0 * lda + k0, lda, bt.ms, pii, ldp, bt.ms, kb, rows);
     if ((rc = launch_check(ctx, "panel_right_kernel"))) return rc;
     GemmArgs g{};
     g.M = rows;
@@ -490,7 +544,7 @@ static gw_status inv_simt(gw_ctx* ctx, gw_prec prec, const typename cpx<T>::t* L
     const int ncols = k0 + kb, rows = n - k0 - kb;
     const int ctas = (k0 + kPR - 1) / kPR + (rows + kPR - 1) / kPR;
     if (ctas > 0) {
-      panel_left_kernel<T><<<dim3(ctas, 1, bt.B), 256, panel_smem<T>(), st>>>(
+      panel_left_kernel<T><<<dim3(ctas, 1, bt.B), 256, panel_smem<T>(false), st>>>(
           p + (long)k0 * ldp + k0, ldp, bt.ms, p + (long)k0 * ldp, kb, k0, Lm + (long)(k0 + kb) * ldl + k0, ldl, bt.ms,
           p + (long)(k0 + kb) * ldp + k0, rows);
       if ((rc = launch_check(ctx, "panel_left_kernel"))) return rc;
