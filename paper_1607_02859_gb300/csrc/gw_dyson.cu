@@ -148,11 +148,12 @@ __global__ void __launch_bounds__(256) potrf_inv_kernel(typename cpx<T>::t* A, l
 #pragma unroll
       for (int a = jb; a < 4; ++a) {
         if (16 * a >= kb) break;                // rows past a short block
-        const C nl = mk(-l[a].x, -l[a].y);
+        // the product first: one rounding at the size of S per update.  As two multiply-adds onto S
+        // each left W~ 10 to 15% further off.
 #pragma unroll
-        for (int b = jb; b <= a; ++b) S[a][b] = cfmac(nl, lc[b], S[a][b]);
+        for (int b = jb; b <= a; ++b) S[a][b] = csub(S[a][b], cmulc(l[a], lc[b]));
 #pragma unroll
-        for (int b = 0; b <= jb; ++b) X[a][b] = cfma(nl, xr[b], X[a][b]);
+        for (int b = 0; b <= jb; ++b) X[a][b] = csub(X[a][b], cmul(l[a], xr[b]));
       }
     }
   }
